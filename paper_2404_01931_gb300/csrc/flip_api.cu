@@ -402,11 +402,18 @@ void carve(flip_handle* h, Carver& cv) {
         L.x = cv.take<float>(ns);
         L.b = cv.take<float>(ns);
         L.code16 = cv.take<uint16_t>(ns);
-        L.seg = cv.take<int4>((size_t)L.nw * L.ny * L.nz);
+        L.seg = cv.take<unsigned int>((size_t)L.nw * L.ny * L.nz);
         L.nseg = cv.take<unsigned int>(1);
+        const size_t blocks = (size_t)L.nbx * L.nby * L.nbz;
+        L.blk = cv.take<int>(blocks);
+        // 512 threads per block, as many blocks as a blocked level can have
+        L.tab = cv.take<uint4>(
+            512 * std::min(blocks, (size_t)MG_BLK_PER_CTA * (size_t)h->pcg_blocks));
         if (l > 0) {
           L.t = cv.take<uint8_t>(n);
           L.bflag = cv.take<uint8_t>((size_t)L.nbx * L.nby * L.nbz);
+          L.nblk = cv.take<unsigned int>(1);
+          L.x2 = cv.take<float>(ns);
         }
         if (l == 0) {
           m.pa0 = cv.take<float>(ns);

@@ -104,6 +104,8 @@ constexpr int MG_MAX_LEVELS = 12;
 constexpr int MG_COARSE_SWEEPS = 2;   // red-black pairs each way on the coarsest level
 constexpr int MG_CTA_CELLS = 4800;    // the coarsest levels, up to this many cells in
                                       // total, run inside one CTA in shared memory
+constexpr int MG_BLK_PER_CTA = 6;     // a level with at most this many blocks holding
+                                      // fluid per CTA is smoothed blocked (block_pass)
 constexpr float MG_OMEGA = 2.0f;      // over-correction of the coarse correction
 
 // One level of the hierarchy.  The grid-wide levels (l < lgrid) are stored
@@ -136,10 +138,15 @@ struct MgLevel {
   int nbx, nby, nbz;  // 8x8x8 blocks of this level's cells
   uint16_t* code16;   // per slot: the code bits above plus the count of
                       // neighbours inside the grid in bits 8..10
-  int4* seg;          // active segments {row j + ny k, segment in row, j, k}
+  unsigned int* seg;  // active segments (seg_pack: segment in row, j, k)
   unsigned int* nseg; // their number (device)
   uint8_t* bflag;     // levels >= 1: block holds a fluid cell (level 0 reads the
                       // brick fluid counts of the binning)
+  int* blk;           // the blocks holding fluid (bx | by << 8 | bz << 16), for the
+                      // blocked smoothing
+  uint4* tab;         // per block and thread of its tile: the codes of its eight cells
+  unsigned int* nblk; // levels >= 1: their number (level 0: the binning's active bricks)
+  float* x2;          // levels >= 1: the level's x after blocked post-smoothing
 };
 
 struct MgArgs {

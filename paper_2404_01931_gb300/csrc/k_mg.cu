@@ -111,8 +111,16 @@ __device__ __forceinline__ void load_tables(const MgArgs& M) {
 // the copy of level l's slice (nullptr: read the list in global memory) and
 // s_segb[l] the index of its first segment.
 constexpr int SEG_CACHE = 1024;
-__shared__ const int4* s_segc[MG_MAX_LEVELS];
+__shared__ const unsigned int* s_segc[MG_MAX_LEVELS];
 __shared__ int s_segb[MG_MAX_LEVELS];
+
+// Levels whose smoothing runs blocked (block_pass): their number of blocks holding
+// fluid, 0 for the levels swept pass by pass.  s_z0 and s_q0 are the arrays that hold
+// level 0's z after a V-cycle and A p: z in lv[0].x and A p in q0, or the other way
+// round when level 0 is blocked (a blocked post-smoothing writes to a second array).
+__shared__ int s_nblk[MG_MAX_LEVELS];
+__shared__ float* s_z0;
+__shared__ float* s_q0;
 
 // The fields of a colour-split level a pass uses, read once into registers at
 // the start of the pass (the level descriptions live in parameter or shared
@@ -122,14 +130,14 @@ struct SV {
   float* x;
   float* b;
   uint16_t* code;
-  const int4* seg;
+  const unsigned int* seg;
   int seg_base;
   int nx, ny, hx, half, margin, pl;
   float s;
 };
 
 __device__ __forceinline__ SV sview(const MgLevel& L) {
-  const int4* c = s_segc[L.lvl];
+  const unsigned int* c = s_segc[L.lvl];
   return SV{L.x, L.b, L.code16, c ? c : L.seg, c ? s_segb[L.lvl] : 0, L.nx, L.ny, L.hx,
             L.half, L.margin, L.hx * L.ny, L.s};
 }
@@ -141,7 +149,7 @@ struct PV {
 };
 
 __device__ __forceinline__ PV pview(const MgLevel& C) {
-  return PV{C.x, C.split, C.nx, C.ny, C.nz, C.hx, C.half, C.margin};
+  return PV{s_nblk[C.lvl] > 0 ? C.x2 : C.x, C.split, C.nx, C.ny, C.nz, C.hx, C.half, C.margin};
 }
 
 // Runs items first, first + stride, ... < end in batches of U: pre(e, ok)
@@ -186,9 +194,21 @@ struct SCell {
   bool ok;
 };
 
-// Lane 'lane' of colour c in segment sg = {row, segment in row, j, k}.
+// A segment {segment in row, j, k}: 5, 11 and 11 bits (extents up to 2048 cells).
+__device__ __forceinline__ unsigned int seg_pack(int w, int j, int k) {
+  return (unsigned)w | (unsigned)j << 5 | (unsigned)k << 16;
+}
+
+// {row, segment in row, j, k} of a segment of a level with ny rows per plane.
+__device__ __forceinline__ int4 seg_unpack(unsigned int v, int ny) {
+  const int j = (int)((v >> 5) & 2047u), k = (int)(v >> 16);
+  return make_int4(j + ny * k, (int)(v & 31u), j, k);
+}
+
+// Lane 'lane' of colour c in segment v.
 template <class LV>
-__device__ __forceinline__ SCell scell(const LV& L, int4 sg, int c, int lane) {
+__device__ __forceinline__ SCell scell(const LV& L, unsigned int v, int c, int lane) {
+  const int4 sg = seg_unpack(v, L.ny);
   SCell e;
   const int s = sg.y * SEG_SLOTS + lane;
   e.j = sg.z;
@@ -257,7 +277,7 @@ __device__ __forceinline__ PCell pcell(const LV& L, int2 q, unsigned int pair, i
   int sq = q.x + 2 * (int)pair + (lane >> 4);
   const bool seg_ok = sq < q.y;
   if (!seg_ok) sq = q.x;
-  const int4 sg = L.seg[sq - L.seg_base];
+  const int4 sg = seg_unpack(L.seg[sq - L.seg_base], L.ny);
   PCell e;
   e.j = sg.z;
   e.k = sg.w;
@@ -708,7 +728,7 @@ __device__ __noinline__ void restrict_split(const MgLevel& Fl, const MgLevel& Cl
   const int lc = Cl.lvl;
   const Items it = seg_items(Cl, 1);
   for (unsigned int t = it.first; t < it.end; t += PCG_WARPS) {
-    const int4 sg = C.seg[t - C.seg_base];
+    const int4 sg = seg_unpack(C.seg[t - C.seg_base], C.ny);
     const int J = sg.z, K = sg.w;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -763,6 +783,312 @@ __device__ __noinline__ void restrict_split_nat(const MgLevel& Fl, const MgLevel
     if (!(code[c] & CODE_SELF)) continue;
     const int i = c % nx, j = (c / nx) % ny, k = c / (nx * ny);
     cb[c] = restrict_sum(F, fnz, i, j, k);
+  }
+}
+
+// ---------------------------------------------------------------- blocked smoothing
+//
+// On a level with few cells per CTA a half-sweep is all latency: a grid barrier
+// (~1.5 us) and a round trip to L2 for a few hundred cells.  There the whole
+// pre-smoothing with the restriction, and the whole correction with the
+// post-smoothing, run as one pass each: half a CTA takes an 8^3 block with a halo of
+// TILE_H = 4 cells into shared memory and makes all the half-sweeps there, between
+// barriers of its 512 threads, on the cells that the block's own still depend on
+// (those within L1 distance 3, 2, 1, 0 of the block).  Every cell gets gs_sum's
+// operations on the same values in its order, so the results are those of the
+// pass-by-pass form.
+//
+// The tile (16^3 cells) is colour-split like the level: cell (tx, ty, tz) of colour c
+// is slot tx >> 1 of row (ty, tz).  Thread t owns slot s = t & 7 of row y = (t >> 3) & 15
+// in the four planes 4 g .. 4 g + 3, g = t >> 7, of both colours, in registers: as float2
+// A (planes 4 g, 4 g + 2) and B (4 g + 1, 4 g + 3), since the x neighbour that is not the
+// thread's own slot is slot s - 1 in one pair and s + 1 in the other.  Of a cell's six
+// neighbours one along x and all but the group's outermost along z are then in
+// registers; the others come from the shared copies a and b, whole pairs at a time.
+// Cells that are not fluid hold 0, with 0 coefficients, so nothing is masked; cells
+// farther out than a half-sweep's results are needed get values nobody uses.
+// A solve's neighbour codes per thread are laid out once per solve (MgLevel::tab), so a
+// pass loads them, and the cells they mark, without index or bounds logic.
+//
+// Bound by latency: with one block per CTA a pass takes 6.2 us (down) or 6.7 us (up),
+// 1.5 us of it the grid barrier, against four or five passes of 3.3 us each; with two
+// blocks per CTA 9.8 and 6.7 us.  Solve at 64^3 (two dam blocks, mixed) 1.20 -> 0.85 ms,
+// 128^3 dam break (FP32) 1.55 -> 1.28, 256^3 pool (levels 2 and 3 blocked) 6.13 -> 5.92.
+// A first form with 1024 threads per tile, one slot in two planes each and scalar
+// shared loads took 7.1 and 8.8 us, 5.5 us for each further block: issue-bound.
+constexpr int TILE_H = 4;
+constexpr int TILE_W = 8 + 2 * TILE_H;
+constexpr int TILE_THREADS = 512;
+constexpr int TILE_GROUPS = PCG_THREADS / TILE_THREADS;
+// The halo is deep enough for two smoothing pairs.
+constexpr int BLK_MAX_NU = TILE_H / 2;
+static_assert(TILE_W * TILE_W * 2 == TILE_THREADS, "8 slots x 16 rows x 4 plane groups");
+
+struct MgTile {
+  float2 a[2][TILE_THREADS], b[2][TILE_THREADS];
+};
+
+__device__ __forceinline__ MgTile& mg_tile(int group);
+
+__device__ __forceinline__ void tile_sync(int group) {
+  asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(TILE_THREADS) : "memory");
+}
+
+// Distance of a tile coordinate from the block's own [TILE_H, TILE_H + 8).
+__device__ __forceinline__ int tile_dist(int t) {
+  return max(max(TILE_H - t, t - (TILE_H + 7)), 0);
+}
+
+// A thread's place in its tile and in the level.
+struct TilePos {
+  int s, y, g;    // slot, row, plane group
+  int wdist;      // smallest L1 distance of the warp's rows from the block
+  bool own;       // the thread's cells are the block's own
+};
+
+__device__ __forceinline__ TilePos tile_pos() {
+  const int t = threadIdx.x & (TILE_THREADS - 1);
+  TilePos p;
+  p.s = t & 7;
+  p.y = (t >> 3) & 15;
+  p.g = t >> 7;
+  const int y0 = p.y & ~3;  // the warp's rows y0 .. y0 + 3
+  p.wdist = (y0 == 0 || y0 == 12) + (p.g == 0 || p.g == 3);
+  p.own = p.s >= 2 && p.s < 6 && p.y >= 4 && p.y < 12 && (p.g == 1 || p.g == 2);
+  return p;
+}
+
+// The block's first cell, and a thread's first red slot (plane 4 g) in the level.
+struct BlkPos {
+  int b0, b1, b2, gi;
+};
+
+__device__ __forceinline__ BlkPos blk_pos(const SV& v, const TilePos& p, int e) {
+  BlkPos q;
+  q.b0 = (e & 255) * 8;
+  q.b1 = ((e >> 8) & 255) * 8;
+  q.b2 = (e >> 16) * 8;
+  const int j = q.b1 - TILE_H + p.y, k = q.b2 - TILE_H + 4 * p.g;
+  q.gi = v.margin + v.hx * (j + v.ny * k) + (q.b0 >> 1) - TILE_H / 2 + p.s;
+  return q;
+}
+
+// Code of plane z (0..3 in the thread's group), colour c.
+__device__ __forceinline__ unsigned int tab_code(const uint4& w, int z, int c) {
+  const unsigned int v = z == 0 ? w.x : z == 1 ? w.y : z == 2 ? w.z : w.w;
+  return c ? v >> 16 : v & 0xffffu;
+}
+
+__device__ __forceinline__ float& plane(float2& a, float2& b, int z) {
+  return z == 0 ? a.x : z == 1 ? b.x : z == 2 ? a.y : b.y;
+}
+
+// One half-sweep of colour c (compile-time) over the tile: x = inv (sum of the six
+// neighbours) + base.
+template <int c>
+__device__ __forceinline__ void tile_sweep(MgTile& T, const TilePos& p, float2 (&xa)[2],
+                                           float2 (&xb)[2], const float2 (&ia)[2],
+                                           const float2 (&ib)[2], const float2 (&ba)[2],
+                                           const float2 (&bb)[2]) {
+  constexpr int o = 1 - c;
+  if (p.y == 0 || p.y == TILE_W - 1) return;  // the outermost rows are never updated
+  const int t = threadIdx.x & (TILE_THREADS - 1);
+  const int d = ((c + p.y) & 1) ? 1 : -1;
+  const float2* ta = T.a[o] + t;
+  const float2* tb = T.b[o] + t;
+  const float zprev = p.g > 0 ? tb[-TILE_W * 8].y : 0.0f;
+  const float znext = p.g < 3 ? ta[TILE_W * 8].x : 0.0f;
+  float2 sa = __fadd2_rn(xa[o], ta[d]);
+  float2 sb = __fadd2_rn(xb[o], tb[-d]);
+  sa = __fadd2_rn(sa, ta[-8]);
+  sb = __fadd2_rn(sb, tb[-8]);
+  sa = __fadd2_rn(sa, ta[8]);
+  sb = __fadd2_rn(sb, tb[8]);
+  sa = __fadd2_rn(sa, make_float2(zprev, xb[o].x));
+  sb = __fadd2_rn(sb, xa[o]);
+  sa = __fadd2_rn(sa, xb[o]);
+  sb = __fadd2_rn(sb, make_float2(xa[o].y, znext));
+  xa[c] = __ffma2_rn(sa, ia[c], ba[c]);
+  xb[c] = __ffma2_rn(sb, ib[c], bb[c]);
+  T.a[c][t] = xa[c];
+  T.b[c][t] = xb[c];
+}
+
+// Blocked pre-smoothing and restriction (POST false: level l's b -> its x and level
+// l + 1's b), or blocked correction and post-smoothing (POST true: x and level l + 1's
+// final x -> xout; RZ: b x over the block's cells is added to rz).  The caller meets a
+// grid barrier after it.
+template <bool POST, bool RZ>
+__device__ __noinline__ void block_pass(const MgArgs& M, int l, FF* rz) {
+  const int group = threadIdx.x / TILE_THREADS;
+  MgTile& T = mg_tile(group);
+  const MgLevel& L = M.lv[l];
+  const MgLevel& Cl = M.lv[l + 1];
+  const SV v = sview(L);
+  const PV C = pview(Cl);
+  float* xout = POST ? (l == 0 ? s_z0 : L.x2) : v.x;
+  const int* blk = L.blk;
+  const uint4* tab = L.tab + (threadIdx.x & (TILE_THREADS - 1));
+  const float omega = M.omega;
+  const int n = s_nblk[l], step = TILE_GROUPS * (int)team_size();
+  const TilePos p = tile_pos();
+  const int t = threadIdx.x & (TILE_THREADS - 1);
+  FF acc;
+  int q = (int)team_rank() + group * (int)team_size();
+  int e_next = 0;
+  uint4 w_next = make_uint4(0u, 0u, 0u, 0u);
+  if (q < n) {
+    e_next = blk[q];
+    w_next = tab[(size_t)q * TILE_THREADS];
+  }
+  for (; q < n; q += step) {
+    const uint4 w = w_next;
+    const BlkPos bp = blk_pos(v, p, e_next);
+    float2 ra[2], rb[2];  // the right-hand side
+    float2 xa[2], xb[2], ia[2], ib[2], ba[2], bb[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int z = 0; z < 4; ++z)
+        plane(ra[c], rb[c], z) = tab_code(w, z, c) ? v.b[c * v.half + bp.gi + z * v.pl] : 0.0f;
+    if constexpr (POST) {
+      float2 pa = make_float2(0.0f, 0.0f);  // parents of planes 0, 1 and of 2, 3
+      const int I = (bp.b0 >> 1) - TILE_H / 2 + p.s, J = (bp.b1 - TILE_H + p.y) >> 1,
+                K = (bp.b2 - TILE_H + 4 * p.g) >> 1;
+      if ((w.x | w.y) & 0xffffu) pa.x = C.x[level_index(C, I, J, K)];
+      if ((w.z | w.w) & 0xffffu) pa.y = C.x[level_index(C, I, J, K + 1)];
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const bool f = tab_code(w, z, 0) != 0u;
+        const float x = f ? v.x[bp.gi + z * v.pl] : 0.0f;
+        plane(xa[0], xb[0], z) = f ? __fmaf_rn(omega, z < 2 ? pa.x : pa.y, x) : 0.0f;
+      }
+    }
+    if (q + step < n) {
+      e_next = blk[q + step];
+      w_next = tab[(size_t)(q + step) * TILE_THREADS];
+    }
+    // coefficients: a warp whose cells are all interior or 0 takes them without the tables
+    bool plain = true;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const unsigned int cd = tab_code(w, z, c);
+        plain = plain && (cd == 0u || cd == CODE_FULL);
+      }
+    if (__all_sync(0xffffffffu, plain)) {
+      const float i6 = s_inv_cnt[6], s6 = s_inv_scnt[l][6];
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          plane(ia[c], ib[c], z) = tab_code(w, z, c) ? i6 : 0.0f;
+          plane(ba[c], bb[c], z) = __fmul_rn(plane(ra[c], rb[c], z), s6);
+        }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const int cnt = code_cnt(tab_code(w, z, c));  // 0 where there is no fluid cell
+          plane(ia[c], ib[c], z) = s_inv_cnt[cnt];
+          plane(ba[c], bb[c], z) = __fmul_rn(plane(ra[c], rb[c], z), s_inv_scnt[l][cnt]);
+        }
+    }
+    if constexpr (!POST) {
+      xa[0] = ba[0];
+      xb[0] = bb[0];
+    }
+    tile_sync(group);  // the last block's readers are done
+    T.a[0][t] = xa[0];
+    T.b[0][t] = xb[0];
+    xa[1] = xb[1] = make_float2(0.0f, 0.0f);
+    tile_sync(group);
+    int reach = 2 * M.nu - 1;
+    for (int h = 0; h < M.nu; ++h) {
+      if (p.wdist <= reach) tile_sweep<1>(T, p, xa, xb, ia, ib, ba, bb);
+      tile_sync(group);
+      --reach;
+      if (POST || h + 1 < M.nu) {
+        if (p.wdist <= reach) tile_sweep<0>(T, p, xa, xb, ia, ib, ba, bb);
+        --reach;
+        if (!POST || h + 1 < M.nu) tile_sync(group);
+      }
+    }
+    if (p.own) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int z = 0; z < 4; ++z)
+          if (tab_code(w, z, c)) {
+            const int gi = c * v.half + bp.gi + z * v.pl;
+            const float x = plane(xa[c], xb[c], z);
+            xout[gi] = x;
+            if constexpr (RZ) acc.add_prod(v.b[gi], x);
+          }
+    }
+    if constexpr (!POST) {
+      if (p.wdist == 0) {
+        // residuals of the red cells (0 where there is no fluid cell)
+        float r[4];
+        const int d = (p.y & 1) ? 1 : -1;
+        const float2* ta = T.a[1] + t;
+        const float2* tb = T.b[1] + t;
+        const float2 xoa = ta[d], xob = tb[-d], yma = ta[-8], ymb = tb[-8], ypa = ta[8],
+                     ypb = tb[8];
+        const float zprev = tb[-TILE_W * 8].y, znext = ta[TILE_W * 8].x;
+        bool full = true;
+#pragma unroll
+        for (int z = 0; z < 4; ++z) full = full && tab_code(w, z, 0) == CODE_FULL;
+        full = __all_sync(0xffffffffu, full || !p.own);
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const unsigned int cd = tab_code(w, z, 0);
+          const float x = plane(xa[0], xb[0], z);
+          const float own = plane(xa[1], xb[1], z);
+          float2 oa = xoa, ob = xob, ma = yma, mb = ymb, pa = ypa, pb = ypb;
+          const float other = plane(oa, ob, z);
+          const bool low = ((z + p.y) & 1) == 0;  // the other slot is the -x neighbour
+          const float xv[6] = {low ? other : own,
+                               low ? own : other,
+                               plane(ma, mb, z),
+                               plane(pa, pb, z),
+                               z == 0 ? zprev : plane(xa[1], xb[1], z > 0 ? z - 1 : 0),
+                               z == 3 ? znext : plane(xa[1], xb[1], z < 3 ? z + 1 : 3)};
+          const float bv = plane(ra[0], rb[0], z);
+          if (full) r[z] = resid_full(v.s, bv, x, xv);
+          else r[z] = cd ? resid(v.s, code_cnt(cd), cd, bv, x, xv) : 0.0f;
+        }
+        // b of the coarse cells: restrict_sum's sum over the red children in order, the
+        // (dy = 1) children being the next row's, eight lanes on
+        float r1[4];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) r1[z] = __shfl_down_sync(0xffffffffu, r[z], 8);
+        if (p.own && (p.y & 1) == 0) {
+          const int I = (bp.b0 >> 1) - TILE_H / 2 + p.s, J = (bp.b1 - TILE_H + p.y) >> 1,
+                    K0 = (bp.b2 - TILE_H + 4 * p.g) >> 1;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int K = K0 + h;
+            if (I >= C.nx || J >= C.ny || K >= C.nz) continue;
+            const int ci = level_index(C, I, J, K);
+            const unsigned int cd = C.split ? (unsigned int)Cl.code16[ci] : (unsigned int)Cl.code[ci];
+            if (!(cd & CODE_SELF)) continue;
+            const float sum = __fadd_rn(__fadd_rn(__fadd_rn(r[2 * h], r1[2 * h]), r[2 * h + 1]),
+                                        r1[2 * h + 1]);
+            const float bv = __fmul_rn(sum, 0.0625f);
+            Cl.b[ci] = bv;
+            // the coarse level's first red half-sweep, as in restrict_split
+            if (C.split && ((I + J + K) & 1) == 0) Cl.x[ci] = gs_first(Cl.lvl, code_cnt(cd), bv);
+          }
+        }
+      }
+    }
+  }
+  if constexpr (RZ) {
+    rz->add_prod(acc.hi, 1.0f);
+    rz->add_prod(acc.lo, 1.0f);
   }
 }
 
@@ -1146,30 +1472,49 @@ __device__ bool vcycle_rest(const PcgArgs& A, FF& rz) {
     return true;
   }
   const MgLevel& L1 = M.lv[1];
-  sweep_split<NORMAL>(M, L0, L1, 0, 1, nullptr);
-  if (!gsync(A)) return false;
-  SOLVE_TRACE(TR_V_PRE1);
-  for (int s = 1; s < M.nu; ++s) {
-    sweep_split<NORMAL>(M, L0, L1, 0, 0, nullptr);
-    if (!gsync(A)) return false;
+  const bool blocked0 = s_nblk[0] > 0;
+  if (blocked0) {
+    block_pass<false, false>(M, 0, nullptr);
+  } else {
     sweep_split<NORMAL>(M, L0, L1, 0, 1, nullptr);
     if (!gsync(A)) return false;
+    SOLVE_TRACE(TR_V_PRE1);
+    for (int s = 1; s < M.nu; ++s) {
+      sweep_split<NORMAL>(M, L0, L1, 0, 0, nullptr);
+      if (!gsync(A)) return false;
+      sweep_split<NORMAL>(M, L0, L1, 0, 1, nullptr);
+      if (!gsync(A)) return false;
+    }
+    SOLVE_TRACE(TR_V_PRE);
+    if (L1.split) restrict_split(L0, L1);
+    else restrict_split_nat(L0, L1);
   }
-  SOLVE_TRACE(TR_V_PRE);
-  if (L1.split) restrict_split(L0, L1);
-  else restrict_split_nat(L0, L1);
   if (!gsync(A)) return false;
   SOLVE_TRACE(TR_V_RESTRICT);
   for (int l = 1; l < M.lgrid; ++l) {
-    if (!down_split(A, l)) return false;
+    if (s_nblk[l] > 0) {
+      block_pass<false, false>(M, l, nullptr);
+      if (!gsync(A)) return false;
+    } else if (!down_split(A, l)) {
+      return false;
+    }
     SOLVE_TRACE(TR_V_DOWN + min(l, 11));
   }
   if (team_rank() == 0) cta_cycle(A);
   if (!gsync(A)) return false;
   SOLVE_TRACE(TR_V_CTA);
   for (int l = M.lgrid - 1; l >= 1; --l) {
-    if (!up_split(A, l)) return false;
+    if (s_nblk[l] > 0) {
+      block_pass<true, false>(M, l, nullptr);
+      if (!gsync(A)) return false;
+    } else if (!up_split(A, l)) {
+      return false;
+    }
     SOLVE_TRACE(TR_V_UP + min(l, 11));
+  }
+  if (blocked0) {
+    block_pass<true, true>(M, 0, &rz);
+    return true;
   }
   sweep_split<CORRECT>(M, L0, L1, 0, 1, M.nu == 1 ? &rz : nullptr);
   if (!gsync(A)) return false;
@@ -1194,8 +1539,8 @@ __device__ __noinline__ void phase_a_v(const PcgArgs& A, const float* pold, floa
                                      FF& pq) {
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
-  const float* z = v.x;
-  float* q0 = M.q0;
+  const float* z = s_z0;
+  float* q0 = s_q0;
   const float s_a = A.s;
   const int lane = threadIdx.x & 31;
   const int2 q = seg_slice(M.lv[0]);
@@ -1266,7 +1611,8 @@ __device__ __noinline__ void phase_b_v(const PcgArgs& A, const float* pnew, floa
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
   float* d0 = M.d0;
-  const float* q0 = M.q0;
+  const float* q0 = s_q0;
+  const bool first_red = s_nblk[0] == 0;  // a blocked level 0 makes it from r itself
   const int lane = threadIdx.x & 31;
   const float invs6 = s_inv_scnt[0][6];
   const int2 q = seg_slice(M.lv[0]);
@@ -1311,7 +1657,8 @@ __device__ __noinline__ void phase_b_v(const PcgArgs& A, const float* pnew, floa
           }
           *reinterpret_cast<float2*>(d0 + st.e.idx) = make_float2(dn[0], dn[1]);
           *reinterpret_cast<float2*>(v.b + st.e.idx) = make_float2(rn[0], rn[1]);
-          if (st.c == 0) *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(zn[0], zn[1]);
+          if (first_red && st.c == 0)
+            *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(zn[0], zn[1]);
           return;
         }
 #pragma unroll
@@ -1329,7 +1676,8 @@ __device__ __noinline__ void phase_b_v(const PcgArgs& A, const float* pnew, floa
         if (st.e.okA || st.e.okB) {
           *reinterpret_cast<float2*>(d0 + st.e.idx) = make_float2(dn[0], dn[1]);
           *reinterpret_cast<float2*>(v.b + st.e.idx) = make_float2(rn[0], rn[1]);
-          if (st.c == 0) *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(zn[0], zn[1]);
+          if (first_red && st.c == 0)
+            *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(zn[0], zn[1]);
         }
       });
   rr.add_prod(acc.hi, 1.0f);
@@ -1342,8 +1690,8 @@ __device__ __noinline__ void phase_a_s(const PcgArgs& A, const float* pold, floa
                                      FF& pq) {
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
-  const float* z = v.x;
-  float* q0 = M.q0;
+  const float* z = s_z0;
+  float* q0 = s_q0;
   const float s_a = A.s;
   const int lane = threadIdx.x & 31;
   const Items it = seg_items(M.lv[0], 2);
@@ -1402,7 +1750,8 @@ __device__ __noinline__ void phase_b_s(const PcgArgs& A, const float* pnew, floa
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
   float* d0 = M.d0;
-  const float* q0 = M.q0;
+  const float* q0 = s_q0;
+  const bool first_red = s_nblk[0] == 0;  // a blocked level 0 makes it from r itself
   const int lane = threadIdx.x & 31;
   const Items it = seg_items(M.lv[0], 2);
   struct S {
@@ -1433,7 +1782,7 @@ __device__ __noinline__ void phase_b_s(const PcgArgs& A, const float* pnew, floa
         d0[s.idx] = __fmaf_rn(alpha, s.p, s.d);
         const float rc = __fmaf_rn(-alpha, s.q, s.r);
         v.b[s.idx] = rc;
-        if (s.c == 0) v.x[s.idx] = gs_first(0, code_cnt(s.code), rc);
+        if (first_red && s.c == 0) v.x[s.idx] = gs_first(0, code_cnt(s.code), rc);
         acc.add_prod(rc, rc);
       });
   rr.add_prod(acc.hi, 1.0f);
@@ -1486,13 +1835,13 @@ __device__ __forceinline__ float2 residual_pair(const SV& v, const float2* x2, c
 // ---------------------------------------------------------------- set-up
 
 // Whether segment g (flat: row g / nw, segment g % nw) of split level L meets a
-// block holding fluid; sg receives {row, segment in row, j, k}.  Level 0 reads
+// block holding fluid; sg receives the packed segment.  Level 0 reads
 // the binning's brick fluid counts.
 __device__ __forceinline__ bool seg_active(const PcgArgs& A, const MgLevel& L, int l, int g,
-                                           int4& sg) {
+                                           unsigned int& sg) {
   const int r = g / L.nw, w = g - r * L.nw;
   const int j = r % L.ny, k = r / L.ny;
-  sg = make_int4(r, w, j, k);
+  sg = seg_pack(w, j, k);
   const int by = j >> 3, bz = k >> 3;
   const int b0 = w * 8, b1 = min(L.nbx, b0 + 8);
   bool any = false;
@@ -1501,6 +1850,105 @@ __device__ __forceinline__ bool seg_active(const PcgArgs& A, const MgLevel& L, i
     any |= (l == 0) ? (A.brick_fluid[bi] > 0u) : (L.bflag[bi] != 0);
   }
   return any;
+}
+
+// Whether a level with n blocks holding fluid is smoothed blocked.  The line: a block
+// takes ~1.2 us of a CTA (two at a time), a pass-by-pass half-sweep ~3.3 us plus the
+// cells' own time.  Solves with the limit at 2, 4, 6 and 10 blocks per CTA: 101 x 67 x 83
+// pool 1.63, 1.51, 1.51, 1.51 ms; 128^3 dam break (3.4 blocks) 1.29, 1.27, 1.28, 1.28;
+// 128^3 pool (8.7 blocks) 1.80, 1.81, 1.81, 2.02.
+__device__ __forceinline__ bool blocked(const MgArgs& M, unsigned int n) {
+  return M.nlev > 1 && M.nu <= BLK_MAX_NU && n > 0u && n <= (unsigned)MG_BLK_PER_CTA * team_size();
+}
+
+// The grid-wide levels' lists of blocks holding fluid.  Level 0's follows the
+// binning's active list, so the sums that blocks of one CTA share keep their order; on
+// the coarser levels the order decides nothing and blocks append as they come.
+__device__ __forceinline__ void block_lists(const PcgArgs& A) {
+  const MgArgs& M = A.mg;
+  {
+    const MgLevel& L = M.lv[0];
+    const unsigned int n = *A.n_active;
+    if (blocked(M, n)) {
+      const Part p = level_part((int)n, false);
+      for (int c = p.begin; c < p.end; c += p.stride) {
+        const int b = (int)A.active[c];
+        L.blk[c] = b % L.nbx | ((b / L.nbx) % L.nby) << 8 | (b / (L.nbx * L.nby)) << 16;
+      }
+    }
+  }
+  for (int l = 1; l < M.lgrid; ++l) {
+    const MgLevel& L = M.lv[l];
+    const Part p = level_part(L.nbx * L.nby * L.nbz, false);
+    for (int c = p.begin; c < p.end; c += p.stride)
+      if (L.bflag[c])
+        L.blk[atomicAdd(L.nblk, 1u)] =
+            c % L.nbx | ((c / L.nbx) % L.nby) << 8 | (c / (L.nbx * L.nby)) << 16;
+  }
+}
+
+// The codes that each thread of a block's tile works with (MgLevel::tab): those of its
+// eight cells within L1 distance TILE_H of the block, 0 elsewhere, off the grid and
+// where there is no fluid.  A thread's cells lie in one of the 27 blocks around, and
+// codes are this solve's only where that block holds fluid.
+__device__ __noinline__ void block_tables(const PcgArgs& A) {
+  const MgArgs& M = A.mg;
+  const TilePos p = tile_pos();
+  const int group = threadIdx.x / TILE_THREADS, t = threadIdx.x & (TILE_THREADS - 1);
+  const int nbx = ((p.s + 2) >> 2) - 1, nby = ((p.y + 4) >> 3) - 1, nbz = ((p.g + 1) >> 1) - 1;
+  for (int l = 0; l < M.lgrid; ++l) {
+    const MgLevel& L = M.lv[l];
+    const SV v = sview(L);
+    const int nz = L.nz;
+    for (int q = (int)team_rank() + group * (int)team_size(); q < s_nblk[l];
+         q += TILE_GROUPS * (int)team_size()) {
+      const int e = L.blk[q];
+      const BlkPos bp = blk_pos(v, p, e);
+      const int x = (e & 255) + nbx, y = ((e >> 8) & 255) + nby, z = (e >> 16) + nbz;
+      uint4 w = make_uint4(0u, 0u, 0u, 0u);
+      bool any = x >= 0 && y >= 0 && z >= 0 && x < L.nbx && y < L.nby && z < L.nbz;
+      if (any) {
+        const int b = x + L.nbx * (y + L.nby * z);
+        any = l == 0 ? A.brick_fluid[b] > 0u : L.bflag[b] != 0;
+      }
+      const int j = bp.b1 - TILE_H + p.y;
+      if (any && j < v.ny) {
+        unsigned int cd[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int k = bp.b2 - TILE_H + 4 * p.g + u;
+          const int dyz = tile_dist(p.y) + tile_dist(4 * p.g + u);
+          cd[u] = 0u;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int tx = 2 * p.s + ((c + p.y + u) & 1), i = bp.b0 - TILE_H + tx;
+            if (k < nz && i < v.nx && tile_dist(tx) + dyz <= TILE_H) {
+              const unsigned int code = v.code[c * v.half + bp.gi + u * v.pl];
+              if (code & CODE_SELF) cd[u] |= code << (16 * c);
+            }
+          }
+        }
+        w = make_uint4(cd[0], cd[1], cd[2], cd[3]);
+      }
+      L.tab[(size_t)q * TILE_THREADS + t] = w;
+    }
+  }
+}
+
+// After build_levels: which levels are smoothed blocked, and level 0's arrays.
+__device__ __forceinline__ void block_rule(const PcgArgs& A) {
+  const MgArgs& M = A.mg;
+  if (threadIdx.x < MG_MAX_LEVELS) {
+    const int l = threadIdx.x;
+    const unsigned int n = l >= M.lgrid ? 0u : l == 0 ? *A.n_active : *M.lv[l].nblk;
+    s_nblk[l] = blocked(M, n) ? (int)n : 0;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_z0 = s_nblk[0] > 0 ? M.q0 : M.lv[0].x;
+    s_q0 = s_nblk[0] > 0 ? M.lv[0].x : M.q0;
+  }
+  __syncthreads();
 }
 
 // Builds, once per solve: the fluid flags of levels 1.. (a coarse cell is fluid
@@ -1514,6 +1962,7 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
     const MgLevel& L = M.lv[l];
     const Part p = level_part(L.nbx * L.nby * L.nbz, false);
     for (int c = p.begin; c < p.end; c += p.stride) L.bflag[c] = 0;
+    if (team_rank() == 0 && threadIdx.x == 0) *L.nblk = 0u;
   }
   if (!gsync(A)) return false;
   SOLVE_TRACE(TR_BFLAG);
@@ -1534,6 +1983,7 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
     if (!gsync(A)) return false;
     SOLVE_TRACE(TR_FLAGS + min(l, 11));
   }
+  block_lists(A);
   // active segments: count per CTA, then write them in segment order
   __shared__ unsigned int s_wsum[PCG_WARPS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1544,7 +1994,7 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
     const int g0 = min(nsegs, (int)team_rank() * per), g1 = min(nsegs, g0 + per);
     unsigned int cnt = 0;
     for (int g = g0 + (int)threadIdx.x; g < g1; g += PCG_THREADS) {
-      int4 sg;
+      unsigned int sg;
       cnt += seg_active(A, L, l, g, sg);
     }
     cnt = __reduce_add_sync(0xffffffffu, cnt);
@@ -1584,7 +2034,7 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
     __syncthreads();
     for (int g00 = g0; g00 < g1; g00 += PCG_THREADS) {
       const int g = g00 + (int)threadIdx.x;
-      int4 sg = make_int4(0, 0, 0, 0);
+      unsigned int sg = 0u;
       const bool act = g < g1 && seg_active(A, L, l, g, sg);
       const unsigned int bal = __ballot_sync(0xffffffffu, act);
       if (lane == 0) s_wsum[warp] = __popc(bal);
@@ -1625,7 +2075,7 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
 
 // Copies this CTA's slice of each grid-wide level's segment list into the
 // shared-memory cache, level 0 first, while it fits (after build_levels).
-__device__ __noinline__ void seg_cache_fill(const MgArgs& M, int4* cache) {
+__device__ __noinline__ void seg_cache_fill(const MgArgs& M, unsigned int* cache) {
   int used = 0;
   for (int l = 0; l < M.lgrid; ++l) {
     const MgLevel& L = M.lv[l];
@@ -1644,12 +2094,20 @@ __device__ __noinline__ void seg_cache_fill(const MgArgs& M, int4* cache) {
 }
 
 // The shared-memory cache of the segment slices sits after the CTA-local levels
-// in the kernel's dynamic shared memory.
+// in the kernel's dynamic shared memory, the tiles of the blocked smoothing after it.
 constexpr size_t MG_DYN_CTA = (sizeof(CtaMg) + 15) / 16 * 16;
-constexpr size_t MG_DYN_BYTES = MG_DYN_CTA + sizeof(int4) * SEG_CACHE;
+constexpr size_t MG_DYN_TILE = MG_DYN_CTA + sizeof(unsigned int) * SEG_CACHE;
+constexpr size_t MG_DYN_BYTES = MG_DYN_TILE + TILE_GROUPS * sizeof(MgTile);
+// one carve-out step up (132 KB) would take L1 from the level-0 passes
+static_assert(MG_DYN_BYTES + 4096 <= 100 * 1024, "the kernel stays in the 100 KB carve-out");
 
-__device__ __forceinline__ int4* seg_cache_of(unsigned char* dyn) {
-  return reinterpret_cast<int4*>(dyn + MG_DYN_CTA);
+__device__ __forceinline__ unsigned int* seg_cache_of(unsigned char* dyn) {
+  return reinterpret_cast<unsigned int*>(dyn + MG_DYN_CTA);
+}
+
+__device__ __forceinline__ MgTile& mg_tile(int group) {
+  extern __shared__ __align__(16) unsigned char mg_dyn[];
+  return reinterpret_cast<MgTile*>(mg_dyn + MG_DYN_TILE)[group];
 }
 
 // The mixed mode's refinement, over level 0's slot pairs with two items in flight
@@ -1779,15 +2237,17 @@ struct SolveState {
 // recomputed residual's norm (refinement).  A slot's readers always pass another barrier before the slot
 // is written again.
 template <bool MIXED>
-__device__ void solve_mg(const PcgArgs& A, Shared& sh, int4* segc, SolveState& S) {
+__device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, SolveState& S) {
   const MgArgs& M = A.mg;
   const MgLevel& L0 = M.lv[0];
   float* d = M.d0;
   float* z = L0.x;
   float* r = L0.b;
   if (!build_levels(A, sh)) { S.ok = false; return; }
+  block_rule(A);
   seg_cache_fill(M, segc);
   SOLVE_TRACE(TR_SEG_CACHE);
+  block_tables(A);  // visible to the V-cycles after the start pass's barrier
   if (M.nlev > 1 && team_rank() == 0) cta_levels_init(M);
   SOLVE_TRACE(TR_CTA_LISTS);
   // ---- start: r = b (cold) or b - A x0 (warm start from the last solve's x),
@@ -1987,7 +2447,7 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, int4* segc, SolveState& S
 // RBGS_CHECK sweep pairs and the sweep pairs are capped at max_iter.
 constexpr int RBGS_CHECK = 8;
 
-__device__ __noinline__ void solve_rbgs(const PcgArgs& A, Shared& sh, int4* segc, SolveState& S) {
+__device__ __noinline__ void solve_rbgs(const PcgArgs& A, Shared& sh, unsigned int* segc, SolveState& S) {
   const MgArgs& M = A.mg;
   const MgLevel& L0 = M.lv[0];
   const MgLevel& L1 = M.nlev > 1 ? M.lv[1] : M.lv[0];
@@ -2067,8 +2527,11 @@ __device__ __noinline__ void solve_rbgs(const PcgArgs& A, Shared& sh, int4* segc
 
 template <bool MIXED>
 __device__ void solve_scene_mg(const PcgArgs& A, Shared& sh, unsigned char* dyn) {
-  int4* segc = seg_cache_of(dyn);
-  if (threadIdx.x < MG_MAX_LEVELS) s_segc[threadIdx.x] = nullptr;  // no cache until filled
+  unsigned int* segc = seg_cache_of(dyn);
+  if (threadIdx.x < MG_MAX_LEVELS) {
+    s_segc[threadIdx.x] = nullptr;  // no cache until filled
+    s_nblk[threadIdx.x] = 0;        // no blocked level until block_rule
+  }
   __syncthreads();
   const long long ncells = (long long)A.g.nx * A.g.ny * A.g.nz;
   const bool singular = A.check_singular && ((long long)A.stats->n_fluid == ncells);

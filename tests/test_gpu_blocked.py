@@ -1,0 +1,44 @@
+"""The multigrid levels that are smoothed blocked (csrc/k_mg.cu, block_pass and the levels
+inside one CTA): shapes where a tile's edges, remainders or halo can go wrong, against the
+oracle's V-cycle.  After one MG-PCG iteration (tolerance out of reach, cap 1 on both sides)
+the pressure is a multiple of one V-cycle of the right-hand side, whose values are about
+4 levels x 4 half-sweeps x 8 additions deep: 1e-5 relative allows each of those roundings
+(6e-8) once.  Later iterates subtract nearly equal residuals and have no such bound."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2404_01931_gb300 import flip as F
+from paper_2404_01931_gb300 import scenes as S
+
+from parity_util import gpu_step, matched, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+def masked_scene(n, fill, seed):
+    """Random fluid cells (single cells, holes, cells at every wall) with random velocities."""
+    mask = S.random_mask(n, fill, seed)
+    sc = S.seed_mask(mask, 1.0 / max(n), 1, seed)
+    return S.random_velocities(sc, 0.3, seed + 1)
+
+
+@pytest.mark.parametrize("nu", [1, 2, 3])  # 3: deeper than the halo, pass by pass
+@pytest.mark.parametrize("n,fill", [
+    ((9, 17, 8), 0.5),       # one cell past a block, the smallest level above the CTA-local ones
+    ((33, 7, 24), 0.9),      # an extent below a block
+    ((40, 25, 31), 0.15),    # mostly isolated cells
+    ((64, 48, 72), 0.97),    # several blocks a CTA group, holes in the interior
+    ((16, 160, 16), 0.6),    # CTA-local levels longer than 16 cells
+    ((144, 96, 80), 0.95),   # level 0 above the limit, the coarser levels blocked
+])
+def test_blocked_smoothing_matches_the_oracle(n, fill, nu):
+    sc = masked_scene(n, fill, 11)
+    op, fp = matched(n, cg_tol=1e-30, cg_max_iter=1, mg_smooth=nu)
+    ref = O.step(op, *sc.arrays())
+    with pytest.warns(RuntimeWarning):
+        got = gpu_step(fp, sc.arrays())
+    assert got["rc"] == F.FLIP_E_NOT_CONVERGED and got["stats"].cg_iterations == 1
+    assert np.array_equal(got["type"], ref.type.ravel())
+    e = rel_l2(got["p"], ref.pressure)
+    assert e <= 1e-5, f"pressure after one MG-PCG iteration: rel L2 {e:.3e}"
