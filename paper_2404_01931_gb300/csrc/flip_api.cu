@@ -406,9 +406,9 @@ void carve(flip_handle* h, Carver& cv) {
         L.nseg = cv.take<unsigned int>(1);
         const size_t blocks = (size_t)L.nbx * L.nby * L.nbz;
         L.blk = cv.take<int>(blocks);
-        // 512 threads per block, as many blocks as a blocked level can have
-        L.tab = cv.take<uint4>(
-            512 * std::min(blocks, (size_t)MG_BLK_PER_CTA * (size_t)h->pcg_blocks));
+        // 1024 threads per block, as many blocks as a blocked level can have
+        L.tab = cv.take<uint2>(
+            1024 * std::min(blocks, (size_t)MG_BLK_PER_CTA * (size_t)h->pcg_blocks));
         if (l > 0) {
           L.t = cv.take<uint8_t>(n);
           L.bflag = cv.take<uint8_t>((size_t)L.nbx * L.nby * L.nbz);

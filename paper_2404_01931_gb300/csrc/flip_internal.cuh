@@ -135,6 +135,10 @@ struct FF {
     hi = s;
     lo = __fadd_rn(lo, e);
   }
+  __device__ __forceinline__ void add(const FF& f) {
+    add_prod(f.hi, 1.0f);
+    add_prod(f.lo, 1.0f);
+  }
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
@@ -199,15 +203,22 @@ __device__ __forceinline__ void red_add_release_gpu(unsigned int* p, unsigned in
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ bool grid_barrier(unsigned int* bar, int* status, unsigned int nblocks,
-                                             unsigned long long timeout_ns) {
-  __shared__ int s_ok;
+// The two halves of a barrier: between them a CTA may load what earlier barriers have
+// made visible (it must not write anything that others read before the barrier ends).
+__device__ __forceinline__ void grid_arrive(unsigned int* bar) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    int ok = 1;
-    const unsigned int target = (s_bar_gen + 1u) * nblocks;
     s_bar_gen += 1u;
     red_add_release_gpu(bar, 1u);
+  }
+}
+
+__device__ __forceinline__ bool grid_wait(unsigned int* bar, int* status, unsigned int nblocks,
+                                          unsigned long long timeout_ns) {
+  __shared__ int s_ok;
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    const unsigned int target = s_bar_gen * nblocks;
     const unsigned long long t0 = global_timer_ns();
     while ((int)(ld_acquire_gpu(bar) - target) < 0) {
       if (*(volatile int*)status & DEV_TIMEOUT) { ok = 0; break; }
@@ -222,6 +233,12 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* bar, int* status, uns
   }
   __syncthreads();
   return s_ok != 0;
+}
+
+__device__ __forceinline__ bool grid_barrier(unsigned int* bar, int* status, unsigned int nblocks,
+                                             unsigned long long timeout_ns) {
+  grid_arrive(bar);
+  return grid_wait(bar, status, nblocks, timeout_ns);
 }
 
 // Number of a cell's neighbours that are not solid walls (the domain planes

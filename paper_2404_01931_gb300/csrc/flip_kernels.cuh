@@ -144,7 +144,7 @@ struct MgLevel {
                       // brick fluid counts of the binning)
   int* blk;           // the blocks holding fluid (bx | by << 8 | bz << 16), for the
                       // blocked smoothing
-  uint4* tab;         // per block and thread of its tile: the codes of its eight cells
+  uint2* tab;         // per block and thread of its tile: the codes of its four cells
   unsigned int* nblk; // levels >= 1: their number (level 0: the binning's active bricks)
   float* x2;          // levels >= 1: the level's x after blocked post-smoothing
 };

@@ -493,8 +493,8 @@ __device__ __forceinline__ bool gs_apply(float* x, int l, float omega, GsIn& s, 
 // grid-wide level never sweeps from zero here: its first red half-sweep is made
 // by the pass that produces its right-hand side.)
 template <int MODE, bool RZ>
-__device__ __noinline__ void sweep_split_v(const MgArgs& M, const MgLevel& L, const MgLevel& C,
-                                         int l, int colour, FF* rz) {
+__device__ __noinline__ FF sweep_split_v(const MgArgs& M, const MgLevel& L, const MgLevel& C,
+                                         int l, int colour) {
   static_assert(MODE != FIRST, "grid-wide levels start from the fused first half-sweep");
   constexpr int U = (MODE == CORRECT) ? 1 : 2;
   const int lane = threadIdx.x & 31;
@@ -576,17 +576,14 @@ __device__ __noinline__ void sweep_split_v(const MgArgs& M, const MgLevel& L, co
         if (st.e.okA || st.e.okB)
           *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(out[0], out[1]);
       });
-  if constexpr (RZ) {
-    rz->add_prod(acc.hi, 1.0f);
-    rz->add_prod(acc.lo, 1.0f);
-  }
+  return acc;
 }
 
 // Scalar form: a lane takes one slot (levels with few segments per CTA, where
 // more items in flight matter more than wider loads).
 template <int MODE>
-__device__ __noinline__ void sweep_split_s(const MgArgs& M, const MgLevel& L, const MgLevel& C,
-                                         int l, int colour, FF* rz) {
+__device__ __noinline__ FF sweep_split_s(const MgArgs& M, const MgLevel& L, const MgLevel& C,
+                                         int l, int colour, bool rz) {
   static_assert(MODE != FIRST, "grid-wide levels start from the fused first half-sweep");
   constexpr int U = (MODE == CORRECT) ? 1 : 2;
   const int lane = threadIdx.x & 31;
@@ -637,10 +634,7 @@ __device__ __noinline__ void sweep_split_s(const MgArgs& M, const MgLevel& L, co
         float xv;
         if (gs_apply<MODE>(v.x, l, omega, s, xv) && rz) acc.add_prod(s.b, xv);
       });
-  if (rz) {
-    rz->add_prod(acc.hi, 1.0f);
-    rz->add_prod(acc.lo, 1.0f);
-  }
+  return acc;
 }
 
 // Levels with many segments per CTA take the paired form (8-byte accesses, half
@@ -652,15 +646,15 @@ __device__ __forceinline__ bool use_pairs(const MgLevel& L) {
 }
 
 template <int MODE>
-__device__ __forceinline__ void sweep_split(const MgArgs& M, const MgLevel& L, const MgLevel& C,
-                                            int l, int colour, FF* rz) {
+__device__ __forceinline__ FF sweep_split(const MgArgs& M, const MgLevel& L, const MgLevel& C,
+                                          int l, int colour, bool rz) {
   if (use_pairs(L)) {
     // the r.z accumulation only where asked (its registers would make the other
     // half-sweeps spill)
-    if (rz) sweep_split_v<MODE, true>(M, L, C, l, colour, rz);
-    else sweep_split_v<MODE, false>(M, L, C, l, colour, nullptr);
+    if (rz) return sweep_split_v<MODE, true>(M, L, C, l, colour);
+    return sweep_split_v<MODE, false>(M, L, C, l, colour);
   }
-  else sweep_split_s<MODE>(M, L, C, l, colour, rz);
+  return sweep_split_s<MODE>(M, L, C, l, colour, rz);
 }
 
 // ---------------------------------------------------------------- restriction
@@ -730,7 +724,7 @@ __device__ __noinline__ void restrict_split(const MgLevel& Fl, const MgLevel& Cl
   for (unsigned int t = it.first; t < it.end; t += PCG_WARPS) {
     const int4 sg = seg_unpack(C.seg[t - C.seg_base], C.ny);
     const int J = sg.z, K = sg.w;
-#pragma unroll
+#pragma unroll 1  // half the code, and nothing lost: 5.29 -> 5.24 ms per solve at 256^3
     for (int h = 0; h < 2; ++h) {
       // every lane takes part (a lane past the row's end on its last cell, whose
       // result it drops), so that a warp can vote
@@ -786,79 +780,87 @@ __device__ __noinline__ void restrict_split_nat(const MgLevel& Fl, const MgLevel
   }
 }
 
+// ---------------------------------------------------------------- barriers
+
+// Out of line: one copy of it stays in the instruction cache for an iteration's ~30
+// barriers.
+__device__ __noinline__ bool gsync(const PcgArgs& A) {
+  return grid_barrier(A.bar, A.status, team_size(), A.timeout_ns);
+}
+
+__device__ __forceinline__ void garrive(const PcgArgs& A) { grid_arrive(A.bar); }
+
+__device__ __forceinline__ bool gwait(const PcgArgs& A) {
+  return grid_wait(A.bar, A.status, team_size(), A.timeout_ns);
+}
+
 // ---------------------------------------------------------------- blocked smoothing
 //
 // On a level with few cells per CTA a half-sweep is all latency: a grid barrier
 // (~1.5 us) and a round trip to L2 for a few hundred cells.  There the whole
 // pre-smoothing with the restriction, and the whole correction with the
-// post-smoothing, run as one pass each: half a CTA takes an 8^3 block with a halo of
-// TILE_H = 4 cells into shared memory and makes all the half-sweeps there, between
-// barriers of its 512 threads, on the cells that the block's own still depend on
-// (those within L1 distance 3, 2, 1, 0 of the block).  Every cell gets gs_sum's
-// operations on the same values in its order, so the results are those of the
-// pass-by-pass form.
+// post-smoothing, run as one pass each: a CTA takes an 8^3 block with a halo of
+// TILE_H = 4 cells into registers and shared memory and makes all the half-sweeps there,
+// between CTA barriers, on the cells that the block's own still depend on (those within
+// L1 distance 3, 2, 1, 0 of the block).  Every cell gets gs_sum's operations on the same
+// values in its order, so the results are those of the pass-by-pass form.
 //
 // The tile (16^3 cells) is colour-split like the level: cell (tx, ty, tz) of colour c
 // is slot tx >> 1 of row (ty, tz).  Thread t owns slot s = t & 7 of row y = (t >> 3) & 15
-// in the four planes 4 g .. 4 g + 3, g = t >> 7, of both colours, in registers: as float2
-// A (planes 4 g, 4 g + 2) and B (4 g + 1, 4 g + 3), since the x neighbour that is not the
-// thread's own slot is slot s - 1 in one pair and s + 1 in the other.  Of a cell's six
-// neighbours one along x and all but the group's outermost along z are then in
-// registers; the others come from the shared copies a and b, whole pairs at a time.
-// Cells that are not fluid hold 0, with 0 coefficients, so nothing is masked; cells
-// farther out than a half-sweep's results are needed get values nobody uses.
-// A solve's neighbour codes per thread are laid out once per solve (MgLevel::tab), so a
-// pass loads them, and the cells they mark, without index or bounds logic.
+// in the planes 2 g and 2 g + 1, g = t >> 7, of both colours, in registers, as one float2
+// per colour.  Of a cell's six neighbours one along x and one along z are then its own
+// thread's; the others come from the shared copy, along y both planes at a time.  The
+// other x neighbour is slot s - 1 in one plane and s + 1 in the other.  Cells that are not
+// fluid hold 0, with 0 coefficients, so nothing is masked; cells farther out than a
+// half-sweep's results are needed get values nobody uses.  The neighbour codes of each
+// thread's cells are laid out once per solve (MgLevel::tab), so a pass loads them, and the
+// cells they mark, without index or bounds logic.
 //
-// Bound by latency: with one block per CTA a pass takes 6.2 us (down) or 6.7 us (up),
-// 1.5 us of it the grid barrier, against four or five passes of 3.3 us each; with two
-// blocks per CTA 9.8 and 6.7 us.  Solve at 64^3 (two dam blocks, mixed) 1.20 -> 0.85 ms,
-// 128^3 dam break (FP32) 1.55 -> 1.28, 256^3 pool (levels 2 and 3 blocked) 6.13 -> 5.92.
-// A first form with 1024 threads per tile, one slot in two planes each and scalar
-// shared loads took 7.1 and 8.8 us, 5.5 us for each further block: issue-bound.
+// Bound by latency (one block per CTA: 4.5-5 us a pass with its 1.5 us grid barrier, against
+// four or five passes of 3.3 us) and, from two blocks on, by issue (2 us per further block).
+// What counts is that nothing spills: 1024 threads have 64 registers each, and a spilled
+// value costs every warp a trip to L1.  With four planes per thread and two 512-thread
+// tiles side by side (68-140 bytes of spills) a pass took 6.2-6.7 us, with one plane twice
+// and scalar shared loads 7.1-8.8.  Solve per step, pass by pass -> four planes -> this:
+// 64^3 double dam (mixed) 1.20 -> 0.77 -> 0.61 ms, 128^3 dam break (FP32) 1.55 -> 1.12 ->
+// 1.00, 101 x 67 x 83 pool 2.06 -> 1.37 -> 1.20, 256^3 pool 6.13 -> 5.43 -> 5.24.
 constexpr int TILE_H = 4;
 constexpr int TILE_W = 8 + 2 * TILE_H;
-constexpr int TILE_THREADS = 512;
-constexpr int TILE_GROUPS = PCG_THREADS / TILE_THREADS;
+constexpr int TILE_PLANE = TILE_W * 8;        // threads (and slots of a colour) per plane
 // The halo is deep enough for two smoothing pairs.
 constexpr int BLK_MAX_NU = TILE_H / 2;
-static_assert(TILE_W * TILE_W * 2 == TILE_THREADS, "8 slots x 16 rows x 4 plane groups");
+static_assert(TILE_PLANE * TILE_W / 2 == PCG_THREADS, "a thread per slot and two planes");
 
 struct MgTile {
-  float2 a[2][TILE_THREADS], b[2][TILE_THREADS];
+  float2 x[2][PCG_THREADS];  // by colour
 };
 
-__device__ __forceinline__ MgTile& mg_tile(int group);
-
-__device__ __forceinline__ void tile_sync(int group) {
-  asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(TILE_THREADS) : "memory");
-}
+__device__ __forceinline__ MgTile& mg_tile();
 
 // Distance of a tile coordinate from the block's own [TILE_H, TILE_H + 8).
 __device__ __forceinline__ int tile_dist(int t) {
   return max(max(TILE_H - t, t - (TILE_H + 7)), 0);
 }
 
-// A thread's place in its tile and in the level.
+// A thread's place in its tile.
 struct TilePos {
-  int s, y, g;    // slot, row, plane group
+  int s, y, g;    // slot, row, pair of planes
   int wdist;      // smallest L1 distance of the warp's rows from the block
   bool own;       // the thread's cells are the block's own
 };
 
 __device__ __forceinline__ TilePos tile_pos() {
-  const int t = threadIdx.x & (TILE_THREADS - 1);
   TilePos p;
-  p.s = t & 7;
-  p.y = (t >> 3) & 15;
-  p.g = t >> 7;
+  p.s = (int)threadIdx.x & 7;
+  p.y = ((int)threadIdx.x >> 3) & 15;
+  p.g = (int)threadIdx.x >> 7;
   const int y0 = p.y & ~3;  // the warp's rows y0 .. y0 + 3
-  p.wdist = (y0 == 0 || y0 == 12) + (p.g == 0 || p.g == 3);
-  p.own = p.s >= 2 && p.s < 6 && p.y >= 4 && p.y < 12 && (p.g == 1 || p.g == 2);
+  p.wdist = (y0 == 0 || y0 == 12) + min(tile_dist(2 * p.g), tile_dist(2 * p.g + 1));
+  p.own = p.s >= 2 && p.s < 6 && p.y >= 4 && p.y < 12 && p.g >= 2 && p.g < 6;
   return p;
 }
 
-// The block's first cell, and a thread's first red slot (plane 4 g) in the level.
+// The block's first cell, and a thread's first red slot (plane 2 g) in the level.
 struct BlkPos {
   int b0, b1, b2, gi;
 };
@@ -868,9 +870,282 @@ __device__ __forceinline__ BlkPos blk_pos(const SV& v, const TilePos& p, int e) 
   q.b0 = (e & 255) * 8;
   q.b1 = ((e >> 8) & 255) * 8;
   q.b2 = (e >> 16) * 8;
-  const int j = q.b1 - TILE_H + p.y, k = q.b2 - TILE_H + 4 * p.g;
+  const int j = q.b1 - TILE_H + p.y, k = q.b2 - TILE_H + 2 * p.g;
   q.gi = v.margin + v.hx * (j + v.ny * k) + (q.b0 >> 1) - TILE_H / 2 + p.s;
   return q;
+}
+
+// Code of plane z (0 or 1 of the thread's two), colour c.
+__device__ __forceinline__ unsigned int tab_code(uint2 w, int z, int c) {
+  const unsigned int v = z == 0 ? w.x : w.y;
+  return c ? v >> 16 : v & 0xffffu;
+}
+
+__device__ __forceinline__ float& plane(float2& a, int z) { return z == 0 ? a.x : a.y; }
+
+// The sum of the six neighbours in colour o of a thread's two cells of the other colour:
+// (-x) + (+x), -y, +y, -z, +z.  zprev and znext are the planes below and above the two.
+__device__ __forceinline__ float2 tile_sum(const float2 own, const float2* t, int d, float zprev,
+                                           float znext) {
+  float2 s = __fadd2_rn(own, make_float2(t[d].x, t[-d].y));
+  s = __fadd2_rn(s, t[-8]);
+  s = __fadd2_rn(s, t[8]);
+  s = __fadd2_rn(s, make_float2(zprev, own.x));
+  return __fadd2_rn(s, make_float2(own.y, znext));
+}
+
+// One half-sweep of colour c (compile-time) over the tile: x = inv (sum of the six
+// neighbours) + base.
+template <int c>
+__device__ __forceinline__ void tile_sweep(MgTile& T, const TilePos& p, float2 (&x)[2],
+                                           const float2 (&inv)[2], const float2 (&base)[2]) {
+  if (p.y == 0 || p.y == TILE_W - 1) return;  // the outermost rows are never updated
+  const float2* t = T.x[1 - c] + threadIdx.x;
+  const float zprev = p.g > 0 ? t[-TILE_PLANE].y : 0.0f;
+  const float znext = p.g < TILE_W / 2 - 1 ? t[TILE_PLANE].x : 0.0f;
+  const float2 s = tile_sum(x[1 - c], t, ((c + p.y) & 1) ? 1 : -1, zprev, znext);
+  x[c] = __ffma2_rn(s, inv[c], base[c]);
+  T.x[c][threadIdx.x] = x[c];
+}
+
+struct PassSum {  // a pass's dot product, and whether its barrier held
+  FF sum;
+  bool ok;
+};
+
+// Blocked pre-smoothing and restriction (POST false: level l's b -> its x and level
+// l + 1's b), or blocked correction and post-smoothing (POST true: x and level l + 1's
+// final x -> xout; RZ: returns b x over the CTA's cells).  With `wait`, the grid barrier
+// before it has only been arrived at (garrive): the CTA loads what does not depend on the
+// pass before (the tables; for the post-smoothing b and x too), then waits.  ok is false if
+// the barrier failed.  The caller meets a grid barrier after it.
+template <bool POST, bool RZ>
+__device__ __noinline__ PassSum block_pass(const PcgArgs& A, int l, bool wait) {
+  const MgArgs& M = A.mg;
+  MgTile& T = mg_tile();
+  const MgLevel& L = M.lv[l];
+  const MgLevel& Cl = M.lv[l + 1];
+  const SV v = sview(L);
+  const PV C = pview(Cl);
+  float* xout = POST ? (l == 0 ? s_z0 : L.x2) : v.x;
+  const int n = s_nblk[l];
+  const TilePos p = tile_pos();
+  FF acc;
+  int q = (int)team_rank();
+  int e = 0;
+  uint2 w = make_uint2(0u, 0u);
+  float2 r[2];  // the right-hand side
+  float2 x0;    // POST: the red cells' x
+  auto load = [&](const BlkPos& bp) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int z = 0; z < 2; ++z)
+        plane(r[c], z) = tab_code(w, z, c) ? v.b[c * v.half + bp.gi + z * v.pl] : 0.0f;
+    if constexpr (POST) {
+#pragma unroll
+      for (int z = 0; z < 2; ++z)
+        plane(x0, z) = tab_code(w, z, 0) ? v.x[bp.gi + z * v.pl] : 0.0f;
+    }
+  };
+  if (q < n) {
+    e = L.blk[q];
+    w = L.tab[(size_t)q * PCG_THREADS + threadIdx.x];
+    if (POST) load(blk_pos(v, p, e));
+  }
+  if (wait && !gwait(A)) return PassSum{FF(), false};
+  for (; q < n; q += (int)team_size()) {
+    const BlkPos bp = blk_pos(v, p, e);
+    float2 x[2], inv[2], base[2];
+    if (!POST) load(bp);
+    const int I = (bp.b0 >> 1) - TILE_H / 2 + p.s, J = (bp.b1 - TILE_H + p.y) >> 1,
+              K = (bp.b2 - TILE_H + 2 * p.g) >> 1;  // the two red cells' parent
+    if constexpr (POST) {
+      const float px = ((w.x | w.y) & 0xffffu) ? C.x[level_index(C, I, J, K)] : 0.0f;
+#pragma unroll
+      for (int z = 0; z < 2; ++z)
+        plane(x[0], z) = tab_code(w, z, 0) ? __fmaf_rn(M.omega, px, plane(x0, z)) : 0.0f;
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        const int cnt = code_cnt(tab_code(w, z, c));  // 0 where there is no fluid cell
+        plane(inv[c], z) = s_inv_cnt[cnt];
+        plane(base[c], z) = __fmul_rn(plane(r[c], z), s_inv_scnt[l][cnt]);
+      }
+    if constexpr (!POST) x[0] = base[0];
+    x[1] = make_float2(0.0f, 0.0f);
+    __syncthreads();  // the last block's readers are done
+    T.x[0][threadIdx.x] = x[0];
+    __syncthreads();
+    int reach = 2 * M.nu - 1;
+#pragma unroll 1
+    for (int h = 0; h < M.nu; ++h) {
+      if (p.wdist <= reach) tile_sweep<1>(T, p, x, inv, base);
+      __syncthreads();
+      --reach;
+      if (POST || h + 1 < M.nu) {
+        if (p.wdist <= reach) tile_sweep<0>(T, p, x, inv, base);
+        --reach;
+        if (!POST || h + 1 < M.nu) __syncthreads();
+      }
+    }
+    if (p.own) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int z = 0; z < 2; ++z)
+          if (tab_code(w, z, c)) {
+            xout[c * v.half + bp.gi + z * v.pl] = plane(x[c], z);
+            if constexpr (RZ) acc.add_prod(plane(r[c], z), plane(x[c], z));
+          }
+    }
+    if constexpr (!POST) {
+      if (p.wdist == 0) {
+        // residuals of the red cells (0 where there is no fluid cell)
+        const float2* t = T.x[1] + threadIdx.x;
+        const int d = (p.y & 1) ? 1 : -1;
+        const float2 other = make_float2(t[d].x, t[-d].y), ym = t[-8], yp = t[8];
+        const float zprev = t[-TILE_PLANE].y, znext = t[TILE_PLANE].x;
+        const bool low = (p.y & 1) == 0;  // plane 0: the other slot is the -x neighbour
+        const float xv0[6] = {low ? other.x : x[1].x, low ? x[1].x : other.x, ym.x, yp.x, zprev,
+                              x[1].y};
+        const float xv1[6] = {low ? x[1].y : other.y, low ? other.y : x[1].y, ym.y, yp.y, x[1].x,
+                              znext};
+        const unsigned int c0 = tab_code(w, 0, 0), c1 = tab_code(w, 1, 0);
+        float r0 = resid(v.s, code_cnt(c0), c0, r[0].x, x[0].x, xv0);
+        float r1 = resid(v.s, code_cnt(c1), c1, r[0].y, x[0].y, xv1);
+        r0 = c0 ? r0 : 0.0f;
+        r1 = c1 ? r1 : 0.0f;
+        // b of the coarse cell: restrict_sum's sum over the red children in order, the
+        // (dy = 1) children being the next row's, eight lanes on
+        const float q0 = __shfl_down_sync(0xffffffffu, r0, 8);
+        const float q1 = __shfl_down_sync(0xffffffffu, r1, 8);
+        if (p.own && (p.y & 1) == 0 && I < C.nx && J < C.ny && K < C.nz) {
+          const int ci = level_index(C, I, J, K);
+          const unsigned int cd = C.split ? (unsigned int)Cl.code16[ci] : (unsigned int)Cl.code[ci];
+          if (cd & CODE_SELF) {
+            const float bv =
+                __fmul_rn(__fadd_rn(__fadd_rn(__fadd_rn(r0, q0), r1), q1), 0.0625f);
+            Cl.b[ci] = bv;
+            // the coarse level's first red half-sweep, as in restrict_split
+            if (C.split && ((I + J + K) & 1) == 0) Cl.x[ci] = gs_first(Cl.lvl, code_cnt(cd), bv);
+          }
+        }
+      }
+    }
+    if (q + (int)team_size() < n) {
+      e = L.blk[q + team_size()];
+      w = L.tab[(size_t)(q + team_size()) * PCG_THREADS + threadIdx.x];
+      if (POST) load(blk_pos(v, p, e));
+    }
+  }
+  return PassSum{acc, true};
+}
+
+// ---------------------------------------------------------------- cycle pieces
+
+// Pre-smoothing from zero and restriction, colour-split level l -> l+1.  The
+// first red half-sweep from zero was made by the restriction into level l
+// (restrict_split), behind the barrier that followed it.  Ends arrived at a barrier.
+__device__ __forceinline__ bool down_split(const PcgArgs& A, int l) {
+  const MgArgs& M = A.mg;
+  const MgLevel& L = M.lv[l];
+  const MgLevel& C = M.lv[l + 1];
+  sweep_split<NORMAL>(M, L, C, l, 1, false);
+  if (!gsync(A)) return false;
+  for (int s = 1; s < M.nu; ++s) {
+    sweep_split<NORMAL>(M, L, C, l, 0, false);
+    if (!gsync(A)) return false;
+    sweep_split<NORMAL>(M, L, C, l, 1, false);
+    if (!gsync(A)) return false;
+  }
+  if (C.split) restrict_split(L, C);
+  else restrict_split_nat(L, C);
+  garrive(A);
+  return true;
+}
+
+// Coarse correction from level l+1 and post-smoothing, colour-split level l.  Ends arrived
+// at a barrier.
+__device__ __forceinline__ bool up_split(const PcgArgs& A, int l) {
+  const MgArgs& M = A.mg;
+  const MgLevel& L = M.lv[l];
+  const MgLevel& C = M.lv[l + 1];
+  sweep_split<CORRECT>(M, L, C, l, 1, false);
+  if (!gsync(A)) return false;
+  sweep_split<NORMAL>(M, L, C, l, 0, false);
+  for (int s = 1; s < M.nu; ++s) {
+    if (!gsync(A)) return false;
+    sweep_split<NORMAL>(M, L, C, l, 1, false);
+    if (!gsync(A)) return false;
+    sweep_split<NORMAL>(M, L, C, l, 0, false);
+  }
+  garrive(A);
+  return true;
+}
+
+// ---------------------------------------------------------------- CTA-local levels in tiles
+//
+// Up to three CTA-local levels (their extents are then at most 16, 8 and 4 cells: all
+// but long thin grids) run in the manner of block_pass's tiles, whole level and no halo:
+// the 16^3 level on warps 0..15, the 8^3 level on warps 16 and 17, the 4^3 level on
+// warp 18, each thread with a slot's eight cells in four planes in registers, as float2 a
+// (planes 4 g, 4 g + 2) and b (4 g + 1, 4 g + 3), and the neighbours in shared memory.  A half-sweep waits only for its own level's warps, and the levels hand over
+// by barriers of the two levels' warps.  The values are those of the list form below,
+// sum for sum.
+//
+// Bound by latency: 22 dependent half-sweeps and residuals, and by instruction fetch,
+// since one SM runs this code once per V-cycle: all levels share one copy of it (15 KB),
+// with the level's shape in registers.  With its grid barrier 8.5 us at 64^3 and 11.1 at
+// 256^3, where the solve's other code takes more of the instruction cache; a copy per
+// level with constant shapes (37 KB) took 9.2 and 17.7, the list form 14 and 17-19.
+constexpr int CT_THREADS = 512 + 64 + 8;
+
+// The tile of each level's threads: 8 >> v slots, 16 >> v rows, 4 >> v plane groups; the
+// entries of the arrays below are thread numbers (level v's from ct_first(v)).
+struct CtaTiles {
+  uint4 tab[CT_THREADS];                           // codes
+  float2 a[2][CT_THREADS], b[2][CT_THREADS];       // x by colour (planes 4 g, 4 g + 2; 4 g + 1,
+                                                   // 4 g + 3)
+  float2 ra[2][CT_THREADS], rb[2][CT_THREADS];     // right-hand side, in the same form
+};
+
+__device__ __forceinline__ CtaTiles& cta_tiles();
+
+__device__ __forceinline__ bool cta_tiled(const MgArgs& M) { return M.nlev - M.lgrid <= 3; }
+
+__device__ __forceinline__ int ct_first(int v) { return v == 0 ? 0 : v == 1 ? 512 : 576; }
+
+// A thread's level v (0: up to 16^3 cells, 1: 8^3, 2: 4^3; 3: none) and place in its tile.
+struct CtPos {
+  int v, ns, ny, ng;  // slots, rows, plane groups
+  int s, y, g;
+  bool live;          // owns cells (of the 4^3 level's warp only eight threads do)
+};
+
+__device__ __forceinline__ CtPos ct_pos() {
+  const int id = (int)threadIdx.x;
+  CtPos p;
+  p.v = id < 512 ? 0 : id < 576 ? 1 : id < 608 ? 2 : 3;
+  p.ns = 8 >> p.v;
+  p.ny = 16 >> p.v;
+  p.ng = 4 >> p.v;
+  const int t = id - ct_first(p.v);
+  p.s = t & (p.ns - 1);
+  p.y = (t >> (3 - p.v)) & (p.ny - 1);
+  p.g = t >> (7 - 2 * p.v);
+  p.live = id < CT_THREADS;
+  return p;
+}
+
+// Barrier of level v's warps, or (hand) of the warps of levels v and v + 1.
+__device__ __forceinline__ void ct_sync(int v) {
+  asm volatile("bar.sync %0, %1;" ::"r"(3 + v), "r"(v == 0 ? 512 : v == 1 ? 64 : 32) : "memory");
+}
+__device__ __forceinline__ void ct_hand(int v) {
+  asm volatile("bar.sync %0, %1;" ::"r"(6 + v), "r"(v == 0 ? 512 + 64 : 64 + 32) : "memory");
 }
 
 // Code of plane z (0..3 in the thread's group), colour c.
@@ -883,260 +1158,207 @@ __device__ __forceinline__ float& plane(float2& a, float2& b, int z) {
   return z == 0 ? a.x : z == 1 ? b.x : z == 2 ? a.y : b.y;
 }
 
-// One half-sweep of colour c (compile-time) over the tile: x = inv (sum of the six
-// neighbours) + base.
-template <int c>
-__device__ __forceinline__ void tile_sweep(MgTile& T, const TilePos& p, float2 (&xa)[2],
-                                           float2 (&xb)[2], const float2 (&ia)[2],
-                                           const float2 (&ib)[2], const float2 (&ba)[2],
-                                           const float2 (&bb)[2]) {
-  constexpr int o = 1 - c;
-  if (p.y == 0 || p.y == TILE_W - 1) return;  // the outermost rows are never updated
-  const int t = threadIdx.x & (TILE_THREADS - 1);
-  const int d = ((c + p.y) & 1) ? 1 : -1;
-  const float2* ta = T.a[o] + t;
-  const float2* tb = T.b[o] + t;
-  const float zprev = p.g > 0 ? tb[-TILE_W * 8].y : 0.0f;
-  const float znext = p.g < 3 ? ta[TILE_W * 8].x : 0.0f;
-  float2 sa = __fadd2_rn(xa[o], ta[d]);
-  float2 sb = __fadd2_rn(xb[o], tb[-d]);
-  sa = __fadd2_rn(sa, ta[-8]);
-  sb = __fadd2_rn(sb, tb[-8]);
-  sa = __fadd2_rn(sa, ta[8]);
-  sb = __fadd2_rn(sb, tb[8]);
-  sa = __fadd2_rn(sa, make_float2(zprev, xb[o].x));
-  sb = __fadd2_rn(sb, xa[o]);
-  sa = __fadd2_rn(sa, xb[o]);
-  sb = __fadd2_rn(sb, make_float2(xa[o].y, znext));
-  xa[c] = __ffma2_rn(sa, ia[c], ba[c]);
-  xb[c] = __ffma2_rn(sb, ib[c], bb[c]);
-  T.a[c][t] = xa[c];
-  T.b[c][t] = xb[c];
+// The float of plane z (0..3) of a pair of arrays at entry t.
+__device__ __forceinline__ float& pair_at(float2* a, float2* b, int t, int z) {
+  float2& v = (z & 1) ? b[t] : a[t];
+  return (z & 2) ? v.y : v.x;
 }
 
-// Blocked pre-smoothing and restriction (POST false: level l's b -> its x and level
-// l + 1's b), or blocked correction and post-smoothing (POST true: x and level l + 1's
-// final x -> xout; RZ: b x over the block's cells is added to rz).  The caller meets a
-// grid barrier after it.
-template <bool POST, bool RZ>
-__device__ __noinline__ void block_pass(const MgArgs& M, int l, FF* rz) {
-  const int group = threadIdx.x / TILE_THREADS;
-  MgTile& T = mg_tile(group);
+// The neighbours in colour o's arrays of a thread's cells of colour 1 - o, but for those
+// that are its own cells: along x (oa, ob), y (ma, mb below, pa, pb above), and the
+// plane before and after its four.  Beyond the tile's faces they are 0.
+struct CtNbr {
+  float2 oa, ob, ma, mb, pa, pb;
+  float zprev, znext;
+};
+
+__device__ __forceinline__ CtNbr ct_nbr(const CtaTiles& S, const CtPos& p, int o) {
+  const float2 zero = make_float2(0.0f, 0.0f);
+  const float2* ta = S.a[o] + threadIdx.x;
+  const float2* tb = S.b[o] + threadIdx.x;
+  const bool up = (1 - o + p.y) & 1;  // the a planes' other x neighbour is the next slot
+  const bool lo = p.s > 0, hi = p.s < p.ns - 1;
+  const int pl = p.ns * p.ny;
+  CtNbr n;
+  n.oa = (up ? hi : lo) ? ta[up ? 1 : -1] : zero;
+  n.ob = (up ? lo : hi) ? tb[up ? -1 : 1] : zero;
+  n.ma = p.y > 0 ? ta[-p.ns] : zero;
+  n.mb = p.y > 0 ? tb[-p.ns] : zero;
+  n.pa = p.y < p.ny - 1 ? ta[p.ns] : zero;
+  n.pb = p.y < p.ny - 1 ? tb[p.ns] : zero;
+  n.zprev = p.g > 0 ? tb[-pl].y : 0.0f;
+  n.znext = p.g < p.ng - 1 ? ta[pl].x : 0.0f;
+  return n;
+}
+
+// The same sums as tile_sum, in the same order.
+template <int c>
+__device__ __forceinline__ void ct_sweep(CtaTiles& S, const CtPos& p, float2 (&xa)[2],
+                                         float2 (&xb)[2], const float2 (&ia)[2],
+                                         const float2 (&ib)[2], const float2 (&ba)[2],
+                                         const float2 (&bb)[2]) {
+  constexpr int o = 1 - c;
+  if (!p.live) return;
+  const CtNbr n = ct_nbr(S, p, o);
+  float2 sa = __fadd2_rn(xa[o], n.oa), sb = __fadd2_rn(xb[o], n.ob);
+  sa = __fadd2_rn(sa, n.ma);
+  sb = __fadd2_rn(sb, n.mb);
+  sa = __fadd2_rn(sa, n.pa);
+  sb = __fadd2_rn(sb, n.pb);
+  sa = __fadd2_rn(sa, make_float2(n.zprev, xb[o].x));
+  sb = __fadd2_rn(sb, xa[o]);
+  sa = __fadd2_rn(sa, xb[o]);
+  sb = __fadd2_rn(sb, make_float2(xa[o].y, n.znext));
+  xa[c] = __ffma2_rn(sa, ia[c], ba[c]);
+  xb[c] = __ffma2_rn(sb, ib[c], bb[c]);
+  S.a[c][threadIdx.x] = xa[c];
+  S.b[c][threadIdx.x] = xb[c];
+}
+
+// Levels [lgrid, nlev) inside CTA 0 in tile form, from level lgrid's global b to its
+// global x, as cta_cycle.
+__device__ __noinline__ void cta_cycle_tiled(const MgArgs& M) {
+  const CtPos p = ct_pos();
+  const int l = M.nlev - 3 + p.v;  // the thread's level
+  if (p.v == 3 || l < M.lgrid) return;
+  CtaTiles& S = cta_tiles();
   const MgLevel& L = M.lv[l];
-  const MgLevel& Cl = M.lv[l + 1];
-  const SV v = sview(L);
-  const PV C = pview(Cl);
-  float* xout = POST ? (l == 0 ? s_z0 : L.x2) : v.x;
-  const int* blk = L.blk;
-  const uint4* tab = L.tab + (threadIdx.x & (TILE_THREADS - 1));
-  const float omega = M.omega;
-  const int n = s_nblk[l], step = TILE_GROUPS * (int)team_size();
-  const TilePos p = tile_pos();
-  const int t = threadIdx.x & (TILE_THREADS - 1);
-  FF acc;
-  int q = (int)team_rank() + group * (int)team_size();
-  int e_next = 0;
-  uint4 w_next = make_uint4(0u, 0u, 0u, 0u);
-  if (q < n) {
-    e_next = blk[q];
-    w_next = tab[(size_t)q * TILE_THREADS];
-  }
-  for (; q < n; q += step) {
-    const uint4 w = w_next;
-    const BlkPos bp = blk_pos(v, p, e_next);
-    float2 ra[2], rb[2];  // the right-hand side
-    float2 xa[2], xb[2], ia[2], ib[2], ba[2], bb[2];
+  const bool top = l == M.lgrid, coarsest = p.v == 2;
+  const uint4 w = p.live ? S.tab[threadIdx.x] : make_uint4(0u, 0u, 0u, 0u);
+  const int nat = L.nx * (p.y + L.ny * 4 * p.g) + 2 * p.s, nsl = L.nx * L.ny;  // natural index
+  float2 xa[2], xb[2], ia[2], ib[2], ba[2], bb[2], ra[2], rb[2];
+  if (top) {
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
       for (int z = 0; z < 4; ++z)
-        plane(ra[c], rb[c], z) = tab_code(w, z, c) ? v.b[c * v.half + bp.gi + z * v.pl] : 0.0f;
-    if constexpr (POST) {
-      float2 pa = make_float2(0.0f, 0.0f);  // parents of planes 0, 1 and of 2, 3
-      const int I = (bp.b0 >> 1) - TILE_H / 2 + p.s, J = (bp.b1 - TILE_H + p.y) >> 1,
-                K = (bp.b2 - TILE_H + 4 * p.g) >> 1;
-      if ((w.x | w.y) & 0xffffu) pa.x = C.x[level_index(C, I, J, K)];
-      if ((w.z | w.w) & 0xffffu) pa.y = C.x[level_index(C, I, J, K + 1)];
+        plane(ra[c], rb[c], z) =
+            tab_code(w, z, c) ? L.b[nat + z * nsl + ((c + p.y + z) & 1)] : 0.0f;
+  } else {
+    ct_hand(p.v - 1);  // the finer level's restriction is done
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float2 zero = make_float2(0.0f, 0.0f);
+      ra[c] = p.live ? S.ra[c][threadIdx.x] : zero;
+      rb[c] = p.live ? S.rb[c][threadIdx.x] : zero;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const int cnt = code_cnt(tab_code(w, z, c));  // 0 where there is no fluid cell
+      plane(ia[c], ib[c], z) = s_inv_cnt[cnt];
+      plane(ba[c], bb[c], z) = __fmul_rn(plane(ra[c], rb[c], z), s_inv_scnt[l][cnt]);
+    }
+  xa[0] = ba[0];
+  xb[0] = bb[0];
+  xa[1] = xb[1] = make_float2(0.0f, 0.0f);
+  const int cfirst = ct_first(p.v + 1), cns = p.ns >> 1, cny = p.ny >> 1;  // the coarser tile
+  const int I = p.s, J = p.y >> 1;  // the red cells' parents: (I, J, 2 g) and (I, J, 2 g + 1)
+#pragma unroll 1
+  for (int post = 0;; ++post) {
+    if (p.live) {
+      S.a[0][threadIdx.x] = xa[0];
+      S.b[0][threadIdx.x] = xb[0];
+    }
+    ct_sync(p.v);
+    // the coarsest level: MG_COARSE_SWEEPS (red, black) pairs from zero, then as many
+    // (black, red) pairs, as one alternating sequence (see coarsest_cta)
+    const int pairs = coarsest ? 2 * MG_COARSE_SWEEPS - 1 : M.nu;
+#pragma unroll 1
+    for (int h = 0; h < pairs; ++h) {
+      ct_sweep<1>(S, p, xa, xb, ia, ib, ba, bb);
+      ct_sync(p.v);
+      if (!coarsest && post == 0 && h + 1 == pairs) break;
+      ct_sweep<0>(S, p, xa, xb, ia, ib, ba, bb);
+      ct_sync(p.v);
+    }
+    if (coarsest || post == 1) break;
+    // residuals of the red cells and the coarser level's right-hand side (restrict_cta)
+    float r[4], r1[4];
+    {
+      CtNbr n = ct_nbr(S, p, 1);
 #pragma unroll
       for (int z = 0; z < 4; ++z) {
-        const bool f = tab_code(w, z, 0) != 0u;
-        const float x = f ? v.x[bp.gi + z * v.pl] : 0.0f;
-        plane(xa[0], xb[0], z) = f ? __fmaf_rn(omega, z < 2 ? pa.x : pa.y, x) : 0.0f;
+        const unsigned int cd = tab_code(w, z, 0);
+        const float own = plane(xa[1], xb[1], z), other = plane(n.oa, n.ob, z);
+        const bool low = ((z + p.y) & 1) == 0;  // the other slot is the -x neighbour
+        const float xv[6] = {low ? other : own,
+                             low ? own : other,
+                             plane(n.ma, n.mb, z),
+                             plane(n.pa, n.pb, z),
+                             z == 0 ? n.zprev : plane(xa[1], xb[1], z > 0 ? z - 1 : 0),
+                             z == 3 ? n.znext : plane(xa[1], xb[1], z < 3 ? z + 1 : 3)};
+        const float rr = resid(L.s, code_cnt(cd), cd, plane(ra[0], rb[0], z),
+                               plane(xa[0], xb[0], z), xv);
+        r[z] = cd ? rr : 0.0f;
       }
     }
-    if (q + step < n) {
-      e_next = blk[q + step];
-      w_next = tab[(size_t)(q + step) * TILE_THREADS];
+#pragma unroll
+    for (int z = 0; z < 4; ++z) r1[z] = __shfl_down_sync(0xffffffffu, r[z], p.ns);
+    int pt[2], pz[2];  // the parents' entries and planes
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int K = 2 * p.g + h;
+      pt[h] = cfirst + ((K >> 2) * cny + J) * cns + (I >> 1) + ((I + J + K) & 1) * CT_THREADS;
+      pz[h] = K & 3;
     }
-    // coefficients: a warp whose cells are all interior or 0 takes them without the tables
-    bool plain = true;
+    if ((p.y & 1) == 0) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float sum = __fadd_rn(__fadd_rn(__fadd_rn(r[2 * h], r1[2 * h]), r[2 * h + 1]),
+                                    r1[2 * h + 1]);
+        pair_at(S.ra[0], S.rb[0], pt[h], pz[h]) = __fmul_rn(sum, 0.0625f);
+      }
+    }
+    ct_hand(p.v);  // to the coarser level
+    ct_hand(p.v);  // and back
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      float& x = plane(xa[0], xb[0], z);
+      const float px = pair_at(S.a[0], S.b[0], pt[z >> 1], pz[z >> 1]);
+      x = tab_code(w, z, 0) ? __fmaf_rn(M.omega, px, x) : 0.0f;
+    }
+  }
+  if (top) {
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
-      for (int z = 0; z < 4; ++z) {
-        const unsigned int cd = tab_code(w, z, c);
-        plain = plain && (cd == 0u || cd == CODE_FULL);
-      }
-    if (__all_sync(0xffffffffu, plain)) {
-      const float i6 = s_inv_cnt[6], s6 = s_inv_scnt[l][6];
-#pragma unroll
-      for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int z = 0; z < 4; ++z) {
-          plane(ia[c], ib[c], z) = tab_code(w, z, c) ? i6 : 0.0f;
-          plane(ba[c], bb[c], z) = __fmul_rn(plane(ra[c], rb[c], z), s6);
-        }
-    } else {
-#pragma unroll
-      for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int z = 0; z < 4; ++z) {
-          const int cnt = code_cnt(tab_code(w, z, c));  // 0 where there is no fluid cell
-          plane(ia[c], ib[c], z) = s_inv_cnt[cnt];
-          plane(ba[c], bb[c], z) = __fmul_rn(plane(ra[c], rb[c], z), s_inv_scnt[l][cnt]);
-        }
-    }
-    if constexpr (!POST) {
-      xa[0] = ba[0];
-      xb[0] = bb[0];
-    }
-    tile_sync(group);  // the last block's readers are done
-    T.a[0][t] = xa[0];
-    T.b[0][t] = xb[0];
-    xa[1] = xb[1] = make_float2(0.0f, 0.0f);
-    tile_sync(group);
-    int reach = 2 * M.nu - 1;
-    for (int h = 0; h < M.nu; ++h) {
-      if (p.wdist <= reach) tile_sweep<1>(T, p, xa, xb, ia, ib, ba, bb);
-      tile_sync(group);
-      --reach;
-      if (POST || h + 1 < M.nu) {
-        if (p.wdist <= reach) tile_sweep<0>(T, p, xa, xb, ia, ib, ba, bb);
-        --reach;
-        if (!POST || h + 1 < M.nu) tile_sync(group);
-      }
-    }
-    if (p.own) {
-#pragma unroll
-      for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int z = 0; z < 4; ++z)
-          if (tab_code(w, z, c)) {
-            const int gi = c * v.half + bp.gi + z * v.pl;
-            const float x = plane(xa[c], xb[c], z);
-            xout[gi] = x;
-            if constexpr (RZ) acc.add_prod(v.b[gi], x);
-          }
-    }
-    if constexpr (!POST) {
-      if (p.wdist == 0) {
-        // residuals of the red cells (0 where there is no fluid cell)
-        float r[4];
-        const int d = (p.y & 1) ? 1 : -1;
-        const float2* ta = T.a[1] + t;
-        const float2* tb = T.b[1] + t;
-        const float2 xoa = ta[d], xob = tb[-d], yma = ta[-8], ymb = tb[-8], ypa = ta[8],
-                     ypb = tb[8];
-        const float zprev = tb[-TILE_W * 8].y, znext = ta[TILE_W * 8].x;
-        bool full = true;
-#pragma unroll
-        for (int z = 0; z < 4; ++z) full = full && tab_code(w, z, 0) == CODE_FULL;
-        full = __all_sync(0xffffffffu, full || !p.own);
-#pragma unroll
-        for (int z = 0; z < 4; ++z) {
-          const unsigned int cd = tab_code(w, z, 0);
-          const float x = plane(xa[0], xb[0], z);
-          const float own = plane(xa[1], xb[1], z);
-          float2 oa = xoa, ob = xob, ma = yma, mb = ymb, pa = ypa, pb = ypb;
-          const float other = plane(oa, ob, z);
-          const bool low = ((z + p.y) & 1) == 0;  // the other slot is the -x neighbour
-          const float xv[6] = {low ? other : own,
-                               low ? own : other,
-                               plane(ma, mb, z),
-                               plane(pa, pb, z),
-                               z == 0 ? zprev : plane(xa[1], xb[1], z > 0 ? z - 1 : 0),
-                               z == 3 ? znext : plane(xa[1], xb[1], z < 3 ? z + 1 : 3)};
-          const float bv = plane(ra[0], rb[0], z);
-          if (full) r[z] = resid_full(v.s, bv, x, xv);
-          else r[z] = cd ? resid(v.s, code_cnt(cd), cd, bv, x, xv) : 0.0f;
-        }
-        // b of the coarse cells: restrict_sum's sum over the red children in order, the
-        // (dy = 1) children being the next row's, eight lanes on
-        float r1[4];
-#pragma unroll
-        for (int z = 0; z < 4; ++z) r1[z] = __shfl_down_sync(0xffffffffu, r[z], 8);
-        if (p.own && (p.y & 1) == 0) {
-          const int I = (bp.b0 >> 1) - TILE_H / 2 + p.s, J = (bp.b1 - TILE_H + p.y) >> 1,
-                    K0 = (bp.b2 - TILE_H + 4 * p.g) >> 1;
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int K = K0 + h;
-            if (I >= C.nx || J >= C.ny || K >= C.nz) continue;
-            const int ci = level_index(C, I, J, K);
-            const unsigned int cd = C.split ? (unsigned int)Cl.code16[ci] : (unsigned int)Cl.code[ci];
-            if (!(cd & CODE_SELF)) continue;
-            const float sum = __fadd_rn(__fadd_rn(__fadd_rn(r[2 * h], r1[2 * h]), r[2 * h + 1]),
-                                        r1[2 * h + 1]);
-            const float bv = __fmul_rn(sum, 0.0625f);
-            Cl.b[ci] = bv;
-            // the coarse level's first red half-sweep, as in restrict_split
-            if (C.split && ((I + J + K) & 1) == 0) Cl.x[ci] = gs_first(Cl.lvl, code_cnt(cd), bv);
-          }
-        }
-      }
-    }
-  }
-  if constexpr (RZ) {
-    rz->add_prod(acc.hi, 1.0f);
-    rz->add_prod(acc.lo, 1.0f);
+      for (int z = 0; z < 4; ++z)
+        if (tab_code(w, z, c))
+          L.x[nat + z * nsl + ((c + p.y + z) & 1)] = plane(xa[c], xb[c], z);
+  } else {
+    ct_hand(p.v - 1);  // x is in shared memory for the finer level
   }
 }
 
-// ---------------------------------------------------------------- cycle pieces
-
-__device__ __forceinline__ bool gsync(const PcgArgs& A) {
-  return grid_barrier(A.bar, A.status, team_size(), A.timeout_ns);
-}
-
-// Pre-smoothing from zero and restriction, colour-split level l -> l+1.  The
-// first red half-sweep from zero was made by the restriction into level l
-// (restrict_split), behind the barrier that followed it.
-__device__ __forceinline__ bool down_split(const PcgArgs& A, int l) {
-  const MgArgs& M = A.mg;
+// Once per solve, after build_levels: CTA 0's codes, code bits plus the count of
+// neighbours inside the grid, 0 where there is no fluid cell; x starts as 0.
+__device__ __noinline__ void cta_tiles_init(const MgArgs& M) {
+  const CtPos p = ct_pos();
+  const int l = M.nlev - 3 + p.v;
+  if (!p.live || l < M.lgrid) return;
+  CtaTiles& S = cta_tiles();
   const MgLevel& L = M.lv[l];
-  const MgLevel& C = M.lv[l + 1];
-  sweep_split<NORMAL>(M, L, C, l, 1, nullptr);
-  if (!gsync(A)) return false;
-  for (int s = 1; s < M.nu; ++s) {
-    sweep_split<NORMAL>(M, L, C, l, 0, nullptr);
-    if (!gsync(A)) return false;
-    sweep_split<NORMAL>(M, L, C, l, 1, nullptr);
-    if (!gsync(A)) return false;
+  unsigned int cd[4];
+#pragma unroll
+  for (int z = 0; z < 4; ++z) {
+    cd[z] = 0u;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int i = 2 * p.s + ((c + p.y + z) & 1), j = p.y, k = 4 * p.g + z;
+      if (i >= L.nx || j >= L.ny || k >= L.nz) continue;
+      const unsigned int code = L.code[i + L.nx * (j + L.ny * k)];
+      const int cnt = (i > 0) + (i < L.nx - 1) + (j > 0) + (j < L.ny - 1) + (k > 0) +
+                      (k < L.nz - 1);
+      if (code & CODE_SELF) cd[z] |= (code | (unsigned)cnt << 8) << (16 * c);
+    }
   }
-  if (C.split) restrict_split(L, C);
-  else restrict_split_nat(L, C);
-  return gsync(A);
+  S.tab[threadIdx.x] = make_uint4(cd[0], cd[1], cd[2], cd[3]);
 }
 
-// Coarse correction from level l+1 and post-smoothing, colour-split level l.
-__device__ __forceinline__ bool up_split(const PcgArgs& A, int l) {
-  const MgArgs& M = A.mg;
-  const MgLevel& L = M.lv[l];
-  const MgLevel& C = M.lv[l + 1];
-  sweep_split<CORRECT>(M, L, C, l, 1, nullptr);
-  if (!gsync(A)) return false;
-  sweep_split<NORMAL>(M, L, C, l, 0, nullptr);
-  if (!gsync(A)) return false;
-  for (int s = 1; s < M.nu; ++s) {
-    sweep_split<NORMAL>(M, L, C, l, 1, nullptr);
-    if (!gsync(A)) return false;
-    sweep_split<NORMAL>(M, L, C, l, 0, nullptr);
-    if (!gsync(A)) return false;
-  }
-  return true;
-}
-
-// ---------------------------------------------------------------- CTA-local levels
+// ---------------------------------------------------------------- CTA-local levels by lists
 
 // The CTA-local levels [lgrid, nlev) live in CTA 0's (dynamic) shared memory:
 // x, b and the neighbour codes of every such level (MG_CTA_CELLS cells in all),
@@ -1163,6 +1385,13 @@ struct CtaMg {
 __device__ __forceinline__ CtaMg& cta_mg() {
   extern __shared__ __align__(16) unsigned char mg_dyn[];
   return *reinterpret_cast<CtaMg*>(mg_dyn);
+}
+
+// The tile form's arrays lie in the same place.
+__device__ __forceinline__ CtaTiles& cta_tiles() {
+  static_assert(sizeof(CtaTiles) <= sizeof(CtaMg), "shares the list form's memory");
+  extern __shared__ __align__(16) unsigned char mg_dyn[];
+  return *reinterpret_cast<CtaTiles*>(mg_dyn);
 }
 
 __device__ __forceinline__ int bits_for(int n) {  // bits of n - 1 (0 for n = 1)
@@ -1443,91 +1672,100 @@ __device__ __noinline__ void cta_cycle(const PcgArgs& A) {
 
 // z = V(r), given that the first red half-sweep of level 0 (from zero) has been
 // done in the phase that produced r, and that a grid barrier has passed since.
-// The last black and the last red half-sweeps of level 0 accumulate r.z over
-// their cells into rz.  The caller publishes rz and meets the next barrier.
-// Returns false if a barrier failed.
-__device__ bool vcycle_rest(const PcgArgs& A, FF& rz) {
+// Returns r.z over the CTA's cells, from the last black and the last red half-sweeps of
+// level 0 (the caller publishes it and meets the next barrier); ok is false if a barrier
+// failed.
+__device__ __noinline__ PassSum vcycle_rest(const PcgArgs& A) {
+  PassSum V{FF(), false};
   const MgArgs& M = A.mg;
   const MgLevel& L0 = M.lv[0];
   if (M.nlev == 1) {  // level 0 is the coarsest level
     // rest of the pre pairs (red, black) after the fused first red half-sweep
     for (int s = 0; s < MG_COARSE_SWEEPS; ++s) {
-      sweep_split<NORMAL>(M, L0, L0, 0, 1, nullptr);
-      if (!gsync(A)) return false;
+      sweep_split<NORMAL>(M, L0, L0, 0, 1, false);
+      if (!gsync(A)) return V;
       if (s + 1 < MG_COARSE_SWEEPS) {
-        sweep_split<NORMAL>(M, L0, L0, 0, 0, nullptr);
-        if (!gsync(A)) return false;
+        sweep_split<NORMAL>(M, L0, L0, 0, 0, false);
+        if (!gsync(A)) return V;
       }
     }
     // post pairs (black, red); the last black and the last red give r.z
     for (int s = 0; s < MG_COARSE_SWEEPS; ++s) {
-      sweep_split<NORMAL>(M, L0, L0, 0, 1, s + 1 == MG_COARSE_SWEEPS ? &rz : nullptr);
-      if (!gsync(A)) return false;
+      V.sum = sweep_split<NORMAL>(M, L0, L0, 0, 1, s + 1 == MG_COARSE_SWEEPS);
+      if (!gsync(A)) return V;
       if (s + 1 < MG_COARSE_SWEEPS) {
-        sweep_split<NORMAL>(M, L0, L0, 0, 0, nullptr);
-        if (!gsync(A)) return false;
+        sweep_split<NORMAL>(M, L0, L0, 0, 0, false);
+        if (!gsync(A)) return V;
       }
     }
-    sweep_split<NORMAL>(M, L0, L0, 0, 0, &rz);
-    return true;
+    V.sum.add(sweep_split<NORMAL>(M, L0, L0, 0, 0, true));
+    V.ok = true;
+    return V;
   }
   const MgLevel& L1 = M.lv[1];
   const bool blocked0 = s_nblk[0] > 0;
   if (blocked0) {
-    block_pass<false, false>(M, 0, nullptr);
+    if (!block_pass<false, false>(A, 0, false).ok) return V;
   } else {
-    sweep_split<NORMAL>(M, L0, L1, 0, 1, nullptr);
-    if (!gsync(A)) return false;
+    sweep_split<NORMAL>(M, L0, L1, 0, 1, false);
+    if (!gsync(A)) return V;
     SOLVE_TRACE(TR_V_PRE1);
     for (int s = 1; s < M.nu; ++s) {
-      sweep_split<NORMAL>(M, L0, L1, 0, 0, nullptr);
-      if (!gsync(A)) return false;
-      sweep_split<NORMAL>(M, L0, L1, 0, 1, nullptr);
-      if (!gsync(A)) return false;
+      sweep_split<NORMAL>(M, L0, L1, 0, 0, false);
+      if (!gsync(A)) return V;
+      sweep_split<NORMAL>(M, L0, L1, 0, 1, false);
+      if (!gsync(A)) return V;
     }
     SOLVE_TRACE(TR_V_PRE);
     if (L1.split) restrict_split(L0, L1);
     else restrict_split_nat(L0, L1);
   }
-  if (!gsync(A)) return false;
-  SOLVE_TRACE(TR_V_RESTRICT);
+  garrive(A);  // from here to level 0, every pass waits for the barrier before it
   for (int l = 1; l < M.lgrid; ++l) {
     if (s_nblk[l] > 0) {
-      block_pass<false, false>(M, l, nullptr);
-      if (!gsync(A)) return false;
-    } else if (!down_split(A, l)) {
-      return false;
+      if (!block_pass<false, false>(A, l, true).ok) return V;
+      SOLVE_TRACE(l == 1 ? TR_V_RESTRICT : TR_V_DOWN + min(l - 1, 11));
+      garrive(A);
+    } else {
+      if (!gwait(A)) return V;
+      SOLVE_TRACE(l == 1 ? TR_V_RESTRICT : TR_V_DOWN + min(l - 1, 11));
+      if (!down_split(A, l)) return V;
     }
-    SOLVE_TRACE(TR_V_DOWN + min(l, 11));
   }
-  if (team_rank() == 0) cta_cycle(A);
-  if (!gsync(A)) return false;
-  SOLVE_TRACE(TR_V_CTA);
+  if (!gwait(A)) return V;
+  SOLVE_TRACE(M.lgrid == 1 ? TR_V_RESTRICT : TR_V_DOWN + min(M.lgrid - 1, 11));
+  if (team_rank() == 0) {
+    if (cta_tiled(M)) cta_cycle_tiled(M);
+    else cta_cycle(A);
+  }
+  garrive(A);
   for (int l = M.lgrid - 1; l >= 1; --l) {
     if (s_nblk[l] > 0) {
-      block_pass<true, false>(M, l, nullptr);
-      if (!gsync(A)) return false;
-    } else if (!up_split(A, l)) {
-      return false;
+      if (!block_pass<true, false>(A, l, true).ok) return V;
+      SOLVE_TRACE(l == M.lgrid - 1 ? TR_V_CTA : TR_V_UP + min(l + 1, 11));
+      garrive(A);
+    } else {
+      if (!gwait(A)) return V;
+      SOLVE_TRACE(l == M.lgrid - 1 ? TR_V_CTA : TR_V_UP + min(l + 1, 11));
+      if (!up_split(A, l)) return V;
     }
-    SOLVE_TRACE(TR_V_UP + min(l, 11));
   }
-  if (blocked0) {
-    block_pass<true, true>(M, 0, &rz);
-    return true;
-  }
-  sweep_split<CORRECT>(M, L0, L1, 0, 1, M.nu == 1 ? &rz : nullptr);
-  if (!gsync(A)) return false;
+  if (blocked0) return block_pass<true, true>(A, 0, true);
+  if (!gwait(A)) return V;
+  SOLVE_TRACE(M.lgrid == 1 ? TR_V_CTA : TR_V_UP + 1);
+  V.sum = sweep_split<CORRECT>(M, L0, L1, 0, 1, M.nu == 1);
+  if (!gsync(A)) return V;
   SOLVE_TRACE(TR_V_CORRECT);
   for (int s = 1; s < M.nu; ++s) {
-    sweep_split<NORMAL>(M, L0, L1, 0, 0, nullptr);
-    if (!gsync(A)) return false;
-    sweep_split<NORMAL>(M, L0, L1, 0, 1, s + 1 == M.nu ? &rz : nullptr);
-    if (!gsync(A)) return false;
+    sweep_split<NORMAL>(M, L0, L1, 0, 0, false);
+    if (!gsync(A)) return V;
+    V.sum = sweep_split<NORMAL>(M, L0, L1, 0, 1, s + 1 == M.nu);
+    if (!gsync(A)) return V;
   }
   SOLVE_TRACE(TR_V_POST);
-  sweep_split<NORMAL>(M, L0, L1, 0, 0, &rz);  // the last red half-sweep
-  return true;
+  V.sum.add(sweep_split<NORMAL>(M, L0, L1, 0, 0, true));  // the last red half-sweep
+  V.ok = true;
+  return V;
 }
 
 // ---------------------------------------------------------------- level-0 passes
@@ -1535,8 +1773,7 @@ __device__ bool vcycle_rest(const PcgArgs& A, FF& rz) {
 // Phase A with z from the V-cycle: p_new = z + beta p_old (recomputed for the
 // neighbours), q = A p_new in difference form, partial p.q.  Both colours; paired
 // form.
-__device__ __noinline__ void phase_a_v(const PcgArgs& A, const float* pold, float* pnew, float beta,
-                                     FF& pq) {
+__device__ __noinline__ FF phase_a_v(const PcgArgs& A, const float* pold, float* pnew, float beta) {
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
   const float* z = s_z0;
@@ -1601,13 +1838,12 @@ __device__ __noinline__ void phase_a_v(const PcgArgs& A, const float* pold, floa
       *reinterpret_cast<float2*>(q0 + e.idx) = make_float2(qn[0], qn[1]);
     }
   }
-  pq.add_prod(acc.hi, 1.0f);
-  pq.add_prod(acc.lo, 1.0f);
+  return acc;
 }
 
 // Phase B: d += alpha p, r -= alpha q, partial r.r, and the next V-cycle's first
 // red half-sweep (from zero) z = r / (s n) on red cells.  Both colours.
-__device__ __noinline__ void phase_b_v(const PcgArgs& A, const float* pnew, float alpha, FF& rr) {
+__device__ __noinline__ FF phase_b_v(const PcgArgs& A, const float* pnew, float alpha) {
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
   float* d0 = M.d0;
@@ -1680,14 +1916,12 @@ __device__ __noinline__ void phase_b_v(const PcgArgs& A, const float* pnew, floa
             *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(zn[0], zn[1]);
         }
       });
-  rr.add_prod(acc.hi, 1.0f);
-  rr.add_prod(acc.lo, 1.0f);
+  return acc;
 }
 
 // Phase A with z from the V-cycle: p_new = z + beta p_old (recomputed for the
 // neighbours), q = A p_new in difference form, partial p.q.  Both colours.
-__device__ __noinline__ void phase_a_s(const PcgArgs& A, const float* pold, float* pnew, float beta,
-                                     FF& pq) {
+__device__ __noinline__ FF phase_a_s(const PcgArgs& A, const float* pold, float* pnew, float beta) {
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
   const float* z = s_z0;
@@ -1740,13 +1974,12 @@ __device__ __noinline__ void phase_a_s(const PcgArgs& A, const float* pold, floa
         q0[s.idx] = qc;
         acc.add_prod(pc, qc);
       });
-  pq.add_prod(acc.hi, 1.0f);
-  pq.add_prod(acc.lo, 1.0f);
+  return acc;
 }
 
 // Phase B: d += alpha p, r -= alpha q, partial r.r, and the next V-cycle's first
 // red half-sweep (from zero) z = r / (s n) on red cells.  Both colours.
-__device__ __noinline__ void phase_b_s(const PcgArgs& A, const float* pnew, float alpha, FF& rr) {
+__device__ __noinline__ FF phase_b_s(const PcgArgs& A, const float* pnew, float alpha) {
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
   float* d0 = M.d0;
@@ -1785,19 +2018,16 @@ __device__ __noinline__ void phase_b_s(const PcgArgs& A, const float* pnew, floa
         if (first_red && s.c == 0) v.x[s.idx] = gs_first(0, code_cnt(s.code), rc);
         acc.add_prod(rc, rc);
       });
-  rr.add_prod(acc.hi, 1.0f);
-  rr.add_prod(acc.lo, 1.0f);
+  return acc;
 }
 
-__device__ __forceinline__ void phase_a(const PcgArgs& A, const float* pold, float* pnew,
-                                        float beta, FF& pq) {
-  if (use_pairs(A.mg.lv[0])) phase_a_v(A, pold, pnew, beta, pq);
-  else phase_a_s(A, pold, pnew, beta, pq);
+__device__ __forceinline__ FF phase_a(const PcgArgs& A, const float* pold, float* pnew,
+                                      float beta) {
+  return use_pairs(A.mg.lv[0]) ? phase_a_v(A, pold, pnew, beta) : phase_a_s(A, pold, pnew, beta);
 }
 
-__device__ __forceinline__ void phase_b(const PcgArgs& A, const float* pnew, float alpha, FF& rr) {
-  if (use_pairs(A.mg.lv[0])) phase_b_v(A, pnew, alpha, rr);
-  else phase_b_s(A, pnew, alpha, rr);
+__device__ __forceinline__ FF phase_b(const PcgArgs& A, const float* pnew, float alpha) {
+  return use_pairs(A.mg.lv[0]) ? phase_b_v(A, pnew, alpha) : phase_b_s(A, pnew, alpha);
 }
 
 // One pass over this thread's fluid cells of level 0, both colours (start of the
@@ -1853,10 +2083,10 @@ __device__ __forceinline__ bool seg_active(const PcgArgs& A, const MgLevel& L, i
 }
 
 // Whether a level with n blocks holding fluid is smoothed blocked.  The line: a block
-// takes ~1.2 us of a CTA (two at a time), a pass-by-pass half-sweep ~3.3 us plus the
-// cells' own time.  Solves with the limit at 2, 4, 6 and 10 blocks per CTA: 101 x 67 x 83
-// pool 1.63, 1.51, 1.51, 1.51 ms; 128^3 dam break (3.4 blocks) 1.29, 1.27, 1.28, 1.28;
-// 128^3 pool (8.7 blocks) 1.80, 1.81, 1.81, 2.02.
+// takes ~2 us of a CTA, a pass-by-pass half-sweep ~3.3 us plus the cells' own time.  Solves
+// with the limit at 3, 6, 10 and 16 blocks per CTA: 128^3 dam break (3.4 blocks) 1.03, 1.00,
+// 1.00, 0.98 ms; 128^3 pool (8.7 blocks) 1.52, 1.52, 1.79, 1.80; 256^3 pool (level 1: 8.4
+// blocks) 5.29, 5.29, 5.55, 5.54; 101 x 67 x 83 pool 1.28, 1.20, 1.21, 1.23.
 __device__ __forceinline__ bool blocked(const MgArgs& M, unsigned int n) {
   return M.nlev > 1 && M.nu <= BLK_MAX_NU && n > 0u && n <= (unsigned)MG_BLK_PER_CTA * team_size();
 }
@@ -1888,37 +2118,33 @@ __device__ __forceinline__ void block_lists(const PcgArgs& A) {
 }
 
 // The codes that each thread of a block's tile works with (MgLevel::tab): those of its
-// eight cells within L1 distance TILE_H of the block, 0 elsewhere, off the grid and
-// where there is no fluid.  A thread's cells lie in one of the 27 blocks around, and
-// codes are this solve's only where that block holds fluid.
+// four cells within L1 distance TILE_H of the block, 0 elsewhere, off the grid and where
+// there is no fluid.  A thread's cells lie in one of the 27 blocks around, and codes are
+// this solve's only where that block holds fluid.
 __device__ __noinline__ void block_tables(const PcgArgs& A) {
   const MgArgs& M = A.mg;
   const TilePos p = tile_pos();
-  const int group = threadIdx.x / TILE_THREADS, t = threadIdx.x & (TILE_THREADS - 1);
-  const int nbx = ((p.s + 2) >> 2) - 1, nby = ((p.y + 4) >> 3) - 1, nbz = ((p.g + 1) >> 1) - 1;
+  const int nbx = ((p.s + 2) >> 2) - 1, nby = ((p.y + 4) >> 3) - 1, nbz = ((p.g + 2) >> 2) - 1;
   for (int l = 0; l < M.lgrid; ++l) {
     const MgLevel& L = M.lv[l];
     const SV v = sview(L);
     const int nz = L.nz;
-    for (int q = (int)team_rank() + group * (int)team_size(); q < s_nblk[l];
-         q += TILE_GROUPS * (int)team_size()) {
+    for (int q = (int)team_rank(); q < s_nblk[l]; q += (int)team_size()) {
       const int e = L.blk[q];
       const BlkPos bp = blk_pos(v, p, e);
       const int x = (e & 255) + nbx, y = ((e >> 8) & 255) + nby, z = (e >> 16) + nbz;
-      uint4 w = make_uint4(0u, 0u, 0u, 0u);
       bool any = x >= 0 && y >= 0 && z >= 0 && x < L.nbx && y < L.nby && z < L.nbz;
       if (any) {
         const int b = x + L.nbx * (y + L.nby * z);
         any = l == 0 ? A.brick_fluid[b] > 0u : L.bflag[b] != 0;
       }
       const int j = bp.b1 - TILE_H + p.y;
+      unsigned int cd[2] = {0u, 0u};
       if (any && j < v.ny) {
-        unsigned int cd[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int k = bp.b2 - TILE_H + 4 * p.g + u;
-          const int dyz = tile_dist(p.y) + tile_dist(4 * p.g + u);
-          cd[u] = 0u;
+        for (int u = 0; u < 2; ++u) {
+          const int k = bp.b2 - TILE_H + 2 * p.g + u;
+          const int dyz = tile_dist(p.y) + tile_dist(2 * p.g + u);
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             const int tx = 2 * p.s + ((c + p.y + u) & 1), i = bp.b0 - TILE_H + tx;
@@ -1928,9 +2154,8 @@ __device__ __noinline__ void block_tables(const PcgArgs& A) {
             }
           }
         }
-        w = make_uint4(cd[0], cd[1], cd[2], cd[3]);
       }
-      L.tab[(size_t)q * TILE_THREADS + t] = w;
+      L.tab[(size_t)q * PCG_THREADS + threadIdx.x] = make_uint2(cd[0], cd[1]);
     }
   }
 }
@@ -2094,10 +2319,10 @@ __device__ __noinline__ void seg_cache_fill(const MgArgs& M, unsigned int* cache
 }
 
 // The shared-memory cache of the segment slices sits after the CTA-local levels
-// in the kernel's dynamic shared memory, the tiles of the blocked smoothing after it.
+// in the kernel's dynamic shared memory, the tile of the blocked smoothing after it.
 constexpr size_t MG_DYN_CTA = (sizeof(CtaMg) + 15) / 16 * 16;
 constexpr size_t MG_DYN_TILE = MG_DYN_CTA + sizeof(unsigned int) * SEG_CACHE;
-constexpr size_t MG_DYN_BYTES = MG_DYN_TILE + TILE_GROUPS * sizeof(MgTile);
+constexpr size_t MG_DYN_BYTES = MG_DYN_TILE + sizeof(MgTile);
 // one carve-out step up (132 KB) would take L1 from the level-0 passes
 static_assert(MG_DYN_BYTES + 4096 <= 100 * 1024, "the kernel stays in the 100 KB carve-out");
 
@@ -2105,9 +2330,9 @@ __device__ __forceinline__ unsigned int* seg_cache_of(unsigned char* dyn) {
   return reinterpret_cast<unsigned int*>(dyn + MG_DYN_CTA);
 }
 
-__device__ __forceinline__ MgTile& mg_tile(int group) {
+__device__ __forceinline__ MgTile& mg_tile() {
   extern __shared__ __align__(16) unsigned char mg_dyn[];
-  return reinterpret_cast<MgTile*>(mg_dyn + MG_DYN_TILE)[group];
+  return *reinterpret_cast<MgTile*>(mg_dyn + MG_DYN_TILE);
 }
 
 // The mixed mode's refinement, over level 0's slot pairs with two items in flight
@@ -2157,7 +2382,7 @@ __device__ __noinline__ void refine_update(const PcgArgs& A) {
 
 // refine_residual: r = b - A x in float pairs (residual_pair_cell) on fluid cells,
 // the next V-cycle's first red half-sweep z = r / (s n) on red ones, and r.r.
-__device__ __noinline__ void refine_residual(const PcgArgs& A, FF& rr) {
+__device__ __noinline__ FF refine_residual(const PcgArgs& A) {
   const MgArgs& M = A.mg;
   const MgLevel& L0 = M.lv[0];
   const SV v = sview(L0);
@@ -2219,8 +2444,7 @@ __device__ __noinline__ void refine_residual(const PcgArgs& A, FF& rr) {
       acc.add_prod(r32, r32);
     }
   }
-  rr.add_prod(acc.hi, 1.0f);
-  rr.add_prod(acc.lo, 1.0f);
+  return acc;
 }
 
 struct SolveState {
@@ -2248,7 +2472,10 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, Solve
   seg_cache_fill(M, segc);
   SOLVE_TRACE(TR_SEG_CACHE);
   block_tables(A);  // visible to the V-cycles after the start pass's barrier
-  if (M.nlev > 1 && team_rank() == 0) cta_levels_init(M);
+  if (M.nlev > 1 && team_rank() == 0) {
+    if (cta_tiled(M)) cta_tiles_init(M);
+    else cta_levels_init(M);
+  }
   SOLVE_TRACE(TR_CTA_LISTS);
   // ---- start: r = b (cold) or b - A x0 (warm start from the last solve's x),
   // p_old = 0, first red half-sweep of the V-cycle; mixed mode: b as a float pair,
@@ -2306,7 +2533,8 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, Solve
   }
   if (!gsync(A)) { S.ok = false; return; }
   SOLVE_TRACE(TR_START);
-  double rz = 0.0, bnorm = 0.0, rnorm = 0.0, rmax = 0.0;
+  // thread 0's, in shared memory to keep every thread's registers free
+  double &rz = sh.dscal[0], &bnorm = sh.dscal[1], &rnorm = sh.dscal[2], &rmax = sh.dscal[3];
   const double target = MIXED ? A.ir_tol : A.tol;
   {
     double s0[2];
@@ -2323,10 +2551,10 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, Solve
   float* pold = M.pa0;
   float* pnew = M.pb0;
   while (!conv) {
-    FF rzp;
-    if (!vcycle_rest(A, rzp)) { S.ok = false; return; }
+    const PassSum V = vcycle_rest(A);
+    if (!V.ok) { S.ok = false; return; }
     {
-      F2 v[1] = {f2_of(rzp)};
+      F2 v[1] = {f2_of(V.sum)};
       publish<1>(A, 3, v, sh);
     }
     if (!gsync(A)) { S.ok = false; return; }
@@ -2347,8 +2575,7 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, Solve
     ++it;
     const float beta = sh.beta;
     // ---- phase A
-    FF pq;
-    phase_a(A, pold, pnew, beta, pq);
+    const FF pq = phase_a(A, pold, pnew, beta);
     {
       F2 v[1] = {f2_of(pq)};
       publish<1>(A, 0, v, sh);
@@ -2363,8 +2590,7 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, Solve
     __syncthreads();
     const float alpha = sh.alpha;
     // ---- phase B (+ the next V-cycle's first red half-sweep)
-    FF rr;
-    phase_b(A, pnew, alpha, rr);
+    const FF rr = phase_b(A, pnew, alpha);
     {
       F2 v[1] = {f2_of(rr)};
       publish<1>(A, 1, v, sh);
@@ -2392,14 +2618,15 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, Solve
         refine_update(A);
         if (!gsync(A)) { S.ok = false; return; }
         if (refinements == 0) SOLVE_TRACE(TR_REFINE + 1);
-        FF rr64;
-        refine_residual(A, rr64);
-        F2 v[1] = {f2_of(rr64)};
-        publish<1>(A, 5, v, sh);
+        const FF rr64 = refine_residual(A);
+        {
+      F2 v[1] = {f2_of(rr64)};
+      publish<1>(A, 5, v, sh);
+    }
         if (!gsync(A)) { S.ok = false; return; }
         if (refinements == 0) SOLVE_TRACE(TR_REFINE + 2);
         double s[1];
-        gather<1>(A, 5, s, sh);
+      gather<1>(A, 5, s, sh);
         ++refinements;
         if (threadIdx.x == 0) {
           rnorm = sqrt(fmax(s[0], 0.0));
@@ -2437,8 +2664,10 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, Solve
   S.iters = it;
   S.refinements = refinements;
   S.conv = conv;
-  S.rel = bnorm > 0.0 ? rnorm / bnorm : 0.0;
-  S.bnorm = bnorm;
+  if (threadIdx.x == 0) {
+    S.rel = bnorm > 0.0 ? rnorm / bnorm : 0.0;
+    S.bnorm = bnorm;
+  }
 }
 
 // The paper's GPU solver (Sec. 3.2.3): red-black Gauss-Seidel sweeps on A p = b
@@ -2482,9 +2711,9 @@ __device__ __noinline__ void solve_rbgs(const PcgArgs& A, Shared& sh, unsigned i
   int it = 0;
   while (!conv) {
     for (int k = 0; k < RBGS_CHECK; ++k) {
-      sweep_split<NORMAL>(M, L0, L1, 0, 0, nullptr);
+      sweep_split<NORMAL>(M, L0, L1, 0, 0, false);
       if (!gsync(A)) { S.ok = false; return; }
-      sweep_split<NORMAL>(M, L0, L1, 0, 1, nullptr);
+      sweep_split<NORMAL>(M, L0, L1, 0, 1, false);
       if (!gsync(A)) { S.ok = false; return; }
     }
     it += RBGS_CHECK;
@@ -2554,15 +2783,30 @@ __device__ void solve_scene_mg(const PcgArgs& A, Shared& sh, unsigned char* dyn)
   }
 }
 
+// The scene's arguments in shared memory.  The passes take them by reference; read from
+// the parameter space (or, in a batch, from global memory) through that reference, the
+// level descriptions would cost every pass an L2 round trip, since a grid barrier's
+// acquire empties L1.
+__shared__ PcgArgs s_args;
+
+__device__ __forceinline__ void load_args(const PcgArgs& A) {
+  static_assert(sizeof(PcgArgs) % 8 == 0 && alignof(PcgArgs) == 8, "copied by 8-byte words");
+  const unsigned long long* src = reinterpret_cast<const unsigned long long*>(&A);
+  unsigned long long* dst = reinterpret_cast<unsigned long long*>(&s_args);
+  for (int i = threadIdx.x; i < (int)(sizeof(PcgArgs) / 8); i += PCG_THREADS) dst[i] = src[i];
+  __syncthreads();
+}
+
 template <bool MIXED>
 __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg_mg(const __grid_constant__ PcgArgs A) {
   __shared__ Shared sh;
   extern __shared__ __align__(16) unsigned char mg_dyn[];
   team_enter(blockIdx.x, gridDim.x);
   SOLVE_TRACE(TR_ENTRY);
-  load_tables(A.mg);
+  load_args(A);
+  load_tables(s_args.mg);
   SOLVE_TRACE(TR_TABLES);
-  solve_scene_mg<MIXED>(A, sh, mg_dyn);
+  solve_scene_mg<MIXED>(s_args, sh, mg_dyn);
   SOLVE_TRACE(TR_EXIT);
 }
 
@@ -2574,8 +2818,9 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg_mg_batch(const __grid_co
   extern __shared__ __align__(16) unsigned char mg_dyn[];
   const int s = B.block_scene[blockIdx.x];
   team_enter(blockIdx.x - B.team_first[s], B.team_first[s + 1] - B.team_first[s]);
-  load_tables(B.args[s].mg);
-  solve_scene_mg<MIXED>(B.args[s], sh, mg_dyn);
+  load_args(B.args[s]);
+  load_tables(s_args.mg);
+  solve_scene_mg<MIXED>(s_args, sh, mg_dyn);
 }
 
 }  // namespace
