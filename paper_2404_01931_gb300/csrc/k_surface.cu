@@ -7,9 +7,9 @@
 //                   the histogram atomic returns its rank in the bin
 //   scan            exclusive scan of the bin counts (tile scan below)
 //   k_sbin_scatter  positions into bin order as float4
-//   k_sdf           one warp per 4 corners along x: the bin rows that meet their
-//                   balls of radius R, read as coalesced particle ranges; kernel
-//                   sums of k and k (x_i - x), phi = |sum k d| / sum k - r
+//   k_sdf           one warp per 2 x 2 corners: the bin rows that meet their balls of
+//                   radius R, read as coalesced particle ranges; kernel sums of k and
+//                   k (x_i - x), phi = |sum k d| / sum k - r
 // Pipeline of flip_surface_mesh:
 //   tile scan over corners of one packed count per corner: (vertices on the
 //   corner's 3 outgoing edges) + (triangles of the cube it is the lowest corner
@@ -374,142 +374,169 @@ __global__ void k_sbin_scatter(const PartView p, long long np, const int* __rest
   pos[start[b] + prank[i]] = make_float4(p.x[i], p.y[i], p.z[i], 0.0f);
 }
 
-// One warp per group of SDF_G corners consecutive along x (same j, k).  With bins
-// of edge R/2 the balls meet at most 5 bins along y and along z, so at most 25 bin
-// rows (fixed y, z bin): lane r finds row r's particle range (the row's bins
-// within the balls' x extent are one contiguous range), a warp scan lays the rows
-// end to end in a per-warp shared table, and the lanes stride over that flat
-// range, so every load is independent and a warp's loads are consecutive
-// float4s.  Each particle is tested against all SDF_G corners, whose sums stay in
-// registers until a warp reduction.  A bin whose nearest point is R or farther
-// from the corners holds no particle closer than R and is skipped.
-constexpr int SDF_G = 4;
+// One warp per group of GX x GY corners of one z plane (2 x 2 where the corners are no
+// farther apart than a bin, else 2 x 1).  With bins of edge R/2 the balls meet at most 6
+// bins along y and 5 along z, so at most 30 bin rows (fixed y, z bin): lane r finds row
+// r's particle range (the row's bins within the balls' x extent are one contiguous range;
+// a bin whose nearest point is R or farther from the corners holds no particle closer
+// than R and is skipped), the nonempty rows are packed into a per-warp list, and the
+// warp's four groups of eight lanes take a row each, eight particles (128 bytes) at a
+// time.  Each particle is tested against all the group's corners, whose sums stay in
+// registers until a reduction that halves the values with every step.  The eight warps of
+// a CTA take neighbouring groups (4 x 4 x 2 corners), so that most of a CTA's particle
+// reads hit L1.
+//
+// Bound by issue (66 % of the slots, the FP32 pipe half busy): about 50 instructions per
+// particle and four corners, 640-800 particles tested per corner of which 268 lie in its
+// ball (8 per cell, R = 2 h).  A whole flip_surface_sdf of 42 M particles at 257^3 corners
+// 6.80 -> 4.81 ms, of 2.1 M at 129^3 0.555 -> 0.414, against one warp per 4 corners along x
+// whose lanes walked one flat range over all rows (row search and 160 shuffles per group);
+// without the load ahead 5.10 ms, 16 lanes a row 5.56, 6 CTAs per SM 5.14.
 constexpr int SDF_THREADS = 256;
 constexpr int SDF_WARPS = SDF_THREADS / 32;
+constexpr int SDF_ROW_LANES = 8;
 
+template <int GX, int GY>
 __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins B,
                                                      const unsigned int* __restrict__ start,
                                                      const float4* __restrict__ pos,
                                                      float* __restrict__ phi) {
-  __shared__ unsigned int s_end[SDF_WARPS][32], s_beg[SDF_WARPS][32], s_p0[SDF_WARPS][32];
+  static_assert(GX == 2 && (GY == 1 || GY == 2), "a packed pair along x");
+  __shared__ uint2 s_row[SDF_WARPS][32];  // {first particle, end} of the nonempty rows
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int gx = (g.c[0] + SDF_G - 1) / SDF_G;
-  const long long ngroups = (long long)gx * g.c[1] * g.c[2];
-  const long long warps = (long long)gridDim.x * SDF_WARPS;
+  // a CTA's groups: 2 x 2 x 2
+  constexpr int CX = 2 * GX, CY = 2 * GY, CZ = 2;
+  const int tx = (g.c[0] + CX - 1) / CX, ty = (g.c[1] + CY - 1) / CY, tz = (g.c[2] + CZ - 1) / CZ;
+  const long long ntiles = (long long)tx * ty * tz;
   constexpr float Rb = 2.0f;  // R in bins (the bin edge is R/2)
-  for (long long grp = blockIdx.x * (long long)SDF_WARPS + wid; grp < ngroups; grp += warps) {
-    const int i0 = (int)(grp % gx) * SDF_G;
-    const int j = (int)((grp / gx) % g.c[1]);
-    const int k = (int)(grp / ((long long)gx * g.c[1]));
-    const int ng = min(SDF_G, g.c[0] - i0);
-    const float x0 = g.o[0] + g.h * (float)i0, xl = g.o[0] + g.h * (float)(i0 + ng - 1);
-    const float yc = g.o[1] + g.h * (float)j, zc = g.o[2] + g.h * (float)k;
-    const float ry = (yc - B.o[1]) * B.inv_b, rz = (zc - B.o[2]) * B.inv_b;
-    const int by0 = max(0, (int)floorf(ry - Rb)), by1 = min(B.nb[1] - 1, (int)floorf(ry + Rb));
+  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int i0 = (int)(tile % tx) * CX + (wid & 1) * GX;
+    const int j0 = (int)((tile / tx) % ty) * CY + ((wid >> 1) & 1) * GY;
+    const int k = (int)(tile / ((long long)tx * ty)) * CZ + (wid >> 2);
+    if (i0 >= g.c[0] || j0 >= g.c[1] || k >= g.c[2]) continue;
+    const float x0 = g.o[0] + g.h * (float)i0, x1 = g.o[0] + g.h * (float)(i0 + 1);
+    const float y0 = g.o[1] + g.h * (float)j0, y1 = g.o[1] + g.h * (float)(j0 + GY - 1);
+    const float zc = g.o[2] + g.h * (float)k;
+    const float ry0 = (y0 - B.o[1]) * B.inv_b, ry1 = (y1 - B.o[1]) * B.inv_b;
+    const float rz = (zc - B.o[2]) * B.inv_b;
+    const int by0 = max(0, (int)floorf(ry0 - Rb)), by1 = min(B.nb[1] - 1, (int)floorf(ry1 + Rb));
     const int bz0 = max(0, (int)floorf(rz - Rb)), bz1 = min(B.nb[2] - 1, (int)floorf(rz + Rb));
     const int nyr = max(by1 - by0 + 1, 1);
     const int nrows = min(nyr * (bz1 - bz0 + 1), 32);
-    unsigned int p0 = 0, cnt = 0;
+    unsigned int p0 = 0, p1 = 0;
     if (lane < nrows) {
       const int by = by0 + lane % nyr, bz = bz0 + lane / nyr;
-      const float dy = fmaxf(fmaxf(B.o[1] + B.b * by - yc, yc - (B.o[1] + B.b * (by + 1))), 0.0f);
+      const float dy = fmaxf(fmaxf(B.o[1] + B.b * by - y1, y0 - (B.o[1] + B.b * (by + 1))), 0.0f);
       const float dz = fmaxf(fmaxf(B.o[2] + B.b * bz - zc, zc - (B.o[2] + B.b * (bz + 1))), 0.0f);
       const float dyz = dy * dy + dz * dz;
       if (dyz < B.R2) {
         const float rx = sqrtf(B.R2 - dyz) * B.inv_b;
         const int bx0 = max(0, (int)floorf((x0 - B.o[0]) * B.inv_b - rx));
-        const int bx1 = min(B.nb[0] - 1, (int)floorf((xl - B.o[0]) * B.inv_b + rx));
+        // (a bin that begins at the balls' end holds nothing closer than R)
+        const int bx1 = min(B.nb[0] - 1, (int)ceilf((x1 - B.o[0]) * B.inv_b + rx) - 1);
         if (bx0 <= bx1) {
           const long long row = (long long)B.nb[0] * (by + (long long)B.nb[1] * bz);
           p0 = start[row + bx0];
-          cnt = start[row + bx1 + 1] - p0;
+          p1 = start[row + bx1 + 1];
         }
       }
     }
-    unsigned int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    const unsigned int total = __shfl_sync(0xffffffffu, incl, 31);
+    const unsigned int some = __ballot_sync(0xffffffffu, p0 < p1);
+    const int nrow = __popc(some);
+    __syncwarp();  // the last group's reads of the list are done
+    if (p0 < p1) s_row[wid][__popc(some & ((1u << lane) - 1u))] = make_uint2(p0, p1);
     __syncwarp();
-    s_end[wid][lane] = incl;
-    s_beg[wid][lane] = incl - cnt;
-    s_p0[wid][lane] = p0;
-    __syncwarp();
-    // per corner q: (sum k, sum k ex) and (sum k ey, sum k ez); corners go in
-    // pairs through packed two-lane FP32 operations, each lane rounded like the
-    // scalar operation
-    static_assert(SDF_G % 2 == 0, "corners in pairs");
-    float2 a01[SDF_G], a23[SDF_G];
-    float2 xq[SDF_G / 2];  // minus the corners' x (P.x + (-x) rounds as P.x - x)
+    // per corner: sum k and sum k e; corners (0, y) and (1, y) go as the two lanes of packed
+    // FP32 operations, each rounded like the scalar operation
+    float2 sk[GY], sx[GY], sy[GY], sz[GY];
 #pragma unroll
-    for (int q = 0; q < SDF_G; ++q) a01[q] = a23[q] = make_float2(0.0f, 0.0f);
+    for (int q = 0; q < GY; ++q) sk[q] = sx[q] = sy[q] = sz[q] = make_float2(0.0f, 0.0f);
+    // minus the corners' coordinates (P.x + (-x) rounds as P.x - x)
+    const float2 mx = make_float2(-x0, -x1), mz = make_float2(-zc, -zc);
+    float2 my[GY];
 #pragma unroll
-    for (int u = 0; u < SDF_G / 2; ++u)
-      xq[u] = make_float2(-(x0 + g.h * (float)(2 * u)), -(x0 + g.h * (float)(2 * u + 1)));
-    const float2 one = make_float2(1.0f, 1.0f), m_inv = make_float2(-B.inv_R2, -B.inv_R2);
-    int r = 0;  // this lane's current row: only moves forward
-    for (unsigned int f = lane; f < total; f += 32) {
-      while (f >= s_end[wid][r]) ++r;
-      const float4 P = pos[s_p0[wid][r] + (f - s_beg[wid][r])];
-      const float ey = __fsub_rn(P.y, yc), ez = __fsub_rn(P.z, zc);
-      const float r2 = __fmaf_rn(ez, ez, __fmul_rn(ey, ey));
-      const float2 eyz = make_float2(ey, ez);
+    for (int q = 0; q < GY; ++q) my[q] = make_float2(q == 0 ? -y0 : -y1, q == 0 ? -y0 : -y1);
+    for (int r = lane / SDF_ROW_LANES; r < nrow; r += 32 / SDF_ROW_LANES) {
+      const uint2 row = s_row[wid][r];
+      unsigned int f = row.x + lane % SDF_ROW_LANES;
+      float4 next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (f < row.y) next = pos[f];
+      for (; f < row.y; f += SDF_ROW_LANES) {
+        const float4 P = next;  // the next particle's load is in flight during this one's sums
+        if (f + SDF_ROW_LANES < row.y) next = pos[f + SDF_ROW_LANES];
+        const float2 ex = __fadd2_rn(make_float2(P.x, P.x), mx);
+        const float2 ez = __fadd2_rn(make_float2(P.z, P.z), mz);
+        const float2 xx = __fmul2_rn(ex, ex), zz = __fmul2_rn(ez, ez);
 #pragma unroll
-      for (int u = 0; u < SDF_G / 2; ++u) {
-        const float2 ex = __fadd2_rn(make_float2(P.x, P.x), xq[u]);
-        const float2 dd = __ffma2_rn(ex, ex, make_float2(r2, r2));
-        const float2 t = __ffma2_rn(dd, m_inv, one);
-        float2 kk = __fmul2_rn(__fmul2_rn(t, t), t);
-        if (!(2 * u < ng && dd.x < B.R2)) kk.x = 0.0f;
-        if (!(2 * u + 1 < ng && dd.y < B.R2)) kk.y = 0.0f;
-        a01[2 * u] = __ffma2_rn(make_float2(kk.x, kk.x), make_float2(1.0f, ex.x), a01[2 * u]);
-        a23[2 * u] = __ffma2_rn(make_float2(kk.x, kk.x), eyz, a23[2 * u]);
-        a01[2 * u + 1] = __ffma2_rn(make_float2(kk.y, kk.y), make_float2(1.0f, ex.y), a01[2 * u + 1]);
-        a23[2 * u + 1] = __ffma2_rn(make_float2(kk.y, kk.y), eyz, a23[2 * u + 1]);
-      }
-    }
-    float sk[SDF_G], s0[SDF_G], s1[SDF_G], s2[SDF_G];
-#pragma unroll
-    for (int q = 0; q < SDF_G; ++q) {
-      sk[q] = a01[q].x;
-      s0[q] = a01[q].y;
-      s1[q] = a23[q].x;
-      s2[q] = a23[q].y;
-    }
-#pragma unroll
-    for (int q = 0; q < SDF_G; ++q) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sk[q] += __shfl_xor_sync(0xffffffffu, sk[q], o);
-        s0[q] += __shfl_xor_sync(0xffffffffu, s0[q], o);
-        s1[q] += __shfl_xor_sync(0xffffffffu, s1[q], o);
-        s2[q] += __shfl_xor_sync(0xffffffffu, s2[q], o);
-      }
-    }
-    if (lane < ng) {
-      float a = 0.0f, b0 = 0.0f, b1 = 0.0f, b2 = 0.0f;
-#pragma unroll
-      for (int q = 0; q < SDF_G; ++q)
-        if (q == lane) {
-          a = sk[q];
-          b0 = s0[q];
-          b1 = s1[q];
-          b2 = s2[q];
+        for (int q = 0; q < GY; ++q) {
+          const float2 ey = __fadd2_rn(make_float2(P.y, P.y), my[q]);
+          const float2 dd = __fadd2_rn(__ffma2_rn(ey, ey, zz), xx);
+          // k = max(0, 1 - d^2 / R^2)^3 (saturating: d^2 >= 0); at d = R the terms vanish
+          const float2 t = make_float2(__saturatef(__fmaf_rn(dd.x, -B.inv_R2, 1.0f)),
+                                       __saturatef(__fmaf_rn(dd.y, -B.inv_R2, 1.0f)));
+          const float2 kk = __fmul2_rn(__fmul2_rn(t, t), t);
+          sk[q] = __fadd2_rn(sk[q], kk);
+          sx[q] = __ffma2_rn(kk, ex, sx[q]);
+          sy[q] = __ffma2_rn(kk, ey, sy[q]);
+          sz[q] = __ffma2_rn(kk, ez, sz[q]);
         }
-      const float v = (a > 0.0f) ? sqrtf(b0 * b0 + b1 * b1 + b2 * b2) / a - B.r : B.R - B.r;
-      phi[(i0 + lane) + (long long)g.c[0] * (j + (long long)g.c[1] * k)] = v;
+      }
+    }
+    // reduction: with every step a lane keeps half of its values and adds its partner's
+    // halves of them; then lane l holds corner l / 4's value l % 4 (for 4 corners; with 2
+    // corners l / 4 is 0 or 1)
+    constexpr int NV = 4 * GX * GY;
+    float v[NV];
+#pragma unroll
+    for (int q = 0; q < GY; ++q) {
+      v[8 * q] = sk[q].x;
+      v[8 * q + 1] = sx[q].x;
+      v[8 * q + 2] = sy[q].x;
+      v[8 * q + 3] = sz[q].x;
+      v[8 * q + 4] = sk[q].y;
+      v[8 * q + 5] = sx[q].y;
+      v[8 * q + 6] = sy[q].y;
+      v[8 * q + 7] = sz[q].y;
+    }
+#pragma unroll
+    for (int n = NV / 2; n >= 1; n >>= 1) {
+      const bool hi = lane & n;
+#pragma unroll
+      for (int q = 0; q < n; ++q) {
+        const float send = hi ? v[q] : v[q + n];
+        const float keep = hi ? v[q + n] : v[q];
+        v[q] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, n));
+      }
+    }
+    // lanes equal modulo NV hold partial sums of the same value
+    float s = v[0];
+#pragma unroll
+    for (int n = NV; n < 32; n <<= 1) s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, n));
+    const float a = __shfl_sync(0xffffffffu, s, 4 * lane);  // lane c < corners: corner c's sums
+    const float b0 = __shfl_sync(0xffffffffu, s, 4 * lane + 1);
+    const float b1 = __shfl_sync(0xffffffffu, s, 4 * lane + 2);
+    const float b2 = __shfl_sync(0xffffffffu, s, 4 * lane + 3);
+    const int i = i0 + (lane & 1), j = j0 + (lane >> 1);
+    if (lane < GX * GY && i < g.c[0] && j < g.c[1]) {
+      const float d = (a > 0.0f) ? sqrtf(b0 * b0 + b1 * b1 + b2 * b2) / a - B.r : B.R - B.r;
+      phi[i + (long long)g.c[0] * (j + (long long)g.c[1] * k)] = d;
     }
   }
 }
 
-int sdf_blocks() {
+// The corners of a 2 x 2 group share most of their bins while h is at most a bin edge
+// (R >= 2 h), and its rows fit a warp's list (6 x 5); wider grids take pairs along x.
+using SdfKernel = void (*)(const SGrid, const SBins, const unsigned int*, const float4*, float*);
+
+SdfKernel sdf_kernel(const SGrid& g, const SBins& B) {
+  return g.h <= 1.001f * B.b ? (SdfKernel)k_sdf<2, 2> : (SdfKernel)k_sdf<2, 1>;
+}
+
+int sdf_blocks(SdfKernel k) {
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sdf, SDF_THREADS, 0) != cudaSuccess) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, SDF_THREADS, 0) != cudaSuccess) {
     cudaGetLastError();
     return 152 * 8;
   }
@@ -879,7 +906,8 @@ int flip_surface_sdf(flip_surface* s, flip_handle* h) {
     k_sbin_scatter<<<blocks_for(np, 256), 256, 0, st>>>(P, np, s->pbin, s->prank, s->bin_start,
                                                         s->pos);
   }
-  k_sdf<<<sdf_blocks(), SDF_THREADS, 0, st>>>(s->g, s->B, s->bin_start, s->pos, s->phi);
+  const SdfKernel sdf = sdf_kernel(s->g, s->B);
+  sdf<<<sdf_blocks(sdf), SDF_THREADS, 0, st>>>(s->g, s->B, s->bin_start, s->pos, s->phi);
   SURF_CUDA(cudaGetLastError());
   return FLIP_OK;
 }

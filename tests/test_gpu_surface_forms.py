@@ -1,0 +1,37 @@
+"""The scalar field's two kernel forms (2 x 2 and 2 x 1 corners per warp) at the line between
+them and on corner counts that leave groups and tiles part empty, against the oracle."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2404_01931_gb300 import flip as F
+from paper_2404_01931_gb300 import scenes as S
+
+from parity_util import matched
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,h,ratio", [
+    ((31, 18, 7), 1 / 24, 2.0),      # R = 2 h: corners a bin apart, 2 x 2
+    ((32, 17, 8), 1 / 24, 1.9),      # just past the line, 2 x 1
+    ((9, 5, 6), 1 / 8, 0.7),         # balls that do not meet, 2 x 1
+    ((60, 55, 3), 1 / 72, 6.5),      # corners far closer than a bin, 2 x 2
+    ((1, 1, 1), 1 / 2, 2.0),         # eight corners
+])
+def test_sdf_forms_match_the_oracle(n, h, ratio):
+    sc = S.random_velocities(S.water_drop(24, centre=(0.4, 0.45, 0.3), radius=0.25), 0.1, 3)
+    sp = F.FlipSurfaceParams()
+    for a in range(3):
+        sp.n[a] = n[a]
+        sp.origin[a] = (-0.01, 0.003, 0.02)[a]
+    sp.h, sp.search_radius = h, ratio * h
+    sp.radius, sp.iso = 0.25 * sp.search_radius, 0.0
+    with F.Simulation(matched(24)[1], *sc.arrays()) as sim, F.Surface(sp) as s:
+        s.sdf(sim)
+        phi = s.read(F.SURF_FIELD).astype(np.float64)
+    ref = O.sdf(sc.x, sc.y, sc.z, tuple(sp.n), tuple(sp.origin), sp.h, sp.radius,
+                sp.search_radius)
+    # FP32 kernel sums: relative rounding ~1e-6 of the lengths involved (R), the bar of
+    # test_gpu_surface.py
+    assert np.abs(phi - ref).max() <= 2e-5 * sp.search_radius
