@@ -2783,20 +2783,6 @@ __device__ void solve_scene_mg(const PcgArgs& A, Shared& sh, unsigned char* dyn)
   }
 }
 
-// The scene's arguments in shared memory.  The passes take them by reference; read from
-// the parameter space (or, in a batch, from global memory) through that reference, the
-// level descriptions would cost every pass an L2 round trip, since a grid barrier's
-// acquire empties L1.
-__shared__ PcgArgs s_args;
-
-__device__ __forceinline__ void load_args(const PcgArgs& A) {
-  static_assert(sizeof(PcgArgs) % 8 == 0 && alignof(PcgArgs) == 8, "copied by 8-byte words");
-  const unsigned long long* src = reinterpret_cast<const unsigned long long*>(&A);
-  unsigned long long* dst = reinterpret_cast<unsigned long long*>(&s_args);
-  for (int i = threadIdx.x; i < (int)(sizeof(PcgArgs) / 8); i += PCG_THREADS) dst[i] = src[i];
-  __syncthreads();
-}
-
 template <bool MIXED>
 __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg_mg(const __grid_constant__ PcgArgs A) {
   __shared__ Shared sh;

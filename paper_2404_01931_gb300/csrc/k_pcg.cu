@@ -195,13 +195,187 @@ __device__ void solve(const PcgArgs& A, const Chunk& ch, Shared& sh, SolveState&
   S.rel = bnorm > 0.0 ? rnorm / bnorm : 0.0;
 }
 
-template <bool MIXED>
+// The same FP32 solve with every thread's cells in registers (at most U each): per cell
+// its index, the fluid neighbours, x, r, p and the preconditioned residual z = r / diag.
+// Only what neighbours read goes to memory, p (double-buffered) and z (in A.r: a
+// neighbour's p_new is then fma(beta, p_old, z), p_update's operations), so phase A is one
+// round of loads and phase B has none.  The values are solve()'s, operation for operation.
+//
+// Bound by latency: two grid barriers (~1.5 us) with a reduction (~1.1 us) each.  Read per
+// phase through the active list, the types and the arrays (three dependent L2 trips, which
+// the barriers' acquires keep cold) an iteration took 12.2 us at 14.7 k fluid cells, 14.9
+// at 166 k; this way 9.2 and 9.5.
+template <int U>
+__device__ void solve_regs(const PcgArgs& A, const Chunk& ch, Shared& sh, SolveState& S) {
+  const Grid& g = A.g;
+  const int sy = g.nx, sz = g.nx * g.ny;
+  int cell[U];              // -1: none
+  unsigned int nb[U];       // bits 0..5: fluid neighbours, bits 8..10: neighbours in the grid
+  float x[U], r[U], p[U], z[U];
+  float* zg = A.r;
+  FF bb, rz0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    cell[u] = -1;
+    nb[u] = 0u;
+    x[u] = r[u] = p[u] = z[u] = 0.0f;
+    const unsigned int e = ch.begin + threadIdx.x + u * PCG_THREADS;
+    if (e >= ch.end) continue;
+    const unsigned int brick = A.active[e >> 9];
+    const int l = (int)(e & 511u);
+    const int i = (int)(brick % (unsigned)g.bx) * BRICK + (l & 7);
+    const int j = (int)((brick / (unsigned)g.bx) % (unsigned)g.by) * BRICK + ((l >> 3) & 7);
+    const int k = (int)(brick / ((unsigned)g.bx * (unsigned)g.by)) * BRICK + (l >> 6);
+    if (i >= g.nx || j >= g.ny || k >= g.nz) continue;
+    const int c = i + sy * (j + g.ny * k);
+    if (A.type[c] != 1) continue;
+    cell[u] = c;
+    const bool in[6] = {i > 0, i < g.nx - 1, j > 0, j < g.ny - 1, k > 0, k < g.nz - 1};
+    const int off[6] = {-1, 1, -sy, sy, -sz, sz};
+    int cnt = 0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      cnt += in[q];
+      if (in[q] && A.type[c + off[q]] == 1) nb[u] |= 1u << q;
+    }
+    nb[u] |= (unsigned)cnt << 8;
+    r[u] = A.b32[c];
+    z[u] = __fmul_rn(r[u], A.minv_tab[cnt]);
+    zg[c] = z[u];
+    A.pa[c] = 0.0f;
+    bb.add_prod(r[u], r[u]);
+    rz0.add_prod(r[u], z[u]);
+  }
+  // thread 0's scalars, in shared memory
+  double &rz = sh.dscal[0], &bnorm = sh.dscal[1], &rnorm = sh.dscal[2];
+  {
+    F2 v[2] = {f2_of(bb), f2_of(rz0)};
+    publish<2>(A, 1, v, sh);
+  }
+  if (!grid_barrier(A.bar, A.status, team_size(), A.timeout_ns)) { S.ok = false; return; }
+  {
+    double s[2];
+    gather<2>(A, 1, s, sh);
+    if (threadIdx.x == 0) {
+      rz = s[1];
+      bnorm = rnorm = sqrt(fmax(s[0], 0.0));
+      sh.flag = (bnorm == 0.0) ? 1 : 0;
+      sh.beta = 0.0f;
+    }
+  }
+  __syncthreads();
+  bool conv = sh.flag != 0;
+  int it = 0;
+  float* pold = A.pa;
+  float* pnew = A.pb;
+  while (!conv && it < A.max_iter) {
+    ++it;
+    const float beta = sh.beta;
+    // ---- phase A
+    float q[U];
+    FF pq;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int c = cell[u];
+      q[u] = 0.0f;
+      if (c < 0) continue;
+      const int off[6] = {-1, 1, -sy, sy, -sz, sz};
+      float zn[6], pn[6];
+#pragma unroll
+      for (int h = 0; h < 6; ++h) {
+        const bool f = (nb[u] >> h) & 1u;
+        zn[h] = f ? zg[c + off[h]] : 0.0f;
+        pn[h] = f ? pold[c + off[h]] : 0.0f;
+      }
+      const float pc = __fmaf_rn(beta, p[u], z[u]);
+      float d = 0.0f;
+      int nfl = 0;
+#pragma unroll
+      for (int h = 0; h < 6; ++h) {
+        const bool f = (nb[u] >> h) & 1u;
+        d += f ? __fsub_rn(pc, __fmaf_rn(beta, pn[h], zn[h])) : 0.0f;
+        nfl += f;
+      }
+      const int cnt = (int)(nb[u] >> 8);
+      q[u] = __fmul_rn(A.s, __fmaf_rn((float)(cnt - nfl), pc, d));
+      p[u] = pc;
+      pnew[c] = pc;
+      pq.add_prod(pc, q[u]);
+    }
+    {
+      F2 v[1] = {f2_of(pq)};
+      publish<1>(A, 0, v, sh);
+    }
+    if (!grid_barrier(A.bar, A.status, team_size(), A.timeout_ns)) { S.ok = false; return; }
+    {
+      double s[1];
+      gather<1>(A, 0, s, sh);
+      if (threadIdx.x == 0) sh.alpha = (float)(rz / s[0]);
+    }
+    __syncthreads();
+    const float alpha = sh.alpha;
+    // ---- phase B
+    FF rr, rzn;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (cell[u] < 0) continue;
+      x[u] = __fmaf_rn(alpha, p[u], x[u]);
+      r[u] = __fmaf_rn(-alpha, q[u], r[u]);
+      z[u] = __fmul_rn(r[u], A.minv_tab[nb[u] >> 8]);
+      zg[cell[u]] = z[u];
+      rr.add_prod(r[u], r[u]);
+      rzn.add_prod(r[u], z[u]);
+    }
+    {
+      F2 v[2] = {f2_of(rr), f2_of(rzn)};
+      publish<2>(A, 1, v, sh);
+    }
+    if (!grid_barrier(A.bar, A.status, team_size(), A.timeout_ns)) { S.ok = false; return; }
+    {
+      double s[2];
+      gather<2>(A, 1, s, sh);
+      if (threadIdx.x == 0) {
+        rnorm = sqrt(fmax(s[0], 0.0));
+        sh.flag = rnorm <= A.tol * bnorm ? 1 : 0;
+        if (sh.flag == 0) {
+          sh.beta = (float)(s[1] / rz);
+          rz = s[1];
+        }
+      }
+    }
+    __syncthreads();
+    if (sh.flag == 1) conv = true;
+    float* t = pold; pold = pnew; pnew = t;
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (cell[u] >= 0) A.x32[cell[u]] = x[u];
+  S.iters = it;
+  S.conv = conv;
+  if (threadIdx.x == 0) {
+    S.rel = bnorm > 0.0 ? rnorm / bnorm : 0.0;
+    S.bnorm = bnorm;
+  }
+}
+
+// Up to UMAX cells per thread a solve keeps them in registers: 4 in a single solve (100^3,
+// 4.3 cells: 21.4 -> 11.9 us an iteration); 2 in a batch, where the arguments' addresses
+// take the registers and the 4-cell form spills 580 bytes.
+
+template <bool MIXED, int UMAX>
 __device__ void solve_scene(const PcgArgs& A, Shared& sh) {
   const unsigned int nact = *A.n_active;
   const long long ncells = (long long)A.g.nx * A.g.ny * A.g.nz;
   const bool singular = A.check_singular && ((long long)A.stats->n_fluid == ncells);
   SolveState S;
-  if (!singular) solve<MIXED>(A, my_chunk(nact), sh, S);
+  if (!singular) {
+    const Chunk ch = my_chunk(nact);
+    // the same for every CTA of the team: the longest chunk
+    const unsigned int per = ((nact * BRICK_CELLS + team_size() - 1) / team_size() + 31u) & ~31u;
+    if (!MIXED && per <= 2 * PCG_THREADS) solve_regs<2>(A, ch, sh, S);
+    else if (!MIXED && per <= UMAX * PCG_THREADS) solve_regs<UMAX>(A, ch, sh, S);
+    else solve<MIXED>(A, ch, sh, S);
+  }
   if (team_rank() == 0 && threadIdx.x == 0) {
     int st = 0;
     if (singular) st |= DEV_SINGULAR;
@@ -220,7 +394,7 @@ template <bool MIXED>
 __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(const __grid_constant__ PcgArgs A) {
   __shared__ Shared sh;
   team_enter(blockIdx.x, gridDim.x);
-  solve_scene<MIXED>(A, sh);
+  solve_scene<MIXED, 4>(A, sh);
 }
 
 // Several scenes in one launch (see k_pcg_mg_batch).
@@ -229,7 +403,8 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg_batch(const __grid_const
   __shared__ Shared sh;
   const int s = B.block_scene[blockIdx.x];
   team_enter(blockIdx.x - B.team_first[s], B.team_first[s + 1] - B.team_first[s]);
-  solve_scene<MIXED>(B.args[s], sh);
+  load_args(B.args[s]);
+  solve_scene<MIXED, 2>(s_args, sh);
 }
 
 int pcg_block_size() { return PCG_THREADS; }
