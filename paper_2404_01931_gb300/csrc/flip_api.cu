@@ -403,7 +403,7 @@ void carve(flip_handle* h, Carver& cv) {
         L.b = cv.take<float>(ns);
         L.code16 = cv.take<uint16_t>(ns);
         L.seg = cv.take<unsigned int>((size_t)L.nw * L.ny * L.nz);
-        L.nseg = cv.take<unsigned int>(1);
+        L.segmask = cv.take<unsigned int>((size_t)L.nby * L.nbz);
         const size_t blocks = (size_t)L.nbx * L.nby * L.nbz;
         L.blk = cv.take<int>(blocks);
         // 1024 threads per block, as many blocks as a blocked level can have

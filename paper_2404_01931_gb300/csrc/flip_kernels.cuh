@@ -138,8 +138,9 @@ struct MgLevel {
   int nbx, nby, nbz;  // 8x8x8 blocks of this level's cells
   uint16_t* code16;   // per slot: the code bits above plus the count of
                       // neighbours inside the grid in bits 8..10
+  unsigned int* segmask;  // per block-row J + nby K: the segments (bits) that meet a block
+                      // holding fluid
   unsigned int* seg;  // active segments (seg_pack: segment in row, j, k)
-  unsigned int* nseg; // their number (device)
   uint8_t* bflag;     // levels >= 1: block holds a fluid cell (level 0 reads the
                       // brick fluid counts of the binning)
   int* blk;           // the blocks holding fluid (bx | by << 8 | bz << 16), for the

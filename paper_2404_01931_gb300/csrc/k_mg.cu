@@ -52,8 +52,8 @@ enum TraceSlot {
   TR_ENTRY = 0,       // kernel entry
   TR_TABLES = 1,      // shared tables loaded
   TR_BFLAG = 2,       // block flags cleared
-  TR_FLAGS = 2,       // + l: fluid flags of level l (l = 1 .. 11) built
-  TR_SEG_COUNT = 14,  // active segments counted
+  TR_FLAGS = 2,       // + 1: fluid flags of all levels built
+  TR_SEG_COUNT = 14,  // active segments counted (large grids)
   TR_SEG_WRITE = 15,  // active-segment lists written
   TR_CODES = 16,      // neighbour codes built
   TR_SEG_CACHE = 17,  // segment slices cached
@@ -110,9 +110,20 @@ __device__ __forceinline__ void load_tables(const MgArgs& M) {
 // every item of a pass, the segment, is then a shared-memory read.  s_segc[l] is
 // the copy of level l's slice (nullptr: read the list in global memory) and
 // s_segb[l] the index of its first segment.
-constexpr int SEG_CACHE = 1024;
+constexpr int SEG_CACHE = 4096;
 __shared__ const unsigned int* s_segc[MG_MAX_LEVELS];
 __shared__ int s_segb[MG_MAX_LEVELS];
+// A level's number of active segments and this CTA's slice of them.
+__shared__ int s_nseg[MG_MAX_LEVELS];
+__shared__ int2 s_slice[MG_MAX_LEVELS];
+
+// One thread: the slice of a level with n active segments.
+__device__ __forceinline__ void set_slice(int l, int n) {
+  const int per = (n + (int)team_size() - 1) / (int)team_size();
+  const int q0 = min(n, (int)team_rank() * per);
+  s_nseg[l] = n;
+  s_slice[l] = make_int2(q0, min(n, q0 + per));
+}
 
 // Levels whose smoothing runs blocked (block_pass): their number of blocks holding
 // fluid, 0 for the levels swept pass by pass.  s_z0 and s_q0 are the arrays that hold
@@ -237,12 +248,7 @@ __device__ __forceinline__ void snbr(const LV& L, const SCell& e, int (&nb)[6]) 
 }
 
 // This CTA's slice [q0, q1) of a level's active segments.
-__device__ __forceinline__ int2 seg_slice(const MgLevel& L) {
-  const int n = (int)*L.nseg;
-  const int per = (n + (int)team_size() - 1) / (int)team_size();
-  const int q0 = min(n, (int)team_rank() * per);
-  return make_int2(q0, min(n, q0 + per));
-}
+__device__ __forceinline__ int2 seg_slice(const MgLevel& L) { return s_slice[L.lvl]; }
 
 // Items (segment, colour) of this CTA for ncol colours: item t is segment
 // t / ncol, colour t % ncol (ncol = 2) or the pass's colour (ncol = 1).  Each
@@ -642,7 +648,7 @@ __device__ __noinline__ FF sweep_split_s(const MgArgs& M, const MgLevel& L, cons
 constexpr int VEC_SEGS_PER_CTA = 256;
 
 __device__ __forceinline__ bool use_pairs(const MgLevel& L) {
-  return *L.nseg >= (unsigned)VEC_SEGS_PER_CTA * team_size();
+  return s_nseg[L.lvl] >= VEC_SEGS_PER_CTA * (int)team_size();
 }
 
 template <int MODE>
@@ -2176,40 +2182,10 @@ __device__ __forceinline__ void block_rule(const PcgArgs& A) {
   __syncthreads();
 }
 
-// Builds, once per solve: the fluid flags of levels 1.. (a coarse cell is fluid
-// when any child is) with their block flags, the active-segment lists of the
-// colour-split levels (in segment order, so the work split is deterministic),
-// the codes of every level.  Ends with a grid barrier.
-__device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
+// The active segments of large grids: counted per CTA, then written in segment order into
+// the levels' lists.  Ends with a grid barrier.
+__device__ __noinline__ bool seg_lists(const PcgArgs& A, Shared& sh) {
   const MgArgs& M = A.mg;
-  // block flags of the split coarse levels start clear
-  for (int l = 1; l < M.lgrid; ++l) {
-    const MgLevel& L = M.lv[l];
-    const Part p = level_part(L.nbx * L.nby * L.nbz, false);
-    for (int c = p.begin; c < p.end; c += p.stride) L.bflag[c] = 0;
-    if (team_rank() == 0 && threadIdx.x == 0) *L.nblk = 0u;
-  }
-  if (!gsync(A)) return false;
-  SOLVE_TRACE(TR_BFLAG);
-  for (int l = 1; l < M.nlev; ++l) {
-    const MgLevel& F = M.lv[l - 1];
-    const MgLevel& C = M.lv[l];
-    const Part p = level_part(C.ncells, false);
-    for (int c = p.begin; c < p.end; c += p.stride) {
-      const int i = c % C.nx, j = (c / C.nx) % C.ny, k = c / (C.nx * C.ny);
-      uint8_t f = 0;
-      for (int d = 0; d < 8; ++d) {
-        const int fi = 2 * i + (d & 1), fj = 2 * j + ((d >> 1) & 1), fk = 2 * k + (d >> 2);
-        if (fi < F.nx && fj < F.ny && fk < F.nz && F.t[fi + F.nx * (fj + F.ny * fk)] == 1) f = 1;
-      }
-      C.t[c] = f;
-      if (f && C.split) C.bflag[(i >> 3) + C.nbx * ((j >> 3) + C.nby * (k >> 3))] = 1;
-    }
-    if (!gsync(A)) return false;
-    SOLVE_TRACE(TR_FLAGS + min(l, 11));
-  }
-  block_lists(A);
-  // active segments: count per CTA, then write them in segment order
   __shared__ unsigned int s_wsum[PCG_WARPS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int l = 0; l < M.lgrid; ++l) {
@@ -2251,7 +2227,7 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
       total = __reduce_add_sync(0xffffffffu, total);
       if (lane == 0) {
         sh.dscal[0] = (double)before;
-        if (team_rank() == 0) *L.nseg = total;
+        set_slice(l, (int)total);
       }
     }
     __syncthreads();
@@ -2274,15 +2250,240 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
       __syncthreads();
     }
   }
+  return gsync(A);
+}
+
+// Copies this CTA's slice of each grid-wide level's segment list into the
+// shared-memory cache, level 0 first, while it fits (after build_levels).
+__device__ __noinline__ void seg_cache_fill(const MgArgs& M, unsigned int* cache) {
+  int used = 0;
+  for (int l = 0; l < M.lgrid; ++l) {
+    const MgLevel& L = M.lv[l];
+    const int2 q = s_slice[l];
+    const int n = q.y - q.x;
+    const bool fits = used + n <= SEG_CACHE;
+    if (fits)
+      for (int i = threadIdx.x; i < n; i += PCG_THREADS) cache[used + i] = L.seg[q.x + i];
+    if (threadIdx.x == 0) {
+      s_segc[l] = fits ? cache + used : nullptr;
+      s_segb[l] = q.x;
+    }
+    if (fits) used += n;
+  }
+  __syncthreads();
+}
+
+// The fluid flags of levels 1.. (a coarse cell is fluid when any child is) and their block
+// flags and segment masks, all of them straight from the binning's active bricks, a warp
+// per brick: lane l has rows 2 (l & 3) and the next of plane l >> 2 of the brick's cells as
+// bits; the rows, planes and bits that share a coarse cell are or-ed.  From level 3 on a
+// brick lies in one cell.  All flags start clear.
+__device__ __noinline__ void level_flags(const PcgArgs& A) {
+  const MgArgs& M = A.mg;
+  const MgLevel& L0 = M.lv[0];
+  const int lane = threadIdx.x & 31;
+  const int n = (int)*A.n_active;
+  for (int q = (int)team_rank() * PCG_WARPS + (int)(threadIdx.x >> 5); q < n;
+       q += (int)team_size() * PCG_WARPS) {
+    const int b = (int)A.active[q];
+    const int bx = b % L0.nbx, by = (b / L0.nbx) % L0.nby, bz = b / (L0.nbx * L0.nby);
+    const int k = bz * 8 + (lane >> 2);
+    unsigned int m = 0u;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int j = by * 8 + 2 * (lane & 3) + h;
+      if (j >= L0.ny || k >= L0.nz) continue;
+      const uint8_t* row = A.type + bx * 8 + L0.nx * (j + L0.ny * k);
+      if (bx * 8 + 8 <= L0.nx && (reinterpret_cast<uintptr_t>(row) & 7u) == 0) {
+        const unsigned long long v = *reinterpret_cast<const unsigned long long*>(row);
+#pragma unroll
+        for (int x = 0; x < 8; ++x) m |= ((unsigned)(v >> (8 * x)) & 255u) == 1u ? 1u << x : 0u;
+      } else {
+        for (int x = 0; x < 8 && bx * 8 + x < L0.nx; ++x) m |= row[x] == 1 ? 1u << x : 0u;
+      }
+    }
+    m |= __shfl_xor_sync(0xffffffffu, m, 4);
+    if (M.nlev > 1 && (lane & 4) == 0) {
+      const MgLevel& L = M.lv[1];
+      const int j = by * 4 + (lane & 3), kk = bz * 4 + (lane >> 3);
+      if (j < L.ny && kk < L.nz) {
+        // the brick's four cells of the row: one word where it is aligned
+        uint8_t* t = L.t + bx * 4 + L.nx * (j + L.ny * kk);
+        const unsigned int c = m | m >> 1;
+        if (bx * 4 + 4 <= L.nx && (reinterpret_cast<uintptr_t>(t) & 3u) == 0) {
+          *reinterpret_cast<unsigned int*>(t) = (c & 1u) | (c >> 2 & 1u) << 8 |
+                                                (c >> 4 & 1u) << 16 | (c >> 6 & 1u) << 24;
+        } else {
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+            if ((c >> (2 * x)) & 1u) t[x] = 1;
+        }
+      }
+    }
+    m |= __shfl_xor_sync(0xffffffffu, m, 1);
+    m |= __shfl_xor_sync(0xffffffffu, m, 8);
+    if (M.nlev > 2 && (lane & 13) == 0) {
+      const MgLevel& L = M.lv[2];
+      const int j = by * 2 + ((lane >> 1) & 1), kk = bz * 2 + (lane >> 4);
+      if (j < L.ny && kk < L.nz)
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+          if ((m >> (4 * x)) & 15u) L.t[bx * 2 + x + L.nx * (j + L.ny * kk)] = 1;
+    }
+    if (lane >= 1 && lane < M.nlev) {
+      const MgLevel& L = M.lv[lane];
+      if (lane >= 3) {
+        const int sh = lane - 3;
+        L.t[(bx >> sh) + L.nx * ((by >> sh) + L.ny * (bz >> sh))] = 1;
+      }
+      if (L.split) L.bflag[(bx >> lane) + L.nbx * ((by >> lane) + L.nby * (bz >> lane))] = 1;
+    }
+    if (lane < M.lgrid) {
+      const MgLevel& L = M.lv[lane];
+      atomicOr(L.segmask + (by >> lane) + L.nby * (bz >> lane), 1u << (bx >> lane >> 3));
+    }
+  }
+}
+
+// Block-rows (the 8 x 8 rows of cells of blocks (*, J, K)) of level 0 up to which every CTA
+// finds its own slices by itself.
+constexpr int SEG_ROWS_PER_THREAD = 8;
+
+// This CTA's slice of each level's active segments, found by every CTA for itself: each
+// counts the segments of all block-rows (MgLevel::segmask: which segments of a row meet a
+// block holding fluid, the same for its 64 rows), scans the counts, and writes those of its
+// own slice, row by row, into the shared-memory cache while the slices fit, else into its
+// part of the level's list.  No CTA reads another's slice, so no grid barrier follows
+// (counting per CTA and writing in segment order took two).
+__device__ __noinline__ void seg_slices(const PcgArgs& A, unsigned int* cache) {
+  const MgArgs& M = A.mg;
+  constexpr int ROUND = 256;  // block-rows written at a time
+  __shared__ int s_scan[PCG_WARPS + 1], s_ra, s_rb, s_at[ROUND];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int used = 0;
+  for (int l = 0; l < M.lgrid; ++l) {
+    const MgLevel& L = M.lv[l];
+    const int nr = L.nby * L.nbz, per_thread = (nr + PCG_THREADS - 1) / PCG_THREADS;
+    const int r0 = (int)threadIdx.x * per_thread;
+    int cnt = 0;
+    for (int u = 0; u < per_thread && r0 + u < nr; ++u) {
+      const int J = (r0 + u) % L.nby, K = (r0 + u) / L.nby;
+      cnt += __popc(L.segmask[r0 + u]) * min(8, L.ny - 8 * J) * min(8, L.nz - 8 * K);
+    }
+    int inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    __syncthreads();
+    if (lane == 31) s_scan[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+      const int t = s_scan[lane];
+      int w = t;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += x;
+      }
+      s_scan[lane] = w - t;
+      if (lane == 31) {
+        const int per = (w + (int)team_size() - 1) / (int)team_size();
+        const bool fits = used + per <= SEG_CACHE;
+        set_slice(l, w);
+        s_segc[l] = fits ? cache + used : nullptr;
+        s_segb[l] = s_slice[l].x;
+        s_scan[PCG_WARPS] = fits ? per : 0;
+        s_ra = nr;
+        s_rb = 0;
+      }
+    }
+    __syncthreads();
+    const int2 q = s_slice[l];
+    unsigned int* dst = s_segc[l] ? cache + used - q.x : L.seg;
+    used += s_scan[PCG_WARPS];
+    // the block-rows that the slice meets are consecutive: [s_ra, s_rb)
+    const int at0 = s_scan[warp] + inc - cnt;
+    const bool mine = cnt > 0 && at0 < q.y && at0 + cnt > q.x;
+    if (mine) {
+      atomicMin(&s_ra, r0);
+      atomicMax(&s_rb, min(nr, r0 + per_thread));
+    }
+    __syncthreads();
+    const int ra = s_ra, rb = s_rb;
+    for (int base = ra; base < rb; base += ROUND) {
+      if (mine) {
+        int at = at0;
+        for (int u = 0; u < per_thread && r0 + u < nr; ++u) {
+          const int J = (r0 + u) % L.nby, K = (r0 + u) / L.nby, r = r0 + u - base;
+          if (r >= 0 && r < ROUND) s_at[r] = at;
+          at += __popc(L.segmask[r0 + u]) * min(8, L.ny - 8 * J) * min(8, L.nz - 8 * K);
+        }
+      }
+      __syncthreads();
+      for (int r = warp; r < min(ROUND, rb - base); r += PCG_WARPS) {  // a warp per block-row
+        const int J = (base + r) % L.nby, K = (base + r) / L.nby;
+        const unsigned int mask = L.segmask[base + r];
+        const int nw = __popc(mask), nj = min(8, L.ny - 8 * J);
+        const int n = nw * nj * min(8, L.nz - 8 * K), at = s_at[r];
+        for (int i = max(0, q.x - at) + lane; i < min(n, q.y - at); i += 32) {
+          const int row = i / nw;
+          dst[at + i] = seg_pack(__fns(mask, 0, i - row * nw + 1), 8 * J + row % nj,
+                                 8 * K + row / nj);
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// Builds, once per solve: the fluid flags of levels 1.. with their block flags, the
+// active-segment slices and the block lists of the colour-split levels, the codes of every
+// level.  Ends with a grid barrier.  All latency: three barriers instead of one per level
+// and five more took the set-up up to the start pass from 41 to 25 us at 64^3, from 155 to
+// 84 us at 256^3 (of which the codes 34 and the flags 20).
+__device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh, unsigned int* cache) {
+  const MgArgs& M = A.mg;
+  // flags start clear (16 bytes at a time: the arrays are padded to 256)
+  for (int l = 1; l < M.nlev; ++l) {
+    const MgLevel& L = M.lv[l];
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const Part p = level_part((L.ncells + 15) / 16, false);
+    for (int c = p.begin; c < p.end; c += p.stride) reinterpret_cast<uint4*>(L.t)[c] = zero;
+    if (L.split) {
+      const Part pb = level_part((L.nbx * L.nby * L.nbz + 15) / 16, false);
+      for (int c = pb.begin; c < pb.end; c += pb.stride) reinterpret_cast<uint4*>(L.bflag)[c] = zero;
+      if (team_rank() == 0 && threadIdx.x == 0) *L.nblk = 0u;
+    }
+  }
+  for (int l = 0; l < M.lgrid; ++l) {
+    const MgLevel& L = M.lv[l];
+    const Part p = level_part(L.nby * L.nbz, false);
+    for (int c = p.begin; c < p.end; c += p.stride) L.segmask[c] = 0u;
+  }
   if (!gsync(A)) return false;
+  SOLVE_TRACE(TR_BFLAG);
+  level_flags(A);
+  if (!gsync(A)) return false;
+  SOLVE_TRACE(TR_FLAGS + 1);
+  block_lists(A);
+  const int lane = threadIdx.x & 31;
+  if (M.lv[0].nby * M.lv[0].nbz <= SEG_ROWS_PER_THREAD * PCG_THREADS) {
+    seg_slices(A, cache);
+  } else {
+    if (!seg_lists(A, sh)) return false;
+    seg_cache_fill(M, cache);
+  }
   SOLVE_TRACE(TR_SEG_WRITE);
   // codes: split levels over their active segments, CTA-local levels over all cells
   for (int l = 0; l < M.lgrid; ++l) {
     const MgLevel& L = M.lv[l];
+    const SV v = sview(L);
     const Items it = seg_items(L, 2);
     for (unsigned int t = it.first; t < it.end; t += PCG_WARPS) {
-      const SCell e = scell(L, L.seg[t >> 1], (int)(t & 1u), lane);
-      if (e.ok) L.code16[e.idx] = (uint16_t)make_code(L, L.t, e.i, e.j, e.k);
+      const SCell e = scell(v, v.seg[(int)(t >> 1) - v.seg_base], (int)(t & 1u), lane);
+      if (e.ok) v.code[e.idx] = (uint16_t)make_code(L, L.t, e.i, e.j, e.k);
     }
   }
   for (int l = M.lgrid; l < M.nlev; ++l) {
@@ -2296,26 +2497,6 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh) {
   const bool ok = gsync(A);
   SOLVE_TRACE(TR_CODES);
   return ok;
-}
-
-// Copies this CTA's slice of each grid-wide level's segment list into the
-// shared-memory cache, level 0 first, while it fits (after build_levels).
-__device__ __noinline__ void seg_cache_fill(const MgArgs& M, unsigned int* cache) {
-  int used = 0;
-  for (int l = 0; l < M.lgrid; ++l) {
-    const MgLevel& L = M.lv[l];
-    const int2 q = seg_slice(L);
-    const int n = q.y - q.x;
-    const bool fits = used + n <= SEG_CACHE;
-    if (fits)
-      for (int i = threadIdx.x; i < n; i += PCG_THREADS) cache[used + i] = L.seg[q.x + i];
-    if (threadIdx.x == 0) {
-      s_segc[l] = fits ? cache + used : nullptr;
-      s_segb[l] = q.x;
-    }
-    if (fits) used += n;
-  }
-  __syncthreads();
 }
 
 // The shared-memory cache of the segment slices sits after the CTA-local levels
@@ -2467,9 +2648,8 @@ __device__ void solve_mg(const PcgArgs& A, Shared& sh, unsigned int* segc, Solve
   float* d = M.d0;
   float* z = L0.x;
   float* r = L0.b;
-  if (!build_levels(A, sh)) { S.ok = false; return; }
+  if (!build_levels(A, sh, segc)) { S.ok = false; return; }
   block_rule(A);
-  seg_cache_fill(M, segc);
   SOLVE_TRACE(TR_SEG_CACHE);
   block_tables(A);  // visible to the V-cycles after the start pass's barrier
   if (M.nlev > 1 && team_rank() == 0) {
@@ -2682,8 +2862,7 @@ __device__ __noinline__ void solve_rbgs(const PcgArgs& A, Shared& sh, unsigned i
   const MgLevel& L1 = M.nlev > 1 ? M.lv[1] : M.lv[0];
   float* z = L0.x;
   float* r = L0.b;
-  if (!build_levels(A, sh)) { S.ok = false; return; }
-  seg_cache_fill(M, segc);
+  if (!build_levels(A, sh, segc)) { S.ok = false; return; }
   {
     FF bb;
     for_fluid0(A, [&](const SCell& e, unsigned int, int n) {

@@ -33,12 +33,30 @@ def masked_scene(n, fill, seed):
     ((144, 96, 80), 0.95),   # level 0 above the limit, the coarser levels blocked
 ])
 def test_blocked_smoothing_matches_the_oracle(n, fill, nu):
-    sc = masked_scene(n, fill, 11)
+    check_one_iteration(masked_scene(n, fill, 11), n, nu)
+
+
+@pytest.mark.parametrize("n,fill", [
+    ((16, 1040, 512), 0.02),  # more segment groups than a CTA scans by itself
+    ((5, 6, 7), 0.7),         # two levels, both in one CTA but the first
+    ((3, 4, 2), 0.6),         # one level
+    ((130, 40, 24), 0.9),     # three segments a row, the last with two cells
+])
+def test_level_set_up_matches_the_oracle(n, fill):
+    """Level flags, segment slices and codes: a wrong one changes the V-cycle at O(1)."""
+    check_one_iteration(masked_scene(n, fill, 7), n, 2)
+
+
+def check_one_iteration(sc, n, nu):
+    """One iteration on the step's own cell types and right-hand side, so that the solve alone
+    is compared (at faces that only vanishing weights reach, P2G's FP32 and FP64 velocities,
+    and with them b, differ at O(1))."""
     op, fp = matched(n, cg_tol=1e-30, cg_max_iter=1, mg_smooth=nu)
-    ref = O.step(op, *sc.arrays())
     with pytest.warns(RuntimeWarning):
         got = gpu_step(fp, sc.arrays())
     assert got["rc"] == F.FLIP_E_NOT_CONVERGED and got["stats"].cg_iterations == 1
-    assert np.array_equal(got["type"], ref.type.ravel())
-    e = rel_l2(got["p"], ref.pressure)
+    typ = got["type"].reshape(n[2], n[1], n[0])
+    ref, _, _ = O.pcg_mg(op, typ, got["rhs"].astype(np.float64).reshape(typ.shape), tol=1e-30,
+                         max_iter=1, nu=nu)
+    e = rel_l2(got["p"], ref)
     assert e <= 1e-5, f"pressure after one MG-PCG iteration: rel L2 {e:.3e}"
