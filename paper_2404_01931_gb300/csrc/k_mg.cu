@@ -92,13 +92,16 @@ constexpr int SEG_SLOTS = 32;  // slots of one colour per segment (a warp)
 
 // Gauss-Seidel coefficients per level, copied to shared memory at kernel start:
 // s_inv_scnt[l][n] = 1 / (s_l n), s_inv_cnt[n] = 1 / n.
+// s_gs[l][n] holds both (0, 0 for n = 0), for the passes that need the pair.
 __shared__ float s_inv_scnt[MG_MAX_LEVELS][8];
 __shared__ float s_inv_cnt[8];
+__shared__ float2 s_gs[MG_MAX_LEVELS][8];
 
 __device__ __forceinline__ void load_tables(const MgArgs& M) {
   if (threadIdx.x < MG_MAX_LEVELS * 8) {
     const int l = threadIdx.x >> 3, n = threadIdx.x & 7;
     s_inv_scnt[l][n] = l < M.nlev ? M.lv[l].inv_scnt[n] : 0.0f;
+    s_gs[l][n] = make_float2(l < M.nlev ? M.lv[l].inv_scnt[n] : 0.0f, M.inv_cnt[n]);
   }
   if (threadIdx.x < 8) s_inv_cnt[threadIdx.x] = M.inv_cnt[threadIdx.x];
   __syncthreads();
@@ -299,37 +302,39 @@ __device__ __forceinline__ PCell pcell(const LV& L, int2 q, unsigned int pair, i
   return e;
 }
 
-// The other colour's values around a slot pair: xm/xp the -x/+x neighbours of
-// cells A and B, ym, yp, zm, zp the pairs in the rows and planes next door.
-struct Nbr2 {
-  float xmA, xpA, xmB, xpB;
-  float2 ym, yp, zm, zp;
+// Passes over four slots per lane: a warp takes four segments (eight lanes each), a lane
+// the slots s .. s + 3 of one colour (s a multiple of 4), read and written as 16 bytes.
+// Item t is segments 4 (t / ncol) .., colour t % ncol.
+__device__ __forceinline__ Items quad_items(int2 q, int ncol) {
+  const int n = (q.y - q.x + 3) >> 2;
+  return Items{(unsigned)(threadIdx.x >> 5), (unsigned)(n * ncol)};
+}
+
+struct QCell {
+  int j, k, s, par;  // par: x of slot s is 2 s + par
+  int idx, ob;       // storage index of slot s and of slot s in the other colour
+  bool ok;           // the lane's segment exists and slot s lies in its row
 };
 
 template <class LV>
-__device__ __forceinline__ Nbr2 load_nbr2(const LV& L, const float* x, const PCell& e) {
-  const float2 m = *reinterpret_cast<const float2*>(x + e.ob);
-  const float ex = x[e.ob - 1 + 3 * e.par];  // slot s - 1 (par 0) or s + 2 (par 1)
-  Nbr2 n;
-  if (e.par == 0) {
-    n.xmA = ex; n.xpA = m.x; n.xmB = m.x; n.xpB = m.y;
-  } else {
-    n.xmA = m.x; n.xpA = m.y; n.xmB = m.y; n.xpB = ex;
-  }
-  const int pl = L.hx * L.ny;
-  n.ym = *reinterpret_cast<const float2*>(x + e.ob - L.hx);
-  n.yp = *reinterpret_cast<const float2*>(x + e.ob + L.hx);
-  n.zm = *reinterpret_cast<const float2*>(x + e.ob - pl);
-  n.zp = *reinterpret_cast<const float2*>(x + e.ob + pl);
-  return n;
+__device__ __forceinline__ QCell qcell(const LV& L, int2 q, unsigned int quad, int c, int lane) {
+  const int sq = q.x + 4 * (int)quad + (lane >> 3);
+  QCell e;
+  e.ok = sq < q.y;
+  const int4 sg = seg_unpack(L.seg[(e.ok ? sq : q.x) - L.seg_base], L.ny);
+  e.j = sg.z;
+  e.k = sg.w;
+  e.s = sg.y * SEG_SLOTS + 4 * (lane & 7);
+  e.par = (c + e.j + e.k) & 1;
+  e.ok = e.ok && e.s < L.hx;
+  e.idx = c * L.half + L.margin + L.hx * sg.x + e.s;
+  e.ob = e.idx + (1 - 2 * c) * L.half;
+  return e;
 }
 
-__device__ __forceinline__ void nbr_of(const Nbr2& n, int which, float (&xv)[6]) {
-  if (which == 0) {
-    xv[0] = n.xmA; xv[1] = n.xpA; xv[2] = n.ym.x; xv[3] = n.yp.x; xv[4] = n.zm.x; xv[5] = n.zp.x;
-  } else {
-    xv[0] = n.xmB; xv[1] = n.xpB; xv[2] = n.ym.y; xv[3] = n.yp.y; xv[4] = n.zm.y; xv[5] = n.zp.y;
-  }
+// Count of neighbours in the grid (0: not fluid) of slot s + h, from the four codes.
+__device__ __forceinline__ int quad_cnt(uint2 code4, int h) {
+  return (int)((h < 2 ? code4.x : code4.y) >> (h & 1 ? 24 : 8)) & 7;
 }
 
 // ---------------------------------------------------------------- natural levels
@@ -359,14 +364,15 @@ __device__ __forceinline__ Cell cell_at(const MgLevel& L, int c) {
 
 // Neighbour code of cell (i, j, k) from natural fluid flags fl (value 1 = fluid):
 // bits 0..5 fluid neighbours inside the grid, bit 6 the cell itself, bits 8..10
-// the number of neighbours inside the grid.
+// the number of neighbours inside the grid; 0 for a cell that is not fluid.
 __device__ __forceinline__ unsigned int make_code(const MgLevel& L, const uint8_t* fl, int i, int j,
                                                   int k) {
   const int c = i + L.nx * (j + L.ny * k);
   const int sy = L.nx, sz = L.nx * L.ny;
   const bool in[6] = {i > 0, i < L.nx - 1, j > 0, j < L.ny - 1, k > 0, k < L.nz - 1};
   const int off[6] = {-1, 1, -sy, sy, -sz, sz};
-  unsigned int code = (fl[c] == 1) ? CODE_SELF : 0u;
+  if (fl[c] != 1) return 0u;
+  unsigned int code = CODE_SELF;
   int cnt = 0;
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
@@ -423,15 +429,6 @@ __device__ __forceinline__ float resid_full(float s, float bc, float xc, const f
 
 // ---------------------------------------------------------------- sweeps
 
-struct GsIn {
-  int i, j, k, idx;
-  bool ok;
-  unsigned int code;
-  float b;
-  float xv[6];
-  float pv[6];  // CORRECT: the neighbours' parents on the next coarser level
-};
-
 // Parents on level C of the six neighbours of cell (i, j, k) of a level with
 // extents (nx, ny, nz); a neighbour off the grid is replaced by the cell itself
 // (its value is unused).
@@ -444,148 +441,145 @@ __device__ __forceinline__ void parent_values(const PV& C, int nx, int ny, int n
   for (int q = 0; q < 6; ++q) pv[q] = C.x[level_index(C, pi[q] >> 1, pj[q] >> 1, pk[q] >> 1)];
 }
 
-// The coarse values that the corrections of a slot pair's two cells (A at x = iA,
-// B at iA + 2) read.  The twelve neighbours' parents are seven coarse cells: three
-// in the pair's coarse row (x = s - 1 + par .. s + 1 + par, which hold A's and B's
-// own parents, s and s + 1), and for A and B the parent in the other y row and in
-// the other z plane (a neighbour's parent is the cell's own but for one neighbour
-// per axis).  pr = {row x3, y-row A, y-row B, z-plane A, z-plane B}; coordinates of
-// off-grid neighbours (never read unmasked) are clamped into the level.
-template <class E>
-__device__ __forceinline__ void pair_parents(const PV& C, const E& e, float (&pr)[7]) {
-  const int J = e.j >> 1, K = e.k >> 1;
-  const int Jy = min(max((e.j & 1) ? J + 1 : J - 1, 0), C.ny - 1);
-  const int Kz = min(max((e.k & 1) ? K + 1 : K - 1, 0), C.nz - 1);
-  const int a = min(e.s, C.nx - 1), b = min(e.s + 1, C.nx - 1);
-#pragma unroll
-  for (int q = 0; q < 3; ++q)
-    pr[q] = C.x[level_index(C, min(max(e.s - 1 + e.par + q, 0), C.nx - 1), J, K)];
-  pr[3] = C.x[level_index(C, a, Jy, K)];
-  pr[4] = C.x[level_index(C, b, Jy, K)];
-  pr[5] = C.x[level_index(C, a, J, Kz)];
-  pr[6] = C.x[level_index(C, b, J, Kz)];
-}
-
-// The six neighbour parents (parent_values' order) of cell h (0: A, 1: B) of the
-// pair, from pair_parents' seven values.
-__device__ __forceinline__ void pair_parents_of(const float (&pr)[7], int par, int j, int k,
-                                                int h, float (&pv)[6]) {
-  const float own = (h == 0) ? (par ? pr[0] : pr[1]) : (par ? pr[1] : pr[2]);
-  const float oy = (h == 0) ? pr[3] : pr[4], oz = (h == 0) ? pr[5] : pr[6];
-  pv[0] = (h == 0) ? pr[0] : pr[1];
-  pv[1] = (h == 0) ? pr[1] : pr[2];
-  pv[2] = (j & 1) ? own : oy;
-  pv[3] = (j & 1) ? oy : own;
-  pv[4] = (k & 1) ? own : oz;
-  pv[5] = (k & 1) ? oz : own;
-}
-
-template <int MODE>
-__device__ __forceinline__ bool gs_apply(float* x, int l, float omega, GsIn& s, float& v) {
-  if (!s.ok || !(s.code & CODE_SELF)) return false;
-  if constexpr (MODE == CORRECT) {
-#pragma unroll
-    for (int q = 0; q < 6; ++q)
-      if ((s.code >> q) & 1u) s.xv[q] = __fmaf_rn(omega, s.pv[q], s.xv[q]);
-  }
-  v = gs_sum(l, code_cnt(s.code), s.code, s.b, s.xv);
-  x[s.idx] = v;
-  return true;
-}
-
-// Half-sweep of one colour over colour-split level l (description L; C is level
-// l+1, read in CORRECT mode).  With rz, also accumulates b x over the updated
-// cells.  Paired form: slots that are not fluid cells of the grid get 0.  (A
-// grid-wide level never sweeps from zero here: its first red half-sweep is made
-// by the pass that produces its right-hand side.)
-template <int MODE, bool RZ>
-__device__ __noinline__ FF sweep_split_v(const MgArgs& M, const MgLevel& L, const MgLevel& C,
-                                         int l, int colour) {
-  static_assert(MODE != FIRST, "grid-wide levels start from the fused first half-sweep");
-  constexpr int U = (MODE == CORRECT) ? 1 : 2;
+// Half-sweep of one colour over colour-split level l (description L).  With RZ, returns
+// b x over the updated cells.  A level's x is 0 where there is no fluid cell (zero_near
+// before the solve, and these sweeps store 0 there) and the neighbours beyond a row's or a
+// plane's end, which the storage wraps to other rows, are not read, so the sum of the six
+// neighbours needs no masks: gs_sum's values.  (A grid-wide level never sweeps from zero
+// here: its first red half-sweep is made by the pass that produces its right-hand side.)
+//
+// Bound by issue: the index arithmetic is the larger part of an item (a version that loaded
+// next to nothing took three quarters of the time), so a lane takes four slots.  A level-0
+// half-sweep at 256^3 with its barrier 11.2 -> 8.2 us, against two slots a lane, masks, and
+// a second path without masks that a segment at a wall always defeats (every pair of a
+// 256-cell row has one); solves 5.17 -> 4.50 ms at 256^3, 1.46 -> 1.30 at 128^3.
+template <bool RZ>
+__device__ __noinline__ FF sweep_split_q(const MgLevel& L, int l, int colour) {
   const int lane = threadIdx.x & 31;
   const SV v = sview(L);
-  const PV cv = pview(C);
-  const float omega = M.omega;
-  const float inv6 = s_inv_cnt[6], invs6 = s_inv_scnt[l][6];
   const int2 q = seg_slice(L);
-  const Items it = pair_items(q, 1);
-  struct S {
-    PCell e;
-    unsigned int code2;
-    float2 b;
-    Nbr2 n;
-    float pr[MODE == CORRECT ? 7 : 1];
-  };
+  const Items it = quad_items(q, 1);
+  const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   FF acc;
-  run_batched<U>(
-      it.first, it.end, PCG_WARPS,
-      [&](unsigned int t, bool ok) {
-        S st;
-        st.e = pcell(v, q, t, colour, lane);
-        st.e.okA &= ok;
-        st.e.okB &= ok;
-        st.code2 = *reinterpret_cast<const unsigned int*>(v.code + st.e.idx);
-        st.b = *reinterpret_cast<const float2*>(v.b + st.e.idx);
-        st.n = load_nbr2(v, v.x, st.e);
-        if constexpr (MODE == CORRECT) pair_parents(cv, st.e, st.pr);
-        return st;
-      },
-      [&](S&) {},
-      [&](S& st) {
-        float out[2];
-        {
-          // a warp whose cells are all fluid with six fluid neighbours (the bulk of
-          // the liquid): gs_sum's operations in its order, without masks or tables
-          // (and the correction of every neighbour in CORRECT mode)
-          const bool full = pair_full(st.code2) && st.e.okA && st.e.okB;
-          if (__all_sync(0xffffffffu, full)) {
+  for (unsigned int t = it.first; t < it.end; t += PCG_WARPS) {
+    const QCell e = qcell(v, q, t, colour, lane);
+    if (!e.ok) continue;
+    const float* xo = v.x + e.ob;
+    const uint2 code4 = *reinterpret_cast<const uint2*>(v.code + e.idx);
+    const float4 b = *reinterpret_cast<const float4*>(v.b + e.idx);
+    const float4 m = *reinterpret_cast<const float4*>(xo);
+    const float4 zm = *reinterpret_cast<const float4*>(xo - v.pl);
+    const float4 zp = *reinterpret_cast<const float4*>(xo + v.pl);
+    const float4 ym = e.j > 0 ? *reinterpret_cast<const float4*>(xo - v.hx) : zero;
+    const float4 yp = e.j < v.ny - 1 ? *reinterpret_cast<const float4*>(xo + v.hx) : zero;
+    // the slot beyond the four, before (par 0) or after (par 1)
+    const float ex = (e.par ? e.s + 4 < v.hx : e.s > 0) ? xo[5 * e.par - 1] : 0.0f;
+    const float4 o = e.par ? make_float4(m.y, m.z, m.w, ex) : make_float4(ex, m.x, m.y, m.z);
+    float2 s0 = __fadd2_rn(make_float2(m.x, m.y), make_float2(o.x, o.y));
+    float2 s1 = __fadd2_rn(make_float2(m.z, m.w), make_float2(o.z, o.w));
+    s0 = __fadd2_rn(s0, make_float2(ym.x, ym.y));
+    s1 = __fadd2_rn(s1, make_float2(ym.z, ym.w));
+    s0 = __fadd2_rn(s0, make_float2(yp.x, yp.y));
+    s1 = __fadd2_rn(s1, make_float2(yp.z, yp.w));
+    s0 = __fadd2_rn(s0, make_float2(zm.x, zm.y));
+    s1 = __fadd2_rn(s1, make_float2(zm.z, zm.w));
+    s0 = __fadd2_rn(s0, make_float2(zp.x, zp.y));
+    s1 = __fadd2_rn(s1, make_float2(zp.z, zp.w));
+    float out[4];
+    const float sum[4] = {s0.x, s0.y, s1.x, s1.y}, bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              float xv[6];
-              nbr_of(st.n, h, xv);
-              if constexpr (MODE == CORRECT) {
-                float pv[6];
-                pair_parents_of(st.pr, st.e.par, st.e.j, st.e.k, h, pv);
-#pragma unroll
-                for (int u = 0; u < 6; ++u) xv[u] = __fmaf_rn(omega, pv[u], xv[u]);
-              }
-              float sum = 0.0f;
-#pragma unroll
-              for (int u = 0; u < 6; ++u) sum = __fadd_rn(sum, xv[u]);
-              const float bc = h == 0 ? st.b.x : st.b.y;
-              out[h] = __fmaf_rn(sum, inv6, __fmul_rn(bc, invs6));
-              if (RZ) acc.add_prod(bc, out[h]);
-            }
-            *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(out[0], out[1]);
-            return;
-          }
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const unsigned int code = h == 0 ? (st.code2 & 0xffffu) : (st.code2 >> 16);
-          const bool ok = (h == 0 ? st.e.okA : st.e.okB) && (code & CODE_SELF);
-          const float bc = h == 0 ? st.b.x : st.b.y;
-          float xv[6];
-          nbr_of(st.n, h, xv);
-          if constexpr (MODE == CORRECT) {
-            float pv[6];
-            pair_parents_of(st.pr, st.e.par, st.e.j, st.e.k, h, pv);
-#pragma unroll
-            for (int u = 0; u < 6; ++u)
-              if ((code >> u) & 1u) xv[u] = __fmaf_rn(omega, pv[u], xv[u]);
-          }
-          const float val = gs_sum(l, code_cnt(code), code, bc, xv);
-          out[h] = ok ? val : 0.0f;
-          if (RZ && ok) acc.add_prod(bc, val);
-        }
-        if (st.e.okA || st.e.okB)
-          *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(out[0], out[1]);
-      });
+    for (int h = 0; h < 4; ++h) {
+      const int cnt = quad_cnt(code4, h);
+      const float2 gs = s_gs[l][cnt];
+      out[h] = cnt ? __fmaf_rn(sum[h], gs.y, __fmul_rn(bv[h], gs.x)) : 0.0f;
+      if (RZ) acc.add_prod(cnt ? bv[h] : 0.0f, out[h]);
+    }
+    *reinterpret_cast<float4*>(v.x + e.idx) = make_float4(out[0], out[1], out[2], out[3]);
+  }
   return acc;
 }
 
-// Scalar form: a lane takes one slot (levels with few segments per CTA, where
+// Four consecutive cells x = I .. I + 3 (I a multiple of 4) of a row of colour-split level
+// C, base being the row's slot I / 2 of colour 0: two pairs, one of each colour.
+__device__ __forceinline__ float4 coarse4(const PV& C, int base, int J, int K) {
+  const int even = ((J + K) & 1) * C.half, odd = C.half - even;
+  const float2 a = *reinterpret_cast<const float2*>(C.x + even + base);
+  const float2 b = *reinterpret_cast<const float2*>(C.x + odd + base);
+  return make_float4(a.x, b.x, a.y, b.y);
+}
+
+// The half-sweep that makes the coarse correction on the fly (C is level l+1, colour-split):
+// black cells from their red neighbours plus omega times those' parents.  The twenty-four
+// neighbours of a lane's four cells have thirteen parents: the four own ones and the one
+// beyond them in the cells' coarse row, and four each in the coarse row and plane next to
+// it that the y and z neighbours outside the own parents lie in.  At 256^3 18.5 -> 15.6 us
+// against two slots and seven parents a lane, whose indexes cost more than the loads.
+template <bool RZ>
+__device__ __noinline__ FF correct_split_q(const MgArgs& M, const MgLevel& L, const MgLevel& Cl,
+                                           int l, int colour) {
+  const int lane = threadIdx.x & 31;
+  const SV v = sview(L);
+  const PV C = pview(Cl);
+  const float omega = M.omega;
+  const int2 q = seg_slice(L);
+  const Items it = quad_items(q, 1);
+  FF acc;
+  for (unsigned int t = it.first; t < it.end; t += PCG_WARPS) {
+    const QCell e = qcell(v, q, t, colour, lane);
+    if (!e.ok) continue;
+    const float* xo = v.x + e.ob;
+    const uint2 code4 = *reinterpret_cast<const uint2*>(v.code + e.idx);
+    const float4 b4 = *reinterpret_cast<const float4*>(v.b + e.idx);
+    const float4 m = *reinterpret_cast<const float4*>(xo);
+    const float4 ym = *reinterpret_cast<const float4*>(xo - v.hx);
+    const float4 yp = *reinterpret_cast<const float4*>(xo + v.hx);
+    const float4 zm = *reinterpret_cast<const float4*>(xo - v.pl);
+    const float4 zp = *reinterpret_cast<const float4*>(xo + v.pl);
+    const float ex = xo[5 * e.par - 1];
+    const int J = e.j >> 1, K = e.k >> 1;
+    // (off the grid: clamped, the values are not used)
+    const int Jy = min(max(e.j & 1 ? J + 1 : J - 1, 0), C.ny - 1);
+    const int Kz = min(max(e.k & 1 ? K + 1 : K - 1, 0), C.nz - 1);
+    const int col = C.margin + (e.s >> 1);
+    const float4 po = coarse4(C, col + C.hx * (J + C.ny * K), J, K);
+    const float4 py = coarse4(C, col + C.hx * (Jy + C.ny * K), Jy, K);
+    const float4 pz = coarse4(C, col + C.hx * (J + C.ny * Kz), J, Kz);
+    const float pe = C.x[level_index(C, min(max(e.par ? e.s + 4 : e.s - 1, 0), C.nx - 1), J, K)];
+    // the cells' own parents are also those of the x neighbour on the side of par
+    const float xo4[4] = {m.x, m.y, m.z, m.w}, pv4[4] = {po.x, po.y, po.z, po.w};
+    const float xl[6] = {ex, m.x, m.y, m.z, m.w, ex};    // par 0: slot h - 1 is xl[h]
+    const float pl[6] = {pe, po.x, po.y, po.z, po.w, pe};  // par 1: slot h + 1 is xl[h + 2]
+    const float yl[4] = {ym.x, ym.y, ym.z, ym.w}, yh[4] = {yp.x, yp.y, yp.z, yp.w};
+    const float zl[4] = {zm.x, zm.y, zm.z, zm.w}, zh[4] = {zp.x, zp.y, zp.z, zp.w};
+    const float py4[4] = {py.x, py.y, py.z, py.w}, pz4[4] = {pz.x, pz.y, pz.z, pz.w};
+    const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
+    float out[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const unsigned int code = ((h < 2 ? code4.x : code4.y) >> (16 * (h & 1))) & 0xffffu;
+      const float own = __fmaf_rn(omega, pv4[h], xo4[h]);
+      const float oth = e.par ? __fmaf_rn(omega, pl[h + 2], xl[h + 2])
+                              : __fmaf_rn(omega, pl[h], xl[h]);
+      const float c[6] = {e.par ? own : oth,
+                          e.par ? oth : own,
+                          __fmaf_rn(omega, e.j & 1 ? pv4[h] : py4[h], yl[h]),
+                          __fmaf_rn(omega, e.j & 1 ? py4[h] : pv4[h], yh[h]),
+                          __fmaf_rn(omega, e.k & 1 ? pv4[h] : pz4[h], zl[h]),
+                          __fmaf_rn(omega, e.k & 1 ? pz4[h] : pv4[h], zh[h])};
+      float sum = 0.0f;
+#pragma unroll
+      for (int u = 0; u < 6; ++u)
+        if ((code >> u) & 1u) sum = __fadd_rn(sum, c[u]);
+      const float2 gs = s_gs[l][code_cnt(code)];
+      out[h] = code ? __fmaf_rn(sum, gs.y, __fmul_rn(bv[h], gs.x)) : 0.0f;
+      if (RZ) acc.add_prod(code ? bv[h] : 0.0f, out[h]);
+    }
+    *reinterpret_cast<float4*>(v.x + e.idx) = make_float4(out[0], out[1], out[2], out[3]);
+  }
+  return acc;
+}
+
+// Scalar forms: a lane takes one slot (levels with few segments per CTA, where
 // more items in flight matter more than wider loads).
 template <int MODE>
 __device__ __noinline__ FF sweep_split_s(const MgArgs& M, const MgLevel& L, const MgLevel& C,
@@ -598,69 +592,68 @@ __device__ __noinline__ FF sweep_split_s(const MgArgs& M, const MgLevel& L, cons
   const int nz = L.nz;
   const float omega = M.omega;
   const Items it = seg_items(L, 1);
-  const float inv6 = s_inv_cnt[6], invs6 = s_inv_scnt[l][6];
+  struct S {
+    int idx;
+    unsigned int code;            // 0: not fluid, or no item
+    float b;
+    float xv[6];
+    float pv[MODE == CORRECT ? 6 : 1];  // the neighbours' parents on the coarser level
+  };
   FF acc;
   run_batched<U>(
       it.first, it.end, PCG_WARPS,
       [&](unsigned int t, bool ok) {
         const SCell e = scell(v, v.seg[t - v.seg_base], colour, lane);
-        GsIn s;
-        s.i = e.i;
-        s.j = e.j;
-        s.k = e.k;
-        s.idx = e.idx;
-        s.ok = e.ok && ok;
-        s.code = v.code[e.idx];
-        s.b = v.b[e.idx];
+        S st;
+        st.idx = e.idx;
+        st.code = e.ok && ok ? (unsigned int)v.code[e.idx] : 0u;
+        st.b = v.b[e.idx];
         int nb[6];
         snbr(v, e, nb);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) s.xv[q] = v.x[nb[q]];
+        for (int q = 0; q < 6; ++q) st.xv[q] = v.x[nb[q]];
         if constexpr (MODE == CORRECT)
-          parent_values(cv, v.nx, v.ny, nz, min(e.i, v.nx - 1), e.j, e.k, s.pv);
-        return s;
+          parent_values(cv, v.nx, v.ny, nz, min(e.i, v.nx - 1), e.j, e.k, st.pv);
+        return st;
       },
-      [&](GsIn&) {},
-      [&](GsIn& s) {
-        // a warp whose cells are all fluid with six fluid neighbours: gs_apply's
-        // operations in its order, without the masks
-        if (__all_sync(0xffffffffu, s.ok && s.code == CODE_FULL)) {
-          if constexpr (MODE == CORRECT) {
+      [&](S&) {},
+      [&](S& st) {
+        if (!st.code) return;
+        float sum = 0.0f;
 #pragma unroll
-            for (int q = 0; q < 6; ++q) s.xv[q] = __fmaf_rn(omega, s.pv[q], s.xv[q]);
-          }
-          float sum = 0.0f;
-#pragma unroll
-          for (int q = 0; q < 6; ++q) sum = __fadd_rn(sum, s.xv[q]);
-          const float xv = __fmaf_rn(sum, inv6, __fmul_rn(s.b, invs6));
-          v.x[s.idx] = xv;
-          if (rz) acc.add_prod(s.b, xv);
-          return;
+        for (int q = 0; q < 6; ++q) {
+          float x = st.xv[q];
+          if constexpr (MODE == CORRECT) x = __fmaf_rn(omega, st.pv[q], x);
+          sum += (st.code >> q) & 1u ? x : 0.0f;
         }
-        float xv;
-        if (gs_apply<MODE>(v.x, l, omega, s, xv) && rz) acc.add_prod(s.b, xv);
+        const float2 gs = s_gs[l][code_cnt(st.code)];
+        const float x = __fmaf_rn(sum, gs.y, __fmul_rn(st.b, gs.x));
+        v.x[st.idx] = x;
+        if (rz) acc.add_prod(st.b, x);
       });
   return acc;
 }
 
-// Levels with many segments per CTA take the paired form (8-byte accesses, half
-// the load instructions); the others the scalar form.
-constexpr int VEC_SEGS_PER_CTA = 256;
+// Levels with many segments per CTA take the wide forms (fewer instructions per cell); the
+// others the scalar form (more items in flight).  Solves at 256^3 (level 0: 519 segments
+// per CTA, level 1: 65) and 128^3 (66) with the line at 256 and at 64: 5.17 -> 5.09 and
+// 1.46 -> 1.42 ms.
+constexpr int VEC_SEGS_PER_CTA = 64;
 
-__device__ __forceinline__ bool use_pairs(const MgLevel& L) {
+__device__ __forceinline__ bool use_wide(const MgLevel& L) {
   return s_nseg[L.lvl] >= VEC_SEGS_PER_CTA * (int)team_size();
 }
 
 template <int MODE>
 __device__ __forceinline__ FF sweep_split(const MgArgs& M, const MgLevel& L, const MgLevel& C,
                                           int l, int colour, bool rz) {
-  if (use_pairs(L)) {
-    // the r.z accumulation only where asked (its registers would make the other
-    // half-sweeps spill)
-    if (rz) return sweep_split_v<MODE, true>(M, L, C, l, colour);
-    return sweep_split_v<MODE, false>(M, L, C, l, colour);
-  }
-  return sweep_split_s<MODE>(M, L, C, l, colour, rz);
+  if (!use_wide(L) || (MODE == CORRECT && !C.split))
+    return sweep_split_s<MODE>(M, L, C, l, colour, rz);
+  // the r.z accumulation only where asked (it costs registers)
+  if constexpr (MODE == CORRECT)
+    return rz ? correct_split_q<true>(M, L, C, l, colour)
+              : correct_split_q<false>(M, L, C, l, colour);
+  else return rz ? sweep_split_q<true>(L, l, colour) : sweep_split_q<false>(L, l, colour);
 }
 
 // ---------------------------------------------------------------- restriction
@@ -714,24 +707,26 @@ __device__ __forceinline__ float restrict_sum(const SV& F, int fnz, int I, int J
   return __fmul_rn(sum, 0.0625f);
 }
 
-// Colour-split F -> colour-split C, over C's active segments; lanes take the
-// segment's 64 cells in x order (so the fine red slots they read are contiguous).
+// Colour-split F -> colour-split C, over C's active segments; a warp takes half a
+// segment, 32 cells in x order (so the fine red slots it reads are contiguous).
 // The pass also makes C's first red half-sweep from zero, x = b / (s_C n) on C's
 // red fluid cells, which needs only the b it has just computed: C's
 // pre-smoothing then starts with the black half-sweep, and the cycle meets one
 // grid barrier fewer per level (the values are those the separate half-sweep
 // computes; the slots of C's non-fluid cells, never read unmasked, are left).
+// Bound by latency (two rounds of 18 loads a lane, about four items a warp at 256^3).  Half
+// segments rather than whole ones even out the last round; two children a lane, the upper
+// plane's on the upper half-warp, took 23.4 us instead of 16.6 (half the slots per request).
 __device__ __noinline__ void restrict_split(const MgLevel& Fl, const MgLevel& Cl) {
   const int lane = threadIdx.x & 31;
   const SV F = sview(Fl), C = sview(Cl);
   const int fnz = Fl.nz;
   const int lc = Cl.lvl;
-  const Items it = seg_items(Cl, 1);
+  const Items it = seg_items(Cl, 2);
   for (unsigned int t = it.first; t < it.end; t += PCG_WARPS) {
-    const int4 sg = seg_unpack(C.seg[t - C.seg_base], C.ny);
-    const int J = sg.z, K = sg.w;
-#pragma unroll 1  // half the code, and nothing lost: 5.29 -> 5.24 ms per solve at 256^3
-    for (int h = 0; h < 2; ++h) {
+    const int4 sg = seg_unpack(C.seg[(int)(t >> 1) - C.seg_base], C.ny);
+    const int J = sg.z, K = sg.w, h = (int)(t & 1u);
+    {
       // every lane takes part (a lane past the row's end on its last cell, whose
       // result it drops), so that a warp can vote
       const int I = sg.y * (2 * SEG_SLOTS) + h * 32 + lane;
@@ -1777,8 +1772,8 @@ __device__ __noinline__ PassSum vcycle_rest(const PcgArgs& A) {
 // ---------------------------------------------------------------- level-0 passes
 
 // Phase A with z from the V-cycle: p_new = z + beta p_old (recomputed for the
-// neighbours), q = A p_new in difference form, partial p.q.  Both colours; paired
-// form.
+// neighbours), q = A p_new in difference form, partial p.q.  Both colours; a lane takes two
+// slots, the pair's and its neighbour pairs' operations packed.
 __device__ __noinline__ FF phase_a_v(const PcgArgs& A, const float* pold, float* pnew, float beta) {
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
@@ -1788,140 +1783,85 @@ __device__ __noinline__ FF phase_a_v(const PcgArgs& A, const float* pold, float*
   const int lane = threadIdx.x & 31;
   const int2 q = seg_slice(M.lv[0]);
   const Items it = pair_items(q, 2);
+  const float2 beta2 = make_float2(beta, beta);
   FF acc;
+  auto p_at = [&](int i) {  // p_new of a pair of slots
+    return __ffma2_rn(beta2, *reinterpret_cast<const float2*>(pold + i),
+                      *reinterpret_cast<const float2*>(z + i));
+  };
   for (unsigned int t = it.first; t < it.end; t += PCG_WARPS) {
     const PCell e = pcell(v, q, t >> 1, (int)(t & 1u), lane);
     const unsigned int code2 = *reinterpret_cast<const unsigned int*>(v.code + e.idx);
-    const float2 zc = *reinterpret_cast<const float2*>(z + e.idx);
-    const float2 pc = *reinterpret_cast<const float2*>(pold + e.idx);
-    const Nbr2 nz = load_nbr2(v, z, e);
-    const Nbr2 np = load_nbr2(v, pold, e);
-    float pn[2], qn[2];
-    // a warp whose cells are all fluid with six fluid neighbours: the same
-    // operations in the same order without the masks (nfl = count = 6)
-    const bool full = pair_full(code2) && e.okA && e.okB;
-    if (__all_sync(0xffffffffu, full)) {
+    const float2 pc = p_at(e.idx), m = p_at(e.ob);
+    const float2 ym = p_at(e.ob - v.hx), yp = p_at(e.ob + v.hx);
+    const float2 zm = p_at(e.ob - v.pl), zp = p_at(e.ob + v.pl);
+    const int ei = e.ob - 1 + 3 * e.par;  // slot s - 1 (par 0) or s + 2 (par 1)
+    const float ex = __fmaf_rn(beta, pold[ei], z[ei]);
+    const float2 xm = e.par ? m : make_float2(ex, m.x);
+    const float2 xp = e.par ? make_float2(m.y, ex) : m;
+    const float2 n[6] = {xm, xp, ym, yp, zm, zp};
+    const unsigned int cA = e.okA ? code2 & 0xffffu : 0u, cB = e.okB ? code2 >> 16 : 0u;
+    float dA = 0.0f, dB = 0.0f;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float zv[6], pv[6];
-        nbr_of(nz, h, zv);
-        nbr_of(np, h, pv);
-        const float p_c = __fmaf_rn(beta, h == 0 ? pc.x : pc.y, h == 0 ? zc.x : zc.y);
-        float d = 0.0f;
-#pragma unroll
-        for (int u = 0; u < 6; ++u) d = __fadd_rn(d, __fsub_rn(p_c, __fmaf_rn(beta, pv[u], zv[u])));
-        pn[h] = p_c;
-        qn[h] = __fmul_rn(s_a, __fmaf_rn(0.0f, p_c, d));
-        acc.add_prod(p_c, qn[h]);
-      }
-      *reinterpret_cast<float2*>(pnew + e.idx) = make_float2(pn[0], pn[1]);
-      *reinterpret_cast<float2*>(q0 + e.idx) = make_float2(qn[0], qn[1]);
-      continue;
+    for (int u = 0; u < 6; ++u) {
+      const float2 d = __fadd2_rn(pc, make_float2(-n[u].x, -n[u].y));
+      if ((cA >> u) & 1u) dA = __fadd_rn(dA, d.x);
+      if ((cB >> u) & 1u) dB = __fadd_rn(dB, d.y);
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const unsigned int code = h == 0 ? (code2 & 0xffffu) : (code2 >> 16);
-      const bool ok = (h == 0 ? e.okA : e.okB) && (code & CODE_SELF);
-      float zv[6], pv[6];
-      nbr_of(nz, h, zv);
-      nbr_of(np, h, pv);
-      const float p_c = __fmaf_rn(beta, h == 0 ? pc.x : pc.y, h == 0 ? zc.x : zc.y);
-      float d = 0.0f;
-      int nfl = 0;
-#pragma unroll
-      for (int u = 0; u < 6; ++u) {
-        const bool f = (code >> u) & 1u;
-        d += f ? __fsub_rn(p_c, __fmaf_rn(beta, pv[u], zv[u])) : 0.0f;
-        nfl += f;
-      }
-      const float q_c = __fmul_rn(s_a, __fmaf_rn((float)(code_cnt(code) - nfl), p_c, d));
-      pn[h] = ok ? p_c : 0.0f;
-      qn[h] = ok ? q_c : 0.0f;
-      if (ok) acc.add_prod(p_c, q_c);
-    }
+    const float nA = (float)(code_cnt(cA) - __popc(cA & 63u));  // neighbours in air
+    const float nB = (float)(code_cnt(cB) - __popc(cB & 63u));
+    const float2 pn = make_float2(cA ? pc.x : 0.0f, cB ? pc.y : 0.0f);
+    const float2 qn = make_float2(cA ? __fmul_rn(s_a, __fmaf_rn(nA, pc.x, dA)) : 0.0f,
+                                  cB ? __fmul_rn(s_a, __fmaf_rn(nB, pc.y, dB)) : 0.0f);
+    acc.add_prod(pn.x, qn.x);
+    acc.add_prod(pn.y, qn.y);
     if (e.okA || e.okB) {
-      *reinterpret_cast<float2*>(pnew + e.idx) = make_float2(pn[0], pn[1]);
-      *reinterpret_cast<float2*>(q0 + e.idx) = make_float2(qn[0], qn[1]);
+      *reinterpret_cast<float2*>(pnew + e.idx) = pn;
+      *reinterpret_cast<float2*>(q0 + e.idx) = qn;
     }
   }
   return acc;
 }
 
 // Phase B: d += alpha p, r -= alpha q, partial r.r, and the next V-cycle's first
-// red half-sweep (from zero) z = r / (s n) on red cells.  Both colours.
-__device__ __noinline__ FF phase_b_v(const PcgArgs& A, const float* pnew, float alpha) {
+// red half-sweep (from zero) z = r / (s n) on red cells.  Both colours, four slots a lane.
+__device__ __noinline__ FF phase_b_q(const PcgArgs& A, const float* pnew, float alpha) {
   const MgArgs& M = A.mg;
   const SV v = sview(M.lv[0]);
   float* d0 = M.d0;
   const float* q0 = s_q0;
   const bool first_red = s_nblk[0] == 0;  // a blocked level 0 makes it from r itself
   const int lane = threadIdx.x & 31;
-  const float invs6 = s_inv_scnt[0][6];
   const int2 q = seg_slice(M.lv[0]);
-  const Items it = pair_items(q, 2);
-  struct S {
-    PCell e;
-    int c;
-    unsigned int code2;
-    float2 d, p, qq, r;
-  };
+  const Items it = quad_items(q, 2);
   FF acc;
-  run_batched<2>(
-      it.first, it.end, PCG_WARPS,
-      [&](unsigned int t, bool ok) {
-        S st;
-        st.c = (int)(t & 1u);
-        st.e = pcell(v, q, t >> 1, st.c, lane);
-        st.e.okA &= ok;
-        st.e.okB &= ok;
-        st.code2 = *reinterpret_cast<const unsigned int*>(v.code + st.e.idx);
-        st.d = *reinterpret_cast<const float2*>(d0 + st.e.idx);
-        st.p = *reinterpret_cast<const float2*>(pnew + st.e.idx);
-        st.qq = *reinterpret_cast<const float2*>(q0 + st.e.idx);
-        st.r = *reinterpret_cast<const float2*>(v.b + st.e.idx);
-        return st;
-      },
-      [&](S&) {},
-      [&](S& st) {
-        float dn[2], rn[2], zn[2];
-        // a warp whose cells are all fluid with six fluid neighbours: no selects
-        const bool full = pair_full(st.code2) && st.e.okA && st.e.okB;
-        if (__all_sync(0xffffffffu, full)) {
+  for (unsigned int t = it.first; t < it.end; t += PCG_WARPS) {
+    const int c = (int)(t & 1u);
+    const QCell e = qcell(v, q, t >> 1, c, lane);
+    if (!e.ok) continue;
+    const uint2 code4 = *reinterpret_cast<const uint2*>(v.code + e.idx);
+    const float4 d4 = *reinterpret_cast<const float4*>(d0 + e.idx);
+    const float4 p4 = *reinterpret_cast<const float4*>(pnew + e.idx);
+    const float4 q4 = *reinterpret_cast<const float4*>(q0 + e.idx);
+    const float4 r4 = *reinterpret_cast<const float4*>(v.b + e.idx);
+    const float dd[4] = {d4.x, d4.y, d4.z, d4.w}, pp[4] = {p4.x, p4.y, p4.z, p4.w};
+    const float qq[4] = {q4.x, q4.y, q4.z, q4.w}, rr[4] = {r4.x, r4.y, r4.z, r4.w};
+    float dn[4], rn[4], zn[4];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float dd = h == 0 ? st.d.x : st.d.y, pp = h == 0 ? st.p.x : st.p.y;
-            const float qq = h == 0 ? st.qq.x : st.qq.y, r0 = h == 0 ? st.r.x : st.r.y;
-            const float rc = __fmaf_rn(-alpha, qq, r0);
-            dn[h] = __fmaf_rn(alpha, pp, dd);
-            rn[h] = rc;
-            zn[h] = __fmul_rn(rc, invs6);
-            acc.add_prod(rc, rc);
-          }
-          *reinterpret_cast<float2*>(d0 + st.e.idx) = make_float2(dn[0], dn[1]);
-          *reinterpret_cast<float2*>(v.b + st.e.idx) = make_float2(rn[0], rn[1]);
-          if (first_red && st.c == 0)
-            *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(zn[0], zn[1]);
-          return;
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const unsigned int code = h == 0 ? (st.code2 & 0xffffu) : (st.code2 >> 16);
-          const bool ok = (h == 0 ? st.e.okA : st.e.okB) && (code & CODE_SELF);
-          const float dd = h == 0 ? st.d.x : st.d.y, pp = h == 0 ? st.p.x : st.p.y;
-          const float qq = h == 0 ? st.qq.x : st.qq.y, r0 = h == 0 ? st.r.x : st.r.y;
-          const float rc = __fmaf_rn(-alpha, qq, r0);
-          dn[h] = ok ? __fmaf_rn(alpha, pp, dd) : dd;
-          rn[h] = ok ? rc : r0;
-          zn[h] = ok ? gs_first(0, code_cnt(code), rc) : 0.0f;
-          if (ok) acc.add_prod(rc, rc);
-        }
-        if (st.e.okA || st.e.okB) {
-          *reinterpret_cast<float2*>(d0 + st.e.idx) = make_float2(dn[0], dn[1]);
-          *reinterpret_cast<float2*>(v.b + st.e.idx) = make_float2(rn[0], rn[1]);
-          if (first_red && st.c == 0)
-            *reinterpret_cast<float2*>(v.x + st.e.idx) = make_float2(zn[0], zn[1]);
-        }
-      });
+    for (int h = 0; h < 4; ++h) {
+      const int cnt = quad_cnt(code4, h);  // 0: not fluid
+      const float rc = __fmaf_rn(-alpha, qq[h], rr[h]);
+      dn[h] = cnt ? __fmaf_rn(alpha, pp[h], dd[h]) : dd[h];
+      rn[h] = cnt ? rc : rr[h];
+      zn[h] = cnt ? gs_first(0, cnt, rc) : 0.0f;
+      const float rs = cnt ? rc : 0.0f;
+      acc.add_prod(rs, rs);
+    }
+    *reinterpret_cast<float4*>(d0 + e.idx) = make_float4(dn[0], dn[1], dn[2], dn[3]);
+    *reinterpret_cast<float4*>(v.b + e.idx) = make_float4(rn[0], rn[1], rn[2], rn[3]);
+    if (first_red && c == 0)
+      *reinterpret_cast<float4*>(v.x + e.idx) = make_float4(zn[0], zn[1], zn[2], zn[3]);
+  }
   return acc;
 }
 
@@ -2029,11 +1969,11 @@ __device__ __noinline__ FF phase_b_s(const PcgArgs& A, const float* pnew, float 
 
 __device__ __forceinline__ FF phase_a(const PcgArgs& A, const float* pold, float* pnew,
                                       float beta) {
-  return use_pairs(A.mg.lv[0]) ? phase_a_v(A, pold, pnew, beta) : phase_a_s(A, pold, pnew, beta);
+  return use_wide(A.mg.lv[0]) ? phase_a_v(A, pold, pnew, beta) : phase_a_s(A, pold, pnew, beta);
 }
 
 __device__ __forceinline__ FF phase_b(const PcgArgs& A, const float* pnew, float alpha) {
-  return use_pairs(A.mg.lv[0]) ? phase_b_v(A, pnew, alpha) : phase_b_s(A, pnew, alpha);
+  return use_wide(A.mg.lv[0]) ? phase_b_q(A, pnew, alpha) : phase_b_s(A, pnew, alpha);
 }
 
 // One pass over this thread's fluid cells of level 0, both colours (start of the
@@ -2438,6 +2378,32 @@ __device__ __noinline__ void seg_slices(const PcgArgs& A, unsigned int* cache) {
   }
 }
 
+// x = 0 on the rows of every block-row within one of a block-row that holds fluid, so that
+// the sweeps read 0 from neighbours that are not fluid (what an earlier solve left there).
+// Level 0 only where it will be swept pass by pass: a blocked level masks what it loads.
+__device__ __noinline__ void zero_near(const PcgArgs& A) {
+  const MgArgs& M = A.mg;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool skip0 = A.precond != PRECOND_RBGS && blocked(M, *A.n_active);
+  for (int l = skip0 ? 1 : 0; l < M.lgrid; ++l) {
+    const MgLevel& L = M.lv[l];
+    const int rows = 64 * L.nby * L.nbz;
+    for (int r = (int)team_rank() * PCG_WARPS + warp; r < rows; r += (int)team_size() * PCG_WARPS) {
+      const int J = (r >> 6) % L.nby, K = (r >> 6) / L.nby;
+      const int j = 8 * J + (r & 7), k = 8 * K + ((r >> 3) & 7);
+      if (j >= L.ny || k >= L.nz) continue;
+      const int dj = J + lane % 3 - 1, dk = K + lane / 3 - 1;
+      const bool near = lane < 9 && dj >= 0 && dk >= 0 && dj < L.nby && dk < L.nbz &&
+                        L.segmask[dj + L.nby * dk] != 0u;
+      if (!__any_sync(0xffffffffu, near)) continue;
+      float* x = L.x + L.margin + L.hx * (j + L.ny * k);
+      for (int c = 0; c < 2; ++c)
+        for (int s = 2 * lane; s < L.hx; s += 64)
+          *reinterpret_cast<float2*>(x + c * L.half + s) = make_float2(0.0f, 0.0f);
+    }
+  }
+}
+
 // Builds, once per solve: the fluid flags of levels 1.. with their block flags, the
 // active-segment slices and the block lists of the colour-split levels, the codes of every
 // level.  Ends with a grid barrier.  All latency: three barriers instead of one per level
@@ -2476,6 +2442,7 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh, unsigned
     seg_cache_fill(M, cache);
   }
   SOLVE_TRACE(TR_SEG_WRITE);
+  zero_near(A);
   // codes: split levels over their active segments, CTA-local levels over all cells
   for (int l = 0; l < M.lgrid; ++l) {
     const MgLevel& L = M.lv[l];

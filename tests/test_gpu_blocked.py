@@ -41,6 +41,8 @@ def test_blocked_smoothing_matches_the_oracle(n, fill, nu):
     ((5, 6, 7), 0.7),         # two levels, both in one CTA but the first
     ((3, 4, 2), 0.6),         # one level
     ((130, 40, 24), 0.9),     # three segments a row, the last with two cells
+    ((67, 121, 96), 0.9),     # four slots a lane with rows that end at three of four
+    ((133, 90, 60), 0.6),     # ... and at one, a third segment of five cells
 ])
 def test_level_set_up_matches_the_oracle(n, fill):
     """Level flags, segment slices and codes: a wrong one changes the V-cycle at O(1)."""
