@@ -135,10 +135,9 @@ struct flip_handle {
 
 void flip_set_last_error_(const std::string& msg) { g_last_error = msg; }
 
-// P2G's default grid: 8 CTAs per SM, twice the co-resident 4, so that CTAs
+// P2G's default grid: 8 CTAs per SM, more than twice the co-resident 3, so that CTAs
 // taking heavy bricks are balanced by the scheduler (the kernel loops over the
-// active bricks; measured 8 % faster than one wave on a 128^3 dam break, equal on
-// the 256^3 pool).  G2P's: its co-resident count.
+// active bricks, or over their slabs where they are few).  G2P's: its co-resident count.
 constexpr int kP2gPerSm = 8;
 
 void set_transfer_grids(flip_handle* h) {
@@ -376,9 +375,9 @@ void carve(flip_handle* h, Carver& cv) {
   h->B.active = cv.take<unsigned int>(nb);
   h->type = cv.take<uint8_t>(nc);
   h->hmark = cv.take<uint8_t>(nb);
-  h->hrow = cv.take<unsigned int>((nb + 31) / 32);  // brick-rows <= bricks
+  h->hrow = cv.take<unsigned int>((nb + 31) / 32 + 1);  // brick-rows <= bricks; hlist_n
   h->hlist = cv.take<unsigned int>(nb);
-  h->hlist_n = cv.take<unsigned int>(1);
+  h->hlist_n = h->hrow + ((size_t)h->g.by * h->g.bz + 31) / 32;
   for (int d = 0; d < 3; ++d) {
     h->acc[d] = cv.take<float2>((size_t)h->nf[d]);
     h->uo[d] = cv.take<float>((size_t)h->nf[d]);
@@ -766,7 +765,7 @@ int flip_step(flip_handle* h, int32_t nsteps, flip_stats* stats) {
     if (timed) FLIP_CUDA(cudaEventRecord(ev[1], s));
     launch_p2g(h->g, h->P[h->cur], h->B, h->acc, h->dstats, h->p2g_blocks, s);
     FLIP_CUDA(launch_finalize_near(h->g, h->B.brick_count, h->hmark, h->hrow, h->hlist,
-                                   h->hlist_n, h->acc, h->uo, h->bar, h->dstats, h->sm_count,
+                                   h->acc, h->uo, h->bar, h->dstats, h->sm_count,
                                    h->near_stale, s));
     h->launches += 3;
     if (timed) FLIP_CUDA(cudaEventRecord(ev[2], s));
@@ -1823,7 +1822,7 @@ int batch_step_impl(flip_batch* b, flip_handle* const* hs, int32_t n, int32_t ns
       launch_front(h, h->stream);
       launch_p2g(h->g, h->P[h->cur], h->B, h->acc, h->dstats, h->p2g_blocks, h->stream);
       FLIP_CUDA(launch_finalize_near(h->g, h->B.brick_count, h->hmark, h->hrow, h->hlist,
-                                     h->hlist_n, h->acc, h->uo, h->bar, h->dstats, h->sm_count,
+                                     h->acc, h->uo, h->bar, h->dstats, h->sm_count,
                                      h->near_stale, h->stream));
       launch_divergence_near(h->g, h->K, h->type, uo, h->b32, h->b64, h->x32, h->x64, h->pff,
                              h->bar, h->dstats, h->hlist, h->hlist_n, h->sm_count,

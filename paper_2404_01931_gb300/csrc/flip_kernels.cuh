@@ -286,11 +286,11 @@ void launch_divergence(const Grid& g, const StepConsts& k, const uint8_t* type,
 // this step's or last step's (full: the whole-grid kernels, after which the marks
 // are current again), walked as whole x-rows of the brick-rows holding such a
 // brick.  launch_finalize_near marks the bricks (hmark: [nbricks], kept across
-// steps), lists the brick-rows (rowflag: [ceil(by bz / 32)] words; list: [by bz];
-// list_n: one word), resets the step words and finalizes: two kernels;
+// steps), lists the brick-rows (rowflag: [ceil(by bz / 32)] words and after
+// them their count, list_n of the second; list: [by bz]), resets the step words and finalizes: two kernels;
 // launch_divergence_near: one.
 cudaError_t launch_finalize_near(const Grid& g, const unsigned int* brick_count, uint8_t* hmark,
-                                 unsigned int* rowflag, unsigned int* list, unsigned int* list_n,
+                                 unsigned int* rowflag, unsigned int* list,
                                  float2* const acc[3], float* const uo[3], unsigned int* bar,
                                  DevStats* st, int sm_count, bool full, cudaStream_t s);
 void launch_divergence_near(const Grid& g, const StepConsts& k, const uint8_t* type,

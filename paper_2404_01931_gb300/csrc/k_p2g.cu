@@ -5,173 +5,275 @@
 //     u_node = sum_P u_P k(x_P - x_node) / sum_P k(x_P - x_node)     (0 if no P)
 // The paper gathers per grid point; here the sum is split by particle bricks.
 // One CTA takes one active 8x8x8 brick (its particles are one contiguous range
-// after binning).  A thread owns a cell: it sums the weighted velocities and
-// weights of that cell's particles into registers over the 2x3x3 face nodes
-// they can reach, then adds them to a shared-memory tile of the brick plus its
-// halo (9x10x10 nodes per component), and the CTA adds the tile to the global
-// (num, den) accumulators with vector float2 atomics.  The normalisation
-// num/den happens in k_finalize_rows (over the rows near the liquid; k_finalize
-// sweeps the whole grid), which also clears the accumulators.
-// A warp takes 8 x-cells by 4 z-planes of one y-row, and the tile's planes are
-// TILE_PLANE = 104 nodes apart (8 mod 32 banks): the 32 lanes of every atomic
-// then fall on 32 different banks.
+// after binning), or a slab of its z-planes where the bricks are few.  A warp
+// takes 8 x-cells by 4 y-rows and walks up the planes, a lane per cell: it reads
+// each of the cell's particles once and sums the weighted velocities and weights
+// of all three components in registers, over the face nodes the particle can
+// reach (2x3x3 per component).  The z-window of sums moves with the walk, so that
+// only the plane of nodes left behind is added to the warp's tile in shared
+// memory.  A warp's tile is its own and the lanes take turns over the nodes they
+// share, so these sums need no atomics.  At the end the CTA adds its four tiles and
+// the result to the global (num, den) accumulators with vector float2 atomics.
+// The normalisation num/den happens in k_finalize_rows (over the rows near the
+// liquid; k_finalize sweeps the whole grid), which also clears the accumulators.
 #include <algorithm>
 
 #include "flip_kernels.cuh"
 
 namespace flipk {
 
-constexpr int P2G_THREADS = 256;
-
+// A brick's face nodes that its particles can reach.
 template <int D>
 struct Tile {
   static constexpr int X = (D == 0) ? 9 : 10;
   static constexpr int Y = (D == 1) ? 9 : 10;
-  static constexpr int Z = (D == 2) ? 9 : 10;
-  static constexpr int N = X * Y * Z;
 };
-constexpr int TILE_PLANE = 104;              // >= X * Y of every component; 8 mod 32
-constexpr int TILE_PAD = 10 * TILE_PLANE;     // up to 10 planes
-static_assert(TILE_PLANE % 32 == 8, "lanes 8 apart in z must take the next 8 banks");
-static_assert(Tile<0>::X * Tile<0>::Y <= TILE_PLANE && Tile<1>::X * Tile<1>::Y <= TILE_PLANE &&
-                  Tile<2>::X * Tile<2>::Y <= TILE_PLANE, "a plane of the tile fits");
 
-// Weights of one axis over the node window of a cell: the component's own axis
-// has 2 nodes (c, c+1); the other axes 3 nodes (c-1, c, c+1).
-template <int NN>
-__device__ __forceinline__ void expand(const AxisW& a, float (&w)[NN]) {
-  if constexpr (NN == 2) {
-    w[0] = a.w0;
-    w[1] = a.w1;
-  } else {
-    const bool lo = (a.off == 0);
-    w[0] = lo ? a.w0 : 0.0f;
-    w[1] = lo ? a.w1 : a.w0;
-    w[2] = lo ? 0.0f : a.w1;
-  }
+constexpr int P2G_THREADS = 128;  // 2 halves in y by 2 in z
+constexpr int P2G_MAX_SPLIT = 4;
+
+// A warp's tile: x-rows of 10 nodes, 6 planes, 6 y-rows TILE_ROW apart (8 mod 16
+// float2: the 8-byte accesses of 8 lanes along x and 4 along y take each bank twice,
+// which is what 32 lanes cost).
+constexpr int TILE_ROW = 72;
+constexpr int TILE_N = 6 * TILE_ROW;
+static_assert(TILE_ROW >= 60 && TILE_ROW % 16 == 8, "tile pitch");
+
+struct P2gShared {
+  __align__(16) float2 tile[4][3][TILE_N];  // [warp][component]: (num, den)
+};
+
+// Nodes per axis that a cell's particles can reach: two on the component's own axis
+// (the cell's faces), three on the others (the cell's centre and both neighbours').
+template <int D>
+struct Win {
+  static constexpr int X = (D == 0) ? 2 : 3, Y = (D == 1) ? 2 : 3, Z = (D == 2) ? 2 : 3;
+};
+
+// One axis of the transfer weights of a particle of cell c (axis_weights' values over the
+// cell's window): f[2] on the faces, and h[3] on the centres, with t the distance from the
+// own centre in cells, |t| <= 1/2 and clamped at the domain's ends.  x/dx - c in one rounding.
+struct AxisP {
+  float f[2], h[3];
+};
+
+__device__ __forceinline__ AxisP axis_p(float x, float inv, float c, float lo, float hi) {
+  const float g = __fmaf_rn(x, inv, -c);
+  AxisP a;
+  a.f[1] = fminf(fmaxf(g, 0.0f), 1.0f);
+  a.f[0] = 1.0f - a.f[1];
+  const float t = fminf(fmaxf(g - 0.5f, lo), hi);
+  a.h[0] = fmaxf(-t, 0.0f);
+  a.h[1] = 1.0f - fabsf(t);
+  a.h[2] = fmaxf(t, 0.0f);
+  return a;
 }
 
 template <int D>
-__device__ __forceinline__ void p2g_cell(const Grid& g, const PartView& P, unsigned int beg,
-                                         unsigned int end, int ci, int cj, int ck, int li,
-                                         int lj, int lk, float* tnum, float* tden) {
-  constexpr int NX = (D == 0) ? 2 : 3, NY = (D == 1) ? 2 : 3, NZ = (D == 2) ? 2 : 3;
-  constexpr int TX = Tile<D>::X;
-  // (num, den) of a node accumulate together: one packed two-lane FMA per node,
-  // each lane rounded like __fmaf_rn
-  float2 acc[NZ][NY][NX];
+struct Acc {
+  float2 a[Win<D>::Z][Win<D>::Y][Win<D>::X];  // (num, den)
+};
+
+// (num, den) of a node accumulate together: one packed two-lane FMA per node.
+template <int D>
+__device__ __forceinline__ void p2g_add(Acc<D>& A, const AxisP& ax, const AxisP& ay,
+                                        const AxisP& az, float v) {
+  constexpr int NX = Win<D>::X, NY = Win<D>::Y, NZ = Win<D>::Z;
+  const float* wx = (D == 0) ? ax.f : ax.h;
+  const float* wy = (D == 1) ? ay.f : ay.h;
+  const float* wz = (D == 2) ? az.f : az.h;
 #pragma unroll
-  for (int z = 0; z < NZ; ++z)
+  for (int y = 0; y < NY; ++y) {
+    const float2 vy = make_float2(__fmul_rn(wy[y], v), wy[y]);
 #pragma unroll
-    for (int y = 0; y < NY; ++y)
-#pragma unroll
-      for (int x = 0; x < NX; ++x) acc[z][y][x] = make_float2(0.0f, 0.0f);
-  const float* vel = (D == 0) ? P.u : (D == 1) ? P.v : P.w;
-  for (unsigned int q = beg; q < end; ++q) {
-    const float px = P.x[q], py = P.y[q], pz = P.z[q], pv = vel[q];
-    float wx[NX], wy[NY], wz[NZ];
-    expand<NX>(axis_weights<D, 0>(px, g.inv_dx, ci, g.nx), wx);
-    expand<NY>(axis_weights<D, 1>(py, g.inv_dx, cj, g.ny), wy);
-    expand<NZ>(axis_weights<D, 2>(pz, g.inv_dx, ck, g.nz), wz);
-#pragma unroll
-    for (int z = 0; z < NZ; ++z)
-#pragma unroll
-      for (int y = 0; y < NY; ++y) {
-        const float wyz = __fmul_rn(wy[y], wz[z]);
-        const float2 tw = make_float2(__fmul_rn(wyz, pv), wyz);
-#pragma unroll
-        for (int x = 0; x < NX; ++x)
-          acc[z][y][x] = __ffma2_rn(make_float2(wx[x], wx[x]), tw, acc[z][y][x]);
-      }
-  }
-#pragma unroll
-  for (int z = 0; z < NZ; ++z)
-#pragma unroll
-    for (int y = 0; y < NY; ++y)
+    for (int z = 0; z < NZ; ++z) {
+      const float2 tw = __fmul2_rn(vy, make_float2(wz[z], wz[z]));
 #pragma unroll
       for (int x = 0; x < NX; ++x)
-        if (acc[z][y][x].y != 0.0f) {
-          const int t = (li + x) + TX * (lj + y) + TILE_PLANE * (lk + z);
-          atomicAdd(tnum + t, acc[z][y][x].x);
-          atomicAdd(tden + t, acc[z][y][x].y);
-        }
-}
-
-template <int D>
-__device__ __forceinline__ void flush_tile(const Grid& g, int b0, int b1, int b2,
-                                           const float* tnum, const float* tden, float2* acc) {
-  constexpr int TX = Tile<D>::X, TY = Tile<D>::Y, N = Tile<D>::N;
-  const int o0 = (D == 0) ? b0 : b0 - 1, o1 = (D == 1) ? b1 : b1 - 1, o2 = (D == 2) ? b2 : b2 - 1;
-  const int FX = g.nx + (D == 0), FY = g.ny + (D == 1), FZ = g.nz + (D == 2);
-  for (int t = threadIdx.x; t < N; t += P2G_THREADS) {
-    const int ta = t % TX, tb = (t / TX) % TY, tc = t / (TX * TY);
-    const int ts = ta + TX * tb + TILE_PLANE * tc;
-    const float dn = tden[ts];
-    if (dn == 0.0f) continue;
-    const int a = o0 + ta, b = o1 + tb, c = o2 + tc;
-    if (a < 0 || b < 0 || c < 0 || a >= FX || b >= FY || c >= FZ) continue;
-    atomicAdd(acc + (a + FX * (b + FY * c)), make_float2(tnum[ts], dn));
+        A.a[z][y][x] = __ffma2_rn(make_float2(wx[x], wx[x]), tw, A.a[z][y][x]);
+    }
   }
 }
 
-// One brick: zero the tiles, splat its cells' particles, add the tiles to the
-// global accumulators.  CTA-uniform; ends with a __syncthreads.
+// Adds node (x, y) of the window's lowest plane to the warp's tile.
+template <int D>
+__device__ __forceinline__ void p2g_put(const Acc<D>& A, int x, int y, float2* tile) {
+  if (x < Win<D>::X && y < Win<D>::Y) {
+    float2* n = tile + D * TILE_N + x + TILE_ROW * y;
+    *n = __fadd2_rn(*n, A.a[0][y < Win<D>::Y ? y : 0][x < Win<D>::X ? x : 0]);
+  }
+}
+
+// Moves the window up by a plane.
+template <int D>
+__device__ __forceinline__ void p2g_shift(Acc<D>& A) {
+#pragma unroll
+  for (int z = 0; z < Win<D>::Z; ++z)
+#pragma unroll
+    for (int y = 0; y < Win<D>::Y; ++y)
+#pragma unroll
+      for (int x = 0; x < Win<D>::X; ++x)
+        A.a[z][y][x] = (z + 1 < Win<D>::Z) ? A.a[z + 1 < Win<D>::Z ? z + 1 : 0][y][x]
+                                           : make_float2(0.0f, 0.0f);
+}
+
+// Adds the CTA's four tiles (rows planes per warp from plane z0 of the brick) and the
+// result to component D's accumulators.
+template <int D>
+__device__ __forceinline__ void flush_tiles(const Grid& g, int b0, int b1, int b2, int rows,
+                                            const P2gShared& sh, float2* acc) {
+  constexpr int TX = Tile<D>::X, TY = Tile<D>::Y;
+  constexpr int WY = 4 + Win<D>::Y - 1;  // rows of a warp's tile
+  const int wz = rows + Win<D>::Z - 1;   // ... and planes
+  const int n = TX * TY * (2 * rows + Win<D>::Z - 1);
+  const int o0 = (D == 0) ? b0 : b0 - 1, o1 = (D == 1) ? b1 : b1 - 1, o2 = (D == 2) ? b2 : b2 - 1;
+  const int FX = g.nx + (D == 0), FY = g.ny + (D == 1), FZ = g.nz + (D == 2);
+  for (int t = threadIdx.x; t < n; t += P2G_THREADS) {
+    const int ta = t % TX, tb = (t / TX) % TY, tc = t / (TX * TY);
+    float2 v = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int y = tb - 4 * (w & 1), z = tc - rows * (w >> 1);
+      if (y >= 0 && y < WY && z >= 0 && z < wz)
+        v = __fadd2_rn(v, sh.tile[w][D][ta + 10 * z + TILE_ROW * y]);
+    }
+    if (v.y == 0.0f) continue;
+    const int a = o0 + ta, b = o1 + tb, c = o2 + tc;
+    if (a < 0 || b < 0 || c < 0 || a >= FX || b >= FY || c >= FZ) continue;
+    atomicAdd(acc + (a + FX * (b + FY * c)), v);
+  }
+}
+
+// Slab `part` of the `split` (1, 2, 4) of one brick.  CTA-uniform; ends with a
+// __syncthreads.
 __device__ __forceinline__ void p2g_brick(const Grid& g, const PartView& P, const BinView& B,
                                           float2* acc0, float2* acc1, float2* acc2,
-                                          unsigned int brick, float (*tnum)[TILE_PAD],
-                                          float (*tden)[TILE_PAD]) {
+                                          unsigned int brick, int part, int split,
+                                          P2gShared& sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b0 = (int)(brick % (unsigned)g.bx) * BRICK;
   const int b1 = (int)((brick / (unsigned)g.bx) % (unsigned)g.by) * BRICK;
   const int b2 = (int)(brick / ((unsigned)g.bx * (unsigned)g.by)) * BRICK;
-  for (int t = threadIdx.x; t < 3 * TILE_PAD; t += P2G_THREADS) {
-    (&tnum[0][0])[t] = 0.0f;
-    (&tden[0][0])[t] = 0.0f;
-  }
-  __syncthreads();
+  const int rows = 4 / split, zc = part * 2 * rows;  // planes per warp; the slab's first
+  const int li = lane & 7, lj = (lane >> 3) + 4 * (warp & 1), lk0 = zc + rows * (warp >> 1);
   const unsigned int bstart = B.brick_start[brick], bend = B.brick_start[brick + 1];
-  static_assert(BRICK_CELLS == 2 * P2G_THREADS, "two passes of 8 x 8 x 4 cells");
-  for (int pass = 0; pass < 2; ++pass) {
-    const int li = threadIdx.x & 7, lk = ((threadIdx.x >> 3) & 3) + 4 * pass,
-              lj = threadIdx.x >> 5;
-    const int l = li + BRICK * (lj + BRICK * lk);
-    const unsigned int key = brick * BRICK_CELLS + (unsigned)l;
-    const unsigned int beg = bstart + B.local_start[key];
-    const unsigned int end = (l < BRICK_CELLS - 1) ? bstart + B.local_start[key + 1] : bend;
-    if (beg == end) continue;
-    const int ci = b0 + li, cj = b1 + lj, ck = b2 + lk;
-    p2g_cell<0>(g, P, beg, end, ci, cj, ck, li, lj, lk, tnum[0], tden[0]);
-    p2g_cell<1>(g, P, beg, end, ci, cj, ck, li, lj, lk, tnum[1], tden[1]);
-    p2g_cell<2>(g, P, beg, end, ci, cj, ck, li, lj, lk, tnum[2], tden[2]);
+  const unsigned int* ls = B.local_start + brick * BRICK_CELLS;
+  int l = li + BRICK * (lj + BRICK * lk0);
+  unsigned int beg = bstart + ls[l];
+  unsigned int end = (l < BRICK_CELLS - 1) ? bstart + ls[l + 1] : bend;
+  {
+    float4* t4 = reinterpret_cast<float4*>(&sh.tile[warp][0][0]);
+    for (int t = lane; t < 3 * TILE_N / 2; t += 32) t4[t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  }
+  __syncwarp();
+  const int ci = b0 + li, cj = b1 + lj;
+  const float cx = (float)ci, cy = (float)cj;
+  const float xlo = (ci == 0) ? 0.0f : -0.5f, xhi = (ci == g.nx - 1) ? 0.0f : 0.5f;
+  const float ylo = (cj == 0) ? 0.0f : -0.5f, yhi = (cj == g.ny - 1) ? 0.0f : 0.5f;
+  float2* tile = &sh.tile[warp][0][0] + li + TILE_ROW * (lane >> 3);
+  Acc<0> A0{};
+  Acc<1> A1{};
+  Acc<2> A2{};
+  int pending = 0;  // planes of the window that may hold sums
+  for (int r = 0; r < rows + 2; ++r, tile += 10) {
+    if (r < rows) {
+      unsigned int q = beg;
+      const unsigned int qe = end;
+      const int ck = b2 + lk0 + r;
+      const float cz = (float)ck;
+      const float zlo = (ck == 0) ? 0.0f : -0.5f, zhi = (ck == g.nz - 1) ? 0.0f : 0.5f;
+      float x = 0.0f, y = 0.0f, z = 0.0f, u = 0.0f, v = 0.0f, w = 0.0f;
+      if (q < qe) {
+        x = P.x[q], y = P.y[q], z = P.z[q];
+        u = P.u[q], v = P.v[q], w = P.w[q];
+      }
+      l += BRICK * BRICK;
+      if (r + 1 < rows) {
+        beg = bstart + ls[l];
+        end = (l < BRICK_CELLS - 1) ? bstart + ls[l + 1] : bend;
+      }
+      if (__any_sync(0xffffffffu, q < qe)) pending = 3;
+      while (q < qe) {
+        const AxisP ax = axis_p(x, g.inv_dx, cx, xlo, xhi);
+        const AxisP ay = axis_p(y, g.inv_dx, cy, ylo, yhi);
+        const AxisP az = axis_p(z, g.inv_dx, cz, zlo, zhi);
+        const float pu = u, pv = v, pw = w;
+        // the next particle's loads are in flight during this one's sums
+        if (++q < qe) {
+          x = P.x[q], y = P.y[q], z = P.z[q];
+          u = P.u[q], v = P.v[q], w = P.w[q];
+        }
+        p2g_add<0>(A0, ax, ay, az, pu);
+        p2g_add<1>(A1, ax, ay, az, pv);
+        p2g_add<2>(A2, ax, ay, az, pw);
+      }
+      __syncwarp();
+    }
+    if (pending > 0) {
+      --pending;
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          p2g_put<0>(A0, dx, dy, tile);
+          p2g_put<1>(A1, dx, dy, tile);
+          p2g_put<2>(A2, dx, dy, tile);
+          __syncwarp();  // the next node is another lane's
+        }
+      p2g_shift(A0);
+      p2g_shift(A1);
+      p2g_shift(A2);
+    }
   }
   __syncthreads();
-  flush_tile<0>(g, b0, b1, b2, tnum[0], tden[0], acc0);
-  flush_tile<1>(g, b0, b1, b2, tnum[1], tden[1], acc1);
-  flush_tile<2>(g, b0, b1, b2, tnum[2], tden[2], acc2);
+  flush_tiles<0>(g, b0, b1, b2 + zc, rows, sh, acc0);
+  flush_tiles<1>(g, b0, b1, b2 + zc, rows, sh, acc1);
+  flush_tiles<2>(g, b0, b1, b2 + zc, rows, sh, acc2);
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(P2G_THREADS, 4) k_p2g(const Grid g, const PartView P,
+// Slabs per brick: the walk through a brick is a serial chain, so few bricks are shared out
+// over the launch's CTAs as far as two rounds of them go.  The P2G stage at 16 bricks (32^3
+// dam break) 35 -> 24 us, at 150 (64^3) 43 -> 35, at 450 (ragged 96 x 64 x 100) 56 -> 55; with
+// one round as the line the last takes 59, its slabs' tiles costing more than they gain.
+__device__ __forceinline__ int p2g_split(unsigned int nact, unsigned int ctas) {
+  int split = 1;
+  while (split < P2G_MAX_SPLIT && nact * 2u * (unsigned)split <= ctas) split *= 2;
+  return split;
+}
+
+// Bound by the FMA pipe and the latency of its chains, at 12 warps per SM (the sums of three
+// components take 108 of 168 registers): 5.2 M particles in 92 us with 330 instructions per
+// 32 particles.  A component at a time (64 registers, 32 warps, each particle read three
+// times) and all 54 nodes added to a common tile by shared-memory atomics, which are
+// compare-and-swap loops for floats: 130 us and 572 instructions.  The stage at 256^3
+// (42.3 M) 0.998 -> 0.736 ms.  A thread per column of nodes in flush_tiles (fewer
+// instructions, but a serial chain) took 0.807, loading the next cell's first particle
+// ahead 0.792.
+__global__ void __launch_bounds__(P2G_THREADS, 3) k_p2g(const Grid g, const PartView P,
                                                      const BinView B, float2* acc0, float2* acc1,
                                                      float2* acc2, const DevStats* st) {
-  __shared__ float tnum[3][TILE_PAD];
-  __shared__ float tden[3][TILE_PAD];
+  __shared__ P2gShared sh;
   const unsigned int nact = st->n_active;
-  for (unsigned int bi = blockIdx.x; bi < nact; bi += gridDim.x)
-    p2g_brick(g, P, B, acc0, acc1, acc2, B.active[bi], tnum, tden);
+  const int split = p2g_split(nact, gridDim.x);
+  for (unsigned int bi = blockIdx.x; bi < nact * (unsigned)split; bi += gridDim.x)
+    p2g_brick(g, P, B, acc0, acc1, acc2, B.active[bi / (unsigned)split],
+              (int)(bi % (unsigned)split), split, sh);
 }
 
 // All scenes' active bricks as one list: L.first holds the running sum of the
 // scenes' active-brick counts (k_active_prefix), so the CTAs share the bricks of
 // every scene evenly whatever their sizes.
-__global__ void __launch_bounds__(P2G_THREADS, 4) k_p2g_batch(const BatchLaunch L) {
-  __shared__ float tnum[3][TILE_PAD];
-  __shared__ float tden[3][TILE_PAD];
+__global__ void __launch_bounds__(P2G_THREADS, 3) k_p2g_batch(const BatchLaunch L) {
+  __shared__ P2gShared sh;
   const unsigned int g0 = L.first[0], g1 = L.first[L.n];
-  for (unsigned int gb = g0 + blockIdx.x; gb < g1; gb += gridDim.x) {
+  const int split = p2g_split(g1 - g0, gridDim.x);
+  for (unsigned int q = blockIdx.x; q < (g1 - g0) * (unsigned)split; q += gridDim.x) {
+    const unsigned int gb = g0 + q / (unsigned)split;
     const int s = batch_scene(L, gb);
     const SceneDev& S = L.scenes[s];
-    p2g_brick(S.g, S.dst, S.B, S.acc[0], S.acc[1], S.acc[2], S.B.active[gb - L.first[s]], tnum,
-              tden);
+    p2g_brick(S.g, S.dst, S.B, S.acc[0], S.acc[1], S.acc[2], S.B.active[gb - L.first[s]],
+              (int)(q % (unsigned)split), split, sh);
   }
 }
 
@@ -346,14 +448,15 @@ __global__ void k_halo_bricks(const Grid g, const unsigned int* __restrict__ bri
   const int nb = g.bx * g.by * g.bz;
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
     const int I = b % g.bx, J = (b / g.bx) % g.by, K = b / (g.bx * g.by);
-    bool near = false;
-    for (int dk = -1; dk <= 1 && !near; ++dk)
-      for (int dj = -1; dj <= 1 && !near; ++dj)
-        for (int di = -1; di <= 1 && !near; ++di) {
-          const int i = I + di, j = J + dj, k = K + dk;
-          if (i < 0 || j < 0 || k < 0 || i >= g.bx || j >= g.by || k >= g.bz) continue;
-          near = brick_count[i + g.bx * (j + g.by * k)] > 0u;
-        }
+    // all 27 loads in flight at once: the kernel is one round of latency
+    unsigned int near = 0;
+#pragma unroll
+    for (int d = 0; d < 27; ++d) {
+      const int i = min(max(I + d % 3 - 1, 0), g.bx - 1);
+      const int j = min(max(J + d / 3 % 3 - 1, 0), g.by - 1);
+      const int k = min(max(K + d / 9 - 1, 0), g.bz - 1);
+      near |= __ldg(brick_count + (i + g.bx * (j + g.by * k)));
+    }
     const unsigned int m = ((near ? 1u : 0u) << 1) | ((unsigned)hmark[b] >> 1);
     hmark[b] = (uint8_t)m;
     if (m != 0u) {
@@ -520,15 +623,15 @@ void launch_divergence(const Grid& g, const StepConsts& k, const uint8_t* type,
 }
 
 cudaError_t launch_finalize_near(const Grid& g, const unsigned int* brick_count, uint8_t* hmark,
-                                 unsigned int* rowflag, unsigned int* list, unsigned int* list_n,
-                                 float2* const acc[3], float* const uo[3], unsigned int* bar,
-                                 DevStats* st, int sm_count, bool full, cudaStream_t s) {
+                                 unsigned int* rowflag, unsigned int* list, float2* const acc[3],
+                                 float* const uo[3], unsigned int* bar, DevStats* st, int sm_count, bool full, cudaStream_t s) {
   const long long nb = (long long)g.bx * g.by * g.bz;
   const size_t rows = (size_t)g.by * g.bz;
-  cudaError_t e = cudaMemsetAsync(rowflag, 0, sizeof(unsigned int) * ((rows + 31) / 32), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(list_n, 0, sizeof(unsigned int), s);
+  unsigned int* list_n = rowflag + (rows + 31) / 32;
+  const cudaError_t e =
+      cudaMemsetAsync(rowflag, 0, sizeof(unsigned int) * ((rows + 31) / 32 + 1), s);
   if (e != cudaSuccess) return e;
-  k_halo_bricks<<<(unsigned)std::min<long long>((nb + 255) / 256, 4LL * sm_count), 256, 0, s>>>(
+  k_halo_bricks<<<(unsigned)std::min<long long>((nb + 127) / 128, 4LL * sm_count), 128, 0, s>>>(
       g, brick_count, hmark, rowflag, list, list_n, bar, st);
   if (full) {
     launch_finalize(g, acc, uo, s);
