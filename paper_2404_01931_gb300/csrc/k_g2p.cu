@@ -7,12 +7,14 @@
 // see below).  It first stages in shared memory the
 // pressure of the brick plus a one-cell halo, then, for every component, the
 // face nodes any of the brick's particles can reach (the 9x10x10 tile P2G also
-// uses): u_new (Eq. 5 with gravity and walls, face_unew's arithmetic) and
-// u_new - u_old.  Each face value is so computed once per brick instead of once
-// per particle that touches it.  Then one thread per particle interpolates
-//     U = interp(u_new),  dU = interp(u_new - u_old)
-//     v <- r (v + dU) + (1 - r) U
-//     x <- clamp(x + dt v, skin, n dx - skin)     (or dt U with grid advection)
+// uses).  With u_new from Eq. 5 (gravity and walls, face_unew's arithmetic), the
+// blend v <- r (v + interp(u_new - u_old)) + (1 - r) interp(u_new) is
+//     v <- r v + interp(u_new - r u_old)
+// so that one value per node is interpolated, staged in one rounding.  Each face
+// value is so computed once per brick instead of once per particle that touches it.
+// Then one thread per particle interpolates and moves:
+//     x <- clamp(x + dt v, skin, n dx - skin)
+// or, with grid advection, x + dt interp(u_new), for which the tile holds u_new too.
 // and computes the key of the cell it moved to and its rank there.  Ranks come
 // from one histogram atomic per distinct key in a warp (lanes with the same key
 // take consecutive ranks), which is all the next step's counting sort needs.
@@ -32,6 +34,7 @@
 namespace flipk {
 
 constexpr int G2P_THREADS = 256;
+constexpr unsigned int G2P_MAX_SPLIT = 8;
 constexpr int G2P_TILE = 904;     // >= 9 * 10 * 10 face nodes per component
 
 template <int D>
@@ -85,6 +88,10 @@ __device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
                "r"(bytes)
                : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned int parity) {
@@ -148,14 +155,28 @@ __device__ __forceinline__ float pdiff(float2 hp, float2 hm) {
 }
 __device__ __forceinline__ float pdiff(float hp, float hm) { return __fsub_rn(hp, hm); }
 
+// A node of the staged tiles: u_new - r u_old, and with grid advection u_new.
+template <bool ADV>
+struct NodeOf;
+template <>
+struct NodeOf<false> {
+  using T = float;
+};
+template <>
+struct NodeOf<true> {
+  using T = float2;
+};
+template <bool ADV>
+using NodeV = typename NodeOf<ADV>::T;
+
 // Stages component D's face tile: node (a, b, c) with a in [o0, o0 + X) etc.,
 // o = brick origin on the own axis and origin - 1 on the others.  Nodes outside
 // the face grid are never interpolated (the clamped weights keep every node in
 // range) and are set to 0.
-template <int D, bool PAIR>
+template <int D, bool PAIR, bool ADV>
 __device__ __forceinline__ void stage_faces(const Grid& g, const StepConsts& K, int b0, int b1,
                                             int b2, const float* __restrict__ uo,
-                                            const typename PTile<PAIR>::T* sp, float2* sud) {
+                                            const typename PTile<PAIR>::T* sp, NodeV<ADV>* sud) {
   constexpr int TX = FaceTile<D>::X, TY = FaceTile<D>::Y, N = FaceTile<D>::N;
   const int o0 = (D == 0) ? b0 : b0 - 1, o1 = (D == 1) ? b1 : b1 - 1, o2 = (D == 2) ? b2 : b2 - 1;
   const int FX = g.nx + (D == 0), FY = g.ny + (D == 1), FZ = g.nz + (D == 2);
@@ -163,7 +184,7 @@ __device__ __forceinline__ void stage_faces(const Grid& g, const StepConsts& K, 
   for (int t = threadIdx.x; t < N; t += G2P_THREADS) {
     const int ta = t % TX, tb = (t / TX) % TY, tc = t / (TX * TY);
     const int a = o0 + ta, b = o1 + tb, c = o2 + tc;
-    float un = 0.0f, du = 0.0f;
+    float un = 0.0f, fl = 0.0f;
     if (a >= 0 && b >= 0 && c >= 0 && a < FX && b < FY && c < FZ) {
       const float uov = __ldg(uo + (a + FX * (b + FY * c)));
       const int nd = (D == 0) ? a : (D == 1) ? b : c;
@@ -176,83 +197,138 @@ __device__ __forceinline__ void stage_faces(const Grid& g, const StepConsts& K, 
         const float dp = pdiff(sp[pc], sp[pm]);
         un = __fsub_rn(__fadd_rn(uov, K.gdt[D]), __fmul_rn(K.pscale, dp));
       }
-      du = __fsub_rn(un, uov);
+      fl = __fmaf_rn(-K.flip_ratio, uov, un);
     }
-    sud[t] = make_float2(un, du);
+    if constexpr (ADV) sud[t] = make_float2(fl, un);
+    else sud[t] = fl;
   }
 }
 
-// Interpolates component D of U and dU at a particle of cell (ci, cj, ck),
-// local (li, lj, lk) in the brick, from the staged tile.
-// The particle's weights on each axis, computed once: `face` for the component
-// whose faces are normal to that axis, `cen` (cell-centred nodes) for the others.
-struct PartW {
-  AxisW face[3], cen[3];
+// floor(v) for |v| < 2^22 by an addition rounded down, and the integer in its low bits: the
+// conversion units have a fraction of the FP32 rate.
+constexpr float FLOOR_MAGIC = 12582912.0f;  // 1.5 * 2^23
+__device__ __forceinline__ float floor_small(float v, int& i) {
+  const float m = __fadd_rd(v, FLOOR_MAGIC);
+  i = __float_as_int(m) - __float_as_int(FLOOR_MAGIC);
+  return __fsub_rn(m, FLOOR_MAGIC);
+}
+
+// cell_of for an x inside the domain (the same integer: both floors are exact).
+__device__ __forceinline__ int cell_in(float x, float inv, int n) {
+  const float p = __fmul_rn(x, inv);
+  const float e = __fmaf_rn(x, inv, -p);
+  int i;
+  const float f = floor_small(p, i);
+  if (p == f && e < 0.0f) --i;
+  return min(max(i, 0), n - 1);
+}
+
+// One axis of a particle's interpolation, both kinds of nodes: the two nodes of the tile
+// (lower index, two weights).  Positions are in cells
+// from the brick's origin, x/dx - b0 in one rounding; a rounding that reaches the next cell
+// changes neither nodes nor weights but by that rounding, for the interpolant is continuous.
+struct NodeW {
+  int i;
+  float w0, w1;
+};
+struct AxisG {
+  NodeW face, cen;
 };
 
-template <int D>
-__device__ __forceinline__ void interp_tile(const PartW& W, int li, int lj, int lk,
-                                            const float2* sud, float& U, float& dU) {
+__device__ __forceinline__ NodeW node_w(float v) {
+  NodeW r;
+  r.w1 = __fsub_rn(v, floor_small(v, r.i));
+  r.w0 = __fsub_rn(1.0f, r.w1);
+  return r;
+}
+
+// The faces are the tile's nodes 0 .. 8, the centres (from one below the brick on) its nodes
+// 0 .. 9, of which those outside the domain are not reached: centre 0 at the least, n - 1 at
+// the most (lo, hi: centre positions).
+__device__ __forceinline__ AxisG axis_g(float x, float inv, float b0, float lo, float hi) {
+  constexpr float BELOW_8 = 7.9999995f;
+  const float p = fminf(fmaxf(__fmaf_rn(x, inv, -b0), 0.0f), 8.0f);
+  AxisG a;
+  a.face = node_w(fminf(p, BELOW_8));
+  a.cen = node_w(fminf(fmaxf(__fadd_rn(p, 0.5f), lo), hi));
+  return a;
+}
+
+__device__ __forceinline__ float lerp(const NodeW& n, float a, float b) {
+  return __fmaf_rn(n.w1, b, __fmul_rn(n.w0, a));
+}
+__device__ __forceinline__ float2 lerp(const NodeW& n, float2 a, float2 b) {
+  return __ffma2_rn(make_float2(n.w1, n.w1), b, __fmul2_rn(make_float2(n.w0, n.w0), a));
+}
+
+// Component D: along x, then y, then z.
+template <int D, class T>
+__device__ __forceinline__ T interp_tile(const AxisG& ax, const AxisG& ay, const AxisG& az,
+                                         const T* sud) {
   constexpr int TX = FaceTile<D>::X, TY = FaceTile<D>::Y;
-  const AxisW& ax = (D == 0) ? W.face[0] : W.cen[0];
-  const AxisW& ay = (D == 1) ? W.face[1] : W.cen[1];
-  const AxisW& az = (D == 2) ? W.face[2] : W.cen[2];
-  const int t0 = (li + ax.off) + TX * ((lj + ay.off) + TY * (lk + az.off));
-  const float wx[2] = {ax.w0, ax.w1}, wy[2] = {ay.w0, ay.w1}, wz[2] = {az.w0, az.w1};
-  // (U, dU) accumulate together: one packed two-lane FMA per node, each lane
-  // rounded like __fmaf_rn
-  float2 s = make_float2(0.0f, 0.0f);
-#pragma unroll
-  for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-    for (int dy = 0; dy < 2; ++dy) {
-      const float wyz = __fmul_rn(wy[dy], wz[dz]);
-#pragma unroll
-      for (int dx = 0; dx < 2; ++dx) {
-        const float w = __fmul_rn(wx[dx], wyz);
-        const int t = t0 + dx + TX * (dy + TY * dz);
-        s = __ffma2_rn(make_float2(w, w), sud[t], s);
-      }
-    }
-  U = s.x;
-  dU = s.y;
+  const NodeW& nx = (D == 0) ? ax.face : ax.cen;
+  const NodeW& ny = (D == 1) ? ay.face : ay.cen;
+  const NodeW& nz = (D == 2) ? az.face : az.cen;
+  const T* t = sud + (nx.i + TX * (ny.i + TY * nz.i));
+  const T z0 = lerp(ny, lerp(nx, t[0], t[1]), lerp(nx, t[TX], t[TX + 1]));
+  t += TX * TY;
+  const T z1 = lerp(ny, lerp(nx, t[0], t[1]), lerp(nx, t[TX], t[TX + 1]));
+  return lerp(nz, z0, z1);
 }
 
 // Shared memory of a G2P CTA: the brick's staged tiles and the particle buffers.
-template <bool PAIR>
+template <bool PAIR, bool ADV>
 struct G2pShared {
   __align__(128) typename PTile<PAIR>::T sp[PTILE_N<PAIR>];  // the pressure slab
-  float2 sud[3][G2P_TILE];  // (u_new, u_new - u_old) per face node
+  NodeV<ADV> sud[3][G2P_TILE];
   __align__(16) float pbuf[2][6][G2P_CHUNK_PAD];
   __align__(8) unsigned long long bar[3];  // particle buffers 0, 1; the pressure slab
+  unsigned long long empty[2];             // ... the buffers' readers, one arrival per warp
   int abort;
 };
 
-// A CTA's streaming state, kept across bricks (and across scenes in a batched
-// launch): the mbarrier phases, the buffer of the next chunk, and (thread 0) which
-// barriers have a copy that nobody has waited for.
+// A CTA's streaming state, kept across bricks (and across scenes in a batched launch), a bit
+// per barrier: their phases, and (thread 0) which have a copy that nobody has waited for, the
+// readers' phases, and which buffers have had readers; the buffer of the next chunk.
 struct G2pCta {
-  unsigned int phase[3] = {0u, 0u, 0u};
-  unsigned int kbuf = 0;
-  bool inflight[3] = {false, false, false};
+  unsigned int phase = 0u, inflight = 0u, empty = 0u, used = 0u, kbuf = 0u;
 };
 
-template <bool PAIR>
-__device__ __forceinline__ void g2p_init(G2pShared<PAIR>& sh) {
+template <bool PAIR, bool ADV>
+__device__ __forceinline__ void g2p_init(G2pShared<PAIR, ADV>& sh) {
   if (threadIdx.x == 0) {
     mbar_init(&sh.bar[0], 1);
     mbar_init(&sh.bar[1], 1);
     mbar_init(&sh.bar[2], 1);
+    mbar_init(&sh.empty[0], G2P_THREADS / 32);
+    mbar_init(&sh.empty[1], G2P_THREADS / 32);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     sh.abort = 0;
   }
   __syncthreads();
 }
 
+// Thread 0: particles [q0, q1) into the next buffer, once its readers have left it; false if
+// they have not within the limit.
+template <bool PAIR, bool ADV>
+__device__ __forceinline__ bool g2p_issue(const PartView& P, unsigned int q0, unsigned int q1,
+                                          unsigned long long wait_ns, G2pShared<PAIR, ADV>& sh,
+                                          G2pCta& cs) {
+  const unsigned int k = cs.kbuf, bit = 1u << k;
+  if (cs.used & bit) {
+    if (!mbar_wait(&sh.empty[k], (cs.empty >> k) & 1u, wait_ns)) return false;
+    cs.empty ^= bit;
+  }
+  cs.used |= bit;
+  issue_chunk(P, q0, q1, sh.pbuf[k], &sh.bar[k]);
+  cs.inflight |= bit;
+  return true;
+}
+
 // One brick of one scene (pmap: the tensor map of the scene's pressure, or
 // nullptr for plain loads).  CTA-uniform; returns false once a wait has given up
 // (DEV_TIMEOUT set in the scene's status), after which the CTA takes no more bricks.
-template <bool PAIR>
+template <bool PAIR, bool ADV>
 __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, const PartView& P,
                                           const BinView& B, const float* __restrict__ uo0,
                                           const float* __restrict__ uo1,
@@ -260,17 +336,27 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
                                           const float* __restrict__ p32,
                                           const float2* __restrict__ pff, DevStats* st,
                                           const CUtensorMap* pmap, unsigned int brick,
-                                          G2pShared<PAIR>& sh, G2pCta& cs, float& speed2) {
+                                          unsigned int part, unsigned int split,
+                                          G2pShared<PAIR, ADV>& sh, G2pCta& cs, float& speed2) {
   using PT = typename PTile<PAIR>::T;
   const int lane = threadIdx.x & 31;
   const int b0 = (int)(brick % (unsigned)g.bx) * BRICK;
   const int b1 = (int)((brick / (unsigned)g.bx) % (unsigned)g.by) * BRICK;
   const int b2 = (int)(brick / ((unsigned)g.bx * (unsigned)g.by)) * BRICK;
-  const unsigned int bstart = B.brick_start[brick], bend = B.brick_start[brick + 1];
+  unsigned int bstart = B.brick_start[brick], bend = B.brick_start[brick + 1];
+  if (split > 1) {  // the part's whole chunks
+    const unsigned int chunks = (bend - bstart + G2P_THREADS - 1) / G2P_THREADS;
+    const unsigned int per = (chunks + split - 1) / split * G2P_THREADS;
+    const unsigned int first = min(bend, bstart + part * per);
+    bend = min(bend, first + per);
+    bstart = first;
+    if (bstart == bend) return true;
+  }
   // the brick's first chunk streams in while the tiles are staged
-  if (threadIdx.x == 0 && bstart < bend) {
-    issue_chunk(P, bstart, min(bend, bstart + G2P_THREADS), sh.pbuf[cs.kbuf], &sh.bar[cs.kbuf]);
-    cs.inflight[cs.kbuf] = true;
+  if (threadIdx.x == 0 && bstart < bend &&
+      !g2p_issue(P, bstart, min(bend, bstart + G2P_THREADS), K.wait_ns, sh, cs)) {
+    atomicOr(&st->status, DEV_TIMEOUT);
+    sh.abort = 1;
   }
   // pressure of cells [b0 - XOFF, b0 - XOFF + SPX) x [b1 - 1, b1 + 9) x [b2 - 1, b2 + 9)
   // (0 outside the grid: never used)
@@ -282,11 +368,11 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       mbar_expect_tx(&sh.bar[2], (unsigned)sizeof(sh.sp));
       tma_load_3d(sh.sp, pmap, b0 - XOFF, b1 - 1, b2 - 1, &sh.bar[2]);
-      cs.inflight[2] = true;
+      cs.inflight |= 4u;
     }
-    if (mbar_wait(&sh.bar[2], cs.phase[2], K.wait_ns)) {
-      cs.phase[2] ^= 1u;
-      cs.inflight[2] = false;
+    if (mbar_wait(&sh.bar[2], cs.phase >> 2, K.wait_ns)) {
+      cs.phase ^= 4u;
+      cs.inflight &= ~4u;
     } else {
       atomicOr(&st->status, DEV_TIMEOUT);
       sh.abort = 1;
@@ -305,65 +391,67 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
   }
   __syncthreads();
   if (sh.abort) return false;
-  stage_faces<0, PAIR>(g, K, b0, b1, b2, uo0, sh.sp, sh.sud[0]);
-  stage_faces<1, PAIR>(g, K, b0, b1, b2, uo1, sh.sp, sh.sud[1]);
-  stage_faces<2, PAIR>(g, K, b0, b1, b2, uo2, sh.sp, sh.sud[2]);
+  stage_faces<0, PAIR, ADV>(g, K, b0, b1, b2, uo0, sh.sp, sh.sud[0]);
+  stage_faces<1, PAIR, ADV>(g, K, b0, b1, b2, uo1, sh.sp, sh.sud[1]);
+  stage_faces<2, PAIR, ADV>(g, K, b0, b1, b2, uo2, sh.sp, sh.sud[2]);
   __syncthreads();
-  // chunk loop: CTA-uniform trip count, so every lane takes part in the key match
+  // A particle's rank in its new cell is what the histogram's atomic returns, with its place
+  // among the warp's lanes of that cell; it is written a chunk later, so that the atomic's
+  // round trip passes under the next chunk's arithmetic.
+  unsigned int first = 0u, rank_ofs = 0u, rank_q = ~0u;
+  int rank_lead = 0;
+  const auto put_ranks = [&]() {
+    const unsigned int f = __shfl_sync(0xffffffffu, first, rank_lead);
+    if (rank_q != ~0u) B.rank[rank_q] = f + rank_ofs;
+    rank_q = ~0u;
+  };
+  // chunk loop: warp-uniform trip count, so every lane takes part in the key match; the warps
+  // run apart by up to the buffers' depth
   for (unsigned int c0 = bstart; c0 < bend; c0 += G2P_THREADS) {
     const unsigned int cur = cs.kbuf;
     cs.kbuf ^= 1u;
-    // the next chunk goes into the other buffer, whose readers passed the
-    // __syncthreads that ended the previous chunk
     const unsigned int n0 = c0 + G2P_THREADS;
-    if (threadIdx.x == 0 && n0 < bend) {
-      issue_chunk(P, n0, min(bend, n0 + G2P_THREADS), sh.pbuf[cs.kbuf], &sh.bar[cs.kbuf]);
-      cs.inflight[cs.kbuf] = true;
-    }
-    // a thread whose wait gives up reads nothing of the chunk; one whose wait
+    bool ok = true;
+    if (threadIdx.x == 0 && n0 < bend)
+      ok = g2p_issue(P, n0, min(bend, n0 + G2P_THREADS), K.wait_ns, sh, cs);
+    // a warp with a wait that gave up reads nothing of the chunk; one whose waits
     // succeeded saw the whole chunk land
-    if (mbar_wait(&sh.bar[cur], cs.phase[cur], K.wait_ns)) {
-      cs.phase[cur] ^= 1u;
-      cs.inflight[cur] = false;
+    if (ok && mbar_wait(&sh.bar[cur], (cs.phase >> cur) & 1u, K.wait_ns)) {
+      cs.phase ^= 1u << cur;
+      cs.inflight &= ~(1u << cur);
     } else {
+      ok = false;
       atomicOr(&st->status, DEV_TIMEOUT);
       sh.abort = 1;
     }
+    if (!__all_sync(0xffffffffu, ok)) break;
     const float(*pb)[G2P_CHUNK_PAD] = sh.pbuf[cur];
-    const unsigned int a0 = c0 & ~3u;
     const unsigned int q = c0 + threadIdx.x;
-    const bool valid = q < bend && !sh.abort;
+    const bool valid = q < bend;
+    const unsigned int o = min(q, bend - 1u) - (c0 & ~3u);
+    float x = pb[0][o], y = pb[1][o], z = pb[2][o];
+    const float vp[3] = {pb[3][o], pb[4][o], pb[5][o]};
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&sh.empty[cur]);
     unsigned int key = 0xffffffffu;
     if (valid) {
-      const unsigned int o = q - a0;
-      float x = pb[0][o], y = pb[1][o], z = pb[2][o];
-      const float vp[3] = {pb[3][o], pb[4][o], pb[5][o]};
-      const int ci = cell_of(x, g.inv_dx, g.nx);
-      const int cj = cell_of(y, g.inv_dx, g.ny);
-      const int ck = cell_of(z, g.inv_dx, g.nz);
-      // the particle's cell lies in this brick (its key was taken by the
-      // same cell_of on the same coordinates); the clamp only keeps the
-      // shared-memory indices in range
-      const int li = min(max(ci - b0, 0), BRICK - 1);
-      const int lj = min(max(cj - b1, 0), BRICK - 1);
-      const int lk = min(max(ck - b2, 0), BRICK - 1);
-      PartW W;
-      W.face[0] = axis_weights<0, 0>(x, g.inv_dx, ci, g.nx);
-      W.face[1] = axis_weights<1, 1>(y, g.inv_dx, cj, g.ny);
-      W.face[2] = axis_weights<2, 2>(z, g.inv_dx, ck, g.nz);
-      W.cen[0] = axis_weights<1, 0>(x, g.inv_dx, ci, g.nx);
-      W.cen[1] = axis_weights<0, 1>(y, g.inv_dx, cj, g.ny);
-      W.cen[2] = axis_weights<0, 2>(z, g.inv_dx, ck, g.nz);
-      float U[3], dU[3];
-      interp_tile<0>(W, li, lj, lk, sh.sud[0], U[0], dU[0]);
-      interp_tile<1>(W, li, lj, lk, sh.sud[1], U[1], dU[1]);
-      interp_tile<2>(W, li, lj, lk, sh.sud[2], U[2], dU[2]);
-      const float r = K.flip_ratio, r1 = 1.0f - K.flip_ratio;
+      // the particle lies in this brick (its key was taken from the same coordinates); the
+      // clamps only keep the shared-memory indices in range
+      const AxisG ax = axis_g(x, g.inv_dx, (float)b0, b0 == 0 ? 1.0f : 0.0f, (float)min(g.nx - b0, 9));
+      const AxisG ay = axis_g(y, g.inv_dx, (float)b1, b1 == 0 ? 1.0f : 0.0f, (float)min(g.ny - b1, 9));
+      const AxisG az = axis_g(z, g.inv_dx, (float)b2, b2 == 0 ? 1.0f : 0.0f, (float)min(g.nz - b2, 9));
+      const NodeV<ADV> ud[3] = {interp_tile<0>(ax, ay, az, sh.sud[0]),
+                                interp_tile<1>(ax, ay, az, sh.sud[1]),
+                                interp_tile<2>(ax, ay, az, sh.sud[2])};
       float vn[3], adv[3];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        vn[d] = __fadd_rn(__fmul_rn(r, __fadd_rn(vp[d], dU[d])), __fmul_rn(r1, U[d]));
-        adv[d] = K.advect_grid ? U[d] : vn[d];
+        if constexpr (ADV) {
+          vn[d] = __fmaf_rn(K.flip_ratio, vp[d], ud[d].x);
+          adv[d] = K.advect_grid ? ud[d].y : vn[d];
+        } else {
+          vn[d] = adv[d] = __fmaf_rn(K.flip_ratio, vp[d], ud[d]);
+        }
       }
       x = fminf(fmaxf(__fmaf_rn(K.dt, adv[0], x), g.skin), g.hi[0]);
       y = fminf(fmaxf(__fmaf_rn(K.dt, adv[1], y), g.skin), g.hi[1]);
@@ -375,22 +463,20 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
       P.v[q] = vn[1];
       P.w[q] = vn[2];
       speed2 = fmaxf(speed2, vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
-      key = brick_key(g, cell_of(x, g.inv_dx, g.nx), cell_of(y, g.inv_dx, g.ny),
-                      cell_of(z, g.inv_dx, g.nz));
+      key = brick_key(g, cell_in(x, g.inv_dx, g.nx), cell_in(y, g.inv_dx, g.ny),
+                      cell_in(z, g.inv_dx, g.nz));
     }
+    if (valid) B.key[q] = key;
+    put_ranks();
     // one histogram atomic per distinct key of the warp
     const unsigned int same = __match_any_sync(0xffffffffu, key);
     const int leader = __ffs(same) - 1;
-    unsigned int first = 0u;
     if (valid && lane == leader) first = atomicAdd(B.cell_count + key, (unsigned)__popc(same));
-    first = __shfl_sync(0xffffffffu, first, leader);
-    if (valid) {
-      B.key[q] = key;
-      B.rank[q] = first + (unsigned)__popc(same & ((1u << lane) - 1u));
-    }
-    __syncthreads();
-    if (sh.abort) break;
+    rank_lead = leader;
+    rank_ofs = (unsigned)__popc(same & ((1u << lane) - 1u));
+    rank_q = valid ? q : ~0u;
   }
+  put_ranks();
   __syncthreads();
   return !sh.abort;
 }
@@ -398,12 +484,13 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
 // After an abort, thread 0 drains the copies it issued and nobody waited for
 // (the chunk whose wait gave up, the one issued after it), boundedly; the CTA's
 // shared memory stays allocated until thread 0 leaves.
-template <bool PAIR>
-__device__ __forceinline__ void g2p_drain(G2pShared<PAIR>& sh, const G2pCta& cs) {
+template <bool PAIR, bool ADV>
+__device__ __forceinline__ void g2p_drain(G2pShared<PAIR, ADV>& sh, const G2pCta& cs) {
   if (threadIdx.x == 0)
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-      if (cs.inflight[k]) (void)mbar_wait(&sh.bar[k], cs.phase[k], G2P_DRAIN_NS);
+      if ((cs.inflight >> k) & 1u)
+        (void)mbar_wait(&sh.bar[k], (cs.phase >> k) & 1u, G2P_DRAIN_NS);
 }
 
 // The largest particle speed a CTA saw in a scene, into the scene's statistics.
@@ -416,7 +503,22 @@ __device__ __forceinline__ void g2p_flush_speed(float& speed2, DevStats* st) {
   speed2 = 0.0f;
 }
 
-template <bool PAIR>
+// Parts per brick: a brick's chunks are a serial chain, so few bricks are shared out over the
+// launch's CTAs, each staging the tiles for itself.  The stage at 16 bricks (32^3 dam break)
+// 37 -> 16 us, at 150 (64^3) 42 -> 25.
+__device__ __forceinline__ unsigned int g2p_split(unsigned int nact, unsigned int ctas) {
+  unsigned int split = 1;
+  while (split < G2P_MAX_SPLIT && nact * 2u * split <= ctas) split *= 2;
+  return split;
+}
+
+// Bound by latency (the tiles' loads, the histogram's atomics) and by shared-memory accesses:
+// at 256^3 (42.3 M particles, 2.4 GB) the stage takes 0.64 ms of the 0.34 that the bytes do.
+// 0.745 -> 0.728 by weights and cells without conversions and packed interpolation by axes,
+// 0.705 by writing ranks a chunk late, 0.684 without a CTA barrier per chunk (and with the
+// barriers' state in bits, not in a stack array), 0.641 with one value per node, which halves
+// the shared-memory traffic.  6 CTAs per SM instead of 5 spill (0.692).
+template <bool PAIR, bool ADV>
 __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const StepConsts K0,
                                                      const PartView P, const BinView B,
                                                      const float* __restrict__ uo0,
@@ -427,16 +529,17 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
                                                      DevStats* st,
                                                      const __grid_constant__ CUtensorMap pmap,
                                                      int use_tma) {
-  __shared__ G2pShared<PAIR> sh;
+  __shared__ G2pShared<PAIR, ADV> sh;
   const StepConsts K = step_consts(K0);
   const unsigned int nact = st->n_active;
   g2p_init(sh);
   G2pCta cs;
   float speed2 = 0.0f;
   const CUtensorMap* map = use_tma ? &pmap : nullptr;
-  for (unsigned int bi = blockIdx.x; bi < nact; bi += gridDim.x)
-    if (!g2p_brick<PAIR>(g, K, P, B, uo0, uo1, uo2, p32, pff, st, map, B.active[bi], sh, cs,
-                         speed2))
+  const unsigned int split = g2p_split(nact, gridDim.x);
+  for (unsigned int bi = blockIdx.x; bi < nact * split; bi += gridDim.x)
+    if (!g2p_brick<PAIR, ADV>(g, K, P, B, uo0, uo1, uo2, p32, pff, st, map, B.active[bi / split],
+                         bi % split, split, sh, cs, speed2))
       break;
   g2p_drain(sh, cs);
   g2p_flush_speed(speed2, st);
@@ -444,37 +547,41 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
 
 // All scenes' active bricks as one list (L.first from k_active_prefix): the CTAs
 // share every scene's bricks evenly.  A CTA that gives up on a wait marks every
-// scene whose bricks it leaves undone.
+// scene whose bricks it leaves undone.  4 CTAs per SM (5 spill: 16 scenes 3.85 against
+// 3.71 ms per step).
 template <bool PAIR>
-__global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p_batch(const BatchLaunch L) {
-  __shared__ G2pShared<PAIR> sh;
+__global__ void __launch_bounds__(G2P_THREADS, 4) k_g2p_batch(const BatchLaunch L) {
+  __shared__ G2pShared<PAIR, true> sh;
   g2p_init(sh);
   G2pCta cs;
   float speed2 = 0.0f;
   int cur = -1;
   const unsigned int g0 = L.first[0], g1 = L.first[L.n];
-  unsigned int gb = g0 + blockIdx.x;
-  for (; gb < g1; gb += gridDim.x) {
+  const unsigned int split = g2p_split(g1 - g0, gridDim.x), n = (g1 - g0) * split;
+  unsigned int q = blockIdx.x;
+  for (; q < n; q += gridDim.x) {
+    const unsigned int gb = g0 + q / split;
     const int s = batch_scene(L, gb);
     const SceneDev& S = L.scenes[s];
     if (s != cur) {
       if (cur >= 0) g2p_flush_speed(speed2, L.scenes[cur].st);
       cur = s;
     }
-    if (!g2p_brick<PAIR>(S.g, step_consts(S.K), S.dst, S.B, S.uo[0], S.uo[1], S.uo[2], S.x32,
-                         S.pff, S.st, nullptr, S.B.active[gb - L.first[s]], sh, cs, speed2))
+    if (!g2p_brick<PAIR, true>(S.g, step_consts(S.K), S.dst, S.B, S.uo[0], S.uo[1], S.uo[2], S.x32,
+                         S.pff, S.st, nullptr, S.B.active[gb - L.first[s]], q % split, split, sh, cs,
+                         speed2))
       break;
   }
   g2p_drain(sh, cs);
   if (cur >= 0) g2p_flush_speed(speed2, L.scenes[cur].st);
-  if (gb < g1 && threadIdx.x == 0)  // aborted: the scenes of the bricks left undone
-    for (gb += gridDim.x; gb < g1; gb += gridDim.x)
-      atomicOr(&L.scenes[batch_scene(L, gb)].st->status, DEV_TIMEOUT);
+  if (q < n && threadIdx.x == 0)  // aborted: the scenes of the bricks left undone
+    for (q += gridDim.x; q < n; q += gridDim.x)
+      atomicOr(&L.scenes[batch_scene(L, g0 + q / split)].st->status, DEV_TIMEOUT);
 }
 
 int g2p_blocks(int sm_count) {
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<true>, G2P_THREADS, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<true, true>, G2P_THREADS, 0) !=
           cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
@@ -497,12 +604,9 @@ void launch_g2p(const Grid& g, const StepConsts& k, const PartView& p, const Bin
   std::memset(&none, 0, sizeof(none));
   const CUtensorMap& m = pmap ? *pmap : none;
   const int tma = pmap ? 1 : 0;
-  if (pff)
-    k_g2p<true><<<nblocks, G2P_THREADS, 0, s>>>(g, k, p, b, uo[0], uo[1], uo[2], p32, pff, st, m,
-                                               tma);
-  else
-    k_g2p<false><<<nblocks, G2P_THREADS, 0, s>>>(g, k, p, b, uo[0], uo[1], uo[2], p32, pff, st, m,
-                                                tma);
+  const auto kernel = pff ? (k.advect_grid ? k_g2p<true, true> : k_g2p<true, false>)
+                          : (k.advect_grid ? k_g2p<false, true> : k_g2p<false, false>);
+  kernel<<<nblocks, G2P_THREADS, 0, s>>>(g, k, p, b, uo[0], uo[1], uo[2], p32, pff, st, m, tma);
 }
 
 bool encode_pressure_map(const Grid& g, void* base, bool pair, CUtensorMap* out) {
