@@ -224,9 +224,9 @@ __device__ __forceinline__ int cell_in(float x, float inv, int n) {
 }
 
 // One axis of a particle's interpolation, both kinds of nodes: the two nodes of the tile
-// (lower index, two weights).  Positions are in cells
-// from the brick's origin, x/dx - b0 in one rounding; a rounding that reaches the next cell
-// changes neither nodes nor weights but by that rounding, for the interpolant is continuous.
+// (lower index, two weights).  Positions are in cells from the brick's origin; one that the
+// rounding of x/dx takes into the next cell has weights 1 and 0 there for 0 and 1 here, for
+// the interpolant is continuous.
 struct NodeW {
   int i;
   float w0, w1;
@@ -247,7 +247,7 @@ __device__ __forceinline__ NodeW node_w(float v) {
 // the most (lo, hi: centre positions).
 __device__ __forceinline__ AxisG axis_g(float x, float inv, float b0, float lo, float hi) {
   constexpr float BELOW_8 = 7.9999995f;
-  const float p = fminf(fmaxf(__fmaf_rn(x, inv, -b0), 0.0f), 8.0f);
+  const float p = fminf(fmaxf(__fsub_rn(__fmul_rn(x, inv), b0), 0.0f), 8.0f);
   AxisG a;
   a.face = node_w(fminf(p, BELOW_8));
   a.cen = node_w(fminf(fmaxf(__fadd_rn(p, 0.5f), lo), hi));

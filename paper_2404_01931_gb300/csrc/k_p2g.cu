@@ -50,19 +50,21 @@ struct Win {
   static constexpr int X = (D == 0) ? 2 : 3, Y = (D == 1) ? 2 : 3, Z = (D == 2) ? 2 : 3;
 };
 
-// One axis of the transfer weights of a particle of cell c (axis_weights' values over the
-// cell's window): f[2] on the faces, and h[3] on the centres, with t the distance from the
-// own centre in cells, |t| <= 1/2 and clamped at the domain's ends.  x/dx - c in one rounding.
+// One axis of the transfer weights of a particle of cell c, axis_weights' values bit for bit
+// over the cell's window (past the two roundings of x/dx and x/dx - 1/2 every difference is
+// exact): f[2] on the faces, and h[3] on the centres, with t the distance from the own centre
+// in cells, |t| <= 1/2 and clamped at the domain's ends.  Where only vanishing weights reach a
+// face their ratio is the velocity, so one rounding more or less would show there.
 struct AxisP {
   float f[2], h[3];
 };
 
 __device__ __forceinline__ AxisP axis_p(float x, float inv, float c, float lo, float hi) {
-  const float g = __fmaf_rn(x, inv, -c);
+  const float g = __fmul_rn(x, inv);
   AxisP a;
-  a.f[1] = fminf(fmaxf(g, 0.0f), 1.0f);
+  a.f[1] = fminf(fmaxf(__fsub_rn(g, c), 0.0f), 1.0f);
   a.f[0] = 1.0f - a.f[1];
-  const float t = fminf(fmaxf(g - 0.5f, lo), hi);
+  const float t = fminf(fmaxf(__fsub_rn(__fsub_rn(g, 0.5f), c), lo), hi);
   a.h[0] = fmaxf(-t, 0.0f);
   a.h[1] = 1.0f - fabsf(t);
   a.h[2] = fmaxf(t, 0.0f);

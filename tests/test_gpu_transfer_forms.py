@@ -31,3 +31,22 @@ def test_transfers_match_the_oracle_at_any_launch_width(n, hi, ctas):
     assert np.abs(got[:3] - np.stack([ref.x, ref.y, ref.z])).max() <= 1e-4 * dx
     vel = np.stack([ref.u, ref.v, ref.w])
     assert rel_l2(got[3:], vel, 9.81 / 240 * np.sqrt(vel.size)) <= 1e-5
+
+
+@pytest.mark.parametrize("cell", [2, 100, 250])
+def test_faces_that_only_vanishing_weights_reach(cell):
+    """Two particles a few roundings of x/dx past a face: the next face's velocity is the ratio
+    of FP32 weights, (f1 - f2) / (f1 + f2), within the sums' roundings."""
+    n, inv = (256, 8, 8), np.float32(256)
+    ulp = np.spacing(np.float32(cell)) / np.float32(256)
+    x = np.float32(cell / 256) + np.array([3, 8], np.float32) * ulp
+    c = np.full(2, 3.5 / 256, np.float32)
+    u, o = np.array([1, -1], np.float32), np.zeros(2, np.float32)
+    op, fp = matched(n)
+    with F.Simulation(fp, x, c, c, u, o, o) as sim:
+        sim.step(1)
+        uo = np.asarray(sim.read(F.U_OLD)).reshape(8, 8, 257)[3, 3]
+    f = x * inv - np.float32(cell)
+    assert (f > 0).all()
+    assert abs(uo[cell + 1] - (f[0] - f[1]) / (f[0] + f[1])) <= 8 * 2.0 ** -24
+    assert abs(uo[cell]) <= 1e-4
