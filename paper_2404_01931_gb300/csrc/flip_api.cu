@@ -1744,7 +1744,7 @@ int batch_step_impl(flip_batch* b, flip_handle* const* hs, int32_t n, int32_t ns
       const flip_handle* h = order[q];
       const long long faces = h->nf[0] + h->nf[1] + h->nf[2];
       const unsigned int cnt[5] = {(h->nbricks + 7u) / 8u, 1u,
-                                   (unsigned int)((h->np + 511) / 512),
+                                   (unsigned int)((h->np + 255) / 256),
                                    (unsigned int)((faces + 1023) / 1024),
                                    (unsigned int)h->g.ny * (unsigned int)h->g.nz};
       const int which[5] = {FL_SCAN, FL_ONE, FL_SCATTER, FL_FINALIZE, FL_DIV};

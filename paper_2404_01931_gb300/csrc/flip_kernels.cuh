@@ -261,7 +261,7 @@ void launch_iota(int* id, long long np, cudaStream_t s);
 // Batched forms: every scene of the table in one launch per kernel (no
 // reseeding, fixed time step).  first[] per launch as above; `ctas` its total.
 // Per-scene CTA counts: cell_local_scan ceil(nbricks / 8); brick_scan one; scatter
-// ceil(np / 512); finalize ceil(faces / 1024); divergence ny * nz.
+// ceil(np / 256); finalize ceil(faces / 1024); divergence ny * nz.
 void launch_bin_batch(const BatchLaunch& L_scan, unsigned int ctas_scan, const BatchLaunch& L_one,
                       cudaStream_t s);
 void launch_scatter_batch(const BatchLaunch& L, unsigned int ctas, cudaStream_t s);

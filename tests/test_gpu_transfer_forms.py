@@ -33,6 +33,22 @@ def test_transfers_match_the_oracle_at_any_launch_width(n, hi, ctas):
     assert rel_l2(got[3:], vel, 9.81 / 240 * np.sqrt(vel.size)) <= 1e-5
 
 
+@pytest.mark.parametrize("n", [(8, 8, 8), (24, 8, 8), (33, 8, 8), (64, 8, 9), (168, 168, 160)])
+def test_binning_keeps_every_particle(n):
+    """1, 3, 5, 16 and 8820 bricks: below, across and past the brick scan's vectors and chunks."""
+    rng = np.random.default_rng(11)
+    dx = np.float32(1 / max(n))
+    pos = [(rng.uniform(0.01, n[a] - 0.01, 3001) * dx).astype(np.float32) for a in range(3)]
+    vel = [rng.uniform(-0.5, 0.5, 3001).astype(np.float32) for _ in range(3)]
+    op, fp = matched(n, cg_tol=1e-2)
+    with F.Simulation(fp, *pos, *vel) as sim:
+        rc, st = sim.step(2, stats=True)
+        ids = np.asarray(sim.read(F.PID))
+        typ = np.asarray(sim.read(F.CELL_TYPE)).reshape(n[2], n[1], n[0])
+    assert rc == F.FLIP_OK and np.array_equal(np.sort(ids), np.arange(3001))
+    assert st.n_fluid_cells == np.count_nonzero(typ)
+
+
 @pytest.mark.parametrize("cell", [2, 100, 250])
 def test_faces_that_only_vanishing_weights_reach(cell):
     """Two particles a few roundings of x/dx past a face: the next face's velocity is the ratio
