@@ -7,7 +7,7 @@
 //                   the histogram atomic returns its rank in the bin
 //   scan            exclusive scan of the bin counts (tile scan below)
 //   k_sbin_scatter  positions into bin order as float4
-//   k_sdf           one warp per 2 x 2 corners: the bin rows that meet their balls of
+//   k_sdf           one warp per 2 x 2 x 2 corners: the bin rows that meet their balls of
 //                   radius R, read as coalesced particle ranges; kernel sums of k and
 //                   k (x_i - x), phi = |sum k d| / sum k - r
 // Pipeline of flip_surface_mesh:
@@ -374,88 +374,96 @@ __global__ void k_sbin_scatter(const PartView p, long long np, const int* __rest
   pos[start[b] + prank[i]] = make_float4(p.x[i], p.y[i], p.z[i], 0.0f);
 }
 
-// One warp per group of GX x GY corners of one z plane (2 x 2 where the corners are no
-// farther apart than a bin, else 2 x 1).  With bins of edge R/2 the balls meet at most 6
-// bins along y and 5 along z, so at most 30 bin rows (fixed y, z bin): lane r finds row
-// r's particle range (the row's bins within the balls' x extent are one contiguous range;
-// a bin whose nearest point is R or farther from the corners holds no particle closer
-// than R and is skipped), the nonempty rows are packed into a per-warp list, and the
-// warp's four groups of eight lanes take a row each, eight particles (128 bytes) at a
-// time.  Each particle is tested against all the group's corners, whose sums stay in
-// registers until a reduction that halves the values with every step.  The eight warps of
-// a CTA take neighbouring groups (4 x 4 x 2 corners), so that most of a CTA's particle
-// reads hit L1.
+// One warp per group of 2 x GY x GZ corners (2 x 2 x 2 where the corners are no farther apart
+// than a bin, else 2 x 1 x 1).  With bins of edge R/2 the balls meet at most 6 bins along y
+// and along z, so at most 36 bin rows (fixed y, z bin): lane r finds the particle ranges of
+// rows r and r + 32 (a row's bins within the balls' x extent are one contiguous range; a bin
+// whose nearest point is R or farther from the corners holds no particle closer than R and is
+// skipped), the nonempty rows are packed into a per-warp list, and the warp's four groups of
+// eight lanes take a row each, eight particles (128 bytes) at a time.  Each particle is tested
+// against all the group's corners, whose sums stay in registers until a reduction that halves
+// the values with every step.  The eight warps of a CTA take neighbouring groups (4 x 4 x 4
+// corners), so that most of a CTA's particle reads hit L1.
 //
-// Bound by issue (66 % of the slots, the FP32 pipe half busy): about 50 instructions per
-// particle and four corners, 640-800 particles tested per corner of which 268 lie in its
-// ball (8 per cell, R = 2 h).  A whole flip_surface_sdf of 42 M particles at 257^3 corners
-// 6.80 -> 4.81 ms, of 2.1 M at 129^3 0.555 -> 0.414, against one warp per 4 corners along x
-// whose lanes walked one flat range over all rows (row search and 160 shuffles per group);
-// without the load ahead 5.10 ms, 16 lanes a row 5.56, 6 CTAs per SM 5.14.
+// With e the offset particle minus corner, 1 - |e|^2 / R^2 is taken axis by axis: the two
+// values of 1 - ez^2 / R^2 and the four with y are shared by the corners, so that a corner's
+// weight costs one FMA more.
+//
+// Bound by issue.  A whole flip_surface_sdf of 42 M particles at 257^3 corners takes 4.04 ms,
+// of 2.1 M at 129^3 0.358; with 2 x 2 x 1 corners a warp 4.81 and 0.414 (about 50 instructions
+// per particle and four corners; a wider group tests more particles, but shares more of their
+// arithmetic); with one warp per 4 corners along x, whose lanes walked one flat range over all
+// rows, 6.80 and 0.555.  With t from 1 - |p|^2 / R^2 about the group's centre plus terms linear
+// in p 4.16 and 0.366, at twice the rounding error; 16 lanes a row 4.40; 4 CTAs per SM 4.40.
 constexpr int SDF_THREADS = 256;
 constexpr int SDF_WARPS = SDF_THREADS / 32;
 constexpr int SDF_ROW_LANES = 8;
+constexpr int SDF_ROWS = 40;
 
-template <int GX, int GY>
+template <int GY, int GZ>
 __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins B,
                                                      const unsigned int* __restrict__ start,
                                                      const float4* __restrict__ pos,
                                                      float* __restrict__ phi) {
-  static_assert(GX == 2 && (GY == 1 || GY == 2), "a packed pair along x");
-  __shared__ uint2 s_row[SDF_WARPS][32];  // {first particle, end} of the nonempty rows
+  constexpr int GX = 2, NP = GY * GZ;  // pairs along x
+  static_assert((GY == 1 || GY == 2) && (GZ == 1 || GZ == 2), "offsets in pairs");
+  __shared__ uint2 s_row[SDF_WARPS][SDF_ROWS];  // {first particle, end} of the nonempty rows
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   // a CTA's groups: 2 x 2 x 2
-  constexpr int CX = 2 * GX, CY = 2 * GY, CZ = 2;
+  constexpr int CX = 2 * GX, CY = 2 * GY, CZ = 2 * GZ;
   const int tx = (g.c[0] + CX - 1) / CX, ty = (g.c[1] + CY - 1) / CY, tz = (g.c[2] + CZ - 1) / CZ;
   const long long ntiles = (long long)tx * ty * tz;
   constexpr float Rb = 2.0f;  // R in bins (the bin edge is R/2)
   for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int i0 = (int)(tile % tx) * CX + (wid & 1) * GX;
     const int j0 = (int)((tile / tx) % ty) * CY + ((wid >> 1) & 1) * GY;
-    const int k = (int)(tile / ((long long)tx * ty)) * CZ + (wid >> 2);
-    if (i0 >= g.c[0] || j0 >= g.c[1] || k >= g.c[2]) continue;
+    const int k0 = (int)(tile / ((long long)tx * ty)) * CZ + (wid >> 2) * GZ;
+    if (i0 >= g.c[0] || j0 >= g.c[1] || k0 >= g.c[2]) continue;
     const float x0 = g.o[0] + g.h * (float)i0, x1 = g.o[0] + g.h * (float)(i0 + 1);
     const float y0 = g.o[1] + g.h * (float)j0, y1 = g.o[1] + g.h * (float)(j0 + GY - 1);
-    const float zc = g.o[2] + g.h * (float)k;
+    const float z0 = g.o[2] + g.h * (float)k0, z1 = g.o[2] + g.h * (float)(k0 + GZ - 1);
     const float ry0 = (y0 - B.o[1]) * B.inv_b, ry1 = (y1 - B.o[1]) * B.inv_b;
-    const float rz = (zc - B.o[2]) * B.inv_b;
+    const float rz0 = (z0 - B.o[2]) * B.inv_b, rz1 = (z1 - B.o[2]) * B.inv_b;
     const int by0 = max(0, (int)floorf(ry0 - Rb)), by1 = min(B.nb[1] - 1, (int)floorf(ry1 + Rb));
-    const int bz0 = max(0, (int)floorf(rz - Rb)), bz1 = min(B.nb[2] - 1, (int)floorf(rz + Rb));
+    const int bz0 = max(0, (int)floorf(rz0 - Rb)), bz1 = min(B.nb[2] - 1, (int)floorf(rz1 + Rb));
     const int nyr = max(by1 - by0 + 1, 1);
-    const int nrows = min(nyr * (bz1 - bz0 + 1), 32);
-    unsigned int p0 = 0, p1 = 0;
-    if (lane < nrows) {
-      const int by = by0 + lane % nyr, bz = bz0 + lane / nyr;
-      const float dy = fmaxf(fmaxf(B.o[1] + B.b * by - y1, y0 - (B.o[1] + B.b * (by + 1))), 0.0f);
-      const float dz = fmaxf(fmaxf(B.o[2] + B.b * bz - zc, zc - (B.o[2] + B.b * (bz + 1))), 0.0f);
-      const float dyz = dy * dy + dz * dz;
-      if (dyz < B.R2) {
-        const float rx = sqrtf(B.R2 - dyz) * B.inv_b;
-        const int bx0 = max(0, (int)floorf((x0 - B.o[0]) * B.inv_b - rx));
-        // (a bin that begins at the balls' end holds nothing closer than R)
-        const int bx1 = min(B.nb[0] - 1, (int)ceilf((x1 - B.o[0]) * B.inv_b + rx) - 1);
-        if (bx0 <= bx1) {
-          const long long row = (long long)B.nb[0] * (by + (long long)B.nb[1] * bz);
-          p0 = start[row + bx0];
-          p1 = start[row + bx1 + 1];
+    const int nrows = min(nyr * (bz1 - bz0 + 1), SDF_ROWS);
+    int nrow = 0;
+    __syncwarp();  // the last group's reads of the list are done
+    for (int r0 = 0; r0 < nrows; r0 += 32) {
+      const int r = r0 + lane;
+      unsigned int p0 = 0, p1 = 0;
+      if (r < nrows) {
+        const int by = by0 + r % nyr, bz = bz0 + r / nyr;
+        const float dy = fmaxf(fmaxf(B.o[1] + B.b * by - y1, y0 - (B.o[1] + B.b * (by + 1))), 0.0f);
+        const float dz = fmaxf(fmaxf(B.o[2] + B.b * bz - z1, z0 - (B.o[2] + B.b * (bz + 1))), 0.0f);
+        const float dyz = dy * dy + dz * dz;
+        if (dyz < B.R2) {
+          const float rx = sqrtf(B.R2 - dyz) * B.inv_b;
+          const int bx0 = max(0, (int)floorf((x0 - B.o[0]) * B.inv_b - rx));
+          // (a bin that begins at the balls' end holds nothing closer than R)
+          const int bx1 = min(B.nb[0] - 1, (int)ceilf((x1 - B.o[0]) * B.inv_b + rx) - 1);
+          if (bx0 <= bx1) {
+            const long long row = (long long)B.nb[0] * (by + (long long)B.nb[1] * bz);
+            p0 = start[row + bx0];
+            p1 = start[row + bx1 + 1];
+          }
         }
       }
+      const unsigned int some = __ballot_sync(0xffffffffu, p0 < p1);
+      if (p0 < p1) s_row[wid][nrow + __popc(some & ((1u << lane) - 1u))] = make_uint2(p0, p1);
+      nrow += __popc(some);
     }
-    const unsigned int some = __ballot_sync(0xffffffffu, p0 < p1);
-    const int nrow = __popc(some);
-    __syncwarp();  // the last group's reads of the list are done
-    if (p0 < p1) s_row[wid][__popc(some & ((1u << lane) - 1u))] = make_uint2(p0, p1);
     __syncwarp();
-    // per corner: sum k and sum k e; corners (0, y) and (1, y) go as the two lanes of packed
-    // FP32 operations, each rounded like the scalar operation
-    float2 sk[GY], sx[GY], sy[GY], sz[GY];
+    // minus the corners' coordinates (P.x + (-x) rounds as P.x - x); packed operations round
+    // like the scalar ones
+    const float2 mx = make_float2(-x0, -x1), my = make_float2(-y0, -y1),
+                 mz = make_float2(-z0, -z1);
+    const float2 nr = make_float2(-B.inv_R2, -B.inv_R2);
+    // per corner: sum k and sum k e; corners (0, y, z) and (1, y, z) are the two lanes
+    float2 sk[NP], sx[NP], sy[NP], sz[NP];
 #pragma unroll
-    for (int q = 0; q < GY; ++q) sk[q] = sx[q] = sy[q] = sz[q] = make_float2(0.0f, 0.0f);
-    // minus the corners' coordinates (P.x + (-x) rounds as P.x - x)
-    const float2 mx = make_float2(-x0, -x1), mz = make_float2(-zc, -zc);
-    float2 my[GY];
-#pragma unroll
-    for (int q = 0; q < GY; ++q) my[q] = make_float2(q == 0 ? -y0 : -y1, q == 0 ? -y0 : -y1);
+    for (int q = 0; q < NP; ++q) sk[q] = sx[q] = sy[q] = sz[q] = make_float2(0.0f, 0.0f);
     for (int r = lane / SDF_ROW_LANES; r < nrow; r += 32 / SDF_ROW_LANES) {
       const uint2 row = s_row[wid][r];
       unsigned int f = row.x + lane % SDF_ROW_LANES;
@@ -465,30 +473,36 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
         const float4 P = next;  // the next particle's load is in flight during this one's sums
         if (f + SDF_ROW_LANES < row.y) next = pos[f + SDF_ROW_LANES];
         const float2 ex = __fadd2_rn(make_float2(P.x, P.x), mx);
+        const float2 ey = __fadd2_rn(make_float2(P.y, P.y), my);
         const float2 ez = __fadd2_rn(make_float2(P.z, P.z), mz);
-        const float2 xx = __fmul2_rn(ex, ex), zz = __fmul2_rn(ez, ez);
+        const float2 fx = __fmul2_rn(ex, nr), fy = __fmul2_rn(ey, nr);
+        const float2 wz = __ffma2_rn(ez, __fmul2_rn(ez, nr), make_float2(1.0f, 1.0f));
 #pragma unroll
-        for (int q = 0; q < GY; ++q) {
-          const float2 ey = __fadd2_rn(make_float2(P.y, P.y), my[q]);
-          const float2 dd = __fadd2_rn(__ffma2_rn(ey, ey, zz), xx);
-          // k = max(0, 1 - d^2 / R^2)^3 (saturating: d^2 >= 0); at d = R the terms vanish
-          const float2 t = make_float2(__saturatef(__fmaf_rn(dd.x, -B.inv_R2, 1.0f)),
-                                       __saturatef(__fmaf_rn(dd.y, -B.inv_R2, 1.0f)));
-          const float2 kk = __fmul2_rn(__fmul2_rn(t, t), t);
-          sk[q] = __fadd2_rn(sk[q], kk);
-          sx[q] = __ffma2_rn(kk, ex, sx[q]);
-          sy[q] = __ffma2_rn(kk, ey, sy[q]);
-          sz[q] = __ffma2_rn(kk, ez, sz[q]);
+        for (int z = 0; z < GZ; ++z) {
+          const float e2 = z ? ez.y : ez.x;
+#pragma unroll
+          for (int y = 0; y < GY; ++y) {
+            const int q = y + GY * z;
+            const float e1 = y ? ey.y : ey.x;
+            const float w = __fmaf_rn(e1, y ? fy.y : fy.x, z ? wz.y : wz.x);
+            // k = max(0, 1 - d^2 / R^2)^3 (saturating: d^2 >= 0); at d = R the terms vanish
+            const float2 t = make_float2(__saturatef(__fmaf_rn(ex.x, fx.x, w)),
+                                         __saturatef(__fmaf_rn(ex.y, fx.y, w)));
+            const float2 kk = __fmul2_rn(__fmul2_rn(t, t), t);
+            sk[q] = __fadd2_rn(sk[q], kk);
+            sx[q] = __ffma2_rn(kk, ex, sx[q]);
+            sy[q] = __ffma2_rn(kk, make_float2(e1, e1), sy[q]);
+            sz[q] = __ffma2_rn(kk, make_float2(e2, e2), sz[q]);
+          }
         }
       }
     }
     // reduction: with every step a lane keeps half of its values and adds its partner's
-    // halves of them; then lane l holds corner l / 4's value l % 4 (for 4 corners; with 2
-    // corners l / 4 is 0 or 1)
-    constexpr int NV = 4 * GX * GY;
+    // halves of them; then lane l holds value l % 4 of corner l / 4 (modulo the corners)
+    constexpr int NV = 8 * NP;
     float v[NV];
 #pragma unroll
-    for (int q = 0; q < GY; ++q) {
+    for (int q = 0; q < NP; ++q) {
       v[8 * q] = sk[q].x;
       v[8 * q + 1] = sx[q].x;
       v[8 * q + 2] = sy[q].x;
@@ -516,20 +530,20 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
     const float b0 = __shfl_sync(0xffffffffu, s, 4 * lane + 1);
     const float b1 = __shfl_sync(0xffffffffu, s, 4 * lane + 2);
     const float b2 = __shfl_sync(0xffffffffu, s, 4 * lane + 3);
-    const int i = i0 + (lane & 1), j = j0 + (lane >> 1);
-    if (lane < GX * GY && i < g.c[0] && j < g.c[1]) {
+    const int i = i0 + (lane & 1), j = j0 + (lane >> 1) % GY, k = k0 + (lane >> 1) / GY;
+    if (lane < 2 * NP && i < g.c[0] && j < g.c[1] && k < g.c[2]) {
       const float d = (a > 0.0f) ? sqrtf(b0 * b0 + b1 * b1 + b2 * b2) / a - B.r : B.R - B.r;
       phi[i + (long long)g.c[0] * (j + (long long)g.c[1] * k)] = d;
     }
   }
 }
 
-// The corners of a 2 x 2 group share most of their bins while h is at most a bin edge
-// (R >= 2 h), and its rows fit a warp's list (6 x 5); wider grids take pairs along x.
+// The corners of a 2 x 2 x 2 group share most of their bins while h is at most a bin edge
+// (R >= 2 h), and its rows fit a warp's list (6 x 6); wider grids take pairs along x (5 x 5).
 using SdfKernel = void (*)(const SGrid, const SBins, const unsigned int*, const float4*, float*);
 
 SdfKernel sdf_kernel(const SGrid& g, const SBins& B) {
-  return g.h <= 1.001f * B.b ? (SdfKernel)k_sdf<2, 2> : (SdfKernel)k_sdf<2, 1>;
+  return g.h <= 1.001f * B.b ? (SdfKernel)k_sdf<2, 2> : (SdfKernel)k_sdf<1, 1>;
 }
 
 int sdf_blocks(SdfKernel k) {
