@@ -1,4 +1,4 @@
-"""The scalar field's two kernel forms (2 x 2 and 2 x 1 corners per warp) at the line between
+"""The scalar field's two kernel forms (2 x 2 x 2 and 2 corners per warp) at the line between
 them and on corner counts that leave groups and tiles part empty, against the oracle."""
 import numpy as np
 import pytest
@@ -8,15 +8,16 @@ from paper_2404_01931_gb300 import flip as F
 from paper_2404_01931_gb300 import scenes as S
 
 from parity_util import matched
+from test_gpu_surface import _gpu_mesh, _sp
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,h,ratio", [
-    ((31, 18, 7), 1 / 24, 2.0),      # R = 2 h: corners a bin apart, 2 x 2
-    ((32, 17, 8), 1 / 24, 1.9),      # just past the line, 2 x 1
-    ((9, 5, 6), 1 / 8, 0.7),         # balls that do not meet, 2 x 1
-    ((60, 55, 3), 1 / 72, 6.5),      # corners far closer than a bin, 2 x 2
+    ((31, 18, 7), 1 / 24, 2.0),      # R = 2 h: corners a bin apart, 2 x 2 x 2
+    ((32, 17, 8), 1 / 24, 1.9),      # just past the line, pairs
+    ((9, 5, 6), 1 / 8, 0.7),         # balls that do not meet, pairs
+    ((60, 55, 3), 1 / 72, 6.5),      # corners far closer than a bin, 2 x 2 x 2
     ((1, 1, 1), 1 / 2, 2.0),         # eight corners
 ])
 def test_sdf_forms_match_the_oracle(n, h, ratio):
@@ -35,3 +36,20 @@ def test_sdf_forms_match_the_oracle(n, h, ratio):
     # FP32 kernel sums: relative rounding ~1e-6 of the lengths involved (R), the bar of
     # test_gpu_surface.py
     assert np.abs(phi - ref).max() <= 2e-5 * sp.search_radius
+
+
+@pytest.mark.parametrize("n", [
+    (1, 1, 1024),      # rows of two corners and planes of four: many carries a step
+    (1024, 1, 1),      # the longest rows, four steps and a bit
+    (15, 15, 40),      # planes of 256 corners: no remainder
+    (30, 33, 5),       # planes of four steps and a bit
+])
+def test_mesh_walks_any_grid_shape(n):
+    """Dense crossings, so that the warps' lists are full; topology as the oracle's (the
+    normals' rounding grows with the grid's length over a cell and is bounded elsewhere)."""
+    phi = S.corner_field_random(n, 4, closed=False)
+    sp = _sp(n, 0.2)
+    ref = O.marching_cubes(phi.astype(np.float64), tuple(sp.origin), sp.h, 0.0)
+    nv, nt, got = _gpu_mesh(sp, phi)
+    assert nv > 1000 and nt > 1000
+    assert np.array_equal(got["e"], ref.vertex_edge) and np.array_equal(got["t"], ref.triangles)
