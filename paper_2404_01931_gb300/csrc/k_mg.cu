@@ -18,17 +18,22 @@
 // one colour and its six neighbour runs of the other colour, so it moves half
 // the bytes of a natural-layout sweep, every access coalesced.  Work is a list
 // of active segments per level (64 cells of a row that meet a block holding
-// fluid), built at the start of every solve; a warp takes one segment, a lane
-// one slot, and each CTA a contiguous slice of the list.  Per cell one 16-bit
-// code carries the fluid neighbours and the neighbour count, so value loads
-// never wait on flags, and each warp loads several segments before it computes
-// (memory-level parallelism).  The small coarsest levels (at most MG_CTA_CELLS
-// cells together) run inside CTA 0 from shared memory with __syncthreads; the
-// others use grid barriers between half-sweeps.
+// fluid), found at the start of every solve, each CTA a contiguous slice of it.
+// Per cell one 16-bit code carries the fluid neighbours and the neighbour
+// count, so value loads never wait on flags.  A level takes one of three forms
+// by its size per CTA: with many segments, a warp takes four of them, a lane
+// four slots (sweep_split_q); with fewer, a lane takes one slot and a warp loads
+// several segments before it computes; with few blocks holding fluid, a CTA
+// smooths whole 8x8x8 blocks with a halo in shared memory, everything before the
+// coarse cycle (restriction included) in one pass and everything after it in
+// another (block_pass).  The small coarsest levels (at most MG_CTA_CELLS cells
+// together) run inside CTA 0 from shared memory, in registers (cta_cycle_tiled)
+// or over lists; the others use grid barriers between passes.
 //
-// The correction is never written: the first post-smoothing half-sweep (black)
-// reads its red neighbours plus omega times their parents' values, and the red
-// half-sweep that follows overwrites the red cells anyway.  The first red
+// In the passes over segments the correction is never written: the first
+// post-smoothing half-sweep (black) reads its red neighbours plus omega times
+// their parents' values, and the red half-sweep that follows overwrites the red
+// cells anyway.  The first red
 // half-sweep from zero only needs the residual, so it is fused into the pass
 // that produces it: at level 0 the CG phase that updates r, at a grid-wide
 // coarse level the restriction.  The last black and the last red half-sweeps of

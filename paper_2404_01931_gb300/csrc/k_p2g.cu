@@ -247,8 +247,8 @@ __device__ __forceinline__ int p2g_split(unsigned int nact, unsigned int ctas) {
 // Bound by the FMA pipe and the latency of its chains, at 12 warps per SM (the sums of three
 // components take 108 of 168 registers): 5.2 M particles in 92 us with 330 instructions per
 // 32 particles.  A component at a time (64 registers, 32 warps, each particle read three
-// times) and all 54 nodes added to a common tile by shared-memory atomics, which are
-// compare-and-swap loops for floats: 130 us and 572 instructions.  The stage at 256^3
+// times) and all 54 nodes added to a common tile by shared-memory atomics:
+// 130 us and 572 instructions.  The stage at 256^3
 // (42.3 M) 0.998 -> 0.736 ms.  A thread per column of nodes in flush_tiles (fewer
 // instructions, but a serial chain) took 0.807, loading the next cell's first particle
 // ahead 0.792.
