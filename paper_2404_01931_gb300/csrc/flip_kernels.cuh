@@ -105,7 +105,9 @@ constexpr int MG_COARSE_SWEEPS = 2;   // red-black pairs each way on the coarses
 constexpr int MG_CTA_CELLS = 4800;    // the coarsest levels, up to this many cells in
                                       // total, run inside one CTA in shared memory
 constexpr int MG_BLK_PER_CTA = 6;     // a level with at most this many blocks holding
-                                      // fluid per CTA is smoothed blocked (block_pass)
+                                      // fluid per CTA is smoothed blocked (block_pass),
+constexpr int MG_BLK_PER_CTA_TEAM = 4;  // the same for teams of fewer than
+constexpr int MG_WIDE_TEAM = 128;       // MG_WIDE_TEAM CTAs
 constexpr float MG_OMEGA = 2.0f;      // over-correction of the coarse correction
 
 // One level of the hierarchy.  The grid-wide levels (l < lgrid) are stored

@@ -2038,8 +2038,11 @@ __device__ __forceinline__ bool seg_active(const PcgArgs& A, const MgLevel& L, i
 // with the limit at 3, 6, 10 and 16 blocks per CTA: 128^3 dam break (3.4 blocks) 1.03, 1.00,
 // 1.00, 0.98 ms; 128^3 pool (8.7 blocks) 1.52, 1.52, 1.79, 1.80; 256^3 pool (level 1: 8.4
 // blocks) 5.29, 5.29, 5.55, 5.54; 101 x 67 x 83 pool 1.28, 1.20, 1.21, 1.23.
+// A small team's barriers are cheaper, so its line is lower: a batch of 16 scenes (teams of 2
+// to 27 CTAs) at 2, 3, 4 and 6 blocks per CTA 3.37, 3.33, 3.34, 3.45 ms per step.
 __device__ __forceinline__ bool blocked(const MgArgs& M, unsigned int n) {
-  return M.nlev > 1 && M.nu <= BLK_MAX_NU && n > 0u && n <= (unsigned)MG_BLK_PER_CTA * team_size();
+  const int most = team_size() < (unsigned)MG_WIDE_TEAM ? MG_BLK_PER_CTA_TEAM : MG_BLK_PER_CTA;
+  return M.nlev > 1 && M.nu <= BLK_MAX_NU && n > 0u && n <= (unsigned)most * team_size();
 }
 
 // The grid-wide levels' lists of blocks holding fluid.  Level 0's follows the
