@@ -781,7 +781,8 @@ int flip_step(flip_handle* h, int32_t nsteps, flip_stats* stats) {
     h->launches += 1;
     if (timed) FLIP_CUDA(cudaEventRecord(ev[4], s));
     launch_g2p(h->g, h->K, h->P[h->cur], h->B, uo, h->mixed ? nullptr : h->x32, h->pff,
-               h->dstats, g2p_count(h), h->g2p_blocks, h->has_pmap ? &h->pmap : nullptr, s);
+               h->dstats, g2p_count(h), h->g2p_blocks, h->has_pmap ? &h->pmap : nullptr,
+               reseeding(h), s);
     h->launches += (g2p_count(h) > 0);
     launch_back(h, s);
     if (timed) FLIP_CUDA(cudaEventRecord(ev[5], s));
@@ -1849,7 +1850,7 @@ int batch_step_impl(flip_batch* b, flip_handle* const* hs, int32_t n, int32_t ns
       FLIP_CUDA(cudaStreamWaitEvent(h->stream, b->ev_solved, 0));
       launch_g2p(h->g, h->K, h->P[h->cur], h->B, uo, h->mixed ? nullptr : h->x32, h->pff,
                  h->dstats, g2p_count(h), h->g2p_blocks, h->has_pmap ? &h->pmap : nullptr,
-                 h->stream);
+                 reseeding(h), h->stream);
       h->launches += (g2p_count(h) > 0);
       launch_back(h, h->stream);
       h->stepped = true;

@@ -343,10 +343,12 @@ void launch_spawn(const Grid& g, const StepConsts& k, const PartView& p, const B
 // k_g2p.cu
 int g2p_blocks(int sm_count);
 // pmap (nullable): tensor map of the pressure (encode_pressure_map) for the TMA
-// staging of the pressure slab; plain loads when NULL.
+// staging of the pressure slab; plain loads when NULL.  keep_order: a brick's
+// particles take their ranks in the order of its chunks.
 void launch_g2p(const Grid& g, const StepConsts& k, const PartView& p, const BinView& b,
                 const float* const uo[3], const float* p32, const float2* pff, DevStats* st,
-                long long np, int nblocks, const CUtensorMap* pmap, cudaStream_t s);
+                long long np, int nblocks, const CUtensorMap* pmap, bool keep_order,
+                cudaStream_t s);
 // Tensor map of a pressure field (float pairs when pair, else FP32; natural
 // layout) for G2P's slab staging; false when the grid's pitches do not allow one.
 bool encode_pressure_map(const Grid& g, void* base, bool pair, CUtensorMap* out);

@@ -505,10 +505,12 @@ __device__ __forceinline__ void g2p_flush_speed(float& speed2, DevStats* st) {
 
 // Parts per brick: a brick's chunks are a serial chain, so few bricks are shared out over the
 // launch's CTAs, each staging the tiles for itself.  The stage at 16 bricks (32^3 dam break)
-// 37 -> 16 us, at 150 (64^3) 42 -> 25.
-__device__ __forceinline__ unsigned int g2p_split(unsigned int nact, unsigned int ctas) {
+// 37 -> 16 us, at 150 (64^3) 42 -> 25.  Not with reseeding (most = 1): the parts would take
+// their ranks in no order, and which of a crowded cell's particles are dropped depends on it.
+__device__ __forceinline__ unsigned int g2p_split(unsigned int nact, unsigned int ctas,
+                                                  unsigned int most) {
   unsigned int split = 1;
-  while (split < G2P_MAX_SPLIT && nact * 2u * split <= ctas) split *= 2;
+  while (split < most && nact * 2u * split <= ctas) split *= 2;
   return split;
 }
 
@@ -528,7 +530,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
                                                      const float2* __restrict__ pff,
                                                      DevStats* st,
                                                      const __grid_constant__ CUtensorMap pmap,
-                                                     int use_tma) {
+                                                     int use_tma, unsigned int most) {
   __shared__ G2pShared<PAIR, ADV> sh;
   const StepConsts K = step_consts(K0);
   const unsigned int nact = st->n_active;
@@ -536,7 +538,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
   G2pCta cs;
   float speed2 = 0.0f;
   const CUtensorMap* map = use_tma ? &pmap : nullptr;
-  const unsigned int split = g2p_split(nact, gridDim.x);
+  const unsigned int split = g2p_split(nact, gridDim.x, most);
   for (unsigned int bi = blockIdx.x; bi < nact * split; bi += gridDim.x)
     if (!g2p_brick<PAIR, ADV>(g, K, P, B, uo0, uo1, uo2, p32, pff, st, map, B.active[bi / split],
                          bi % split, split, sh, cs, speed2))
@@ -557,7 +559,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 4) k_g2p_batch(const BatchLaunch 
   float speed2 = 0.0f;
   int cur = -1;
   const unsigned int g0 = L.first[0], g1 = L.first[L.n];
-  const unsigned int split = g2p_split(g1 - g0, gridDim.x), n = (g1 - g0) * split;
+  const unsigned int split = g2p_split(g1 - g0, gridDim.x, G2P_MAX_SPLIT), n = (g1 - g0) * split;
   unsigned int q = blockIdx.x;
   for (; q < n; q += gridDim.x) {
     const unsigned int gb = g0 + q / split;
@@ -598,7 +600,8 @@ void launch_g2p_batch(const BatchLaunch& L, unsigned int ctas, bool pair, cudaSt
 
 void launch_g2p(const Grid& g, const StepConsts& k, const PartView& p, const BinView& b,
                 const float* const uo[3], const float* p32, const float2* pff, DevStats* st,
-                long long np, int nblocks, const CUtensorMap* pmap, cudaStream_t s) {
+                long long np, int nblocks, const CUtensorMap* pmap, bool keep_order,
+                cudaStream_t s) {
   if (np <= 0) return;
   CUtensorMap none;
   std::memset(&none, 0, sizeof(none));
@@ -606,7 +609,8 @@ void launch_g2p(const Grid& g, const StepConsts& k, const PartView& p, const Bin
   const int tma = pmap ? 1 : 0;
   const auto kernel = pff ? (k.advect_grid ? k_g2p<true, true> : k_g2p<true, false>)
                           : (k.advect_grid ? k_g2p<false, true> : k_g2p<false, false>);
-  kernel<<<nblocks, G2P_THREADS, 0, s>>>(g, k, p, b, uo[0], uo[1], uo[2], p32, pff, st, m, tma);
+  kernel<<<nblocks, G2P_THREADS, 0, s>>>(g, k, p, b, uo[0], uo[1], uo[2], p32, pff, st, m, tma,
+                                          keep_order ? 1u : G2P_MAX_SPLIT);
 }
 
 bool encode_pressure_map(const Grid& g, void* base, bool pair, CUtensorMap* out) {
