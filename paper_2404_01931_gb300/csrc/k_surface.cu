@@ -411,9 +411,9 @@ __global__ void k_sbin_scatter(const PartView p, long long np, const int* __rest
 }
 
 // One warp per group of 2 x GY x GZ corners (2 x 2 x 2 where the corners are no farther apart
-// than a bin, else 2 x 1 x 1).  With bins of edge R/2 the balls meet at most 6 bins along y
-// and along z, so at most 36 bin rows (fixed y, z bin): lane r finds the particle ranges of
-// rows r and r + 32 (a row's bins within the balls' x extent are one contiguous range; a bin
+// than a bin, else 2 x 1 x 1).  With bins of edge R/2 the balls' extent along y or z is at most
+// 5.001 bins, which meets at most 7 (corners on bin faces, with roundings either way), so at
+// most 49 bin rows (fixed y, z bin): lane r finds the particle ranges of rows r and r + 32 (a row's bins within the balls' x extent are one contiguous range; a bin
 // whose nearest point is R or farther from the corners holds no particle closer than R and is
 // skipped), the nonempty rows are packed into a per-warp list, and the warp's four groups of
 // eight lanes take a row each, eight particles (128 bytes) at a time.  Each particle is tested
@@ -434,7 +434,7 @@ __global__ void k_sbin_scatter(const PartView p, long long np, const int* __rest
 constexpr int SDF_THREADS = 256;
 constexpr int SDF_WARPS = SDF_THREADS / 32;
 constexpr int SDF_ROW_LANES = 8;
-constexpr int SDF_ROWS = 40;
+constexpr int SDF_ROWS = 49;
 
 template <int GY, int GZ>
 __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins B,
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
 }
 
 // The corners of a 2 x 2 x 2 group share most of their bins while h is at most a bin edge
-// (R >= 2 h), and its rows fit a warp's list (6 x 6); wider grids take pairs along x (5 x 5).
+// (R >= 2 h), and its rows fit a warp's list (7 x 7); wider grids take pairs along x (6 x 6).
 using SdfKernel = void (*)(const SGrid, const SBins, const unsigned int*, const float4*, float*);
 
 SdfKernel sdf_kernel(const SGrid& g, const SBins& B) {

@@ -19,13 +19,16 @@ pytestmark = pytest.mark.gpu
     ((9, 5, 6), 1 / 8, 0.7),         # balls that do not meet, pairs
     ((60, 55, 3), 1 / 72, 6.5),      # corners far closer than a bin, 2 x 2 x 2
     ((1, 1, 1), 1 / 2, 2.0),         # eight corners
+    ((30, 25, 18), 1 / 30, 2.0),     # corners on bin faces, rounded to either side: 2 x 2 x 2
+    ((23, 17, 12), 1 / 23, 2.0),     # ... and 2 x 2 x 1
+    ((55, 50, 45), 1 / 55, 2.0),
 ])
 def test_sdf_forms_match_the_oracle(n, h, ratio):
     sc = S.random_velocities(S.water_drop(24, centre=(0.4, 0.45, 0.3), radius=0.25), 0.1, 3)
     sp = F.FlipSurfaceParams()
     for a in range(3):
         sp.n[a] = n[a]
-        sp.origin[a] = (-0.01, 0.003, 0.02)[a]
+        sp.origin[a] = 0.0 if round(n[0] * h, 6) == 1.0 else (-0.01, 0.003, 0.02)[a]
     sp.h, sp.search_radius = h, ratio * h
     sp.radius, sp.iso = 0.25 * sp.search_radius, 0.0
     with F.Simulation(matched(24)[1], *sc.arrays()) as sim, F.Surface(sp) as s:
