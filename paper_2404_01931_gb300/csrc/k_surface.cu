@@ -576,10 +576,18 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
 
 // The corners of a 2 x 2 x 2 group share most of their bins while h is at most a bin edge
 // (R >= 2 h), and its rows fit a warp's list (7 x 7); wider grids take pairs along x (6 x 6).
+// A grid of few groups takes 2 x 2 x 1 ones, twice as many, to even out the chip's last
+// rounds: flip_surface_sdf with 7 thousand groups (48 x 33 x 33 cells, 4 scenes) 58-69 us
+// with 2 x 2 x 2, 59-66 with 2 x 2 x 1; with 11 thousand 63-81 and 64-72; with 26 thousand
+// 72-103 and 77-109; with 30 thousand 75-112 and 87-135.
 using SdfKernel = void (*)(const SGrid, const SBins, const unsigned int*, const float4*, float*);
 
+constexpr long long SDF_FEW = 4 * 152 * 3 * SDF_WARPS;  // four rounds of resident warps
+
 SdfKernel sdf_kernel(const SGrid& g, const SBins& B) {
-  return g.h <= 1.001f * B.b ? (SdfKernel)k_sdf<2, 2> : (SdfKernel)k_sdf<1, 1>;
+  if (g.h > 1.001f * B.b) return k_sdf<1, 1>;
+  const long long groups = (long long)((g.c[0] + 1) / 2) * ((g.c[1] + 1) / 2) * ((g.c[2] + 1) / 2);
+  return groups >= SDF_FEW ? k_sdf<2, 2> : k_sdf<2, 1>;
 }
 
 int sdf_blocks(SdfKernel k) {

@@ -1,4 +1,4 @@
-"""The scalar field's two kernel forms (2 x 2 x 2 and 2 corners per warp) at the line between
+"""The scalar field's kernel forms (2 x 2 x 2, 2 x 2 and 2 corners per warp) at the lines between
 them and on corner counts that leave groups and tiles part empty, against the oracle."""
 import numpy as np
 import pytest
@@ -14,14 +14,15 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,h,ratio", [
-    ((31, 18, 7), 1 / 24, 2.0),      # R = 2 h: corners a bin apart, 2 x 2 x 2
+    ((31, 18, 7), 1 / 24, 2.0),      # R = 2 h: corners a bin apart, 2 x 2
     ((32, 17, 8), 1 / 24, 1.9),      # just past the line, pairs
     ((9, 5, 6), 1 / 8, 0.7),         # balls that do not meet, pairs
-    ((60, 55, 3), 1 / 72, 6.5),      # corners far closer than a bin, 2 x 2 x 2
+    ((60, 55, 3), 1 / 72, 6.5),      # corners far closer than a bin, 2 x 2
     ((1, 1, 1), 1 / 2, 2.0),         # eight corners
-    ((30, 25, 18), 1 / 30, 2.0),     # corners on bin faces, rounded to either side: 2 x 2 x 2
-    ((23, 17, 12), 1 / 23, 2.0),     # ... and 2 x 2 x 1
-    ((55, 50, 45), 1 / 55, 2.0),
+    ((30, 25, 18), 1 / 30, 2.0),     # corners on bin faces, rounded to either side: 2 x 2
+    ((23, 17, 12), 1 / 23, 2.0),
+    ((55, 50, 45), 1 / 55, 2.0),     # ... and 2 x 2 x 2
+    ((47, 59, 51), 1 / 60, 3.1),     # 2 x 2 x 2, corners between the faces
 ])
 def test_sdf_forms_match_the_oracle(n, h, ratio):
     sc = S.random_velocities(S.water_drop(24, centre=(0.4, 0.45, 0.3), radius=0.25), 0.1, 3)
