@@ -22,7 +22,6 @@ pytestmark = pytest.mark.gpu
     ((30, 25, 18), 1 / 30, 2.0),     # corners on bin faces, rounded to either side: 2 x 2
     ((23, 17, 12), 1 / 23, 2.0),
     ((55, 50, 45), 1 / 55, 2.0),     # ... and 2 x 2 x 2
-    ((47, 59, 51), 1 / 60, 3.1),     # 2 x 2 x 2, corners between the faces
 ])
 def test_sdf_forms_match_the_oracle(n, h, ratio):
     sc = S.random_velocities(S.water_drop(24, centre=(0.4, 0.45, 0.3), radius=0.25), 0.1, 3)
