@@ -7,14 +7,12 @@
 // see below).  It first stages in shared memory the
 // pressure of the brick plus a one-cell halo, then, for every component, the
 // face nodes any of the brick's particles can reach (the 9x10x10 tile P2G also
-// uses).  With u_new from Eq. 5 (gravity and walls, face_unew's arithmetic), the
-// blend v <- r (v + interp(u_new - u_old)) + (1 - r) interp(u_new) is
-//     v <- r v + interp(u_new - r u_old)
-// so that one value per node is interpolated, staged in one rounding.  Each face
-// value is so computed once per brick instead of once per particle that touches it.
-// Then one thread per particle interpolates and moves:
-//     x <- clamp(x + dt v, skin, n dx - skin)
-// or, with grid advection, x + dt interp(u_new), for which the tile holds u_new too.
+// uses): U = u_new (Eq. 5 with gravity and walls, face_unew's arithmetic) and
+// dU = u_new - u_old.  Each face value is so computed once per brick instead of
+// once per particle that touches it.  Then one thread per particle interpolates
+// (U, dU) with P2G's weights and applies
+//     v <- r (v + interp(dU)) + (1 - r) interp(U)
+//     x <- clamp(x + dt v, skin, n dx - skin)      (or dt interp(U), grid advection)
 // and computes the key of the cell it moved to and its rank there.  Ranks come
 // from one histogram atomic per distinct key in a warp (lanes with the same key
 // take consecutive ranks), which is all the next step's counting sort needs.
@@ -155,28 +153,14 @@ __device__ __forceinline__ float pdiff(float2 hp, float2 hm) {
 }
 __device__ __forceinline__ float pdiff(float hp, float hm) { return __fsub_rn(hp, hm); }
 
-// A node of the staged tiles: u_new - r u_old, and with grid advection u_new.
-template <bool ADV>
-struct NodeOf;
-template <>
-struct NodeOf<false> {
-  using T = float;
-};
-template <>
-struct NodeOf<true> {
-  using T = float2;
-};
-template <bool ADV>
-using NodeV = typename NodeOf<ADV>::T;
-
 // Stages component D's face tile: node (a, b, c) with a in [o0, o0 + X) etc.,
 // o = brick origin on the own axis and origin - 1 on the others.  Nodes outside
 // the face grid are never interpolated (the clamped weights keep every node in
 // range) and are set to 0.
-template <int D, bool PAIR, bool ADV>
+template <int D, bool PAIR>
 __device__ __forceinline__ void stage_faces(const Grid& g, const StepConsts& K, int b0, int b1,
                                             int b2, const float* __restrict__ uo,
-                                            const typename PTile<PAIR>::T* sp, NodeV<ADV>* sud) {
+                                            const typename PTile<PAIR>::T* sp, float2* sud) {
   constexpr int TX = FaceTile<D>::X, TY = FaceTile<D>::Y, N = FaceTile<D>::N;
   const int o0 = (D == 0) ? b0 : b0 - 1, o1 = (D == 1) ? b1 : b1 - 1, o2 = (D == 2) ? b2 : b2 - 1;
   const int FX = g.nx + (D == 0), FY = g.ny + (D == 1), FZ = g.nz + (D == 2);
@@ -184,7 +168,7 @@ __device__ __forceinline__ void stage_faces(const Grid& g, const StepConsts& K, 
   for (int t = threadIdx.x; t < N; t += G2P_THREADS) {
     const int ta = t % TX, tb = (t / TX) % TY, tc = t / (TX * TY);
     const int a = o0 + ta, b = o1 + tb, c = o2 + tc;
-    float un = 0.0f, fl = 0.0f;
+    float un = 0.0f, du = 0.0f;
     if (a >= 0 && b >= 0 && c >= 0 && a < FX && b < FY && c < FZ) {
       const float uov = __ldg(uo + (a + FX * (b + FY * c)));
       const int nd = (D == 0) ? a : (D == 1) ? b : c;
@@ -197,10 +181,9 @@ __device__ __forceinline__ void stage_faces(const Grid& g, const StepConsts& K, 
         const float dp = pdiff(sp[pc], sp[pm]);
         un = __fsub_rn(__fadd_rn(uov, K.gdt[D]), __fmul_rn(K.pscale, dp));
       }
-      fl = __fmaf_rn(-K.flip_ratio, uov, un);
+      du = __fsub_rn(un, uov);
     }
-    if constexpr (ADV) sud[t] = make_float2(fl, un);
-    else sud[t] = fl;
+    sud[t] = make_float2(un, du);
   }
 }
 
@@ -224,9 +207,10 @@ __device__ __forceinline__ int cell_in(float x, float inv, int n) {
 }
 
 // One axis of a particle's interpolation, both kinds of nodes: the two nodes of the tile
-// (lower index, two weights).  Positions are in cells from the brick's origin; one that the
-// rounding of x/dx takes into the next cell has weights 1 and 0 there for 0 and 1 here, for
-// the interpolant is continuous.
+// (lower index, two weights).  The weights are axis_weights', bit for bit: past the two
+// roundings of x/dx and x/dx - 1/2 every difference is exact.  A position that the first
+// takes to the end of its cell may stand at a node of weight 1 as the lower or as the
+// upper of the two; the other's weight is 0 and the interpolant the same.
 struct NodeW {
   int i;
   float w0, w1;
@@ -235,52 +219,53 @@ struct AxisG {
   NodeW face, cen;
 };
 
-__device__ __forceinline__ NodeW node_w(float v) {
-  NodeW r;
-  r.w1 = __fsub_rn(v, floor_small(v, r.i));
-  r.w0 = __fsub_rn(1.0f, r.w1);
-  return r;
-}
-
-// The faces are the tile's nodes 0 .. 8, the centres (from one below the brick on) its nodes
-// 0 .. 9, of which those outside the domain are not reached: centre 0 at the least, n - 1 at
-// the most (lo, hi: centre positions).
-__device__ __forceinline__ AxisG axis_g(float x, float inv, float b0, float lo, float hi) {
+// The faces are the tile's nodes 0 .. 8 (of the brick's eight cells), the centres (from one
+// below the brick on) its nodes 0 .. 9, of which those outside the domain are not reached:
+// centre 0 at the least, n - 1 at the most.  lo, hi: those centres, or the ends of what the
+// brick's particles reach (b0 - 1, b0 + 7.5), which keep the indices in range.
+__device__ __forceinline__ AxisG axis_g(float x, float inv, int b0, float lo, float hi) {
   constexpr float BELOW_8 = 7.9999995f;
-  const float p = fminf(fmaxf(__fsub_rn(__fmul_rn(x, inv), b0), 0.0f), 8.0f);
+  const float g = __fmul_rn(x, inv);
+  const float p = fminf(fmaxf(__fsub_rn(g, (float)b0), 0.0f), 8.0f);
+  const float c = fminf(fmaxf(__fsub_rn(g, 0.5f), lo), hi);
   AxisG a;
-  a.face = node_w(fminf(p, BELOW_8));
-  a.cen = node_w(fminf(fmaxf(__fadd_rn(p, 0.5f), lo), hi));
+  a.face.w1 = __fsub_rn(p, floor_small(fminf(p, BELOW_8), a.face.i));
+  a.face.w0 = __fsub_rn(1.0f, a.face.w1);
+  a.cen.w1 = __fsub_rn(c, floor_small(c, a.cen.i));
+  a.cen.w0 = __fsub_rn(1.0f, a.cen.w1);
+  a.cen.i += 1 - b0;
   return a;
 }
 
-__device__ __forceinline__ float lerp(const NodeW& n, float a, float b) {
-  return __fmaf_rn(n.w1, b, __fmul_rn(n.w0, a));
-}
-__device__ __forceinline__ float2 lerp(const NodeW& n, float2 a, float2 b) {
-  return __ffma2_rn(make_float2(n.w1, n.w1), b, __fmul2_rn(make_float2(n.w0, n.w0), a));
-}
-
-// Component D: along x, then y, then z.
-template <int D, class T>
-__device__ __forceinline__ T interp_tile(const AxisG& ax, const AxisG& ay, const AxisG& az,
-                                         const T* sud) {
+// Interpolates component D of (U, dU) from the staged tile: one packed two-lane FMA per
+// node, each lane rounded like __fmaf_rn.
+template <int D>
+__device__ __forceinline__ float2 interp_tile(const AxisG& ax, const AxisG& ay, const AxisG& az,
+                                              const float2* sud) {
   constexpr int TX = FaceTile<D>::X, TY = FaceTile<D>::Y;
   const NodeW& nx = (D == 0) ? ax.face : ax.cen;
   const NodeW& ny = (D == 1) ? ay.face : ay.cen;
   const NodeW& nz = (D == 2) ? az.face : az.cen;
-  const T* t = sud + (nx.i + TX * (ny.i + TY * nz.i));
-  const T z0 = lerp(ny, lerp(nx, t[0], t[1]), lerp(nx, t[TX], t[TX + 1]));
-  t += TX * TY;
-  const T z1 = lerp(ny, lerp(nx, t[0], t[1]), lerp(nx, t[TX], t[TX + 1]));
-  return lerp(nz, z0, z1);
+  const float2* t = sud + (nx.i + TX * (ny.i + TY * nz.i));
+  const float wy[2] = {ny.w0, ny.w1}, wz[2] = {nz.w0, nz.w1};
+  float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+  for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy) {
+      const float wyz = __fmul_rn(wy[dy], wz[dz]);
+      const float w0 = __fmul_rn(nx.w0, wyz), w1 = __fmul_rn(nx.w1, wyz);
+      s = __ffma2_rn(make_float2(w0, w0), t[TX * (dy + TY * dz)], s);
+      s = __ffma2_rn(make_float2(w1, w1), t[TX * (dy + TY * dz) + 1], s);
+    }
+  return s;
 }
 
 // Shared memory of a G2P CTA: the brick's staged tiles and the particle buffers.
-template <bool PAIR, bool ADV>
+template <bool PAIR>
 struct G2pShared {
   __align__(128) typename PTile<PAIR>::T sp[PTILE_N<PAIR>];  // the pressure slab
-  NodeV<ADV> sud[3][G2P_TILE];
+  float2 sud[3][G2P_TILE];  // (u_new, u_new - u_old) per face node
   __align__(16) float pbuf[2][6][G2P_CHUNK_PAD];
   __align__(8) unsigned long long bar[3];  // particle buffers 0, 1; the pressure slab
   unsigned long long empty[2];             // ... the buffers' readers, one arrival per warp
@@ -294,8 +279,8 @@ struct G2pCta {
   unsigned int phase = 0u, inflight = 0u, empty = 0u, used = 0u, kbuf = 0u;
 };
 
-template <bool PAIR, bool ADV>
-__device__ __forceinline__ void g2p_init(G2pShared<PAIR, ADV>& sh) {
+template <bool PAIR>
+__device__ __forceinline__ void g2p_init(G2pShared<PAIR>& sh) {
   if (threadIdx.x == 0) {
     mbar_init(&sh.bar[0], 1);
     mbar_init(&sh.bar[1], 1);
@@ -310,9 +295,9 @@ __device__ __forceinline__ void g2p_init(G2pShared<PAIR, ADV>& sh) {
 
 // Thread 0: particles [q0, q1) into the next buffer, once its readers have left it; false if
 // they have not within the limit.
-template <bool PAIR, bool ADV>
+template <bool PAIR>
 __device__ __forceinline__ bool g2p_issue(const PartView& P, unsigned int q0, unsigned int q1,
-                                          unsigned long long wait_ns, G2pShared<PAIR, ADV>& sh,
+                                          unsigned long long wait_ns, G2pShared<PAIR>& sh,
                                           G2pCta& cs) {
   const unsigned int k = cs.kbuf, bit = 1u << k;
   if (cs.used & bit) {
@@ -328,7 +313,7 @@ __device__ __forceinline__ bool g2p_issue(const PartView& P, unsigned int q0, un
 // One brick of one scene (pmap: the tensor map of the scene's pressure, or
 // nullptr for plain loads).  CTA-uniform; returns false once a wait has given up
 // (DEV_TIMEOUT set in the scene's status), after which the CTA takes no more bricks.
-template <bool PAIR, bool ADV>
+template <bool PAIR>
 __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, const PartView& P,
                                           const BinView& B, const float* __restrict__ uo0,
                                           const float* __restrict__ uo1,
@@ -337,7 +322,7 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
                                           const float2* __restrict__ pff, DevStats* st,
                                           const CUtensorMap* pmap, unsigned int brick,
                                           unsigned int part, unsigned int split,
-                                          G2pShared<PAIR, ADV>& sh, G2pCta& cs, float& speed2) {
+                                          G2pShared<PAIR>& sh, G2pCta& cs, float& speed2) {
   using PT = typename PTile<PAIR>::T;
   const int lane = threadIdx.x & 31;
   const int b0 = (int)(brick % (unsigned)g.bx) * BRICK;
@@ -391,9 +376,9 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
   }
   __syncthreads();
   if (sh.abort) return false;
-  stage_faces<0, PAIR, ADV>(g, K, b0, b1, b2, uo0, sh.sp, sh.sud[0]);
-  stage_faces<1, PAIR, ADV>(g, K, b0, b1, b2, uo1, sh.sp, sh.sud[1]);
-  stage_faces<2, PAIR, ADV>(g, K, b0, b1, b2, uo2, sh.sp, sh.sud[2]);
+  stage_faces<0, PAIR>(g, K, b0, b1, b2, uo0, sh.sp, sh.sud[0]);
+  stage_faces<1, PAIR>(g, K, b0, b1, b2, uo1, sh.sp, sh.sud[1]);
+  stage_faces<2, PAIR>(g, K, b0, b1, b2, uo2, sh.sp, sh.sud[2]);
   __syncthreads();
   // A particle's rank in its new cell is what the histogram's atomic returns, with its place
   // among the warp's lanes of that cell; it is written a chunk later, so that the atomic's
@@ -437,21 +422,19 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
     if (valid) {
       // the particle lies in this brick (its key was taken from the same coordinates); the
       // clamps only keep the shared-memory indices in range
-      const AxisG ax = axis_g(x, g.inv_dx, (float)b0, b0 == 0 ? 1.0f : 0.0f, (float)min(g.nx - b0, 9));
-      const AxisG ay = axis_g(y, g.inv_dx, (float)b1, b1 == 0 ? 1.0f : 0.0f, (float)min(g.ny - b1, 9));
-      const AxisG az = axis_g(z, g.inv_dx, (float)b2, b2 == 0 ? 1.0f : 0.0f, (float)min(g.nz - b2, 9));
-      const NodeV<ADV> ud[3] = {interp_tile<0>(ax, ay, az, sh.sud[0]),
-                                interp_tile<1>(ax, ay, az, sh.sud[1]),
-                                interp_tile<2>(ax, ay, az, sh.sud[2])};
+      const auto axis = [&](float p, int b, int n) {
+        return axis_g(p, g.inv_dx, b, (float)max(b - 1, 0), fminf((float)(n - 1), (float)b + 7.5f));
+      };
+      const AxisG ax = axis(x, b0, g.nx), ay = axis(y, b1, g.ny), az = axis(z, b2, g.nz);
+      const float2 ud[3] = {interp_tile<0>(ax, ay, az, sh.sud[0]),
+                            interp_tile<1>(ax, ay, az, sh.sud[1]),
+                            interp_tile<2>(ax, ay, az, sh.sud[2])};
+      const float r = K.flip_ratio, r1 = 1.0f - K.flip_ratio;
       float vn[3], adv[3];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        if constexpr (ADV) {
-          vn[d] = __fmaf_rn(K.flip_ratio, vp[d], ud[d].x);
-          adv[d] = K.advect_grid ? ud[d].y : vn[d];
-        } else {
-          vn[d] = adv[d] = __fmaf_rn(K.flip_ratio, vp[d], ud[d]);
-        }
+        vn[d] = __fadd_rn(__fmul_rn(r, __fadd_rn(vp[d], ud[d].y)), __fmul_rn(r1, ud[d].x));
+        adv[d] = K.advect_grid ? ud[d].x : vn[d];
       }
       x = fminf(fmaxf(__fmaf_rn(K.dt, adv[0], x), g.skin), g.hi[0]);
       y = fminf(fmaxf(__fmaf_rn(K.dt, adv[1], y), g.skin), g.hi[1]);
@@ -484,8 +467,8 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
 // After an abort, thread 0 drains the copies it issued and nobody waited for
 // (the chunk whose wait gave up, the one issued after it), boundedly; the CTA's
 // shared memory stays allocated until thread 0 leaves.
-template <bool PAIR, bool ADV>
-__device__ __forceinline__ void g2p_drain(G2pShared<PAIR, ADV>& sh, const G2pCta& cs) {
+template <bool PAIR>
+__device__ __forceinline__ void g2p_drain(G2pShared<PAIR>& sh, const G2pCta& cs) {
   if (threadIdx.x == 0)
 #pragma unroll
     for (int k = 0; k < 3; ++k)
@@ -515,12 +498,14 @@ __device__ __forceinline__ unsigned int g2p_split(unsigned int nact, unsigned in
 }
 
 // Bound by latency (the tiles' loads, the histogram's atomics) and by shared-memory accesses:
-// at 256^3 (42.3 M particles, 2.4 GB) the stage takes 0.64 ms of the 0.34 that the bytes do.
-// 0.745 -> 0.728 by weights and cells without conversions and packed interpolation by axes,
-// 0.705 by writing ranks a chunk late, 0.684 without a CTA barrier per chunk (and with the
-// barriers' state in bits, not in a stack array), 0.641 with one value per node, which halves
-// the shared-memory traffic.  6 CTAs per SM instead of 5 spill (0.692).
-template <bool PAIR, bool ADV>
+// at 256^3 (42.3 M particles, 2.4 GB) the stage takes 0.703 ms of the 0.34 that the bytes do.
+// It took 0.745 with conversions to integers in the weights and cells, ranks written in the
+// same chunk, a CTA barrier per chunk, and the barriers' state in a stack array.  One value
+// per node, u_new - r u_old, would give the blend as r v + interp(u_new - r u_old) with half
+// the shared-memory traffic (0.648), but rounds it otherwise than the interpolants of u_new
+// and u_new - u_old: a position's last bit is any change of the velocity of a face that only
+// vanishing weights reach.
+template <bool PAIR>
 __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const StepConsts K0,
                                                      const PartView P, const BinView B,
                                                      const float* __restrict__ uo0,
@@ -531,7 +516,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
                                                      DevStats* st,
                                                      const __grid_constant__ CUtensorMap pmap,
                                                      int use_tma, unsigned int most) {
-  __shared__ G2pShared<PAIR, ADV> sh;
+  __shared__ G2pShared<PAIR> sh;
   const StepConsts K = step_consts(K0);
   const unsigned int nact = st->n_active;
   g2p_init(sh);
@@ -540,7 +525,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
   const CUtensorMap* map = use_tma ? &pmap : nullptr;
   const unsigned int split = g2p_split(nact, gridDim.x, most);
   for (unsigned int bi = blockIdx.x; bi < nact * split; bi += gridDim.x)
-    if (!g2p_brick<PAIR, ADV>(g, K, P, B, uo0, uo1, uo2, p32, pff, st, map, B.active[bi / split],
+    if (!g2p_brick<PAIR>(g, K, P, B, uo0, uo1, uo2, p32, pff, st, map, B.active[bi / split],
                          bi % split, split, sh, cs, speed2))
       break;
   g2p_drain(sh, cs);
@@ -549,11 +534,11 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
 
 // All scenes' active bricks as one list (L.first from k_active_prefix): the CTAs
 // share every scene's bricks evenly.  A CTA that gives up on a wait marks every
-// scene whose bricks it leaves undone.  4 CTAs per SM (5 spill: 16 scenes 3.85 against
-// 3.71 ms per step).
+// scene whose bricks it leaves undone.  4 CTAs per SM (5 spill: 16 scenes 3.65 against
+// 3.62 ms per step).
 template <bool PAIR>
 __global__ void __launch_bounds__(G2P_THREADS, 4) k_g2p_batch(const BatchLaunch L) {
-  __shared__ G2pShared<PAIR, true> sh;
+  __shared__ G2pShared<PAIR> sh;
   g2p_init(sh);
   G2pCta cs;
   float speed2 = 0.0f;
@@ -569,7 +554,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 4) k_g2p_batch(const BatchLaunch 
       if (cur >= 0) g2p_flush_speed(speed2, L.scenes[cur].st);
       cur = s;
     }
-    if (!g2p_brick<PAIR, true>(S.g, step_consts(S.K), S.dst, S.B, S.uo[0], S.uo[1], S.uo[2], S.x32,
+    if (!g2p_brick<PAIR>(S.g, step_consts(S.K), S.dst, S.B, S.uo[0], S.uo[1], S.uo[2], S.x32,
                          S.pff, S.st, nullptr, S.B.active[gb - L.first[s]], q % split, split, sh, cs,
                          speed2))
       break;
@@ -583,7 +568,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 4) k_g2p_batch(const BatchLaunch 
 
 int g2p_blocks(int sm_count) {
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<true, true>, G2P_THREADS, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<true>, G2P_THREADS, 0) !=
           cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
@@ -607,8 +592,7 @@ void launch_g2p(const Grid& g, const StepConsts& k, const PartView& p, const Bin
   std::memset(&none, 0, sizeof(none));
   const CUtensorMap& m = pmap ? *pmap : none;
   const int tma = pmap ? 1 : 0;
-  const auto kernel = pff ? (k.advect_grid ? k_g2p<true, true> : k_g2p<true, false>)
-                          : (k.advect_grid ? k_g2p<false, true> : k_g2p<false, false>);
+  const auto kernel = pff ? k_g2p<true> : k_g2p<false>;
   kernel<<<nblocks, G2P_THREADS, 0, s>>>(g, k, p, b, uo[0], uo[1], uo[2], p32, pff, st, m, tma,
                                           keep_order ? 1u : G2P_MAX_SPLIT);
 }

@@ -66,3 +66,57 @@ def test_faces_that_only_vanishing_weights_reach(cell):
     assert (f > 0).all()
     assert abs(uo[cell + 1] - (f[0] - f[1]) / (f[0] + f[1])) <= 8 * 2.0 ** -24
     assert abs(uo[cell]) <= 1e-4
+
+
+def _axis(x, inv, n):
+    """Float32: (lower node, weight of the upper) on faces and on centres, as P2G weighs a node
+    (csrc/flip_internal.cuh, axis_weights; x/dx is exact in 64 bits, so its floor is the cell)."""
+    cell = np.clip(np.floor(x.astype(np.float64) * inv), 0, n - 1).astype(np.int64)
+    g = x * np.float32(inv)
+    face = np.clip(g - cell.astype(np.float32), np.float32(0), np.float32(1))
+    c = np.clip(g - np.float32(0.5), np.float32(0), np.float32(n - 1))
+    base = np.minimum(np.floor(c).astype(np.int64), n - 2)
+    return (cell, face), (base, c - base.astype(np.float32))
+
+
+def _fma(a, b, c):  # a b is exact in 64 bits
+    return (a.astype(np.float64) * b.astype(np.float64) + c.astype(np.float64)).astype(np.float32)
+
+
+@pytest.mark.parametrize("advect", [F.FLIP_ADVECT_PARTICLE, F.FLIP_ADVECT_GRID])
+@pytest.mark.parametrize("precision", [F.FLIP_PREC_FP32, F.FLIP_PREC_MIXED_IR])
+@pytest.mark.parametrize("n,hi", [
+    ((45, 41, 43), (1.0, 0.85, 1.0)),  # x/dx - 1/2 rounds in every binade but the first brick's
+    ((9, 70, 8), (1.0, 0.5, 1.0)),
+])
+def test_g2p_interpolates_with_p2gs_weights(n, hi, precision, advect):
+    """Velocities and positions bit for bit: the faces that next step's P2G reaches with
+    vanishing weights turn a position's last bit into any change of their velocity."""
+    sc = S.random_velocities(S.box(n, (0.0, 0.0, 0.0), hi, seed=8), 0.5, 9)
+    op, fp = matched(n, cg_tol=1e-7, advect_source=advect)
+    fp.precision = precision
+    with F.Simulation(fp, *sc.arrays()) as sim:
+        sim.step(1)
+        uo = [np.asarray(sim.read(f)) for f in (F.U_OLD, F.V_OLD, F.W_OLD)]
+        un = [np.asarray(sim.read(f)) for f in (F.U_NEW, F.V_NEW, F.W_NEW)]
+        got = sim.particles()
+    pos, vel = sc.arrays()[:3], sc.arrays()[3:]
+    ax = [_axis(pos[a], max(n), n[a]) for a in range(3)]
+    one, r, dt = np.float32(1), np.float32(fp.flip_ratio), np.float32(fp.dt)
+    for d in range(3):
+        dim = [n[a] + (a == d) for a in range(3)]
+        w = [ax[a][0 if a == d else 1] for a in range(3)]
+        U, dU = np.zeros_like(pos[0]), np.zeros_like(pos[0])
+        for q in range(8):  # x fastest
+            o = [(q >> a) & 1 for a in range(3)]
+            k = [w[a][1] if o[a] else one - w[a][1] for a in range(3)]
+            k = k[0] * (k[1] * k[2])
+            # (a node past the grid has weight 0)
+            i = [np.minimum(w[a][0] + o[a], dim[a] - 1) for a in range(3)]
+            i = i[0] + dim[0] * (i[1] + dim[1] * i[2])
+            U, dU = _fma(k, un[d][i], U), _fma(k, un[d][i] - uo[d][i], dU)
+        v = r * (vel[d] + dU) + (one - r) * U
+        x = _fma(np.full_like(v, dt), U if advect == F.FLIP_ADVECT_GRID else v, pos[d])
+        x = np.clip(x, np.float32(fp.skin), np.float32(n[d] * fp.dx - fp.skin))
+        assert np.array_equal(got[3 + d], v), d
+        assert np.array_equal(got[d], x), d
