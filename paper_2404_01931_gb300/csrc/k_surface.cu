@@ -435,6 +435,11 @@ constexpr int SDF_THREADS = 256;
 constexpr int SDF_WARPS = SDF_THREADS / 32;
 constexpr int SDF_ROW_LANES = 8;
 constexpr int SDF_ROWS = 49;
+// A corner whose sum of weights is below this is summed again with the ball's edge taken
+// exactly.  A particle at distance R or more has a rounded 1 - d^2 / R^2 of up to 2^-23, a
+// weight of 2^-69: nothing beside this sum, but all there is at a corner that no particle is
+// closer to than R.
+constexpr float SDF_THIN = 0x1p-30f;
 
 template <int GY, int GZ>
 __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins B,
@@ -521,7 +526,8 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
             const int q = y + GY * z;
             const float e1 = y ? ey.y : ey.x;
             const float w = __fmaf_rn(e1, y ? fy.y : fy.x, z ? wz.y : wz.x);
-            // k = max(0, 1 - d^2 / R^2)^3 (saturating: d^2 >= 0); at d = R the terms vanish
+            // k = max(0, 1 - d^2 / R^2)^3 (saturating: d^2 >= 0), at d >= R to rounding
+            // (SDF_THIN)
             const float2 t = make_float2(__saturatef(__fmaf_rn(ex.x, fx.x, w)),
                                          __saturatef(__fmaf_rn(ex.y, fx.y, w)));
             const float2 kk = __fmul2_rn(__fmul2_rn(t, t), t);
@@ -562,12 +568,42 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
     float s = v[0];
 #pragma unroll
     for (int n = NV; n < 32; n <<= 1) s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, n));
-    const float a = __shfl_sync(0xffffffffu, s, 4 * lane);  // lane c < corners: corner c's sums
-    const float b0 = __shfl_sync(0xffffffffu, s, 4 * lane + 1);
-    const float b1 = __shfl_sync(0xffffffffu, s, 4 * lane + 2);
-    const float b2 = __shfl_sync(0xffffffffu, s, 4 * lane + 3);
+    float a = __shfl_sync(0xffffffffu, s, 4 * lane);  // lane c < corners: corner c's sums
+    float b0 = __shfl_sync(0xffffffffu, s, 4 * lane + 1);
+    float b1 = __shfl_sync(0xffffffffu, s, 4 * lane + 2);
+    float b2 = __shfl_sync(0xffffffffu, s, 4 * lane + 3);
     const int i = i0 + (lane & 1), j = j0 + (lane >> 1) % GY, k = k0 + (lane >> 1) / GY;
-    if (lane < 2 * NP && i < g.c[0] && j < g.c[1] && k < g.c[2]) {
+    const bool in = lane < 2 * NP && i < g.c[0] && j < g.c[1] && k < g.c[2];
+    // (few: no measurable time)
+    for (unsigned int thin = __ballot_sync(0xffffffffu, in && a > 0.0f && a < SDF_THIN); thin;
+         thin &= thin - 1u) {
+      const int c = __ffs(thin) - 1;
+      const float cx = c & 1 ? x1 : x0, cy = (c >> 1) % GY ? y1 : y0, cz = (c >> 1) / GY ? z1 : z0;
+      float w = 0.0f, wx = 0.0f, wy = 0.0f, wz = 0.0f;
+      for (int r = lane / SDF_ROW_LANES; r < nrow; r += 32 / SDF_ROW_LANES) {
+        const uint2 row = s_row[wid][r];
+        for (unsigned int f = row.x + lane % SDF_ROW_LANES; f < row.y; f += SDF_ROW_LANES) {
+          const float4 P = pos[f];
+          const float ex = P.x - cx, ey = P.y - cy, ez = P.z - cz;
+          const float dd = __fmaf_rn(ex, ex, __fmaf_rn(ez, ez, __fmul_rn(ey, ey)));
+          const float t = dd < B.R2 ? fmaxf(__fmaf_rn(dd, -B.inv_R2, 1.0f), 0.0f) : 0.0f;
+          const float kk = t * t * t;
+          w += kk;
+          wx = __fmaf_rn(kk, ex, wx);
+          wy = __fmaf_rn(kk, ey, wy);
+          wz = __fmaf_rn(kk, ez, wz);
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        w += __shfl_xor_sync(0xffffffffu, w, o);
+        wx += __shfl_xor_sync(0xffffffffu, wx, o);
+        wy += __shfl_xor_sync(0xffffffffu, wy, o);
+        wz += __shfl_xor_sync(0xffffffffu, wz, o);
+      }
+      if (lane == c) a = w, b0 = wx, b1 = wy, b2 = wz;
+    }
+    if (in) {
       const float d = (a > 0.0f) ? sqrtf(b0 * b0 + b1 * b1 + b2 * b2) / a - B.r : B.R - B.r;
       phi[i + (long long)g.c[0] * (j + (long long)g.c[1] * k)] = d;
     }

@@ -56,3 +56,23 @@ def test_mesh_walks_any_grid_shape(n):
     nv, nt, got = _gpu_mesh(sp, phi)
     assert nv > 1000 and nt > 1000
     assert np.array_equal(got["e"], ref.vertex_edge) and np.array_equal(got["t"], ref.triangles)
+
+
+@pytest.mark.parametrize("n", [10, 24, 48, 101])
+@pytest.mark.parametrize("ratio", [2.0, 1.9])  # 2 x 2 x 1 corners (n < 48) or 2 x 2 x 2; pairs
+@pytest.mark.parametrize("dirs", [((0, 1), (0, -1)), ((1, 1), (1, -1)), ((2, 1), (2, -1)),
+                                  ((0, 1), (1, 1)), ((2, -1), (1, 1)),
+                                  tuple((a, s) for a in range(3) for s in (-1, 1))])
+def test_particles_at_exactly_the_search_radius_do_not_count(n, ratio, dirs):
+    """Corner 0 lies at (R, R, R), the particles R from it on its axes: the coordinates 0, R
+    and 2 R and their differences are exact, so no particle is closer than R."""
+    R = np.float32(2 / n)
+    pos = np.full((3, len(dirs)), R, np.float32)
+    for q, (a, s) in enumerate(dirs):
+        pos[a, q] = R + np.float32(s) * R
+    sp = _sp((n, n, n), float(R) / ratio, origin=(float(R),) * 3, r=0.25 * float(R), R=float(R))
+    zero = np.zeros(len(dirs), np.float32)
+    with F.Simulation(matched(n)[1], *pos, zero, zero, zero) as sim, F.Surface(sp) as s:
+        s.sdf(sim)
+        phi = s.read(F.SURF_FIELD).reshape(n + 1, n + 1, n + 1)
+    assert phi[0, 0, 0] == R - np.float32(0.25) * R
