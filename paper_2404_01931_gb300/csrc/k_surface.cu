@@ -410,16 +410,16 @@ __global__ void k_sbin_scatter(const PartView p, long long np, const int* __rest
   pos[start[b] + prank[i]] = make_float4(p.x[i], p.y[i], p.z[i], 0.0f);
 }
 
-// One warp per group of 2 x GY x GZ corners (2 x 2 x 2 where the corners are no farther apart
-// than a bin, else 2 x 1 x 1).  With bins of edge R/2 the balls' extent along y or z is at most
-// 5.001 bins, which meets at most 7 (corners on bin faces, with roundings either way), so at
-// most 49 bin rows (fixed y, z bin): lane r finds the particle ranges of rows r and r + 32 (a row's bins within the balls' x extent are one contiguous range; a bin
-// whose nearest point is R or farther from the corners holds no particle closer than R and is
-// skipped), the nonempty rows are packed into a per-warp list, and the warp's four groups of
-// eight lanes take a row each, eight particles (128 bytes) at a time.  Each particle is tested
-// against all the group's corners, whose sums stay in registers until a reduction that halves
-// the values with every step.  The eight warps of a CTA take neighbouring groups (4 x 4 x 4
-// corners), so that most of a CTA's particle reads hit L1.
+// One warp per group of 2 PX x GY x GZ corners (sdf_kernel has the lines between them).  With
+// bins of edge R/2 the balls' extent along y or z is at most 5.98 bins, which meets at most 7
+// (8 with roundings), so at most 64 bin rows (fixed y, z bin): lane r finds the particle
+// ranges of rows r and r + 32 (a row's bins within the balls' x extent are one contiguous
+// range; a bin whose nearest point is R or farther from the corners holds no particle closer
+// than R and is skipped), the nonempty rows are packed into a per-warp list, and the warp's
+// four groups of eight lanes take a row each, eight particles (128 bytes) at a time.  Each
+// particle is tested against all the group's corners, whose sums stay in registers until a
+// reduction that halves the values with every step.  The eight warps of a CTA take
+// neighbouring groups (2 x 2 x 2 of them), so that most of a CTA's particle reads hit L1.
 //
 // With e the offset particle minus corner, 1 - |e|^2 / R^2 is taken axis by axis: the two
 // values of 1 - ez^2 / R^2 and the four with y are shared by the corners, so that a corner's
@@ -434,20 +434,20 @@ __global__ void k_sbin_scatter(const PartView p, long long np, const int* __rest
 constexpr int SDF_THREADS = 256;
 constexpr int SDF_WARPS = SDF_THREADS / 32;
 constexpr int SDF_ROW_LANES = 8;
-constexpr int SDF_ROWS = 49;
+constexpr int SDF_ROWS = 64;
 // A corner whose sum of weights is below this is summed again with the ball's edge taken
 // exactly.  A particle at distance R or more has a rounded 1 - d^2 / R^2 of up to 2^-23, a
 // weight of 2^-69: nothing beside this sum, but all there is at a corner that no particle is
 // closer to than R.
 constexpr float SDF_THIN = 0x1p-30f;
 
-template <int GY, int GZ>
+template <int PX, int GY, int GZ>
 __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins B,
                                                      const unsigned int* __restrict__ start,
                                                      const float4* __restrict__ pos,
                                                      float* __restrict__ phi) {
-  constexpr int GX = 2, NP = GY * GZ;  // pairs along x
-  static_assert((GY == 1 || GY == 2) && (GZ == 1 || GZ == 2), "offsets in pairs");
+  constexpr int GX = 2 * PX, NP = PX * GY * GZ;  // pairs along x
+  static_assert((GY == 1 || GY == 2) && (GZ == 1 || GZ == 2) && NP <= 4, "offsets in pairs");
   __shared__ uint2 s_row[SDF_WARPS][SDF_ROWS];  // {first particle, end} of the nonempty rows
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   // a CTA's groups: 2 x 2 x 2
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
     const int j0 = (int)((tile / tx) % ty) * CY + ((wid >> 1) & 1) * GY;
     const int k0 = (int)(tile / ((long long)tx * ty)) * CZ + (wid >> 2) * GZ;
     if (i0 >= g.c[0] || j0 >= g.c[1] || k0 >= g.c[2]) continue;
-    const float x0 = g.o[0] + g.h * (float)i0, x1 = g.o[0] + g.h * (float)(i0 + 1);
+    const float x0 = g.o[0] + g.h * (float)i0, x1 = g.o[0] + g.h * (float)(i0 + GX - 1);
     const float y0 = g.o[1] + g.h * (float)j0, y1 = g.o[1] + g.h * (float)(j0 + GY - 1);
     const float z0 = g.o[2] + g.h * (float)k0, z1 = g.o[2] + g.h * (float)(k0 + GZ - 1);
     const float ry0 = (y0 - B.o[1]) * B.inv_b, ry1 = (y1 - B.o[1]) * B.inv_b;
@@ -498,10 +498,14 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
     __syncwarp();
     // minus the corners' coordinates (P.x + (-x) rounds as P.x - x); packed operations round
     // like the scalar ones
-    const float2 mx = make_float2(-x0, -x1), my = make_float2(-y0, -y1),
-                 mz = make_float2(-z0, -z1);
+    float2 mx[PX];
+#pragma unroll
+    for (int p = 0; p < PX; ++p)
+      mx[p] = make_float2(-(g.o[0] + g.h * (float)(i0 + 2 * p)),
+                          -(g.o[0] + g.h * (float)(i0 + 2 * p + 1)));
+    const float2 my = make_float2(-y0, -y1), mz = make_float2(-z0, -z1);
     const float2 nr = make_float2(-B.inv_R2, -B.inv_R2);
-    // per corner: sum k and sum k e; corners (0, y, z) and (1, y, z) are the two lanes
+    // per corner: sum k and sum k e; corners (2 p, y, z) and (2 p + 1, y, z) are the two lanes
     float2 sk[NP], sx[NP], sy[NP], sz[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) sk[q] = sx[q] = sy[q] = sz[q] = make_float2(0.0f, 0.0f);
@@ -513,28 +517,36 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
       for (; f < row.y; f += SDF_ROW_LANES) {
         const float4 P = next;  // the next particle's load is in flight during this one's sums
         if (f + SDF_ROW_LANES < row.y) next = pos[f + SDF_ROW_LANES];
-        const float2 ex = __fadd2_rn(make_float2(P.x, P.x), mx);
         const float2 ey = __fadd2_rn(make_float2(P.y, P.y), my);
         const float2 ez = __fadd2_rn(make_float2(P.z, P.z), mz);
-        const float2 fx = __fmul2_rn(ex, nr), fy = __fmul2_rn(ey, nr);
+        const float2 fy = __fmul2_rn(ey, nr);
+        float2 ex[PX], fx[PX];
+#pragma unroll
+        for (int p = 0; p < PX; ++p) {
+          ex[p] = __fadd2_rn(make_float2(P.x, P.x), mx[p]);
+          fx[p] = __fmul2_rn(ex[p], nr);
+        }
         const float2 wz = __ffma2_rn(ez, __fmul2_rn(ez, nr), make_float2(1.0f, 1.0f));
 #pragma unroll
         for (int z = 0; z < GZ; ++z) {
           const float e2 = z ? ez.y : ez.x;
 #pragma unroll
           for (int y = 0; y < GY; ++y) {
-            const int q = y + GY * z;
             const float e1 = y ? ey.y : ey.x;
             const float w = __fmaf_rn(e1, y ? fy.y : fy.x, z ? wz.y : wz.x);
-            // k = max(0, 1 - d^2 / R^2)^3 (saturating: d^2 >= 0), at d >= R to rounding
-            // (SDF_THIN)
-            const float2 t = make_float2(__saturatef(__fmaf_rn(ex.x, fx.x, w)),
-                                         __saturatef(__fmaf_rn(ex.y, fx.y, w)));
-            const float2 kk = __fmul2_rn(__fmul2_rn(t, t), t);
-            sk[q] = __fadd2_rn(sk[q], kk);
-            sx[q] = __ffma2_rn(kk, ex, sx[q]);
-            sy[q] = __ffma2_rn(kk, make_float2(e1, e1), sy[q]);
-            sz[q] = __ffma2_rn(kk, make_float2(e2, e2), sz[q]);
+#pragma unroll
+            for (int p = 0; p < PX; ++p) {
+              const int q = p + PX * (y + GY * z);
+              // k = max(0, 1 - d^2 / R^2)^3 (saturating: d^2 >= 0), at d >= R to rounding
+              // (SDF_THIN)
+              const float2 t = make_float2(__saturatef(__fmaf_rn(ex[p].x, fx[p].x, w)),
+                                           __saturatef(__fmaf_rn(ex[p].y, fx[p].y, w)));
+              const float2 kk = __fmul2_rn(__fmul2_rn(t, t), t);
+              sk[q] = __fadd2_rn(sk[q], kk);
+              sx[q] = __ffma2_rn(kk, ex[p], sx[q]);
+              sy[q] = __ffma2_rn(kk, make_float2(e1, e1), sy[q]);
+              sz[q] = __ffma2_rn(kk, make_float2(e2, e2), sz[q]);
+            }
           }
         }
       }
@@ -572,13 +584,15 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
     float b0 = __shfl_sync(0xffffffffu, s, 4 * lane + 1);
     float b1 = __shfl_sync(0xffffffffu, s, 4 * lane + 2);
     float b2 = __shfl_sync(0xffffffffu, s, 4 * lane + 3);
-    const int i = i0 + (lane & 1), j = j0 + (lane >> 1) % GY, k = k0 + (lane >> 1) / GY;
+    const int i = i0 + lane % GX, j = j0 + lane / GX % GY, k = k0 + lane / (GX * GY);
     const bool in = lane < 2 * NP && i < g.c[0] && j < g.c[1] && k < g.c[2];
     // (few: no measurable time)
     for (unsigned int thin = __ballot_sync(0xffffffffu, in && a > 0.0f && a < SDF_THIN); thin;
          thin &= thin - 1u) {
       const int c = __ffs(thin) - 1;
-      const float cx = c & 1 ? x1 : x0, cy = (c >> 1) % GY ? y1 : y0, cz = (c >> 1) / GY ? z1 : z0;
+      float2 m = mx[0];
+      if (PX > 1 && c % GX >= 2) m = mx[PX - 1];
+      const float cx = -(c & 1 ? m.y : m.x), cy = c / GX % GY ? y1 : y0, cz = c / (GX * GY) ? z1 : z0;
       float w = 0.0f, wx = 0.0f, wy = 0.0f, wz = 0.0f;
       for (int r = lane / SDF_ROW_LANES; r < nrow; r += 32 / SDF_ROW_LANES) {
         const uint2 row = s_row[wid][r];
@@ -610,8 +624,12 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
   }
 }
 
-// The corners of a 2 x 2 x 2 group share most of their bins while h is at most a bin edge
-// (R >= 2 h), and its rows fit a warp's list (7 x 7); wider grids take pairs along x (6 x 6).
+// 2 x 2 x 2 corners share most of their bins and, up to corners 1.98 bins apart (R a little
+// over h), their rows fit a warp's list; wider grids take 4 x 1 x 1, whose rows do not grow
+// with h.  A 128^3 pool at R = 1.9, 1.4, 1.05 and 0.9, 0.7 and 0.5 h: 658, 530, 547 us and
+// 617, 762, 1293; with 2 x 1 x 1 from R < 2 h on 1063, 823, 802 and 835, 999, 1515; with
+// lanes that walk one flat range over the rows of 4 corners along x 962, 699, 653 and 701,
+// 871, 1488.
 // A grid of few groups takes 2 x 2 x 1 ones, twice as many, to even out the chip's last
 // rounds: flip_surface_sdf with 7 thousand groups (48 x 33 x 33 cells, 4 scenes) 58-69 us
 // with 2 x 2 x 2, 59-66 with 2 x 2 x 1; with 11 thousand 63-81 and 64-72; with 26 thousand
@@ -621,9 +639,9 @@ using SdfKernel = void (*)(const SGrid, const SBins, const unsigned int*, const 
 constexpr long long SDF_FEW = 4 * 152 * 3 * SDF_WARPS;  // four rounds of resident warps
 
 SdfKernel sdf_kernel(const SGrid& g, const SBins& B) {
-  if (g.h > 1.001f * B.b) return k_sdf<1, 1>;
+  if (g.h > 1.98f * B.b) return k_sdf<2, 1, 1>;
   const long long groups = (long long)((g.c[0] + 1) / 2) * ((g.c[1] + 1) / 2) * ((g.c[2] + 1) / 2);
-  return groups >= SDF_FEW ? k_sdf<2, 2> : k_sdf<2, 1>;
+  return groups >= SDF_FEW ? k_sdf<1, 2, 2> : k_sdf<1, 2, 1>;
 }
 
 int sdf_blocks(SdfKernel k) {

@@ -76,3 +76,47 @@ def test_particles_at_exactly_the_search_radius_do_not_count(n, ratio, dirs):
         s.sdf(sim)
         phi = s.read(F.SURF_FIELD).reshape(n + 1, n + 1, n + 1)
     assert phi[0, 0, 0] == R - np.float32(0.25) * R
+
+
+@pytest.mark.parametrize("n,h,ratio", [
+    ((60, 52, 57), 1 / 50, 1.9),     # corners over a bin apart, many and few groups
+    ((26, 20, 23), 1 / 50, 1.6),
+    ((56, 49, 51), 1 / 50, 1.02),    # just inside the line: seven bin rows each way
+    ((56, 49, 51), 1 / 50, 1.0),     # past it: four corners along x
+    ((14, 9, 11), 1 / 12, 0.7),      # ... with balls that do not meet, a row's rest of three
+])
+def test_sdf_forms_match_the_oracle_within_each_corners_conditioning(n, h, ratio):
+    check_sdf(n, h, ratio)
+
+
+def check_sdf(n, h, ratio):
+    """The bar of the tests above, and beyond it what the roundings of t = 1 - d^2 / R^2 can
+    change at a corner: phi + r = |sum k e| / sum k, k = t^3, moves by at most
+    2 R sum dk / sum k (|e - mean| <= 2 R), dk = (t + eps)^3 - t^3.  eps: five roundings to
+    within 2^-25 of t's terms (below 2^-22 in all), and the corner's coordinates, within 2^-23
+    of their size.  Only a corner with no particle well inside its ball needs it."""
+    sc = S.random_velocities(S.water_drop(24, centre=(0.4, 0.45, 0.3), radius=0.25), 0.1, 3)
+    sp = F.FlipSurfaceParams()
+    for a in range(3):
+        sp.n[a] = n[a]
+        sp.origin[a] = (-0.01, 0.003, 0.02)[a]
+    sp.h, sp.search_radius = h, ratio * h
+    sp.radius, sp.iso = 0.25 * sp.search_radius, 0.0
+    R = sp.search_radius
+    with F.Simulation(matched(24)[1], *sc.arrays()) as sim, F.Surface(sp) as s:
+        s.sdf(sim)
+        phi = s.read(F.SURF_FIELD).astype(np.float64).reshape(n[2] + 1, n[1] + 1, n[0] + 1)
+    ref = O.sdf(sc.x, sc.y, sc.z, tuple(sp.n), tuple(sp.origin), sp.h, sp.radius, R)
+    assert (ref < 0).any() and (ref == R - sp.radius).any()
+    assert phi.min() >= -sp.radius * (1 + 1e-6) and phi.max() <= (R - sp.radius) * (1 + 1e-6)
+    err = np.abs(phi - ref)
+    far = np.argwhere(err > 2e-5 * R)
+    assert len(far) <= 1e-4 * err.size
+    eps = 2.0 ** -22 + 2 * 2.0 ** -23 * (0.02 + max(n) * h) / R
+    p = np.stack([sc.x, sc.y, sc.z]).astype(np.float64)
+    for k, j, i in far:
+        e = p - (np.array([i, j, k]) * h + np.array(sp.origin))[:, None]
+        t = 1 - (e * e).sum(0) / R ** 2
+        t = t[t > -eps].clip(0)
+        dk = ((t + eps) ** 3 - t ** 3).sum() / max((t ** 3).sum(), 1e-300)
+        assert err[k, j, i] <= 2e-5 * R + 2 * R * dk, (i, j, k)
