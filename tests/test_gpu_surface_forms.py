@@ -89,6 +89,16 @@ def test_sdf_forms_match_the_oracle_within_each_corners_conditioning(n, h, ratio
     check_sdf(n, h, ratio)
 
 
+@pytest.mark.parametrize("n,h,ratio", [
+    ((47, 59, 51), 1 / 60, 3.1),     # bins wider than a cell, corners between bin faces
+    ((63, 50, 55), 1 / 64, 2.7),
+    ((52, 50, 53), 1 / 55, 6.5),     # corners far closer than a bin
+])
+def test_sdf_of_many_corners_matches_the_oracle_at_other_radii(n, h, ratio):
+    """Grids of 15 thousand groups and more, which take 2 x 2 x 2 corners a warp."""
+    check_sdf(n, h, ratio)
+
+
 def check_sdf(n, h, ratio):
     """The bar of the tests above, and beyond it what the roundings of t = 1 - d^2 / R^2 can
     change at a corner: phi + r = |sum k e| / sum k, k = t^3, moves by at most
