@@ -313,7 +313,7 @@ __device__ __forceinline__ bool g2p_issue(const PartView& P, unsigned int q0, un
 // One brick of one scene (pmap: the tensor map of the scene's pressure, or
 // nullptr for plain loads).  CTA-uniform; returns false once a wait has given up
 // (DEV_TIMEOUT set in the scene's status), after which the CTA takes no more bricks.
-template <bool PAIR>
+template <bool PAIR, bool ORDERED>
 __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, const PartView& P,
                                           const BinView& B, const float* __restrict__ uo0,
                                           const float* __restrict__ uo1,
@@ -391,7 +391,8 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
     rank_q = ~0u;
   };
   // chunk loop: warp-uniform trip count, so every lane takes part in the key match; the warps
-  // run apart by up to the buffers' depth
+  // run apart by up to the buffers' depth, or (ORDERED) meet after every chunk, so that a
+  // chunk's atomics come before the next one's
   for (unsigned int c0 = bstart; c0 < bend; c0 += G2P_THREADS) {
     const unsigned int cur = cs.kbuf;
     cs.kbuf ^= 1u;
@@ -409,7 +410,10 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
       atomicOr(&st->status, DEV_TIMEOUT);
       sh.abort = 1;
     }
-    if (!__all_sync(0xffffffffu, ok)) break;
+    if (!__all_sync(0xffffffffu, ok)) {
+      if (ORDERED) (void)__syncthreads_or(1);  // the others meet there, and leave too
+      break;
+    }
     const float(*pb)[G2P_CHUNK_PAD] = sh.pbuf[cur];
     const unsigned int q = c0 + threadIdx.x;
     const bool valid = q < bend;
@@ -458,6 +462,7 @@ __device__ __forceinline__ bool g2p_brick(const Grid& g, const StepConsts& K, co
     rank_lead = leader;
     rank_ofs = (unsigned)__popc(same & ((1u << lane) - 1u));
     rank_q = valid ? q : ~0u;
+    if (ORDERED && __syncthreads_or(0)) break;
   }
   put_ranks();
   __syncthreads();
@@ -488,12 +493,12 @@ __device__ __forceinline__ void g2p_flush_speed(float& speed2, DevStats* st) {
 
 // Parts per brick: a brick's chunks are a serial chain, so few bricks are shared out over the
 // launch's CTAs, each staging the tiles for itself.  The stage at 16 bricks (32^3 dam break)
-// 37 -> 16 us, at 150 (64^3) 42 -> 25.  Not with reseeding (most = 1): the parts would take
-// their ranks in no order, and which of a crowded cell's particles are dropped depends on it.
-__device__ __forceinline__ unsigned int g2p_split(unsigned int nact, unsigned int ctas,
-                                                  unsigned int most) {
+// 37 -> 16 us, at 150 (64^3) 42 -> 25.  Not with reseeding (ORDERED), where the ranks decide
+// which of a crowded cell's particles are dropped: a brick's particles then take theirs in the
+// order of its chunks, on one CTA that meets after every chunk.
+__device__ __forceinline__ unsigned int g2p_split(unsigned int nact, unsigned int ctas) {
   unsigned int split = 1;
-  while (split < most && nact * 2u * split <= ctas) split *= 2;
+  while (split < G2P_MAX_SPLIT && nact * 2u * split <= ctas) split *= 2;
   return split;
 }
 
@@ -505,7 +510,7 @@ __device__ __forceinline__ unsigned int g2p_split(unsigned int nact, unsigned in
 // the shared-memory traffic (0.648), but rounds it otherwise than the interpolants of u_new
 // and u_new - u_old: a position's last bit is any change of the velocity of a face that only
 // vanishing weights reach.
-template <bool PAIR>
+template <bool PAIR, bool ORDERED>
 __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const StepConsts K0,
                                                      const PartView P, const BinView B,
                                                      const float* __restrict__ uo0,
@@ -515,7 +520,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
                                                      const float2* __restrict__ pff,
                                                      DevStats* st,
                                                      const __grid_constant__ CUtensorMap pmap,
-                                                     int use_tma, unsigned int most) {
+                                                     int use_tma) {
   __shared__ G2pShared<PAIR> sh;
   const StepConsts K = step_consts(K0);
   const unsigned int nact = st->n_active;
@@ -523,9 +528,9 @@ __global__ void __launch_bounds__(G2P_THREADS, 5) k_g2p(const Grid g, const Step
   G2pCta cs;
   float speed2 = 0.0f;
   const CUtensorMap* map = use_tma ? &pmap : nullptr;
-  const unsigned int split = g2p_split(nact, gridDim.x, most);
+  const unsigned int split = ORDERED ? 1u : g2p_split(nact, gridDim.x);
   for (unsigned int bi = blockIdx.x; bi < nact * split; bi += gridDim.x)
-    if (!g2p_brick<PAIR>(g, K, P, B, uo0, uo1, uo2, p32, pff, st, map, B.active[bi / split],
+    if (!g2p_brick<PAIR, ORDERED>(g, K, P, B, uo0, uo1, uo2, p32, pff, st, map, B.active[bi / split],
                          bi % split, split, sh, cs, speed2))
       break;
   g2p_drain(sh, cs);
@@ -544,7 +549,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 4) k_g2p_batch(const BatchLaunch 
   float speed2 = 0.0f;
   int cur = -1;
   const unsigned int g0 = L.first[0], g1 = L.first[L.n];
-  const unsigned int split = g2p_split(g1 - g0, gridDim.x, G2P_MAX_SPLIT), n = (g1 - g0) * split;
+  const unsigned int split = g2p_split(g1 - g0, gridDim.x), n = (g1 - g0) * split;
   unsigned int q = blockIdx.x;
   for (; q < n; q += gridDim.x) {
     const unsigned int gb = g0 + q / split;
@@ -554,7 +559,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 4) k_g2p_batch(const BatchLaunch 
       if (cur >= 0) g2p_flush_speed(speed2, L.scenes[cur].st);
       cur = s;
     }
-    if (!g2p_brick<PAIR>(S.g, step_consts(S.K), S.dst, S.B, S.uo[0], S.uo[1], S.uo[2], S.x32,
+    if (!g2p_brick<PAIR, false>(S.g, step_consts(S.K), S.dst, S.B, S.uo[0], S.uo[1], S.uo[2], S.x32,
                          S.pff, S.st, nullptr, S.B.active[gb - L.first[s]], q % split, split, sh, cs,
                          speed2))
       break;
@@ -568,7 +573,7 @@ __global__ void __launch_bounds__(G2P_THREADS, 4) k_g2p_batch(const BatchLaunch 
 
 int g2p_blocks(int sm_count) {
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<true>, G2P_THREADS, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<true, false>, G2P_THREADS, 0) !=
           cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
@@ -592,9 +597,9 @@ void launch_g2p(const Grid& g, const StepConsts& k, const PartView& p, const Bin
   std::memset(&none, 0, sizeof(none));
   const CUtensorMap& m = pmap ? *pmap : none;
   const int tma = pmap ? 1 : 0;
-  const auto kernel = pff ? k_g2p<true> : k_g2p<false>;
-  kernel<<<nblocks, G2P_THREADS, 0, s>>>(g, k, p, b, uo[0], uo[1], uo[2], p32, pff, st, m, tma,
-                                          keep_order ? 1u : G2P_MAX_SPLIT);
+  const auto kernel = pff ? (keep_order ? k_g2p<true, true> : k_g2p<true, false>)
+                          : (keep_order ? k_g2p<false, true> : k_g2p<false, false>);
+  kernel<<<nblocks, G2P_THREADS, 0, s>>>(g, k, p, b, uo[0], uo[1], uo[2], p32, pff, st, m, tma);
 }
 
 bool encode_pressure_map(const Grid& g, void* base, bool pair, CUtensorMap* out) {

@@ -120,3 +120,39 @@ def test_g2p_interpolates_with_p2gs_weights(n, hi, precision, advect):
         x = np.clip(x, np.float32(fp.skin), np.float32(n[d] * fp.dx - fp.skin))
         assert np.array_equal(got[3 + d], v), d
         assert np.array_equal(got[d], x), d
+
+
+def test_reseeding_drops_by_the_order_of_a_bricks_chunks():
+    """In each of 512 bricks, eight cells with two chunks of 256 particles each move half a
+    cell along every axis into one cell that may keep 512: those whose chunks come first."""
+    n, m = 64, 512
+    rng = np.random.default_rng(5)
+    b, c = np.divmod(np.repeat(np.arange((n // 8) ** 3 * 8), m), 8)
+    org = [8 * (b % 8), 8 * (b // 8 % 8), 8 * (b // 64)]
+    # cell 3's upper half or cell 4's lower one
+    pos = [((org[a] + np.where((c >> a) & 1, 4.05, 3.55) + 0.4 * rng.random(c.size)) / n)
+           .astype(np.float32) for a in range(3)]
+    vel = [np.full(c.size, 0.5 / n * 240, np.float32)] * 3
+    op, fp = matched(n, gravity=(0.0, 0.0, 0.0))
+    fp.ppc_min, fp.ppc_max = 1, m
+    with F.Simulation(fp, *pos, *vel) as sim:
+        sim.step(1)
+        stored = np.asarray(sim.read(F.PID)).reshape(-1, 8 * m)  # a brick a row
+        sim.step(1)
+        kept = np.asarray(sim.read(F.PID)).reshape(-1, m)
+    assert np.array_equal(np.sort(kept, axis=1), np.sort(stored[:, :m], axis=1))
+
+
+def test_reseeding_step_ends_when_waits_give_up():
+    """The warps of G2P meet after every chunk with reseeding; a limit of 1 ns on its copies'
+    waits makes them leave in different places, and the step returns FLIP_E_TIMEOUT."""
+    sc = S.dam_break(32)
+    op, fp = matched(32)
+    fp.ppc_min, fp.ppc_max = 3, 12
+    with F.Simulation(fp, *sc.arrays()) as sim:
+        sim.set_wait_timeout(1)
+        with pytest.raises(F.FlipError) as ei:
+            sim.step(1, stats=True)
+        assert ei.value.code == F.FLIP_E_TIMEOUT
+    with F.Simulation(fp, *sc.arrays()) as sim:  # the device is as usable as before
+        assert sim.step(1, stats=True)[0] == F.FLIP_OK
