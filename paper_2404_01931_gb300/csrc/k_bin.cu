@@ -296,6 +296,9 @@ __device__ __forceinline__ void scatter(const PartView& src, const PartView& dst
   const int id = src.id[i];
   if (r >= rank_max) return;
   const unsigned int d = b.brick_start[key / BRICK_CELLS] + b.local_start[key] + r;
+  // a step that timed out leaves keys and ranks that its counts do not hold (and offsets of
+  // bricks that these call empty): their slots may lie past the particles
+  if (d >= np) return;
   dst.x[d] = x;
   dst.y[d] = y;
   dst.z[d] = z;
