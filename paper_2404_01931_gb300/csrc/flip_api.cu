@@ -382,7 +382,8 @@ void carve(flip_handle* h, Carver& cv) {
     h->acc[d] = cv.take<float2>((size_t)h->nf[d]);
     h->uo[d] = cv.take<float>((size_t)h->nf[d]);
   }
-  h->x32 = cv.take<float>(nc);
+  // (the mixed multigrid solve keeps its FP32 vectors in the level-0 layout)
+  if (!h->mixed || h->prm.preconditioner == FLIP_PRECOND_JACOBI) h->x32 = cv.take<float>(nc);
   if (h->mixed) {
     h->b64 = cv.take<double>(nc);
     h->x64 = cv.take<double>(nc);
@@ -391,8 +392,20 @@ void carve(flip_handle* h, Carver& cv) {
     h->b32 = cv.take<float>(nc);
   }
   h->partials = cv.take<double>((size_t)PCG_SLOTS * (size_t)h->pcg_blocks);
+  const size_t nfmax = (size_t)std::max(h->nf[0], std::max(h->nf[1], h->nf[2]));
+  h->tmp_bytes = std::max(nfmax * sizeof(float), nc * sizeof(double));
+  h->tmp = cv.take<char>(h->tmp_bytes);
   if (h->prm.preconditioner != FLIP_PRECOND_JACOBI) {
     MgArgs& m = h->mg;
+    const bool blocked = h->prm.preconditioner == FLIP_PRECOND_MG && m.nu <= MG_BLK_MAX_NU;
+    // memory that holds nothing during a solve: the reads' staging buffer, else its own
+    size_t used = 0;
+    auto idle = [&](size_t bytes) -> char* {
+      const size_t at = (used + 255) & ~(size_t)255;
+      if (at + bytes > h->tmp_bytes) return cv.take<char>(bytes);
+      used = at + bytes;
+      return (char*)h->tmp + at;
+    };
     for (int l = 0; l < m.nlev; ++l) {
       MgLevel& L = m.lv[l];
       const size_t n = (size_t)L.ncells;
@@ -405,14 +418,15 @@ void carve(flip_handle* h, Carver& cv) {
         L.segmask = cv.take<unsigned int>((size_t)L.nby * L.nbz);
         const size_t blocks = (size_t)L.nbx * L.nby * L.nbz;
         L.blk = cv.take<int>(blocks);
-        // 1024 threads per block, as many blocks as a blocked level can have
-        L.tab = cv.take<uint2>(
-            1024 * std::min(blocks, (size_t)MG_BLK_PER_CTA * (size_t)h->pcg_blocks));
+        if (blocked)  // as many blocks as a blocked level can have
+          L.tab = (unsigned int*)idle(
+              sizeof(unsigned int) * MG_BLK_THREADS *
+              std::min(blocks, (size_t)MG_BLK_PER_CTA * (size_t)h->pcg_blocks));
         if (l > 0) {
           L.t = cv.take<uint8_t>(n);
           L.bflag = cv.take<uint8_t>((size_t)L.nbx * L.nby * L.nbz);
           L.nblk = cv.take<unsigned int>(1);
-          L.x2 = cv.take<float>(ns);
+          if (blocked) L.x2 = (float*)idle(sizeof(float) * ns);
         }
         if (l == 0) {
           m.pa0 = cv.take<float>(ns);
@@ -442,9 +456,6 @@ void carve(flip_handle* h, Carver& cv) {
   h->dstats = cv.take<DevStats>(1);
   h->norms = cv.take<double>(2);
   h->diag = cv.take<double>(4 * (size_t)energy_blocks(h->sm_count) + 4);
-  const size_t nfmax = (size_t)std::max(h->nf[0], std::max(h->nf[1], h->nf[2]));
-  h->tmp_bytes = std::max(nfmax * sizeof(float), nc * sizeof(double));
-  h->tmp = cv.take<char>(h->tmp_bytes);
 }
 
 int upload(void* dst, const void* src, size_t bytes, int src_dev, cudaStream_t s) {

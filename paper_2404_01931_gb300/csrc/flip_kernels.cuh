@@ -108,6 +108,8 @@ constexpr int MG_BLK_PER_CTA = 6;     // a level with at most this many blocks h
                                       // fluid per CTA is smoothed blocked (block_pass),
 constexpr int MG_BLK_PER_CTA_TEAM = 4;  // the same for teams of fewer than
 constexpr int MG_WIDE_TEAM = 128;       // MG_WIDE_TEAM CTAs
+constexpr int MG_BLK_MAX_NU = 2;      // ... with at most this many smoothing pairs, since
+constexpr int MG_BLK_THREADS = 1024;  // the halo of its tile (a thread each) is 4 cells
 constexpr float MG_OMEGA = 2.0f;      // over-correction of the coarse correction
 
 // One level of the hierarchy.  The grid-wide levels (l < lgrid) are stored
@@ -147,7 +149,8 @@ struct MgLevel {
                       // brick fluid counts of the binning)
   int* blk;           // the blocks holding fluid (bx | by << 8 | bz << 16), for the
                       // blocked smoothing
-  uint2* tab;         // per block and thread of its tile: the codes of its four cells
+  unsigned int* tab;  // per block and thread of its tile: what a pass needs of the codes of
+                      // its four cells (blk_pack); in memory that is idle during a solve
   unsigned int* nblk; // levels >= 1: their number (level 0: the binning's active bricks)
   float* x2;          // levels >= 1: the level's x after blocked post-smoothing
 };

@@ -833,9 +833,9 @@ __device__ __forceinline__ bool gwait(const PcgArgs& A) {
 constexpr int TILE_H = 4;
 constexpr int TILE_W = 8 + 2 * TILE_H;
 constexpr int TILE_PLANE = TILE_W * 8;        // threads (and slots of a colour) per plane
-// The halo is deep enough for two smoothing pairs.
-constexpr int BLK_MAX_NU = TILE_H / 2;
-static_assert(TILE_PLANE * TILE_W / 2 == PCG_THREADS, "a thread per slot and two planes");
+static_assert(MG_BLK_MAX_NU == TILE_H / 2, "the halo's depth");
+static_assert(TILE_PLANE * TILE_W / 2 == PCG_THREADS && PCG_THREADS == MG_BLK_THREADS,
+              "a thread per slot and two planes");
 
 struct MgTile {
   float2 x[2][PCG_THREADS];  // by colour
@@ -881,10 +881,26 @@ __device__ __forceinline__ BlkPos blk_pos(const SV& v, const TilePos& p, int e) 
   return q;
 }
 
-// Code of plane z (0 or 1 of the thread's two), colour c.
-__device__ __forceinline__ unsigned int tab_code(uint2 w, int z, int c) {
-  const unsigned int v = z == 0 ? w.x : w.y;
-  return c ? v >> 16 : v & 0xffffu;
+// A thread's four codes in a word: the counts of the red cells and of the black ones (a digit
+// each, plane 0 first; 0 where there is no fluid cell), and the red cells' fluid neighbours (a
+// byte each), which the residual needs.  At 8 bytes a thread (the codes themselves) the
+// tables took twice the memory; a pass is no slower.
+__device__ __forceinline__ unsigned int blk_pack(const unsigned int (&red)[2],
+                                                 const unsigned int (&black)[2]) {
+  unsigned int w = 0u;
+#pragma unroll
+  for (int z = 0; z < 2; ++z)
+    w |= (red[z] >> 8 & 7u) << (4 * z) | (black[z] >> 8 & 7u) << (8 + 4 * z) |
+         (red[z] & 63u) << (16 + 8 * z);
+  return w;
+}
+
+// Count of plane z (0 or 1 of the thread's two), colour c; fluid neighbours of a red cell.
+__device__ __forceinline__ int blk_cnt(unsigned int w, int z, int c) {
+  return (int)(w >> (8 * c + 4 * z)) & 7;
+}
+__device__ __forceinline__ unsigned int blk_nbr(unsigned int w, int z) {
+  return w >> (16 + 8 * z);
 }
 
 __device__ __forceinline__ float& plane(float2& a, int z) { return z == 0 ? a.x : a.y; }
@@ -939,7 +955,7 @@ __device__ __noinline__ PassSum block_pass(const PcgArgs& A, int l, bool wait) {
   FF acc;
   int q = (int)team_rank();
   int e = 0;
-  uint2 w = make_uint2(0u, 0u);
+  unsigned int w = 0u;
   float2 r[2];  // the right-hand side
   float2 x0;    // POST: the red cells' x
   auto load = [&](const BlkPos& bp) {
@@ -947,11 +963,11 @@ __device__ __noinline__ PassSum block_pass(const PcgArgs& A, int l, bool wait) {
     for (int c = 0; c < 2; ++c)
 #pragma unroll
       for (int z = 0; z < 2; ++z)
-        plane(r[c], z) = tab_code(w, z, c) ? v.b[c * v.half + bp.gi + z * v.pl] : 0.0f;
+        plane(r[c], z) = blk_cnt(w, z, c) ? v.b[c * v.half + bp.gi + z * v.pl] : 0.0f;
     if constexpr (POST) {
 #pragma unroll
       for (int z = 0; z < 2; ++z)
-        plane(x0, z) = tab_code(w, z, 0) ? v.x[bp.gi + z * v.pl] : 0.0f;
+        plane(x0, z) = blk_cnt(w, z, 0) ? v.x[bp.gi + z * v.pl] : 0.0f;
     }
   };
   if (q < n) {
@@ -967,16 +983,16 @@ __device__ __noinline__ PassSum block_pass(const PcgArgs& A, int l, bool wait) {
     const int I = (bp.b0 >> 1) - TILE_H / 2 + p.s, J = (bp.b1 - TILE_H + p.y) >> 1,
               K = (bp.b2 - TILE_H + 2 * p.g) >> 1;  // the two red cells' parent
     if constexpr (POST) {
-      const float px = ((w.x | w.y) & 0xffffu) ? C.x[level_index(C, I, J, K)] : 0.0f;
+      const float px = (w & 0x77u) ? C.x[level_index(C, I, J, K)] : 0.0f;
 #pragma unroll
       for (int z = 0; z < 2; ++z)
-        plane(x[0], z) = tab_code(w, z, 0) ? __fmaf_rn(M.omega, px, plane(x0, z)) : 0.0f;
+        plane(x[0], z) = blk_cnt(w, z, 0) ? __fmaf_rn(M.omega, px, plane(x0, z)) : 0.0f;
     }
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
       for (int z = 0; z < 2; ++z) {
-        const int cnt = code_cnt(tab_code(w, z, c));  // 0 where there is no fluid cell
+        const int cnt = blk_cnt(w, z, c);  // 0 where there is no fluid cell
         plane(inv[c], z) = s_inv_cnt[cnt];
         plane(base[c], z) = __fmul_rn(plane(r[c], z), s_inv_scnt[l][cnt]);
       }
@@ -1002,7 +1018,7 @@ __device__ __noinline__ PassSum block_pass(const PcgArgs& A, int l, bool wait) {
       for (int c = 0; c < 2; ++c)
 #pragma unroll
         for (int z = 0; z < 2; ++z)
-          if (tab_code(w, z, c)) {
+          if (blk_cnt(w, z, c)) {
             xout[c * v.half + bp.gi + z * v.pl] = plane(x[c], z);
             if constexpr (RZ) acc.add_prod(plane(r[c], z), plane(x[c], z));
           }
@@ -1019,9 +1035,9 @@ __device__ __noinline__ PassSum block_pass(const PcgArgs& A, int l, bool wait) {
                               x[1].y};
         const float xv1[6] = {low ? x[1].y : other.y, low ? other.y : x[1].y, ym.y, yp.y, x[1].x,
                               znext};
-        const unsigned int c0 = tab_code(w, 0, 0), c1 = tab_code(w, 1, 0);
-        float r0 = resid(v.s, code_cnt(c0), c0, r[0].x, x[0].x, xv0);
-        float r1 = resid(v.s, code_cnt(c1), c1, r[0].y, x[0].y, xv1);
+        const int c0 = blk_cnt(w, 0, 0), c1 = blk_cnt(w, 1, 0);
+        float r0 = resid(v.s, c0, blk_nbr(w, 0), r[0].x, x[0].x, xv0);
+        float r1 = resid(v.s, c1, blk_nbr(w, 1), r[0].y, x[0].y, xv1);
         r0 = c0 ? r0 : 0.0f;
         r1 = c1 ? r1 : 0.0f;
         // b of the coarse cell: restrict_sum's sum over the red children in order, the
@@ -2042,7 +2058,7 @@ __device__ __forceinline__ bool seg_active(const PcgArgs& A, const MgLevel& L, i
 // to 27 CTAs) at 2, 3, 4 and 6 blocks per CTA 3.37, 3.33, 3.34, 3.45 ms per step.
 __device__ __forceinline__ bool blocked(const MgArgs& M, unsigned int n) {
   const int most = team_size() < (unsigned)MG_WIDE_TEAM ? MG_BLK_PER_CTA_TEAM : MG_BLK_PER_CTA;
-  return M.nlev > 1 && M.nu <= BLK_MAX_NU && n > 0u && n <= (unsigned)most * team_size();
+  return M.nlev > 1 && M.nu <= MG_BLK_MAX_NU && n > 0u && n <= (unsigned)most * team_size();
 }
 
 // The grid-wide levels' lists of blocks holding fluid.  Level 0's follows the
@@ -2093,7 +2109,7 @@ __device__ __noinline__ void block_tables(const PcgArgs& A) {
         any = l == 0 ? A.brick_fluid[b] > 0u : L.bflag[b] != 0;
       }
       const int j = bp.b1 - TILE_H + p.y;
-      unsigned int cd[2] = {0u, 0u};
+      unsigned int red[2] = {0u, 0u}, black[2] = {0u, 0u};
       if (any && j < v.ny) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -2104,12 +2120,12 @@ __device__ __noinline__ void block_tables(const PcgArgs& A) {
             const int tx = 2 * p.s + ((c + p.y + u) & 1), i = bp.b0 - TILE_H + tx;
             if (k < nz && i < v.nx && tile_dist(tx) + dyz <= TILE_H) {
               const unsigned int code = v.code[c * v.half + bp.gi + u * v.pl];
-              if (code & CODE_SELF) cd[u] |= code << (16 * c);
+              if (code & CODE_SELF) (c ? black : red)[u] = code;
             }
           }
         }
       }
-      L.tab[(size_t)q * PCG_THREADS + threadIdx.x] = make_uint2(cd[0], cd[1]);
+      L.tab[(size_t)q * PCG_THREADS + threadIdx.x] = blk_pack(red, black);
     }
   }
 }

@@ -62,3 +62,16 @@ def check_one_iteration(sc, n, nu):
                          max_iter=1, nu=nu)
     e = rel_l2(got["p"], ref)
     assert e <= 1e-5, f"pressure after one MG-PCG iteration: rel L2 {e:.3e}"
+
+
+@pytest.mark.parametrize("n", [32, 48, 64, 96, 128])
+@pytest.mark.parametrize("nu", [2, 3])
+def test_solver_memory_per_cell(n, nu):
+    """What a multigrid scene takes beyond a Jacobi one: 26 bytes a slot of level 0 (six FP32
+    vectors and the codes), the coarser levels' 11 (a seventh of it), margins, less Jacobi's
+    16; not the blocked smoothing's tables, which lie in memory that is idle in a solve."""
+    fp = matched(n)[1]
+    fp.mg_smooth = nu
+    mg = F.flip_footprint_bytes(fp, n ** 3)
+    fp.preconditioner = F.FLIP_PRECOND_JACOBI
+    assert 0 < mg - F.flip_footprint_bytes(fp, n ** 3) <= 16 * n ** 3
