@@ -2495,8 +2495,12 @@ __device__ __noinline__ bool build_levels(const PcgArgs& A, Shared& sh, unsigned
 constexpr size_t MG_DYN_CTA = (sizeof(CtaMg) + 15) / 16 * 16;
 constexpr size_t MG_DYN_TILE = MG_DYN_CTA + sizeof(unsigned int) * SEG_CACHE;
 constexpr size_t MG_DYN_BYTES = MG_DYN_TILE + sizeof(MgTile);
-// one carve-out step up (132 KB) would take L1 from the level-0 passes
-static_assert(MG_DYN_BYTES + 4096 <= 100 * 1024, "the kernel stays in the 100 KB carve-out");
+// one carve-out step up (132 KB) would take L1 from the level-0 passes; beside the dynamic
+// memory lie the arguments and the sums (3.4 KB), the level tables, slices and the set-up's
+// scratch (3 KB; the kernel's own variables are 6432 bytes in all), and 1 KB of every CTA's
+constexpr size_t MG_STATIC_BYTES = sizeof(PcgArgs) + sizeof(Shared) + 4096;
+static_assert(MG_DYN_BYTES + MG_STATIC_BYTES + 1024 <= 100 * 1024,
+              "the kernel stays in the 100 KB carve-out");
 
 __device__ __forceinline__ unsigned int* seg_cache_of(unsigned char* dyn) {
   return reinterpret_cast<unsigned int*>(dyn + MG_DYN_CTA);
