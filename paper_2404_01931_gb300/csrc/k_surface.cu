@@ -193,7 +193,7 @@ bool build_table(McTable& T) {
 }
 
 // The table is generated once per process and uploaded to each device that
-// creates a surface object (constant memory is per device).
+// creates a surface object (a device variable has a copy on each).
 std::mutex g_table_mutex;
 bool g_table_built = false, g_table_ok = false;
 McTable g_table;
@@ -410,7 +410,7 @@ __global__ void k_sbin_scatter(const PartView p, long long np, const int* __rest
   pos[start[b] + prank[i]] = make_float4(p.x[i], p.y[i], p.z[i], 0.0f);
 }
 
-// One warp per group of 2 PX x GY x GZ corners (sdf_kernel has the lines between them).  With
+// One warp per group of 2 PX x GY x GZ corners (sdf_launch has the lines between them).  With
 // bins of edge R/2 the balls' extent along y or z is at most 5.98 bins, which meets at most 7
 // (8 with roundings), so at most 64 bin rows (fixed y, z bin): lane r finds the particle
 // ranges of rows r and r + 32 (a row's bins within the balls' x extent are one contiguous
@@ -630,29 +630,38 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
 // 617, 762, 1293; with 2 x 1 x 1 from R < 2 h on 1063, 823, 802 and 835, 999, 1515; with
 // lanes that walk one flat range over the rows of 4 corners along x 962, 699, 653 and 701,
 // 871, 1488.
-// A grid of few groups takes 2 x 2 x 1 ones, twice as many, to even out the chip's last
+// A grid of few groups (of less than four rounds of resident warps: 14592 on 152 SMs) takes
+// 2 x 2 x 1 ones, twice as many, to even out the chip's last
 // rounds: flip_surface_sdf with 7 thousand groups (48 x 33 x 33 cells, 4 scenes) 58-69 us
 // with 2 x 2 x 2, 59-66 with 2 x 2 x 1; with 11 thousand 63-81 and 64-72; with 26 thousand
 // 72-103 and 77-109; with 30 thousand 75-112 and 87-135.
 using SdfKernel = void (*)(const SGrid, const SBins, const unsigned int*, const float4*, float*);
 
-constexpr long long SDF_FEW = 4 * 152 * 3 * SDF_WARPS;  // four rounds of resident warps
+struct SdfLaunch {
+  SdfKernel kernel = nullptr;
+  int ctas = 0;
+};
 
-SdfKernel sdf_kernel(const SGrid& g, const SBins& B) {
-  if (g.h > 1.98f * B.b) return k_sdf<2, 1, 1>;
-  const long long groups = (long long)((g.c[0] + 1) / 2) * ((g.c[1] + 1) / 2) * ((g.c[2] + 1) / 2);
-  return groups >= SDF_FEW ? k_sdf<1, 2, 2> : k_sdf<1, 2, 1>;
-}
-
-int sdf_blocks(SdfKernel k) {
+// Once per surface object, on its device.
+cudaError_t sdf_launch(const SGrid& g, const SBins& B, SdfLaunch* out) {
   int dev = 0, sms = 0, per = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, SDF_THREADS, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return 152 * 8;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const auto resident = [&](SdfKernel k) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, SDF_THREADS, 0);
+  };
+  SdfKernel k = k_sdf<2, 1, 1>;
+  if (g.h <= 1.98f * B.b) {
+    k = k_sdf<1, 2, 2>;
+    if (e == cudaSuccess) e = resident(k);
+    const long long groups =
+        (long long)((g.c[0] + 1) / 2) * ((g.c[1] + 1) / 2) * ((g.c[2] + 1) / 2);
+    if (groups < 4ll * sms * per * SDF_WARPS) k = k_sdf<1, 2, 1>;  // four rounds of warps
   }
-  return std::max(1, sms * std::max(per, 1));
+  if (e == cudaSuccess) e = resident(k);
+  out->kernel = k;
+  out->ctas = std::max(1, sms * std::max(per, 1));
+  return e;
 }
 
 // ------------------------------------------------------------------ marching cubes
@@ -975,6 +984,7 @@ struct flip_surface {
   flip_surface_params prm{};
   SGrid g{};
   SBins B{};
+  SdfLaunch sdf;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   float* phi = nullptr;
@@ -1100,6 +1110,7 @@ int flip_surface_create(const flip_surface_params* sp, void* stream, flip_surfac
     step(cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking), "cudaStreamCreate");
     s->own_stream = rc == FLIP_OK;
   }
+  step(sdf_launch(g, B, &s->sdf), "scalar field launch shape");
   const long long nc = g.ncorners;
   step(cudaMalloc(&s->phi, sizeof(float) * nc), "cudaMalloc(phi)");
   step(cudaMalloc(&s->voff, sizeof(unsigned int) * nc), "cudaMalloc(voff)");
@@ -1181,8 +1192,7 @@ int flip_surface_sdf(flip_surface* s, flip_handle* h) {
     k_sbin_scatter<<<blocks_for(np, 256), 256, 0, st>>>(P, np, s->pbin, s->prank, s->bin_start,
                                                         s->pos);
   }
-  const SdfKernel sdf = sdf_kernel(s->g, s->B);
-  sdf<<<sdf_blocks(sdf), SDF_THREADS, 0, st>>>(s->g, s->B, s->bin_start, s->pos, s->phi);
+  s->sdf.kernel<<<s->sdf.ctas, SDF_THREADS, 0, st>>>(s->g, s->B, s->bin_start, s->pos, s->phi);
   SURF_CUDA(cudaGetLastError());
   return FLIP_OK;
 }
