@@ -184,3 +184,41 @@ def test_steps_after_a_timed_out_one_stay_inside_the_particle_arrays(limit):
         assert rel_l2(sim.read(F.PRESSURE_F64), ref.pressure) <= 1e-5
         got = np.stack(sim.particles()[:3]).astype(np.float64)
         assert np.abs(got - np.stack([ref.x, ref.y, ref.z])).max() * n <= 1e-4
+
+
+@pytest.mark.parametrize("n,hi", [((45, 41, 43), (1.0, 0.85, 1.0)), ((70, 9, 33), (0.4, 1.0, 0.5))])
+def test_p2g_face_by_face_weighted_by_the_sum_of_weights(n, hi):
+    """Every face, with the bound that its sum of weights allows (a face that only vanishing
+    weights reach has none of its own): x/dx and x/dx - 1/2 are rounded to within 2^-23 m cells
+    (m the longest extent), so each of a face's k particles' weights, products of three, moves
+    by at most 3 of that, and the numerator by (k + 4) roundings of its terms; a velocity is
+    at most V from the face's mean of them times 2."""
+    sc = S.random_velocities(S.box(n, (0.0, 0.0, 0.0), hi, seed=4), 0.5, 6)
+    op, fp = matched(n)
+    with F.Simulation(fp, *sc.arrays()) as sim:
+        sim.step(1)
+        uo = [np.asarray(sim.read(f), np.float64) for f in (F.U_OLD, F.V_OLD, F.W_OLD)]
+    m, V = max(n), 0.5
+    pos = [a.astype(np.float64) * m for a in sc.arrays()[:3]]
+    for d in range(3):
+        dim = [n[a] + (a == d) for a in range(3)]
+        base, frac = [], []
+        for a in range(3):
+            g = np.clip(pos[a] - (0.0 if a == d else 0.5), 0.0, dim[a] - 1.0)
+            b = np.minimum(np.floor(g), dim[a] - 2).astype(np.int64)
+            base.append(b)
+            frac.append(g - b)
+        num, den, cnt = (np.zeros(dim[0] * dim[1] * dim[2]) for _ in range(3))
+        vel = sc.arrays()[3 + d].astype(np.float64)
+        for q in range(8):
+            o = [(q >> a) & 1 for a in range(3)]
+            w = np.prod([frac[a] if o[a] else 1 - frac[a] for a in range(3)], axis=0)
+            i = (base[0] + o[0]) + dim[0] * ((base[1] + o[1]) + dim[1] * (base[2] + o[2]))
+            np.add.at(num, i, w * vel)
+            np.add.at(den, i, w)
+            np.add.at(cnt, i, 1.0)
+        far = den > 1e-30  # (below, FP32 weights may be 0)
+        err = np.abs(uo[d][far] - num[far] / den[far])
+        bound = 2 * V * (3 * cnt[far] * 2.0 ** -23 * m / den[far] + (cnt[far] + 4) * 2.0 ** -24)
+        assert (err <= np.minimum(bound, 2 * V)).all(), d
+        assert not uo[d][cnt == 0].any(), d
