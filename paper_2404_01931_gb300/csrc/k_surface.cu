@@ -21,7 +21,7 @@
 //   k_mc_normals    the weights gathered per vertex from the four cubes around its edge in a
 //                   fixed order (deterministic sums)
 // A call of 4.2 M corners and 53 thousand vertices, with its field set and its results read,
-// 257 -> 176 us.
+// 258 -> 180 us (174 to 185 from run to run).
 #include <cuda_runtime.h>
 
 #include <algorithm>
