@@ -435,13 +435,20 @@ constexpr int SDF_THREADS = 256;
 constexpr int SDF_WARPS = SDF_THREADS / 32;
 constexpr int SDF_ROW_LANES = 8;
 constexpr int SDF_ROWS = 64;
+// On a grid of few groups the lanes of a warp share every row from this many particles a row
+// on, instead of a row per eight lanes.  Such a grid's balls can meet few rows of up to
+// thousands of particles each: 2^3 cells over 32 thousand particles, R = 4 h, 1010 -> 345 us,
+// 10^3 cells, R = 4, 6 and 8 h, 252, 366 and 508 -> 189, 241 and 260 (with lanes that walk one
+// flat range over the rows of 4 corners along x 401, 186, 281 and 353).  From 32 on, rows that
+// do not fill the lanes cost more (64^3 cells, R = 2 h, 132 -> 162 us).
+constexpr unsigned int SDF_LONG = 64;
 // A corner whose sum of weights is below this is summed again with the ball's edge taken
 // exactly.  A particle at distance R or more has a rounded 1 - d^2 / R^2 of up to 2^-23, a
 // weight of 2^-69: nothing beside this sum, but all there is at a corner that no particle is
 // closer to than R.
 constexpr float SDF_THIN = 0x1p-30f;
 
-template <int PX, int GY, int GZ>
+template <int PX, int GY, int GZ, bool FEW>
 __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins B,
                                                      const unsigned int* __restrict__ start,
                                                      const float4* __restrict__ pos,
@@ -470,6 +477,7 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
     const int nyr = max(by1 - by0 + 1, 1);
     const int nrows = min(nyr * (bz1 - bz0 + 1), SDF_ROWS);
     int nrow = 0;
+    unsigned int npart = 0;
     __syncwarp();  // the last group's reads of the list are done
     for (int r0 = 0; r0 < nrows; r0 += 32) {
       const int r = r0 + lane;
@@ -494,8 +502,14 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
       const unsigned int some = __ballot_sync(0xffffffffu, p0 < p1);
       if (p0 < p1) s_row[wid][nrow + __popc(some & ((1u << lane) - 1u))] = make_uint2(p0, p1);
       nrow += __popc(some);
+      npart += p1 - p0;
     }
     __syncwarp();
+    // the rows a lane walks and its particles of each
+    int row0 = lane / SDF_ROW_LANES, rows = 32 / SDF_ROW_LANES;
+    unsigned int part0 = lane % SDF_ROW_LANES, parts = SDF_ROW_LANES;
+    if (FEW && __reduce_add_sync(0xffffffffu, npart) >= SDF_LONG * (unsigned int)nrow)
+      row0 = 0, rows = 1, part0 = (unsigned int)lane, parts = 32u;
     // minus the corners' coordinates (P.x + (-x) rounds as P.x - x); packed operations round
     // like the scalar ones
     float2 mx[PX];
@@ -509,14 +523,14 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
     float2 sk[NP], sx[NP], sy[NP], sz[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) sk[q] = sx[q] = sy[q] = sz[q] = make_float2(0.0f, 0.0f);
-    for (int r = lane / SDF_ROW_LANES; r < nrow; r += 32 / SDF_ROW_LANES) {
+    for (int r = row0; r < nrow; r += rows) {
       const uint2 row = s_row[wid][r];
-      unsigned int f = row.x + lane % SDF_ROW_LANES;
+      unsigned int f = row.x + part0;
       float4 next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       if (f < row.y) next = pos[f];
-      for (; f < row.y; f += SDF_ROW_LANES) {
+      for (; f < row.y; f += parts) {
         const float4 P = next;  // the next particle's load is in flight during this one's sums
-        if (f + SDF_ROW_LANES < row.y) next = pos[f + SDF_ROW_LANES];
+        if (f + parts < row.y) next = pos[f + parts];
         const float2 ey = __fadd2_rn(make_float2(P.y, P.y), my);
         const float2 ez = __fadd2_rn(make_float2(P.z, P.z), mz);
         const float2 fy = __fmul2_rn(ey, nr);
@@ -594,9 +608,9 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
       if (PX > 1 && c % GX >= 2) m = mx[PX - 1];
       const float cx = -(c & 1 ? m.y : m.x), cy = c / GX % GY ? y1 : y0, cz = c / (GX * GY) ? z1 : z0;
       float w = 0.0f, wx = 0.0f, wy = 0.0f, wz = 0.0f;
-      for (int r = lane / SDF_ROW_LANES; r < nrow; r += 32 / SDF_ROW_LANES) {
+      for (int r = row0; r < nrow; r += rows) {
         const uint2 row = s_row[wid][r];
-        for (unsigned int f = row.x + lane % SDF_ROW_LANES; f < row.y; f += SDF_ROW_LANES) {
+        for (unsigned int f = row.x + part0; f < row.y; f += parts) {
           const float4 P = pos[f];
           const float ex = P.x - cx, ey = P.y - cy, ez = P.z - cz;
           const float dd = __fmaf_rn(ex, ex, __fmaf_rn(ez, ez, __fmul_rn(ey, ey)));
@@ -631,10 +645,14 @@ __global__ void __launch_bounds__(SDF_THREADS) k_sdf(const SGrid g, const SBins 
 // lanes that walk one flat range over the rows of 4 corners along x 962, 699, 653 and 701,
 // 871, 1488.
 // A grid of few groups (of less than four rounds of resident warps: 14592 on 152 SMs) takes
-// 2 x 2 x 1 ones, twice as many, to even out the chip's last
-// rounds: flip_surface_sdf with 7 thousand groups (48 x 33 x 33 cells, 4 scenes) 58-69 us
-// with 2 x 2 x 2, 59-66 with 2 x 2 x 1; with 11 thousand 63-81 and 64-72; with 26 thousand
-// 72-103 and 77-109; with 30 thousand 75-112 and 87-135.
+// 2 x 2 x 1 ones, twice as many, to even out the chip's last rounds, and a CTA per tile, which
+// the device hands out as CTAs end: 40^3 cells (9261 groups), R = 2, 4 and 8 h, 79, 233 and
+// 1200 -> 70, 149 and 678 us; 32^3 (4913) 140, 640 and 3650 -> 129, 577 and 3020, and with
+// 2 x 2 x 2 corners 140, 659 and 3120.  With fewer groups than resident warps it takes pairs:
+// 32 x 25 x 16 cells (1989 groups), R = 1.2, 2, 4 and 8 h, 282, 667, 3319 and 13918 -> 241,
+// 611, 3152 and 13955 us, but 32^3 94, 129, 577 and 3020 -> 91, 130, 614 and 3550.  More groups
+// do not gain by a CTA per tile (256^3 cells 4.01 -> 4.41 ms), nor by the smaller ones (26
+// thousand 72-103 us with 2 x 2 x 2 corners, 77-109 with 2 x 2 x 1).
 using SdfKernel = void (*)(const SGrid, const SBins, const unsigned int*, const float4*, float*);
 
 struct SdfLaunch {
@@ -643,24 +661,22 @@ struct SdfLaunch {
 };
 
 // Once per surface object, on its device.
-cudaError_t sdf_launch(const SGrid& g, const SBins& B, SdfLaunch* out) {
-  int dev = 0, sms = 0, per = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const auto resident = [&](SdfKernel k) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, SDF_THREADS, 0);
-  };
-  SdfKernel k = k_sdf<2, 1, 1>;
-  if (g.h <= 1.98f * B.b) {
-    k = k_sdf<1, 2, 2>;
-    if (e == cudaSuccess) e = resident(k);
-    const long long groups =
-        (long long)((g.c[0] + 1) / 2) * ((g.c[1] + 1) / 2) * ((g.c[2] + 1) / 2);
-    if (groups < 4ll * sms * per * SDF_WARPS) k = k_sdf<1, 2, 1>;  // four rounds of warps
+cudaError_t sdf_launch(const SGrid& g, const SBins& B, int sms, SdfLaunch* out) {
+  int per = 0;
+  const bool wide = g.h > 1.98f * B.b;
+  SdfKernel k = wide ? k_sdf<2, 1, 1, false> : k_sdf<1, 2, 2, false>;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, SDF_THREADS, 0);
+  const long long held = (long long)sms * std::max(per, 1);  // CTAs
+  const auto over = [&](int a, int n) { return (long long)((g.c[a] + n - 1) / n); };
+  const long long groups =
+      wide ? over(0, 4) * g.c[1] * g.c[2] : over(0, 2) * over(1, 2) * over(2, 2);
+  out->ctas = (int)held;
+  if (groups < 4 * SDF_WARPS * held) {  // four rounds of warps
+    const bool pairs = !wide && groups < SDF_WARPS * held;
+    k = wide ? k_sdf<2, 1, 1, true> : pairs ? k_sdf<1, 1, 1, true> : k_sdf<1, 2, 1, true>;
+    out->ctas = (int)(over(0, wide ? 8 : 4) * over(1, wide || pairs ? 2 : 4) * over(2, 2));
   }
-  if (e == cudaSuccess) e = resident(k);
   out->kernel = k;
-  out->ctas = std::max(1, sms * std::max(per, 1));
   return e;
 }
 
@@ -985,6 +1001,7 @@ struct flip_surface {
   SGrid g{};
   SBins B{};
   SdfLaunch sdf;
+  int sms = 0;  // of its device
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   float* phi = nullptr;
@@ -1110,7 +1127,10 @@ int flip_surface_create(const flip_surface_params* sp, void* stream, flip_surfac
     step(cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking), "cudaStreamCreate");
     s->own_stream = rc == FLIP_OK;
   }
-  step(sdf_launch(g, B, &s->sdf), "scalar field launch shape");
+  int dev = 0;
+  step(cudaGetDevice(&dev), "cudaGetDevice");
+  step(cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+  step(sdf_launch(g, B, s->sms, &s->sdf), "scalar field launch shape");
   const long long nc = g.ncorners;
   step(cudaMalloc(&s->phi, sizeof(float) * nc), "cudaMalloc(phi)");
   step(cudaMalloc(&s->voff, sizeof(unsigned int) * nc), "cudaMalloc(voff)");

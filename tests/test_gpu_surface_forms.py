@@ -99,7 +99,20 @@ def test_sdf_of_many_corners_matches_the_oracle_at_other_radii(n, h, ratio):
     check_sdf(n, h, ratio)
 
 
-def check_sdf(n, h, ratio):
+@pytest.mark.parametrize("n,h,ratio", [
+    ((20, 14, 16), 1 / 8, 8.0),      # balls that meet a few rows of a thousand particles
+    ((12, 9, 10), 1 / 8, 4.0),
+    ((10, 11, 9), 1 / 9, 2.0),       # rows longer and shorter than the line
+    ((21, 20, 19), 1 / 18, 2.0),
+    ((11, 12, 9), 1 / 8, 0.9),       # four corners along x
+])
+def test_sdf_of_grids_coarse_against_the_particles(n, h, ratio):
+    """Each lane adds up to 7 thousand / 32 terms before the tree, within the bar; corners
+    beyond it are held to their conditioning, however many of so few there are."""
+    check_sdf(n, h, ratio, most=1.0)
+
+
+def check_sdf(n, h, ratio, most=1e-4):
     """The bar of the tests above, and beyond it what the roundings of t = 1 - d^2 / R^2 can
     change at a corner: phi + r = |sum k e| / sum k, k = t^3, moves by at most
     2 R sum dk / sum k (|e - mean| <= 2 R), dk = (t + eps)^3 - t^3.  eps: five roundings to
@@ -121,7 +134,7 @@ def check_sdf(n, h, ratio):
     assert phi.min() >= -sp.radius * (1 + 1e-6) and phi.max() <= (R - sp.radius) * (1 + 1e-6)
     err = np.abs(phi - ref)
     far = np.argwhere(err > 2e-5 * R)
-    assert len(far) <= 1e-4 * err.size
+    assert len(far) <= most * err.size
     eps = 2.0 ** -22 + 2 * 2.0 ** -23 * (0.02 + max(n) * h) / R
     p = np.stack([sc.x, sc.y, sc.z]).astype(np.float64)
     for k, j, i in far:
