@@ -802,14 +802,16 @@ __global__ void __launch_bounds__(SC_THREADS) k_mc_vertices(const SGrid g,
                                                             unsigned int* __restrict__ voff,
                                                             unsigned int* __restrict__ toff,
                                                             float* __restrict__ vert,
-                                                            long long* __restrict__ vedge) {
+                                                            long long* __restrict__ vedge,
+                                                            unsigned int parts) {
   static_assert(SC_ROWS == 8, "eight corners a thread");
   __shared__ u64 sm[72];
   __shared__ uint8_t s_ntri[256];
   __shared__ ushort4 s_item[SC_THREADS / 32][256];  // {corner, code, vertices, triangles before}
   load_ntri(s_ntri);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long base = (long long)blockIdx.x * SC_TILE;
+  const unsigned int tile = blockIdx.x / parts, part = blockIdx.x % parts;
+  const long long base = (long long)tile * SC_TILE;
   unsigned int cd[8];
   load_codes(code, base + 8 * threadIdx.x, g.ncorners, cd);
   u64 own = 0;
@@ -817,7 +819,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_mc_vertices(const SGrid g,
   for (int q = 0; q < 8; ++q)
     own += (u64)__popc(cd[q] & 7u) | ((u64)s_ntri[cd[q] >> 8] << 32);
   u64 tot;
-  const u64 off = tile_off[blockIdx.x], ex = block_excl_scan(own, tot, sm);
+  const u64 off = tile_off[tile], ex = block_excl_scan(own, tot, sm);
   // the tile's own counts (at most 3 and 12 a corner) fit 16 bits
   unsigned int nv = (unsigned int)(ex & 0xffffffffull), nt = (unsigned int)(ex >> 32);
   int n = 0;
@@ -837,7 +839,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_mc_vertices(const SGrid g,
   if (n == 0) return;
   const TileCorner tc(g, base);
   const long long st[3] = {1, g.c[0], (long long)g.c[0] * g.c[1]};
-  for (int m = lane; m < n; m += 32) {
+  for (int m = (int)part * 32 + lane; m < n; m += 32 * (int)parts) {
     const ushort4 it = s_item[warp][m];
     const long long c = base + it.x;
     unsigned int v = (unsigned int)(off & 0xffffffffull) + it.z;
@@ -900,12 +902,14 @@ __global__ void __launch_bounds__(SC_THREADS) k_mc_triangles(const SGrid g,
                                                              const uint16_t* __restrict__ code,
                                                              const float* __restrict__ vert,
                                                              int* __restrict__ tri,
-                                                             float* __restrict__ tw) {
+                                                             float* __restrict__ tw,
+                                                             unsigned int parts) {
   __shared__ uint16_t s_cube[SC_THREADS / 32][256];
   __shared__ uint8_t s_ntri[256];
   load_ntri(s_ntri);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long c0 = (long long)blockIdx.x * SC_TILE + 256 * warp;
+  const unsigned int tile = blockIdx.x / parts, part = blockIdx.x % parts;
+  const long long c0 = (long long)tile * SC_TILE + 256 * warp;
   unsigned int cd[8];
   load_codes(code, c0 + 8 * lane, g.ncorners, cd);
   int n = 0;
@@ -917,7 +921,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_mc_triangles(const SGrid g,
     n += __popc(some);
   }
   __syncwarp();
-  for (int m = lane >> 2; m < n; m += 8) {
+  for (int m = (int)part * 8 + (lane >> 2); m < n; m += 8 * (int)parts) {
     const long long c = c0 + s_cube[warp][m];
     const int cs = code[c] >> 8;
     const unsigned int t0 = toff[c];
@@ -986,6 +990,18 @@ __global__ void k_mc_normals(const SGrid g, long long nv,
   nrm[3 * v] = s[0] * f;
   nrm[3 * v + 1] = s[1] * f;
   nrm[3 * v + 2] = s[2] * f;
+}
+
+// CTAs per tile in the passes over lists, each with its part of every warp's list: few tiles
+// leave most of the chip idle while a warp has a list of up to 256 corners.  Up to eight CTAs
+// per SM in all: flip_surface_mesh of random fields on 32^3 cells (18 tiles, every corner
+// crosses) 112 -> 71 us, on 16^3 105 -> 67, of a field with a surface around single particles
+// on 150 x 40 x 90 (275 tiles) 99 -> 78 (two per SM 99, four 82, sixteen 79); with a thread
+// per corner 105, 96 and 93.
+unsigned int mc_parts(long long ntiles, int sms) {
+  unsigned int parts = 1;
+  while (parts < 8u && 2 * parts * ntiles <= 8ll * sms) parts *= 2;
+  return parts;
 }
 
 unsigned int blocks_for(long long n, int threads) {
@@ -1260,11 +1276,12 @@ int flip_surface_mesh(flip_surface* s, int64_t* n_vertices, int64_t* n_triangles
     s->tcap = nt;
   }
   if (nv > 0) {  // (a triangle has vertices)
-    k_mc_vertices<<<(unsigned)ntiles, SC_THREADS, 0, st>>>(s->g, s->phi, s->code, s->tile,
-                                                           s->voff, s->toff, s->vert, s->vedge);
+    const unsigned int parts = mc_parts(ntiles, s->sms), ctas = (unsigned int)ntiles * parts;
+    k_mc_vertices<<<ctas, SC_THREADS, 0, st>>>(s->g, s->phi, s->code, s->tile, s->voff, s->toff,
+                                               s->vert, s->vedge, parts);
     if (nt > 0)
-      k_mc_triangles<<<(unsigned)ntiles, SC_THREADS, 0, st>>>(s->g, s->voff, s->toff, s->code,
-                                                              s->vert, s->tri, s->tw);
+      k_mc_triangles<<<ctas, SC_THREADS, 0, st>>>(s->g, s->voff, s->toff, s->code, s->vert,
+                                                  s->tri, s->tw, parts);
     k_mc_normals<<<blocks_for(4 * nv, 256), 256, 0, st>>>(s->g, nv, s->vedge, s->toff, s->code,
                                                           s->tri, s->tw, s->nrm);
   }

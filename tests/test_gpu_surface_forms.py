@@ -112,6 +112,19 @@ def test_sdf_of_grids_coarse_against_the_particles(n, h, ratio):
     check_sdf(n, h, ratio, most=1.0)
 
 
+@pytest.mark.parametrize("n", [(42, 41, 40), (74, 73, 75), (92, 91, 93), (110, 109, 111)])
+def test_mesh_passes_over_lists_shared_by_ctas(n):
+    """37, 206, 393 and 668 tiles: eight, four, two and one CTAs a tile on 152 SMs."""
+    phi = S.corner_field_random(n, 6)
+    sp = _sp(n, 0.2)
+    ref = O.marching_cubes(phi.astype(np.float64), tuple(sp.origin), sp.h, 0.0)
+    nv, nt, got = _gpu_mesh(sp, phi)
+    assert np.array_equal(got["e"], ref.vertex_edge) and np.array_equal(got["t"], ref.triangles)
+    # the bar of test_gpu_surface.py
+    scale = max(abs(o) for o in sp.origin) + sp.h * max(n)
+    assert np.abs(got["v"] - ref.vertices).max() <= 4e-7 * scale + 1e-6 * sp.h
+
+
 def check_sdf(n, h, ratio, most=1e-4):
     """The bar of the tests above, and beyond it what the roundings of t = 1 - d^2 / R^2 can
     change at a corner: phi + r = |sum k e| / sum k, k = t^3, moves by at most
